@@ -24,6 +24,7 @@
 
 #include "mixed.cuh"
 #include "ops.cuh"
+#include "sym.cuh"
 #include "tc_ptx.cuh"
 #include "vfmm_internal.cuh"
 
@@ -103,202 +104,6 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) c0[(size_t)b * R + r] = acc;
     }
-}
-
-// ---------------------------------------------------------------- FP64 gather GEMM tile
-// C_j[r] = scale_j * sum_s A[r][s] B_j[s] for rows r in [row0, row0 + 64), columns j < ncols.
-constexpr int GBM = 64, GBN = 64, GBK = 16;
-
-struct ColPtrs {
-    const double* b[GBN];
-    double* c[GBN];
-    double scale[GBN];
-};
-
-__device__ inline void gemm_tile_fp64(const double* __restrict__ A, int M, int K, int row0, int ncols,
-                                      const ColPtrs& cp) {
-    __shared__ double As[GBK][GBM + 1];
-    __shared__ double Bs[GBK][GBN + 1];
-    const int t = threadIdx.x;
-    const int tx = t % 16, ty = t / 16;
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    const int lr = t / 4, lk = (t % 4) * 4;  // loader: row/column lr, k offset lk
-    for (int k0 = 0; k0 < K; k0 += GBK) {
-        {
-            int r = row0 + lr;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                int kk = k0 + lk + q;
-                As[lk + q][lr] = (r < M && kk < K) ? A[(size_t)r * K + kk] : 0.0;
-            }
-            const double* bp = lr < ncols ? cp.b[lr] : nullptr;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                int kk = k0 + lk + q;
-                Bs[lk + q][lr] = (bp && kk < K) ? bp[kk] : 0.0;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GBK; ++kk) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        int c = tx * 4 + j;
-        if (c >= ncols) continue;
-        double* cptr = cp.c[c];
-        double sc = cp.scale[c];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            int r = row0 + ty * 4 + i;
-            if (r < M) cptr[r] = sc * acc[i][j];
-        }
-    }
-}
-
-// Near field: one tile = (configuration, range of its U entries). Every gather GEMM here takes
-// its column tile from blockIdx.x (no 65,535 limit) and its row tile from blockIdx.y.
-__global__ void __launch_bounds__(256) near_gemm_kernel(const int4* __restrict__ tiles, const double* __restrict__ T,
-                                                        int kk, const int32_t* __restrict__ u_by_cfg,
-                                                        const int32_t* __restrict__ lidxU,
-                                                        const int32_t* __restrict__ leaf_of_box,
-                                                        const double* __restrict__ f, double* __restrict__ slab) {
-    __shared__ ColPtrs cp;
-    const int4 tl = tiles[blockIdx.x];  // cfg, begin, end
-    const int ncols = min(GBN, tl.z - tl.y);
-    if (threadIdx.x < GBN) {
-        int j = threadIdx.x;
-        if (j < ncols) {
-            int e = u_by_cfg[tl.y + j];
-            cp.b[j] = f + (size_t)leaf_of_box[lidxU[e]] * kk;
-            cp.c[j] = slab + (size_t)e * 3 * kk;
-        } else {
-            cp.b[j] = nullptr;
-            cp.c[j] = nullptr;
-        }
-        cp.scale[j] = 1.0;
-    }
-    __syncthreads();
-    gemm_tile_fp64(T + (size_t)tl.x * 3 * kk * kk, 3 * kk, kk, blockIdx.y * GBM, ncols, cp);
-}
-
-// FP64 M2L over the V list: one tile = (offset, run of its V entries in offset order); column j =
-// entry e, slab row e = M2L_real[offset] . multipole of the entry's source box (all 2(p+1) rows).
-__global__ void __launch_bounds__(256) v_gemm_kernel(const int4* __restrict__ tiles, const double* __restrict__ A,
-                                                     int P2, const int32_t* __restrict__ by_cfg,
-                                                     const int32_t* __restrict__ lidxV, const double* __restrict__ Mexp,
-                                                     double* __restrict__ vslab) {
-    __shared__ ColPtrs cp;
-    const int4 tl = tiles[blockIdx.x];  // offset, begin, end
-    const int ncols = min(GBN, tl.z - tl.y);
-    if (threadIdx.x < GBN) {
-        const int j = threadIdx.x;
-        if (j < ncols) {
-            const int e = by_cfg[tl.y + j];
-            cp.b[j] = Mexp + (size_t)lidxV[e] * P2;
-            cp.c[j] = vslab + (size_t)e * P2;
-        } else {
-            cp.b[j] = nullptr;
-            cp.c[j] = nullptr;
-        }
-        cp.scale[j] = 1.0;
-    }
-    __syncthreads();
-    gemm_tile_fp64(A + (size_t)tl.x * P2 * P2, P2, P2, blockIdx.y * GBM, ncols, cp);
-}
-
-// FP64 S2L over the X list: column j = entry e (target box b, source leaf c), slab row e =
-// (2 h_b)^2 S2L_real[configuration] . f_c.
-__global__ void __launch_bounds__(256) x_gemm_kernel(const int4* __restrict__ tiles, const double* __restrict__ A,
-                                                     int P2, int kk, const int32_t* __restrict__ by_cfg,
-                                                     const int32_t* __restrict__ lidxX, const int32_t* __restrict__ x_tgt,
-                                                     const int32_t* __restrict__ level, double width,
-                                                     const int32_t* __restrict__ leaf_of_box,
-                                                     const double* __restrict__ f, double* __restrict__ xslab) {
-    __shared__ ColPtrs cp;
-    const int4 tl = tiles[blockIdx.x];
-    const int ncols = min(GBN, tl.z - tl.y);
-    if (threadIdx.x < GBN) {
-        const int j = threadIdx.x;
-        if (j < ncols) {
-            const int e = by_cfg[tl.y + j];
-            const double h = ldexp(width, -level[x_tgt[e]]);
-            cp.b[j] = f + (size_t)leaf_of_box[lidxX[e]] * kk;
-            cp.c[j] = xslab + (size_t)e * P2;
-            cp.scale[j] = 4.0 * h * h;
-        } else {
-            cp.b[j] = nullptr;
-            cp.c[j] = nullptr;
-            cp.scale[j] = 0.0;
-        }
-    }
-    __syncthreads();
-    gemm_tile_fp64(A + (size_t)tl.x * P2 * kk, P2, kk, blockIdx.y * GBM, ncols, cp);
-}
-
-// S2M: columns are leaves; output row = multipole of the leaf's box, scaled by h^2.
-__global__ void __launch_bounds__(256) s2m_gemm_kernel(const double* __restrict__ S2M, int P2, int kk, int nleaf,
-                                                       const int32_t* __restrict__ box_of_leaf,
-                                                       const int32_t* __restrict__ level, double width,
-                                                       const double* __restrict__ f, double* __restrict__ Mexp) {
-    __shared__ ColPtrs cp;
-    const int col0 = blockIdx.x * GBN;
-    const int ncols = min(GBN, nleaf - col0);
-    if (threadIdx.x < GBN) {
-        int j = threadIdx.x;
-        if (j < ncols) {
-            int leaf = col0 + j;
-            int b = box_of_leaf[leaf];
-            double h = ldexp(width, -level[b]);
-            cp.b[j] = f + (size_t)leaf * kk;
-            cp.c[j] = Mexp + (size_t)b * P2;
-            cp.scale[j] = h * h;
-        } else {
-            cp.b[j] = nullptr;
-            cp.c[j] = nullptr;
-            cp.scale[j] = 0.0;
-        }
-    }
-    __syncthreads();
-    gemm_tile_fp64(S2M, P2, kk, blockIdx.y * GBM, ncols, cp);
-}
-
-// L2T: columns are leaves; input = local expansion of the leaf's box.
-__global__ void __launch_bounds__(256) l2t_gemm_kernel(const double* __restrict__ L2T, int P2, int kk, int nleaf,
-                                                       const int32_t* __restrict__ box_of_leaf,
-                                                       const double* __restrict__ Lexp, double* __restrict__ far) {
-    __shared__ ColPtrs cp;
-    const int col0 = blockIdx.x * GBN;
-    const int ncols = min(GBN, nleaf - col0);
-    if (threadIdx.x < GBN) {
-        int j = threadIdx.x;
-        if (j < ncols) {
-            int leaf = col0 + j;
-            cp.b[j] = Lexp + (size_t)box_of_leaf[leaf] * P2;
-            cp.c[j] = far + (size_t)leaf * 3 * kk;
-        } else {
-            cp.b[j] = nullptr;
-            cp.c[j] = nullptr;
-        }
-        cp.scale[j] = 1.0;
-    }
-    __syncthreads();
-    gemm_tile_fp64(L2T, 3 * kk, P2, blockIdx.y * GBM, ncols, cp);
 }
 
 // Outputs j and P-1-j of one position of a triangular translation (mode 0, M2M: output o takes
@@ -569,8 +374,9 @@ struct DownArgs {
     const int* m2l_E;   // [Rx] row exponents of the M2L tables
     const unsigned* m2l_G;  // [(depth + 1) R] biased level exponents of the multipole operand
     const double* m2l_c0;  // Re of local coefficient 0 from the V and X lists, with the log(h) terms
-    const double* vslab;   // FP64 form: [n_V][2(p+1)] M2L of every V entry
-    const double* xslab;   // FP64 form: [n_X][2(p+1)] S2L of every X entry
+    const double* vslab;   // FP64 form: M2L of every V instance, [2(p+1)]
+    const double* xslab;   // FP64 form: S2L of every X instance, [2(p+1)]
+    const int32_t *viptr, *xiptr;  // instances of each box
     const double* pwloc;   // FP64 form, plane-wave M2L: [n_boxes][2(p+1)] V-list locals (null: vslab)
     int lw;                 // root width = wm 2^lw, wm in [1, 2)
     double wm;
@@ -590,61 +396,61 @@ __device__ __forceinline__ float2 m2l_value(const DownArgs& d, size_t vb, int q)
     return d.m2l_out[vb * d.Rx + q];
 }
 
-__global__ void __launch_bounds__(64) down_kernel(DownArgs d) {
-    const int R = d.R;
-    const int b = d.begin + blockIdx.x / R, r = blockIdx.x % R;
-    if (b >= d.end) return;
-    const size_t vb = (size_t)b * R + r;
-    const int P = d.P, t = threadIdx.x;
-    const double h = ldexp(d.width, -d.level);
-    const double logh = log(h);
-    double re = 0.0, im = 0.0;
-    if (d.level >= 3 && t < P) {
-        // L2L from the parent, written by translate_kernel just before this launch
-        re = d.Lexp[vb * 2 * P + 2 * t];
-        im = d.Lexp[vb * 2 * P + 2 * t + 1];
-    }
-    if (!d.m2l_out && t < P) {
-        // FP64 form: M2L and S2L rows from the per-entry slabs of the V and X GEMMs, in list order,
-        // with the log(h) a_0 terms of the scaling
-        if (d.pwloc) {
-            re += d.pwloc[(size_t)b * 2 * P + 2 * t];
-            im += d.pwloc[(size_t)b * 2 * P + 2 * t + 1];
-        }
-        for (int e = d.vptr[b]; e < d.vptr[b + 1]; ++e) {
-            if (!d.pwloc) {
-                re += d.vslab[(size_t)e * 2 * P + 2 * t];
-                im += d.vslab[(size_t)e * 2 * P + 2 * t + 1];
+// FP64 form: a box's own terms of local coefficients t = lane, lane + 32 (one warp per box): the V and X
+// instances' rows, in order, and the log(h) a_0 terms of the scaling.
+__device__ __forceinline__ void own_terms_fp64(const DownArgs& d, int level, int b, int lane, double2 own[2]) {
+    const int P = d.P;
+    const double h = ldexp(d.width, -level);
+    double a0 = 0.0;
+    for (int e = d.vptr[b] + lane; e < d.vptr[b + 1]; e += 32) a0 += d.Mexp[(size_t)d.vidx[e] * 2 * P];
+    for (int e = d.xptr[b] + lane; e < d.xptr[b + 1]; e += 32) a0 += d.Mexp[(size_t)d.xidx[e] * 2 * P];
+    for (int o = 16; o > 0; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int t = lane + 32 * i;
+        double re = 0.0, im = 0.0;
+        if (t < P) {
+            if (d.xiptr[b + 1] > d.xiptr[b]) {
+                for (int e = d.xiptr[b]; e < d.xiptr[b + 1]; ++e) {
+                    const double2 v = reinterpret_cast<const double2*>(d.xslab)[(size_t)e * P + t];
+                    re += v.x;
+                    im += v.y;
+                }
+                re *= 4.0 * h * h;
+                im *= 4.0 * h * h;
             }
-            if (t == 0) re += d.Mexp[((size_t)d.vidx[e] * R + r) * 2 * P] * logh;
+            if (d.pwloc) {
+                const double2 v = reinterpret_cast<const double2*>(d.pwloc)[(size_t)b * P + t];
+                re += v.x;
+                im += v.y;
+            } else {
+#pragma unroll 4
+                for (int e = d.viptr[b]; e < d.viptr[b + 1]; ++e) {
+                    const double2 v = reinterpret_cast<const double2*>(d.vslab)[(size_t)e * P + t];
+                    re += v.x;
+                    im += v.y;
+                }
+            }
         }
-        for (int e = d.xptr[b]; e < d.xptr[b + 1]; ++e) {
-            re += d.xslab[(size_t)e * 2 * P + 2 * t];
-            im += d.xslab[(size_t)e * 2 * P + 2 * t + 1];
-            if (t == 0) re += logh * d.Mexp[((size_t)d.xidx[e] * R + r) * 2 * P];
-        }
+        own[i] = make_double2(re, im);
     }
-    if (d.m2l_out && t >= 1 && t < P && d.xptr[b + 1] > d.xptr[b]) {
-        const float2 vr = d.s2l_out[vb * d.Rx + 2 * (t - 1)];
-        const float2 vi = d.s2l_out[vb * d.Rx + 2 * (t - 1) + 1];
-        const double sc = 4.0 * h * h * pow2(d.Ef[r]);
-        re += sc * ((double)vr.x + (double)vr.y) * pow2(d.s2l_E[2 * (t - 1)]);
-        im += sc * ((double)vi.x + (double)vi.y) * pow2(d.s2l_E[2 * (t - 1) + 1]);
-    }
-    if (d.m2l_out && t < P && (d.vptr[b + 1] > d.vptr[b] || d.xptr[b + 1] > d.xptr[b])) {
-        if (t == 0) {
-            re += d.m2l_c0[vb];
-        } else if (d.vptr[b + 1] > d.vptr[b]) {
-            const float2 vr = m2l_value(d, vb, 2 * (t - 1));
-            const float2 vi = m2l_value(d, vb, 2 * (t - 1) + 1);
-            const int g = level_exp_value(d.m2l_G[(size_t)d.level * R + r]);
-            re += ((double)vr.x + (double)vr.y) * pow2(g + d.m2l_E[2 * (t - 1)]);
-            im += ((double)vi.x + (double)vi.y) * pow2(g + d.m2l_E[2 * (t - 1) + 1]);
-        }
-    }
-    if (t < P) {
-        d.Lexp[vb * 2 * P + 2 * t] = re;
-        d.Lexp[vb * 2 * P + 2 * t + 1] = im;
+    if (lane == 0) own[0].x += log(h) * a0;
+}
+
+// FP64 form, one level (P <= 64): one warp per box adds its own terms to the L2L values that the
+// translation kernel has just written.
+__global__ void __launch_bounds__(128) down_kernel(DownArgs d) {
+    const int b = d.begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (b >= d.end) return;
+    double2 own[2];
+    own_terms_fp64(d, d.level, b, lane, own);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int t = lane + 32 * i;
+        if (t >= d.P) continue;
+        double2* L = reinterpret_cast<double2*>(d.Lexp) + (size_t)b * d.P + t;
+        const double2 p = d.level >= 3 ? *L : make_double2(0.0, 0.0);
+        *L = make_double2(p.x + own[i].x, p.y + own[i].y);
     }
 }
 
@@ -902,10 +708,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) upward_pass_kernel(PassArgs a
     }
 }
 
-// Mixed form, all downward levels. First every box of level >= 2 gets its own terms (the M2L and
-// S2L outputs and coefficient 0) in one warp unit per virtual box, counted 1 on its readiness word
+// All downward levels. First every box of level >= 2 gets its own terms (the M2L and S2L outputs and
+// coefficient 0) in one warp unit per virtual box, counted 1 on its readiness word
 // (level 2 boxes are then complete). Then, level by level, each non-leaf parent's local is shifted
 // to its 4 children (L2L) and added to their own terms, counted 1 more (complete at 2).
+template <bool kMixed>
 __global__ void __launch_bounds__(kPassThreads, 1) downward_pass_kernel(PassArgs a, DownArgs d) {
     extern __shared__ __align__(128) unsigned char pass_raw[];
     __shared__ int abort_grp[kPassGroups];
@@ -923,7 +730,14 @@ __global__ void __launch_bounds__(kPassThreads, 1) downward_pass_kernel(PassArgs
         const int64_t vb0 = (int64_t)a.level_start[2] * R, vb1 = (int64_t)a.level_start[a.depth + 1] * R;
         for (int64_t vb = vb0 + wslot; vb < vb1; vb += nw) {
             const int b = (int)(vb / R), r = (int)(vb % R), lv = a.level[b];
-            for (int t = lane; t < P; t += 32) a.ex[(size_t)vb * P + t] = combine_local(d, lv, b, r, t, 0.0, 0.0);
+            if constexpr (kMixed) {
+                for (int t = lane; t < P; t += 32) a.ex[(size_t)vb * P + t] = combine_local(d, lv, b, r, t, 0.0, 0.0);
+            } else {
+                double2 own[2];
+                own_terms_fp64(d, lv, b, lane, own);
+                if (lane < P) a.ex[(size_t)vb * P + lane] = own[0];
+                if (lane + 32 < P) a.ex[(size_t)vb * P + lane + 32] = own[1];
+            }
             __threadfence();
             __syncwarp();
             if (lane == 0) red_release_add_u32(a.ready + vb, 1u);
@@ -1108,100 +922,80 @@ __global__ void leaf_mixed_kernel(LeafMixedArgs a) {
 
 // ---------------------------------------------------------------- leaf pass (one CTA per leaf)
 struct LeafArgs {
+    SymOp op;  // rows of the classes
     int nleaf, kk, k, P;
     double width;
     const int32_t* box_of_leaf;
     const int32_t* level;
-    const int32_t *uptr, *uidx;
-    const int32_t *wptr, *widx, *wcfg;
-    const double* xhat;
-    const double* slab;
-    const double* far;
+    const int32_t *uptr, *uidx, *wptr, *widx;
+    const int32_t *uiptr, *wiptr;  // instances of each box
+    const double* slab;            // near field of every U instance, [3kk]
+    const double* wslab;           // M2T of every W instance, [3kk]
+    const double* far;             // L2T of every leaf, [3kk]
     const double* Mexp;
+    const double* Lexp;
     double* u;
     double* ux;
     double* uy;
 };
 
-// FP64 form: one CTA per leaf sums the near-field slab rows, the log(h) term, the far values
-// and the W-list multipoles (direct series) at its nodes.
-__global__ void __launch_bounds__(256) leaf_kernel(LeafArgs a) {
-    __shared__ double sa[2 * 64];
-    const int leaf = blockIdx.x;
-    const int t = threadIdx.x;
-    const int kk = a.kk, P = a.P;
-    const bool act = t < kk;
+// FP64 form: one CTA per leaf sums its instances' rows and the far values class by class, in order,
+// then each node puts its four classes together and adds the scalar log terms
+// -(1/2pi) (log(h) sum_U a_0 + log(h_w) sum_W a_0), h_w = h / 2 (first warp).
+__global__ void __launch_bounds__(256) leaf_kernel(const __grid_constant__ LeafArgs a) {
+    extern __shared__ double rows[];  // [3kk] class rows of u, u_x, u_y
+    __shared__ double s_scal;
+    const int leaf = blockIdx.x, t = threadIdx.x, kk = a.kk, k = a.k;
     const int b = a.box_of_leaf[leaf];
-    const double h = ldexp(a.width, -a.level[b]);
-    double u = 0.0, gx = 0.0, gy = 0.0, mass = 0.0;
-    for (int e = a.uptr[b]; e < a.uptr[b + 1]; ++e) {
-        if (act) {
-            const double* s = a.slab + (size_t)e * 3 * kk;
-            u += s[t];
-            gx += s[kk + t];
-            gy += s[2 * kk + t];
+    const double h = ldexp(a.width, -a.level[b]), ih = 1.0 / h;
+    for (int r = t; r < 3 * kk; r += blockDim.x) {
+        int s = 0;
+        while (r >= a.op.seg[s + 1]) ++s;
+        double n = 0.0, f = a.far[(size_t)leaf * 3 * kk + r];
+        for (int e = a.uiptr[b]; e < a.uiptr[b + 1]; ++e) n += a.slab[(size_t)e * 3 * kk + r];
+        for (int e = a.wiptr[b]; e < a.wiptr[b + 1]; ++e) f += a.wslab[(size_t)e * 3 * kk + r];
+        rows[r] = s % 3 == 0 ? fma(h * h, n, f) : fma(h, n, f * ih);
+    }
+    if (t < 32) {
+        const int P2 = 2 * a.P;
+        double m = 0.0, w0 = 0.0;
+        for (int e = a.uptr[b] + t; e < a.uptr[b + 1]; e += 32) m += a.Mexp[(size_t)a.uidx[e] * P2];
+        for (int e = a.wptr[b] + t; e < a.wptr[b + 1]; e += 32) w0 += a.Mexp[(size_t)a.widx[e] * P2];
+        for (int o = 16; o > 0; o >>= 1) {
+            m += __shfl_xor_sync(0xffffffffu, m, o);
+            w0 += __shfl_xor_sync(0xffffffffu, w0, o);
         }
-        mass += a.Mexp[(size_t)a.uidx[e] * 2 * P];
-    }
-    u = h * h * u - kInv2Pi * log(h) * mass;
-    gx *= h;
-    gy *= h;
-    const double hw = 0.5 * h;
-    if (act) {
-        const double* fr = a.far + (size_t)leaf * 3 * kk;
-        u += fr[t];
-        gx += fr[kk + t] / h;
-        gy += fr[2 * kk + t] / h;
-    }
-    const double xt = act ? a.xhat[t % a.k] : 0.0, yt = act ? a.xhat[t / a.k] : 0.0;
-    for (int e = a.wptr[b]; e < a.wptr[b + 1]; ++e) {
-        const int w = a.widx[e];
-        for (int q = t; q < 2 * P; q += blockDim.x) sa[q] = a.Mexp[(size_t)w * 2 * P + q];
-        __syncthreads();
-        if (act) {
-            int px, py;
-            far_pattern(a.wcfg[e], &px, &py);
-            // zeta = (z - z_w)/h_w = 2 (xhat - D), D = (px, py)/4
-            double zr = 2.0 * (xt - px / 4.0), zi = 2.0 * (yt - py / 4.0);
-            double r2 = zr * zr + zi * zi;
-            double vr = zr / r2, vi = -zi / r2;  // z^-1
-            // S = sum_{n>=1} a_n v^n and S' = sum n a_n v^n by Horner
-            double Sr = 0.0, Si = 0.0, Tr = 0.0, Ti = 0.0;
-            for (int n = P - 1; n >= 1; --n) {
-                double ar = sa[2 * n], ai = sa[2 * n + 1];
-                double nr = Sr + ar, ni = Si + ai;
-                Sr = nr * vr - ni * vi;
-                Si = nr * vi + ni * vr;
-                double mr = Tr + n * ar, mi = Ti + n * ai;
-                Tr = mr * vr - mi * vi;
-                Ti = mr * vi + mi * vr;
-            }
-            const double a0r = sa[0], a0i = sa[1];
-            const double lz = 0.5 * log(r2), th = atan2(zi, zr);
-            // Re Phi = Re(a0 (log h_w + log zeta)) + Re S
-            double phir = a0r * (log(hw) + lz) - a0i * th + Sr;
-            // dPhi/dzeta = v (a0 - S'), Phi' = dPhi/dzeta / h_w
-            double dr = a0r - Tr, di = a0i - Ti;
-            double pr = (vr * dr - vi * di) / hw, pi = (vr * di + vi * dr) / hw;
-            u += -kInv2Pi * phir;
-            gx += -kInv2Pi * pr;
-            gy += kInv2Pi * pi;
+        if (t == 0) {
+            const double logh = log(h);
+            s_scal = -kInv2Pi * (logh * m + (logh - 0.6931471805599453) * w0);
         }
-        __syncthreads();
     }
-    if (act) {
-        const size_t o = (size_t)leaf * kk + t;
-        a.u[o] = u;
-        a.ux[o] = gx;
-        a.uy[o] = gy;
-    }
+    __syncthreads();
+    if (t >= kk) return;
+    const int j = t / k, i = t - j * k;
+    const int i0 = min(i, k - 1 - i), j0 = min(j, k - 1 - j), s = (i > i0 ? 1 : 0) | (j > j0 ? 2 : 0);
+    double v[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int pa = sym_pa(c, q), pb = sym_pb(c, q), nx = sym_half(k, pa);
+            if (i0 >= nx || j0 >= sym_half(k, pb)) continue;  // an odd field's middle line
+            const double x = rows[a.op.seg[3 * c + q] + j0 * nx + i0];
+            v[q] += ((s & pa) ^ ((s >> 1) & pb)) & 1 ? -x : x;
+        }
+    const size_t o = (size_t)leaf * kk + t;
+    a.u[o] = v[0] + s_scal;
+    a.ux[o] = v[1];
+    a.uy[o] = v[2];
 }
 
 // ---------------------------------------------------------------- host side
 struct Workspace {
     bool fork = false;  // mixed form: run the near field and S2L on the thread's second stream
-    double* vslab;      // FP64 form: per V entry M2L rows
-    double* xslab;      // FP64 form: per X entry S2L rows
+    double* vslab;      // FP64 form: per V instance M2L rows
+    double* xslab;      // FP64 form: per X instance S2L rows
+    double* wslab;      // FP64 form: per W instance M2T rows
     double* pwX;        // FP64 form, plane-wave M2L: [n_boxes][4][s] outgoing coefficients (null: dense)
     double* pwL;        // FP64 form, plane-wave M2L: [n_boxes][2(p+1)] V-list local coefficients
     const PlanSet* ps;  // split-contraction plans for the folded right-hand sides (mixed form)
@@ -1253,17 +1047,25 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
             w->ready_words = words;
         }
     }
-    take(w ? &w->slab : &dummy, mixed ? 1 : (size_t)T.llen[VFMM_LIST_U] * 3 * kk);
-    take(w ? &w->far : &dummy, mixed ? 1 : (size_t)T.n_leaves * 3 * kk);
     const bool pw = !mixed && o.m2l_form == VFMM_M2L_PLANEWAVE;
-    take(w ? &w->vslab : &dummy, mixed || pw ? 1 : (size_t)T.llen[VFMM_LIST_V] * P2);
-    if (pw) {
-        take(w ? &w->pwX : &dummy, planewave_work_doubles(T.n_boxes, o));
-        take(w ? &w->pwL : &dummy, (size_t)T.n_boxes * P2);
-    } else if (w) {
-        w->pwX = w->pwL = nullptr;
+    if (w) w->slab = w->far = w->vslab = w->xslab = w->wslab = w->pwX = w->pwL = nullptr;
+    if (!mixed) {
+        take(w ? &w->slab : &dummy, (size_t)T.n_inst[VFMM_LIST_U] * 3 * kk);
+        // the M2L and S2L rows (or plane waves) are read before the leaf far field is written: one region
+        const size_t shared = off;
+        if (pw) {
+            take(w ? &w->pwX : &dummy, planewave_work_doubles(T.n_boxes, o));
+            take(w ? &w->pwL : &dummy, (size_t)T.n_boxes * P2);
+        } else {
+            take(w ? &w->vslab : &dummy, (size_t)T.n_inst[VFMM_LIST_V] * P2);
+        }
+        take(w ? &w->xslab : &dummy, (size_t)T.n_inst[VFMM_LIST_X] * P2);
+        const size_t down_end = off;
+        off = shared;
+        take(w ? &w->far : &dummy, (size_t)T.n_leaves * 3 * kk);
+        take(w ? &w->wslab : &dummy, (size_t)T.n_inst[VFMM_LIST_W] * 3 * kk);
+        off = std::max(off, down_end);
     }
-    take(w ? &w->xslab : &dummy, mixed ? 1 : (size_t)T.llen[VFMM_LIST_X] * P2);
     if (mixed) {
         const MixedOps* mo = (const MixedOps*)o.mixed;
         const PlanSet* PS = nullptr;
@@ -1316,63 +1118,6 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
     return VFMM_OK;
 }
 
-// V or X list grouped by configuration (host counting sort of the entries) and cut into GEMM
-// tiles of at most GBN entries of one configuration; all device arrays in one allocation.
-static int build_list_groups(DeviceTree* T, const std::vector<int32_t>& cfg, const std::vector<int32_t>& ptr, int ncfg,
-                             int32_t** by_cfg, int32_t** tiles_out, int32_t* n_tiles, int32_t** tgt_out,
-                             cudaStream_t st) {
-    const int64_t n = (int64_t)cfg.size();
-    std::vector<int64_t> start(ncfg + 1, 0);
-    for (int64_t e = 0; e < n; ++e) ++start[cfg[e] + 1];
-    for (int c = 0; c < ncfg; ++c) start[c + 1] += start[c];
-    std::vector<int32_t> order(std::max<int64_t>(n, 1));
-    std::vector<int64_t> fill(start.begin(), start.end() - 1);
-    for (int64_t e = 0; e < n; ++e) order[fill[cfg[e]]++] = (int32_t)e;
-    std::vector<int4> tiles;
-    for (int c = 0; c < ncfg; ++c)
-        for (int64_t b = start[c]; b < start[c + 1]; b += GBN)
-            tiles.push_back(make_int4(c, (int)b, (int)std::min<int64_t>(b + GBN, start[c + 1]), 0));
-    *n_tiles = (int32_t)tiles.size();
-    std::vector<int32_t> tgt;
-    if (tgt_out) {
-        tgt.assign(std::max<int64_t>(n, 1), 0);
-        for (int b = 0; b < T->n_boxes; ++b)
-            for (int e = ptr[b]; e < ptr[b + 1]; ++e) tgt[e] = b;
-    }
-    // [tiles (int4)][order][tgt], each piece 16-byte aligned
-    const size_t n_tile_ints = 4 * std::max<size_t>(1, tiles.size());
-    const size_t n_order = (order.size() + 3) / 4 * 4;
-    std::vector<int32_t> host(n_tile_ints + n_order + tgt.size(), 0);
-    if (!tiles.empty()) std::memcpy(host.data(), tiles.data(), tiles.size() * sizeof(int4));
-    std::copy(order.begin(), order.end(), host.begin() + n_tile_ints);
-    std::copy(tgt.begin(), tgt.end(), host.begin() + n_tile_ints + n_order);
-    int32_t* dev = nullptr;
-    VFMM_CHECK(tree_malloc(reinterpret_cast<void**>(&dev), host.size() * sizeof(int32_t), st));
-    VFMM_CUDA(cudaMemcpyAsync(dev, host.data(), host.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    *tiles_out = dev;  // owns the allocation
-    *by_cfg = dev + n_tile_ints;
-    if (tgt_out) *tgt_out = dev + n_tile_ints + n_order;
-    return VFMM_OK;
-}
-
-int build_near_tiles(DeviceTree* T, const HostLists& H, cudaStream_t st) {
-    VFMM_CHECK(build_list_groups(T, H.cfg[VFMM_LIST_V], H.ptr[VFMM_LIST_V], kVCfg, &T->v_by_cfg, &T->v_tiles,
-                                 &T->n_v_tiles, nullptr, st));
-    VFMM_CHECK(build_list_groups(T, H.cfg[VFMM_LIST_X], H.ptr[VFMM_LIST_X], kFarCfg, &T->x_by_cfg, &T->x_tiles,
-                                 &T->n_x_tiles, &T->x_tgt, st));
-    std::vector<int4> tiles;
-    for (int c = 0; c < kNearCfg; ++c)
-        for (int64_t b = T->u_cfg_start[c]; b < T->u_cfg_start[c + 1]; b += GBN)
-            tiles.push_back(make_int4(c, (int)b, (int)std::min<int64_t>(b + GBN, T->u_cfg_start[c + 1]), 0));
-    T->n_near_tiles = (int)tiles.size();
-    tree_free(T->near_tiles);
-    T->near_tiles = nullptr;
-    VFMM_CHECK(tree_malloc(reinterpret_cast<void**>(&T->near_tiles), std::max<size_t>(1, tiles.size()) * sizeof(int4), st));
-    if (!tiles.empty())
-        VFMM_CUDA(cudaMemcpyAsync(T->near_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-    return VFMM_OK;
-}
-
 // Optional stage timing: a start and a stop event around every stage.
 struct StageEvents {
     cudaEvent_t ev[2 * VFMM_N_STAGES];
@@ -1416,6 +1161,8 @@ static void fill_down_args(DownArgs& d, const DeviceTree& T, const vfmm_ops& o, 
     d.Lexp = w.Lexp;
     d.vslab = w.vslab;
     d.xslab = w.xslab;
+    d.viptr = T.inst_ptr[VFMM_LIST_V];
+    d.xiptr = T.inst_ptr[VFMM_LIST_X];
     d.pwloc = w.pwL;
     d.m2l_out = mo ? w.mix.m2l_out : nullptr;
     // a grouped split-K M2L leaves its partial sums to the downward kernels (m2l_mixed defers them)
@@ -1446,8 +1193,9 @@ template <typename... Args>
 static int launch_pass(void (*kernel)(Args...), int R, int P, int widest_items, int cap, cudaStream_t st,
                        Args... args) {
     const size_t smem = pass_smem_bytes(P);
-    static thread_local int attr_dev[2] = {-1, -1};
-    const int slot = (void*)kernel == (void*)upward_pass_kernel ? 0 : 1;
+    static thread_local int attr_dev[3] = {-1, -1, -1};
+    const int slot = (void*)kernel == (void*)upward_pass_kernel ? 0
+                     : (void*)kernel == (void*)downward_pass_kernel<true> ? 1 : 2;
     int dev = 0;
     cudaGetDevice(&dev);
     if (attr_dev[slot] != dev) {
@@ -1558,6 +1306,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     const int R = PS.R;
     if (!mixed && R != 1) return fail(VFMM_ERR_INTERNAL, "the FP64 form solves one right-hand side at a time");
     const MixedOps* mo = (const MixedOps*)o.mixed;
+    const SymTables* sy = (const SymTables*)o.sym;
     int launches = 0;
     const bool passes = use_passes(T, R, P);
     // readiness counters (persistent passes) and level exponents (mixed form) start at zero
@@ -1590,8 +1339,15 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         launches += 1 + gemm_launches(PS.s2m, kDeferSplits);
     } else {
         ++launches;
-        dim3 g((nleaf + GBN - 1) / GBN, (P2 + GBM - 1) / GBM);
-        s2m_gemm_kernel<<<g, 256, 0, st>>>(o.s2m, P2, kk, nleaf, T.box_of_leaf, T.level, T.width, f, w.Mexp);
+        SymRun r;
+        r.src = f;
+        r.src_stride = kk;
+        r.out = w.Mexp;
+        r.out_stride = P2;
+        r.out_map = T.box_of_leaf;
+        r.level = T.level;
+        r.width = T.width;
+        VFMM_CHECK(sym_gemm(T, sy->s2m, r, st));
     }
     mark(se, ST_S2M, true, st);
     // M2M, finest parents first (levels >= 2 are the ones the lists read)
@@ -1662,8 +1418,8 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     }
     if (side) VFMM_CUDA(cudaStreamWaitEvent(st, side->ev[1], 0));
     if (!mixed) {
-        // FP64 form: every M2L (V list) and S2L (X list) product as gather GEMMs grouped by
-        // configuration, one slab row per list entry; the per-level kernels below sum them
+        // FP64 form: M2L (V list) and S2L (X list) in reflection classes, one slab row per instance; the
+        // downward kernels below sum them
         if (w.pwX) {
             // plane-wave form: outgoing waves of every box, then diagonal translations and the
             // incoming conversion per target box
@@ -1672,21 +1428,28 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
                 VFMM_CHECK(planewave_m2l(o, T.level_start[2], T.n_boxes, T.lptr[VFMM_LIST_V],
                                          T.lidx[VFMM_LIST_V], T.lcfg[VFMM_LIST_V], w.Mexp, w.pwX, w.pwL, st));
             }
-        } else if (T.n_v_tiles > 0) {
+        } else if (T.n_inst[VFMM_LIST_V] > 0) {
             ++launches;
-            dim3 g(T.n_v_tiles, (P2 + GBM - 1) / GBM);
-            v_gemm_kernel<<<g, 256, 0, st>>>((const int4*)T.v_tiles, o.m2l_real, P2, T.v_by_cfg,
-                                             T.lidx[VFMM_LIST_V], w.Mexp, w.vslab);
+            SymRun r;
+            r.q = VFMM_LIST_V;
+            r.src = w.Mexp;
+            r.src_stride = P2;
+            r.out = w.vslab;
+            r.out_stride = P2;
+            VFMM_CHECK(sym_gemm(T, sy->m2l, r, st));
         }
-        if (T.n_x_tiles > 0) {
+        if (T.n_inst[VFMM_LIST_X] > 0) {
             ++launches;
-            dim3 g(T.n_x_tiles, (P2 + GBM - 1) / GBM);
-            x_gemm_kernel<<<g, 256, 0, st>>>((const int4*)T.x_tiles, o.s2l_real, P2, kk, T.x_by_cfg,
-                                             T.lidx[VFMM_LIST_X], T.x_tgt, T.level, T.width, T.leaf_of_box, f,
-                                             w.xslab);
+            SymRun r;
+            r.q = VFMM_LIST_X;
+            r.src = f;
+            r.src_stride = kk;
+            r.out = w.xslab;
+            r.out_stride = P2;
+            VFMM_CHECK(sym_gemm(T, sy->s2l, r, st));
         }
     }
-    if (mixed && passes) {
+    if (passes) {
         DownArgs d;
         fill_down_args(d, T, o, f, w, 2, R);
         PassArgs pa;
@@ -1704,10 +1467,12 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         pa.glev = nullptr;
         pa.level = T.level;
         pa.err = w.mix.err;
-        VFMM_CHECK(launch_pass(downward_pass_kernel, R, P, std::max(widest * R, 16 * R), PS.pass_ctas, st, pa, d));
+        const int items = std::max(widest * R, 16 * R);
+        if (mixed) VFMM_CHECK(launch_pass(downward_pass_kernel<true>, R, P, items, PS.pass_ctas, st, pa, d));
+        else VFMM_CHECK(launch_pass(downward_pass_kernel<false>, R, P, items, 0, st, pa, d));
         ++launches;
     }
-    for (int l = 2; l <= T.depth && !(mixed && passes); ++l) {
+    for (int l = 2; l <= T.depth && !passes; ++l) {
         DownArgs d;
         fill_down_args(d, T, o, f, w, l, R);
         int n = d.end - d.begin;
@@ -1722,7 +1487,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
             const int64_t nt = (int64_t)n * R * P;
             down_mixed_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d);
         } else {
-            down_kernel<<<(unsigned)n * R, 64, 0, st>>>(d);
+            down_kernel<<<(unsigned)((n + 3) / 4), 128, 0, st>>>(d);
         }
     }
     if (T.depth < 2) VFMM_CUDA(cudaMemsetAsync(w.Lexp, 0, (size_t)T.n_boxes * R * P2 * sizeof(double), st));
@@ -1730,12 +1495,14 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     mark(se, ST_DOWN, true, st);
     if (!mixed) {
         mark(se, ST_NEAR, false, st);
-        if (T.n_near_tiles > 0) {
-            ++launches;
-            dim3 g(T.n_near_tiles, (3 * kk + GBM - 1) / GBM);
-            near_gemm_kernel<<<g, 256, 0, st>>>((const int4*)T.near_tiles, o.near, kk, T.u_by_cfg,
-                                                T.lidx[VFMM_LIST_U], T.leaf_of_box, f, w.slab);
-        }
+        ++launches;
+        SymRun r;
+        r.q = VFMM_LIST_U;
+        r.src = f;
+        r.src_stride = kk;
+        r.out = w.slab;
+        r.out_stride = 3 * kk;
+        VFMM_CHECK(sym_gemm(T, sy->near, r, st));
         mark(se, ST_NEAR, true, st);
     }
     // far field at the leaves
@@ -1744,32 +1511,22 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         VFMM_CHECK(far_leaf_mixed(T, PS, o, w.Mexp, w.Lexp, w.mix, st));
         launches += 1 + gemm_launches(PS.far, kDeferSegments);
     } else {
-        ++launches;
-        dim3 g((nleaf + GBN - 1) / GBN, (3 * kk + GBM - 1) / GBM);
-        l2t_gemm_kernel<<<g, 256, 0, st>>>(o.l2t, P2, kk, nleaf, T.box_of_leaf, w.Lexp, w.far);
+        launches += T.n_inst[VFMM_LIST_W] > 0 ? 2 : 1;
+        SymRun r;
+        r.src = w.Lexp;
+        r.src_stride = P2;
+        r.src_map = T.box_of_leaf;
+        r.out = w.far;
+        r.out_stride = 3 * kk;
+        VFMM_CHECK(sym_gemm(T, sy->l2t, r, st));
+        r.q = VFMM_LIST_W;
+        r.src = w.Mexp;
+        r.src_map = nullptr;
+        r.out = w.wslab;
+        VFMM_CHECK(sym_gemm(T, sy->m2t, r, st));
     }
     mark(se, ST_L2T, true, st);
     mark(se, ST_LEAF, false, st);
-    LeafArgs a;
-    a.nleaf = nleaf;
-    a.kk = kk;
-    a.k = o.k;
-    a.P = P;
-    a.width = T.width;
-    a.box_of_leaf = T.box_of_leaf;
-    a.level = T.level;
-    a.uptr = T.lptr[VFMM_LIST_U];
-    a.uidx = T.lidx[VFMM_LIST_U];
-    a.wptr = T.lptr[VFMM_LIST_W];
-    a.widx = T.lidx[VFMM_LIST_W];
-    a.wcfg = T.lcfg[VFMM_LIST_W];
-    a.xhat = o.xhat;
-    a.slab = w.slab;
-    a.far = w.far;
-    a.Mexp = w.Mexp;
-    a.u = u;
-    a.ux = ux;
-    a.uy = uy;
     if (mixed) {
         const int64_t nv = (int64_t)nleaf * R;
         int lw = 0;
@@ -1811,7 +1568,30 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         leaf_mixed_kernel<<<(unsigned)nv, std::max(32, ((kk + 31) / 32) * 32), 0, st>>>(la);
         ++launches;
     } else {
-        leaf_kernel<<<(unsigned)nleaf, ((kk + 31) / 32) * 32, 0, st>>>(a);
+        LeafArgs a;
+        a.op = sy->near;
+        a.nleaf = nleaf;
+        a.kk = kk;
+        a.k = o.k;
+        a.P = P;
+        a.width = T.width;
+        a.box_of_leaf = T.box_of_leaf;
+        a.level = T.level;
+        a.uptr = T.lptr[VFMM_LIST_U];
+        a.uidx = T.lidx[VFMM_LIST_U];
+        a.wptr = T.lptr[VFMM_LIST_W];
+        a.widx = T.lidx[VFMM_LIST_W];
+        a.uiptr = T.inst_ptr[VFMM_LIST_U];
+        a.wiptr = T.inst_ptr[VFMM_LIST_W];
+        a.slab = w.slab;
+        a.wslab = w.wslab;
+        a.far = w.far;
+        a.Mexp = w.Mexp;
+        a.Lexp = w.Lexp;
+        a.u = u;
+        a.ux = ux;
+        a.uy = uy;
+        leaf_kernel<<<(unsigned)nleaf, ((kk + 31) / 32) * 32, (size_t)3 * kk * sizeof(double), st>>>(a);
         ++launches;
     }
     mark(se, ST_LEAF, true, st);

@@ -39,6 +39,7 @@
 
 #include "mixed.cuh"
 #include "ops.cuh"
+#include "sym.cuh"
 #include "tc_ptx.cuh"
 #include "vfmm_internal.cuh"
 
@@ -883,7 +884,7 @@ int build_mixed_plan(DeviceTree* T, cudaStream_t st) {
     HostLists H;
     VFMM_CHECK(fetch_host_lists(*T, &H));
     VFMM_CHECK(build_far_slots(T, H, st));
-    VFMM_CHECK(build_near_tiles(T, H, st));  // the FP64 form's GEMM tiles
+    VFMM_CHECK(build_instances(T, st));  // the FP64 form's table products
     T->plans_r = new std::map<int, PlanSet*>();
     T->plans_mu = new std::mutex();
     return build_plans(*T, 1, H, &T->plans, st);

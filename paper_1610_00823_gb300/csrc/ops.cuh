@@ -20,9 +20,8 @@ struct vfmm_ops {
     double* l2l_r = nullptr;  // [in][out] real
     double* m2l_t = nullptr;  // [40][in][out] complex
     double* l2t = nullptr;    // [3kk][2(p+1)] real
-    // real forms for the FP64 form's gather GEMMs: rows 2l (Re), 2l + 1 (Im) of output coefficient l
-    double* m2l_real = nullptr;  // [40][2(p+1)][2(p+1)]: columns 2n, 2n + 1 of input coefficient n
-    double* s2l_real = nullptr;  // [20][2(p+1)][kk]
+    // FP64 form: every table product in the reflection classes of the square (SymTables, sym.cuh)
+    void* sym = nullptr;
     // split-precision near-field operands (VFMM_MIXED)
     void* mixed = nullptr;
     // plane-wave M2L (FP64 form, planewave.cu): rule length s, outgoing [p][s] lambda^(n-1)/(n-1)!,

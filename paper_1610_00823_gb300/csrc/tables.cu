@@ -35,6 +35,7 @@
 
 #include "near_quad.cuh"
 #include "ops.cuh"
+#include "sym.cuh"
 #include "vfmm_internal.cuh"
 
 namespace vfmm {
@@ -451,8 +452,14 @@ static int create(int k, int p, int precision, cudaStream_t st, vfmm_ops* o) {
                     sr[((size_t)c * P2 + 2 * l) * kk + s] = st_[(((size_t)c * kk + s) * P + l) * 2];
                     sr[((size_t)c * P2 + 2 * l + 1) * kk + s] = st_[(((size_t)c * kk + s) * P + l) * 2 + 1];
                 }
-        VFMM_CHECK(dalloc_copy(&o->m2l_real, mr, st));
-        VFMM_CHECK(dalloc_copy(&o->s2l_real, sr, st));
+        double *d_m2l = nullptr, *d_s2l = nullptr;
+        int rc = dalloc_copy(&d_m2l, mr, st);
+        if (rc == VFMM_OK) rc = dalloc_copy(&d_s2l, sr, st);
+        if (rc == VFMM_OK) rc = sym_prepare(o, d_m2l, d_s2l, st);
+        cudaStreamSynchronize(st);
+        cudaFree(d_m2l);
+        cudaFree(d_s2l);
+        VFMM_CHECK(rc);
         VFMM_CHECK(planewave_prepare(o, st));
     }
     VFMM_CUDA(cudaStreamSynchronize(st));
@@ -468,11 +475,12 @@ static int create(int k, int p, int precision, cudaStream_t st, vfmm_ops* o) {
 
 void free_ops(vfmm_ops* o) {
     double* ps[] = {o->xhat,  o->near,  o->s2m, o->s2l_t,    o->m2m_t,   o->l2l_t,
-                    o->m2m_r, o->l2l_r, o->m2l_t, o->l2t, o->m2l_real, o->s2l_real};
+                    o->m2m_r, o->l2l_r, o->m2l_t, o->l2t};
     for (double* p : ps)
         if (p) cudaFree(p);
     mixed_free(o);
     planewave_free(o);
+    sym_free(o);
 }
 
 }  // namespace vfmm

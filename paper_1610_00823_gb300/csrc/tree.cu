@@ -189,8 +189,7 @@ __global__ void scan_add_kernel(int32_t* __restrict__ out, const int32_t* __rest
     }
 }
 
-// out[i] = sum_{j < i} in[j]; *total = sum of all (host). `in` and `out` may alias.
-static int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, cudaStream_t st) {
+int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, cudaStream_t st) {
     if (n <= 0) {
         *total = 0;
         return VFMM_OK;
@@ -676,26 +675,6 @@ __global__ void shift_kernel(int32_t* a, int64_t n, int32_t s) {
     if (i < n) a[i] -= s;
 }
 
-__global__ void cfg_flags_kernel(const int32_t* __restrict__ cfg, int64_t n, int ncfg, int32_t* __restrict__ flags) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    int c = cfg[e];
-    for (int j = 0; j < ncfg; ++j) flags[(int64_t)j * n + e] = (j == c) ? 1 : 0;
-}
-
-__global__ void cfg_scatter_kernel(const int32_t* __restrict__ cfg, const int32_t* __restrict__ pos, int64_t n,
-                                   int32_t* __restrict__ out) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    out[pos[(int64_t)cfg[e] * n + e]] = (int32_t)e;
-}
-
-__global__ void entry_target_kernel(const int32_t* __restrict__ ptr, int n, int32_t* __restrict__ tgt) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    for (int e = ptr[b]; e < ptr[b + 1]; ++e) tgt[e] = b;
-}
-
 static inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
 // ---------------------------------------------------------------- host orchestration
@@ -748,11 +727,6 @@ static int upload_child_basis(int k, BuildCtx& B) {
     return VFMM_OK;
 }
 
-// out[c] = in[c * stride], c < n.
-__global__ void strided_gather_kernel(const int32_t* __restrict__ in, int64_t stride, int n, int32_t* __restrict__ out) {
-    for (int c = threadIdx.x; c < n; c += blockDim.x) out[c] = in[(int64_t)c * stride];
-}
-
 static int compute_lists(DeviceTree* T, cudaStream_t st) {
     const int n = T->n_boxes;
     TreeView V{T->key, T->level_start_dev, T->level, T->ix, T->iy, T->parent, T->child0, T->depth};
@@ -790,34 +764,6 @@ static int compute_lists(DeviceTree* T, cudaStream_t st) {
         T->lcfg[q] = cfg[q].release();
         T->lptr[q] = ptr[q].release();
     }
-    // U entries grouped by configuration, stable (flattened config-major scan)
-    const int64_t nU = T->llen[VFMM_LIST_U];
-    DBuf<int32_t> flags, byc, tgt;
-    VFMM_CHECK(flags.alloc((size_t)kNearCfg * nU, st));
-    VFMM_CHECK(byc.alloc_tree(std::max<int64_t>(1, nU), st));
-    VFMM_CHECK(tgt.alloc_tree(std::max<int64_t>(1, nU), st));
-    cfg_flags_kernel<<<nblk(nU), 256, 0, st>>>(T->lcfg[0], nU, kNearCfg, flags.p);
-    VFMM_CUDA(cudaGetLastError());
-    int64_t tot = 0;
-    VFMM_CHECK(exclusive_scan(flags.p, flags.p, (int64_t)kNearCfg * nU, &tot, st));
-    cfg_scatter_kernel<<<nblk(nU), 256, 0, st>>>(T->lcfg[0], flags.p, nU, byc.p);
-    entry_target_kernel<<<nblk(n), 256, 0, st>>>(T->lptr[0], n, tgt.p);
-    VFMM_CUDA(cudaGetLastError());
-    // first entry of each configuration: flags[c * nU], gathered and read back once
-    T->u_cfg_start.assign(kNearCfg + 1, 0);
-    if (nU > 0) {
-        DBuf<int32_t> starts_dev;
-        VFMM_CHECK(starts_dev.alloc(kNearCfg, st));
-        strided_gather_kernel<<<1, 64, 0, st>>>(flags.p, nU, kNearCfg, starts_dev.p);
-        VFMM_CUDA(cudaGetLastError());
-        int32_t h[kNearCfg];
-        VFMM_CUDA(cudaMemcpyAsync(h, starts_dev.p, kNearCfg * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        VFMM_CUDA(cudaStreamSynchronize(st));
-        for (int c = 0; c < kNearCfg; ++c) T->u_cfg_start[c] = h[c];
-    }
-    T->u_cfg_start[kNearCfg] = nU;
-    T->u_by_cfg = byc.release();
-    T->u_tgt = tgt.release();
     return VFMM_OK;
 }
 
@@ -1141,10 +1087,9 @@ static int finalize(std::vector<DBuf<uint32_t>>& keys, std::vector<int64_t>& cnt
 void free_tree(DeviceTree* t) {
     // work queued on any stream may still read the tree
     cudaDeviceSynchronize();
-    // v_by_cfg, x_by_cfg and x_tgt point into the v_tiles and x_tiles allocations
     void* ps[] = {t->key,         t->level,       t->ix,       t->iy,           t->parent,     t->child0,
-                  t->leaf_of_box, t->box_of_leaf, t->level_start_dev, t->u_by_cfg, t->u_tgt, t->near_tiles,
-                  t->far_slot,    t->nonleaf,     t->nonleaf_start_dev, t->v_tiles, t->x_tiles};
+                  t->leaf_of_box, t->box_of_leaf, t->level_start_dev, t->inst,
+                  t->far_slot,    t->nonleaf,     t->nonleaf_start_dev};
     free_plan_set(&t->plans);
     if (t->plans_r) {
         for (auto& kv : *t->plans_r) {

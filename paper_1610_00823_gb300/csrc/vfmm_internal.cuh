@@ -220,22 +220,14 @@ struct DeviceTree {
     int32_t* lidx[4] = {nullptr, nullptr, nullptr, nullptr};
     int32_t* lcfg[4] = {nullptr, nullptr, nullptr, nullptr};
     int64_t llen[4] = {0, 0, 0, 0};
-    // U entries grouped by near configuration (stable within a configuration)
-    int32_t* u_by_cfg = nullptr;       // [llen[U]] U-entry indices
-    int32_t* u_tgt = nullptr;          // [llen[U]] target leaf box of each U entry
-    std::vector<int64_t> u_cfg_start;  // host, 34 entries
-    // GEMM tile schedule for the near field: per tile (cfg, first column)
-    int32_t* near_tiles = nullptr;
-    int32_t n_near_tiles = 0;
-    // V and X entries grouped by configuration, with GEMM tiles (configuration, first, end) over
-    // the grouped order and each entry's target box (FP64 form's M2L and S2L)
-    int32_t* v_by_cfg = nullptr;
-    int32_t* v_tiles = nullptr;
-    int32_t n_v_tiles = 0;
-    int32_t* x_by_cfg = nullptr;
-    int32_t* x_tiles = nullptr;
-    int32_t* x_tgt = nullptr;
-    int32_t n_x_tiles = 0;
+    // instances of the four lists (sym.cuh): per list the box pointers, the four sources of each
+    // instance, the instances in orbit-major order and each orbit's first place there; one allocation
+    void* inst = nullptr;
+    int32_t* inst_ptr[4] = {nullptr, nullptr, nullptr, nullptr};     // [n_boxes + 1]
+    int4* inst_src[4] = {nullptr, nullptr, nullptr, nullptr};        // [n_inst] source under each reflection or -1
+    int32_t* inst_order[4] = {nullptr, nullptr, nullptr, nullptr};   // [n_inst]
+    int32_t* inst_ostart[4] = {nullptr, nullptr, nullptr, nullptr};  // [orbits + 1]
+    int64_t n_inst[4] = {0, 0, 0, 0};
     // split-precision schedules (VFMM_MIXED): one right-hand side built with the tree, others on
     // first use (plans_for), guarded by plans_mu
     PlanSet plans;
@@ -253,14 +245,14 @@ void free_split_plan(SplitPlan* p);
 void free_plan_set(PlanSet* ps);
 // Plans for R folded right-hand sides (R = 1: the tree's own set); builds and caches on first use.
 int plans_for(const DeviceTree& T, int R, const PlanSet** out);
-struct HostLists;
-int build_near_tiles(DeviceTree* t, const HostLists& h, cudaStream_t st);
 // Device arrays a tree keeps (boxes, lists, schedules) come from a per-device stream-ordered pool:
 // tree_malloc allocates in the order of stream st (the tree build synchronises st before it
 // returns, after which the arrays are valid on every stream); tree_free returns one to the pool
 // and is called once the device has finished with it (free_tree synchronises the device first).
 int tree_malloc(void** p, size_t bytes, cudaStream_t st);
 void tree_free(void* p);
+// out[i] = sum_{j < i} in[j]; *total = sum of all (host; synchronises st). `in` and `out` may alias.
+int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, cudaStream_t st);
 // vfmm_volume_potential with flags: fork = false keeps every launch on `st` (no second stream);
 // reset = false leaves the workspace's status word as it is (a caller solving several right-hand
 // sides one after another clears it once, so that a timeout in an early one is not lost).
