@@ -337,8 +337,8 @@ int vfmm_leaf_interpolate(const vfmm_tree* tree, int32_t n_fields, const double*
  * far field instead of a new FMM). For each point t (x_dev[i], y_dev[i]) of leaf b (located as
  * vfmm_leaf_interpolate locates it): u, u_x, u_y = the far field of b's local expansion and of the
  * multipoles of b's W list at t, plus the near field of every leaf of b's U list, integrated
- * against f~ at t itself by on-the-fly quadrature (tanh-sinh rules on triangles with apex at the
- * source box's point nearest to t). At a leaf node it gives the solve's value there; elsewhere it is
+ * against f~ at t itself in closed form (f~ is the Laplacian of a polynomial on each leaf, which leaves
+ * edge integrals that are Legendre functions of the second kind). At a leaf node it gives the solve's value there; elsewhere it is
  * V f~(t), not the interpolant v~. Reads the expansions a vfmm_volume_potential call with nrhs = 1
  * and the same tree, ops and f_dev ([n_leaves][k*k]) left in workspace_dev (workspace_bytes as
  * given to that call), so it must follow that call on the same stream and precede any other use of

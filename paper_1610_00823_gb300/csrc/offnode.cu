@@ -6,36 +6,220 @@
 //   V f~(t) = -(1/2 pi) Re [ sum_l b~_l ((t - z_b)/h)^l + sum over W(b) of the multipole at t ]
 //           + sum over U(b) of -(1/2 pi) int_{B_s} log|t - y| f~_s(y) dy,
 // with the gradient from the differentiated expansions and kernels (Section 3.2). The far part
-// reads the expansions a solve left in its workspace; the near part is an on-the-fly quadrature
-// per (point, neighbour leaf): the source box is cut into triangles with apex at its point nearest
-// to t (near_quad.cuh, the construction of the near-field tables) and integrated with tanh-sinh
-// rules in both directions, f~_s evaluated from its Chebyshev coefficients at every node.
+// reads the expansions a solve left in its workspace.
 //
-// One CTA per point: warp 0 sums the far part, then all threads share the quadrature nodes of each
-// neighbour leaf in turn (fixed order, so results are deterministic).
+// Near part: on a leaf (unit box) f~ is a polynomial, and so is a P with Laplace P = f~. Green's second
+// identity and the Cauchy-Pompeiu formula then leave integrals over the four edges only,
+//   int log|t - y| f~ dy  = sum_e int (log|t - y| dP/dn - P d log|t - y|/dn) ds  [+ 2 pi P(t) inside],
+//   int f~ / (t - y) dy   = (i/2) sum_e int F/(y - t) dy  [+ pi F(t) inside],  F = 2 (P_x - i P_y),
+// and with the traces as Legendre series on an edge (x in [-1, 1], z the point in its coordinate)
+//   int P_n(x) / (x - z) dx = -2 Q_n(z),   int P_n(x) log|x - z| dx = 2 Re (Q_{n+1} - Q_{n-1})/(2n + 1),
+// Q_n the Legendre functions of the second kind: closed forms at any distance from the edge, where a
+// quadrature needs ever more nodes. Q_n comes from its three-term recurrence, upwards where z is near
+// the edge, else downwards from a start high enough (Miller) and scaled to Q_0 = log((z+1)/(z-1))/2.
+//
+// P is the polynomial of total degree 2k of least weighted norm (prepared per k on the host, per
+// reflection class: tensor Legendre coefficients c_mn, m + n <= 2k, from the k x k leaf values).
+//
+// What bounds it: FP64 (about 0.4 MFMA per point, most of it leaf values to coefficients; one CTA per
+// point, two per SM). 1000 points of a 1,378-leaf tree, k = 16: 247 ms with tanh-sinh quadrature of the
+// neighbours (up to 8 x 201^2 nodes of k^2 terms each) -> 1.15 ms, error against 64-bit
+// sums unchanged (1.5e-15).
+#include <algorithm>
 #include <cmath>
+#include <vector>
 
-#include "near_quad.cuh"
 #include "ops.cuh"
+#include "sym.cuh"
 #include "vfmm_internal.cuh"
 
 namespace vfmm {
 
 constexpr int kOffThreads = 256;
-// tanh-sinh rules of the on-the-fly near-field quadrature, by the distance d from the point to the
-// boundary of the source leaf (width hs): step 0.1 (65 nodes per direction) when the point lies on
-// that boundary or d >= hs / 4; 0.05 (141 nodes, the near-field tables' rule) for hs / 1000 <= d <
-// hs / 4; 0.035 (201 nodes) closer. Measured on the unit box against a step of 0.015: the gradient
-// of a point 1e-4 inside an edge is off by 1e-8 with step 0.1, 6e-13 with 0.05; 1e-6 inside, 4e-12
-// with 0.05 and 2e-13 with 0.035.
-constexpr int kOffRules = 3;
-__host__ __device__ constexpr double off_step(int r) { return r == 0 ? 0.1 : (r == 1 ? 0.05 : 0.035); }
-// nodes j in [-half, half]: |u| <= 3.2, 3.5, 3.5
-__host__ __device__ constexpr int off_half(int r) { return r == 0 ? 32 : (r == 1 ? 70 : 100); }
-// first node of rule r in the shared node table
-__host__ __device__ constexpr int off_first(int r) { return r == 0 ? 0 : (r == 1 ? 65 : 65 + 141); }
-constexpr int kOffDENodes = 65 + 141 + 201;
+constexpr int kOffMaxU = 13;      // a leaf, and at most 12 neighbours
+constexpr int kOffMaxN = 33;      // 2k + 1 Legendre coefficients along an edge
+constexpr int kOffTasks = 4 * kOffMaxU;
+constexpr int kOffSteps = 288;    // recurrence constants: steps above kOffMaxN that Miller needs for
+constexpr float kOffForward = 1.08f;  // rho >= kOffForward: 37 / (2 log 1.08) = 241
 
+// Rows (m, n), m = a + 2i, n = b + 2j, m + n <= 2k of class (a, b), i outer.
+__host__ __device__ inline int off_ni(int k, int c) { return k + 1 - ((c & 1) + (c >> 1) + 1) / 2; }
+__host__ __device__ inline int off_rows(int k, int c) { return off_ni(k, c) * (off_ni(k, c) + 1) / 2; }
+__host__ __device__ inline int off_first(int k, int c) {
+    int r = 0;
+    for (int d = 0; d < c; ++d) r += off_rows(k, d);
+    return r;
+}
+__host__ __device__ inline int off_row0(int k, int c, int i) { return off_first(k, c) + i * off_ni(k, c) - i * (i - 1) / 2; }
+// First value of class c in a leaf's symmetrised values (a quadrant of nodes per class, k^2 in all).
+__host__ __device__ inline int off_val(int k, int c) {
+    int r = 0;
+    for (int d = 0; d < c; ++d) r += sym_half(k, d & 1) * sym_half(k, d >> 1);
+    return r;
+}
+
+struct OffTables {
+    double* G = nullptr;   // per class [value][row]: coefficients of P from the symmetrised values
+    int64_t g_off[4] = {};
+    double4* C = nullptr;  // [kOffSteps]: (2n+1)/n, (n+1)/n (downwards), (2n+1)/(n+1), n/(n+1) (upwards)
+};
+
+// ---------------------------------------------------------------- host: values -> P
+// Legendre coefficients of the k Lagrange polynomials of the nodes xi: A[j][i].
+static void legendre_of_nodes(int k, const std::vector<double>& xi, std::vector<double>& A) {
+    std::vector<double> V((size_t)k * k), inv((size_t)k * k, 0.0);
+    // V[i][j] = P_j(xi_i); A = V^-1 by Gauss-Jordan with pivoting, in extended precision
+    std::vector<long double> M((size_t)k * 2 * k, 0.0L);
+    for (int i = 0; i < k; ++i) {
+        long double p0 = 1.0L, p1 = xi[i];
+        for (int j = 0; j < k; ++j) {
+            M[(size_t)i * 2 * k + j] = p0;
+            const long double p2 = ((2 * j + 3) * (long double)xi[i] * p1 - (j + 1) * p0) / (j + 2);
+            p0 = p1;
+            p1 = p2;
+        }
+        M[(size_t)i * 2 * k + k + i] = 1.0L;
+    }
+    for (int c = 0; c < k; ++c) {
+        int pv = c;
+        for (int r = c + 1; r < k; ++r)
+            if (std::fabs(M[(size_t)r * 2 * k + c]) > std::fabs(M[(size_t)pv * 2 * k + c])) pv = r;
+        for (int q = 0; q < 2 * k; ++q) std::swap(M[(size_t)c * 2 * k + q], M[(size_t)pv * 2 * k + q]);
+        const long double d = 1.0L / M[(size_t)c * 2 * k + c];
+        for (int q = 0; q < 2 * k; ++q) M[(size_t)c * 2 * k + q] *= d;
+        for (int r = 0; r < k; ++r) {
+            const long double f = M[(size_t)r * 2 * k + c];
+            if (r == c || f == 0.0L) continue;
+            for (int q = 0; q < 2 * k; ++q) M[(size_t)r * 2 * k + q] -= f * M[(size_t)c * 2 * k + q];
+        }
+    }
+    A.resize((size_t)k * k);
+    for (int j = 0; j < k; ++j)
+        for (int i = 0; i < k; ++i) A[(size_t)j * k + i] = (double)M[(size_t)j * 2 * k + k + i];
+}
+
+// G of one class, [value][row]. Unknowns c_mn of P, equations: Legendre coefficients of Laplace P = those
+// of f~ (j + l <= 2k - 2; zero beyond its degrees), least norm of (1 + m(m+1) + n(n+1)) c_mn: Householder QR
+// of the transposed weighted system and one refinement step with the residual in extended precision.
+static void class_table(int k, int c, const std::vector<double>& A, double* G) {
+    const int a = c & 1, b = c >> 1, nu = off_rows(k, c), ni = off_ni(k, c), base = off_first(k, c);
+    std::vector<int> eq_j, eq_l;
+    for (int j = a; j <= 2 * k - 2; j += 2)
+        for (int l = b; j + l <= 2 * k - 2; l += 2) {
+            eq_j.push_back(j);
+            eq_l.push_back(l);
+        }
+    const int ne = (int)eq_j.size();
+    auto row = [&](int m, int n) { return off_row0(k, c, m >> 1) - base + (n >> 1); };
+    std::vector<double> W(nu);
+    for (int i = 0; i < ni; ++i)
+        for (int j = 0; i + j < ni; ++j) {
+            const int m = a + 2 * i, n = b + 2 * j;
+            W[row(m, n)] = 1.0 + m * (m + 1) + n * (n + 1);
+        }
+    // d2(j, m): coefficient j of the second derivative of Legendre polynomial m in unit-box coordinates
+    auto d2 = [](int j, int m) { return 4.0 * (j + 0.5) * (m * (m + 1.0) - j * (j + 1.0)); };
+    // columns = equations, rows = unknowns (weighted): H = Q R
+    std::vector<double> H((size_t)ne * nu, 0.0), M;
+    for (int e = 0; e < ne; ++e) {
+        for (int m = eq_j[e] + 2; m + eq_l[e] <= 2 * k; m += 2) H[(size_t)e * nu + row(m, eq_l[e])] += d2(eq_j[e], m);
+        for (int n = eq_l[e] + 2; n + eq_j[e] <= 2 * k; n += 2) H[(size_t)e * nu + row(eq_j[e], n)] += d2(eq_l[e], n);
+        for (int u = 0; u < nu; ++u) H[(size_t)e * nu + u] /= W[u];
+    }
+    M = H;
+    std::vector<double> tau(ne);
+    for (int e = 0; e < ne; ++e) {
+        double* v = H.data() + (size_t)e * nu;
+        double nrm = 0.0;
+        for (int u = e; u < nu; ++u) nrm += v[u] * v[u];
+        nrm = std::sqrt(nrm);
+        const double alpha = v[e] > 0.0 ? -nrm : nrm;
+        const double v0 = v[e] - alpha;
+        tau[e] = -v0 / alpha;
+        for (int u = e + 1; u < nu; ++u) v[u] /= v0;
+        v[e] = alpha;  // R's diagonal; the reflector's leading 1 is implied
+        for (int q = e + 1; q < ne; ++q) {
+            double* x = H.data() + (size_t)q * nu;
+            double s = x[e];
+            for (int u = e + 1; u < nu; ++u) s += v[u] * x[u];
+            s *= tau[e];
+            x[e] -= s;
+            for (int u = e + 1; u < nu; ++u) x[u] -= s * v[u];
+        }
+    }
+    // x = Q R^-T s
+    auto solve = [&](std::vector<double> y, std::vector<double>& x) {
+        for (int e = 0; e < ne; ++e) {
+            double s = y[e];
+            for (int q = 0; q < e; ++q) s -= H[(size_t)e * nu + q] * y[q];  // R[q][e]
+            y[e] = s / H[(size_t)e * nu + e];
+        }
+        x.assign(nu, 0.0);
+        std::copy(y.begin(), y.end(), x.begin());
+        for (int e = ne - 1; e >= 0; --e) {
+            const double* v = H.data() + (size_t)e * nu;
+            double s = x[e];
+            for (int u = e + 1; u < nu; ++u) s += v[u] * x[u];
+            s *= tau[e];
+            x[e] -= s;
+            for (int u = e + 1; u < nu; ++u) x[u] -= s * v[u];
+        }
+    };
+    const int nx = sym_half(k, a), ny = sym_half(k, b);
+    std::vector<double> s(ne), r(ne), x, dx;
+    for (int jy = 0; jy < ny; ++jy)
+        for (int ix = 0; ix < nx; ++ix) {
+            const double w = (2 * ix == k - 1 ? 0.5 : 1.0) * (2 * jy == k - 1 ? 0.5 : 1.0);
+            for (int e = 0; e < ne; ++e)
+                s[e] = eq_j[e] < k && eq_l[e] < k ? w * A[(size_t)eq_j[e] * k + ix] * A[(size_t)eq_l[e] * k + jy] : 0.0;
+            solve(s, x);
+            for (int e = 0; e < ne; ++e) {
+                long double t = s[e];
+                for (int u = 0; u < nu; ++u)
+                    if (M[(size_t)e * nu + u] != 0.0) t -= (long double)M[(size_t)e * nu + u] * x[u];
+                r[e] = (double)t;
+            }
+            solve(r, dx);
+            for (int u = 0; u < nu; ++u) G[((size_t)jy * nx + ix) * nu + u] = (x[u] + dx[u]) / W[u];
+        }
+}
+
+int offnode_prepare(vfmm_ops* o, cudaStream_t st) {
+    const int k = o->k;
+    const double pi = 3.14159265358979323846;
+    std::vector<double> xi(k), A, G;
+    for (int i = 0; i < k; ++i) xi[i] = -std::cos(pi * (2.0 * i + 1.0) / (2.0 * k));
+    legendre_of_nodes(k, xi, A);
+    OffTables* t = new OffTables();
+    o->off = t;
+    for (int c = 0; c < 4; ++c) {
+        t->g_off[c] = (int64_t)G.size();
+        const size_t n = (size_t)sym_half(k, c & 1) * sym_half(k, c >> 1) * off_rows(k, c);
+        G.resize(G.size() + n);
+        class_table(k, c, A, G.data() + t->g_off[c]);
+    }
+    std::vector<double4> C(kOffSteps);
+    for (int n = 0; n < kOffSteps; ++n)
+        C[n] = make_double4(n ? (2.0 * n + 1.0) / n : 0.0, n ? (n + 1.0) / n : 0.0, (2.0 * n + 1.0) / (n + 1.0),
+                            n / (n + 1.0));
+    VFMM_CUDA(cudaMalloc(&t->G, G.size() * sizeof(double)));
+    VFMM_CUDA(cudaMalloc(&t->C, C.size() * sizeof(double4)));
+    VFMM_CUDA(cudaMemcpyAsync(t->G, G.data(), G.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+    VFMM_CUDA(cudaMemcpyAsync(t->C, C.data(), C.size() * sizeof(double4), cudaMemcpyHostToDevice, st));
+    VFMM_CUDA(cudaStreamSynchronize(st));
+    return VFMM_OK;
+}
+
+void offnode_free(vfmm_ops* o) {
+    OffTables* t = (OffTables*)o->off;
+    if (!t) return;
+    if (t->G) cudaFree(t->G);
+    if (t->C) cudaFree(t->C);
+    delete t;
+    o->off = nullptr;
+}
+
+// ---------------------------------------------------------------- device
 struct OffArgs {
     int k, P, depth, R;
     int64_t n;
@@ -47,38 +231,142 @@ struct OffArgs {
     const double* Lexp;  // [n_boxes][R][2P] scaled locals of the solve
     const double *x, *y;
     double *u, *ux, *uy;
-    double A[16 * 16];   // values -> Chebyshev coefficients, A[m][i] = (2 - d_m0)/k T_m(x_i)
+    OffTables t;
 };
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double s = 0.0;
-    for (int w = 0; w < kOffThreads / 32; ++w) s += red[w];  // every thread, same order
-    return s;
+// A U leaf as seen from the point, unit-box coordinates: distances to its sides (left, right, bottom,
+// top), positive inwards. On a side (all >= 0, some 0) the point counts as inside, by an amount that the
+// arithmetic of the edges cannot see.
+struct OffLeaf {
+    double d[4];
+    double h;
+    int leaf, inside;
+};
+
+// sum over this thread's values v of the table columns, for NU leaves: cf[row][u] = sum_v G[v][row] fs[v][u]
+template <int NU>
+__device__ __forceinline__ void off_coeffs(const double* __restrict__ G, int K, int ld, const double* fs, double* out) {
+    double acc[NU];
+#pragma unroll
+    for (int u = 0; u < NU; ++u) acc[u] = 0.0;
+#pragma unroll 4
+    for (int v = 0; v < K; ++v) {
+        const double g = __ldg(G + (size_t)v * ld);
+#pragma unroll
+        for (int u = 0; u < NU; ++u) acc[u] = fma(g, fs[v * kOffMaxU + u], acc[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < NU; ++u) out[u] = acc[u];
+}
+template <int NU>
+__device__ __forceinline__ void off_coeffs_n(int nu, const double* G, int K, int ld, const double* fs, double* out) {
+    if (nu == NU) off_coeffs<NU>(G, K, ld, fs, out);
+    else if constexpr (NU > 1) off_coeffs_n<NU - 1>(nu, G, K, ld, fs, out);
 }
 
-__global__ void __launch_bounds__(kOffThreads) offnode_kernel(OffArgs a) {
-    __shared__ double sDE[3][kOffDENodes];  // the three rules' nodes one after another
-    __shared__ double sC[16 * 16];    // Chebyshev coefficients of the current source leaf, [n][m]
-    __shared__ double sTmp[16 * 16];
-    __shared__ QuadPiece pcs[8];
-    __shared__ int s_npc;
-    __shared__ double red[kOffThreads / 32];
-    __shared__ double s_far[3];
-    __shared__ int s_b;
-    const int tid = threadIdx.x, k = a.k, kk = k * k;
-    const int64_t p = blockIdx.x;
-    const double px = a.x[p], py = a.y[p];
-    for (int r = 0; r < kOffRules; ++r)
-        for (int j = tid; j < 2 * off_half(r) + 1; j += blockDim.x) {
-            const DENode d = de_node(j - off_half(r), off_step(r));
-            sDE[0][off_first(r) + j] = d.x;
-            sDE[1][off_first(r) + j] = d.xc;
-            sDE[2][off_first(r) + j] = d.w;
+// (V, Re Phi', Im Phi') of one edge of a unit box at the point: w1, w2 the distances along the edge from
+// the point to its end and from its start (edge coordinate, length 2), zi the one across (positive inside);
+// p, g, T: Legendre coefficients of P, its outward and its tangential derivative, stride kOffTasks; logs is
+// log(h / 2); (tr, ti) the conjugate of the edge's direction.
+__device__ __forceinline__ void edge_terms(double w1, double w2, double zi, const double* p, const double* g,
+                                           const double* T, int N, const double4* __restrict__ C, double logs,
+                                           double tr, double ti, double* out) {
+    const double zr = 0.5 * (w2 - w1), n1 = w1 * w1 + zi * zi, n2 = w2 * w2 + zi * zi;
+    const double l1 = 0.5 * log(n1);
+    const double dl = zr >= 0.0 ? 0.5 * log1p(4.0 * zr / n1) : -0.5 * log1p(-4.0 * zr / n2);  // log|z+1| - log|z-1|
+    const double ang = atan2(-2.0 * zi, zi * zi - w1 * w2);                                   // arg(z+1) - arg(z-1)
+    const double q0r = 0.5 * dl, q0i = 0.5 * ang;
+    // rho = |z + sqrt(z^2 - 1)|, the growth of the recurrence
+    const float s = 0.5f * (sqrtf((float)n1) + sqrtf((float)n2));
+    const float rho = s + sqrtf(fmaxf(s * s - 1.0f, 0.0f));
+    double Ar = 0.0, Ai = 0.0, Br = 0.0, Bi = 0.0, Sr = 0.0, Si = 0.0;
+    // s_n = g_(n-1)/(2n - 1) - g_(n+1)/(2n + 3), g_0 apart
+    auto add = [&](int n, double qr, double qi, double gm, double gn, double gp) {
+        double sn = 0.0;
+        if (n >= 2) sn = gm / (2 * n - 1);
+        if (n + 1 < N) sn -= gp / (2 * n + 3);
+        Sr = fma(sn, qr, Sr);
+        Si = fma(sn, qi, Si);
+        if (n < N) {
+            const double pn = p[n * kOffTasks], tn = T[n * kOffTasks];
+            Ar = fma(pn, qr, Ar);
+            Ai = fma(pn, qi, Ai);
+            Br = fma(tn, qr, fma(-gn, qi, Br));
+            Bi = fma(tn, qi, fma(gn, qr, Bi));
         }
+    };
+    if (rho < kOffForward) {
+        double qr = q0r, qi = q0i, rr = zr * q0r - zi * q0i - 1.0, ri = zr * q0i + zi * q0r;  // Q_n, Q_(n+1)
+        double gm = 0.0, gn = g[0];
+        for (int n = 0; n <= N; ++n) {
+            const double gp = n + 1 < N ? g[(n + 1) * kOffTasks] : 0.0;
+            add(n, qr, qi, gm, gn, gp);
+            gm = gn;
+            gn = gp;
+            const double4 c = C[n + 1];
+            const double xr = c.z * (zr * rr - zi * ri) - c.w * qr, xi = c.z * (zr * ri + zi * rr) - c.w * qi;
+            qr = rr;
+            qi = ri;
+            rr = xr;
+            ri = xi;
+        }
+    } else {
+        int n = N + 1 + (int)(18.5f / logf(rho));
+        double qr = 1e-100, qi = 0.0, rr = 0.0, ri = 0.0;  // q_n, q_(n+1)
+        for (; n > N; --n) {
+            const double4 c = C[n];
+            const double xr = c.x * (zr * qr - zi * qi) - c.y * rr, xi = c.x * (zr * qi + zi * qr) - c.y * ri;
+            rr = qr;
+            ri = qi;
+            qr = xr;
+            qi = xi;
+        }
+        double gp = 0.0, gn = 0.0;
+        for (; n >= 0; --n) {
+            const double gm = n >= 1 ? g[(n - 1) * kOffTasks] : 0.0;
+            add(n, qr, qi, gm, gn, gp);
+            if (n == 0) break;
+            gp = gn;
+            gn = gm;
+            const double4 c = C[n];
+            const double xr = c.x * (zr * qr - zi * qi) - c.y * rr, xi = c.x * (zr * qi + zi * qr) - c.y * ri;
+            rr = qr;
+            ri = qi;
+            qr = xr;
+            qi = xi;
+        }
+        // all sums times Q_0 / q_0
+        const double m = 1.0 / (qr * qr + qi * qi);
+        const double fr = m * (q0r * qr + q0i * qi), fi = m * (q0i * qr - q0r * qi);
+        const double a = Ar * fi + Ai * fr;
+        Ai = a;
+        const double br = Br * fr - Bi * fi;
+        Bi = Br * fi + Bi * fr;
+        Br = br;
+        Sr = Sr * fr - Si * fi;
+    }
+    const double L0 = w1 * l1 + w2 * (l1 + dl) - zi * ang - 2.0;  // int log|x - z| dx
+    out[0] = fma(logs + 0.5 * L0, g[0], Sr + 2.0 * Ai);
+    // -2 i conj(tau) B
+    const double cr = tr * Br - ti * Bi, ci = tr * Bi + ti * Br;
+    out[1] = 2.0 * ci;
+    out[2] = -2.0 * cr;
+}
+
+__global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_constant__ OffArgs a) {
+    extern __shared__ double off_sm[];
+    __shared__ OffLeaf lf[kOffMaxU];
+    __shared__ double s_far[3], s_in[3], s_edge[2][3];
+    __shared__ double leg[4][kOffMaxN];  // P_m(x), P_m'(x), P_n(y), P_n'(y) at the point in an inside leaf
+    __shared__ int s_b;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, k = a.k, kk = k * k, N = 2 * k + 1;
+    const int nrows = off_first(k, 4);
+    double* cf = off_sm;                            // [nrows][kOffMaxU]
+    double* fs = cf + nrows * kOffMaxU;             // [kk][kOffMaxU], then the traces
+    double* tp = fs;                                // [3][N][kOffTasks]: P, normal, tangential derivative
+    double *tg = tp + N * kOffTasks, *tt = tg + N * kOffTasks;
+    const int64_t pt = blockIdx.x;
+    const double px = a.x[pt], py = a.y[pt];
     if (tid == 0) {
         // the leaf holding the point: integer coordinates at the finest level, a descent from the root
         const double X = (px - a.lox) / a.width, Y = (py - a.loy) / a.width;
@@ -100,36 +388,134 @@ __global__ void __launch_bounds__(kOffThreads) offnode_kernel(OffArgs a) {
     __syncthreads();
     const int b = s_b;
     if (b < 0) {  // outside the closed root box, or a NaN coordinate
-        if (tid == 0) a.u[p] = a.ux[p] = a.uy[p] = __longlong_as_double(0x7ff8000000000000ll);
+        if (tid == 0) a.u[pt] = a.ux[pt] = a.uy[pt] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
+    const int u0 = a.uptr[b], nu = a.uptr[b + 1] - u0;
+    if (tid < nu) {
+        const int s = a.uidx[u0 + tid];
+        const double h = ldexp(a.width, -a.level[s]);
+        OffLeaf L;
+        L.h = h;
+        L.leaf = a.leaf_of_box[s];
+        const double x0 = a.lox + a.ix[s] * h, y0 = a.loy + a.iy[s] * h;
+        L.d[0] = (px - x0) / h;
+        L.d[1] = (x0 + h - px) / h;
+        L.d[2] = (py - y0) / h;
+        L.d[3] = (y0 + h - py) / h;
+        L.inside = L.d[0] >= 0.0 && L.d[1] >= 0.0 && L.d[2] >= 0.0 && L.d[3] >= 0.0;
+        if (L.inside)
+            for (int i = 0; i < 4; ++i) L.d[i] = fmax(L.d[i], 1e-30);
+        lf[tid] = L;
+    }
+    __syncthreads();
+    // the leaves' values in the four classes: sums over the mirrored nodes
+    {
+        const int hx = (k + 1) / 2;
+        for (int q = tid; q < nu * hx * hx; q += kOffThreads) {
+            const int u = q / (hx * hx), e = q - u * hx * hx, j = e / hx, i = e - j * hx;
+            const double* f = a.f + (size_t)lf[u].leaf * kk;
+            const double v0 = f[j * k + i], v1 = f[j * k + k - 1 - i];
+            const double v2 = f[(k - 1 - j) * k + i], v3 = f[(k - 1 - j) * k + k - 1 - i];
+            const double s0 = v0 + v1, d0 = v0 - v1, s1 = v2 + v3, d1 = v2 - v3;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int nx = sym_half(k, c & 1);
+                if (i >= nx || j >= sym_half(k, c >> 1)) continue;
+                const double v = (c & 1) ? ((c >> 1) ? d0 - d1 : d0 + d1) : ((c >> 1) ? s0 - s1 : s0 + s1);
+                fs[(off_val(k, c) + j * nx + i) * kOffMaxU + u] = v;
+            }
+        }
+    }
+    __syncthreads();
+    for (int r = tid; r < nrows; r += kOffThreads) {
+        int c = 0;
+        while (c < 3 && r >= off_first(k, c + 1)) ++c;
+        const int K = sym_half(k, c & 1) * sym_half(k, c >> 1);
+        off_coeffs_n<kOffMaxU>(nu, a.t.G + a.t.g_off[c] + (r - off_first(k, c)), K, off_rows(k, c),
+                               fs + off_val(k, c) * kOffMaxU, cf + r * kOffMaxU);
+    }
+    __syncthreads();
+    // traces. Edges 0..3 = bottom, right, top, left, run around the leaf counterclockwise (top and left
+    // against their coordinate: a factor (-1)^n). (leaf, axis, n): n along the edge, the sum across it
+    for (int q = tid; q < nu * 2 * N; q += kOffThreads) {
+        const int u = q % nu, e = q / nu, axis = e & 1, n = e >> 1;
+        double sp[2] = {0.0, 0.0}, sg[2] = {0.0, 0.0};  // even and odd coefficients across
+#pragma unroll
+        for (int par = 0; par < 2; ++par) {
+            const int c = axis == 0 ? (n & 1) | (par << 1) : par | ((n & 1) << 1);  // axis 0: bottom and top
+            for (int m = par; m + n <= 2 * k; m += 2) {
+                const int row = axis == 0 ? off_row0(k, c, n >> 1) + (m >> 1) : off_row0(k, c, m >> 1) + (n >> 1);
+                const double v = cf[row * kOffMaxU + u];
+                sp[par] += v;
+                sg[par] = fma((double)(m * (m + 1)), v, sg[par]);
+            }
+        }
+        const double sgn = (n & 1) ? -1.0 : 1.0;
+        const int lo = 4 * u + (axis == 0 ? 0 : 3), hi = 4 * u + (axis == 0 ? 2 : 1);
+        const double flo = axis == 0 ? 1.0 : sgn, fhi = axis == 0 ? sgn : 1.0;
+        tp[n * kOffTasks + lo] = flo * (sp[0] - sp[1]);
+        tg[n * kOffTasks + lo] = flo * (sg[0] - sg[1]);
+        tp[n * kOffTasks + hi] = fhi * (sp[0] + sp[1]);
+        tg[n * kOffTasks + hi] = fhi * (sg[0] + sg[1]);
+    }
+    __syncthreads();
+    for (int q = tid; q < 4 * nu * N; q += kOffThreads) {
+        const int e = q % (4 * nu), n = q / (4 * nu);
+        double s = 0.0;
+        for (int m = n + 1; m < N; m += 2) s += tp[m * kOffTasks + e];
+        tt[n * kOffTasks + e] = (4 * n + 2) * s;
+    }
+    __syncthreads();
     const double h = ldexp(a.width, -a.level[b]);
-    const double cxb = a.lox + ((double)a.ix[b] + 0.5) * h, cyb = a.loy + ((double)a.iy[b] + 0.5) * h;
-    const double inv2pi = 0.15915494309189533577;
-    const int P = a.P;
-    if (tid < 32) {
+    const double inv2pi = 0.15915494309189533577, pi = 3.14159265358979323846;
+    if (warp < 2) {
+        // one edge per lane
+        const int e = tid;
+        double v[3] = {0.0, 0.0, 0.0};
+        if (e < 4 * nu) {
+            const OffLeaf L = lf[e >> 2];
+            const int s = e & 3;
+            // (end - point, point - start) along the edge, distance inwards
+            const double w1 = 2.0 * (s == 0 ? L.d[1] : (s == 1 ? L.d[3] : (s == 2 ? L.d[0] : L.d[2])));
+            const double w2 = 2.0 * (s == 0 ? L.d[0] : (s == 1 ? L.d[2] : (s == 2 ? L.d[1] : L.d[3])));
+            const double zi = 2.0 * (s == 0 ? L.d[2] : (s == 1 ? L.d[1] : (s == 2 ? L.d[3] : L.d[0])));
+            edge_terms(w1, w2, zi, tp + e, tg + e, tt + e, N, a.t.C, log(0.5 * L.h),
+                       s == 0 ? 1.0 : (s == 2 ? -1.0 : 0.0), s == 1 ? -1.0 : (s == 3 ? 1.0 : 0.0), v);
+            v[0] *= L.h * L.h;
+            v[1] *= L.h;
+            v[2] *= L.h;
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+            if (lane == 0) s_edge[warp][i] = v[i];
+        }
+    } else if (warp == 2) {
         // far part: b's local expansion at zeta = (t - z_b)/h (lanes split the coefficients), then the
         // W multipoles (lanes split the boxes); fixed-order shuffle sums
+        const int P = a.P;
+        const double cxb = a.lox + ((double)a.ix[b] + 0.5) * h, cyb = a.loy + ((double)a.iy[b] + 0.5) * h;
         const double zr = (px - cxb) / h, zi = (py - cyb) / h;
         double phr = 0.0, dr = 0.0, di = 0.0;
         const double* L = a.Lexp + (size_t)b * a.R * 2 * P;
-        for (int l = tid; l < P; l += 32) {
+        for (int l = lane; l < P; l += 32) {
             // zeta^l and l zeta^(l-1) by repeated multiplication (l <= 63)
-            double pr = 1.0, pi = 0.0, qr = 0.0, qi = 0.0;  // zeta^l, zeta^(l-1)
+            double pr = 1.0, pi_ = 0.0, qr = 0.0, qi = 0.0;  // zeta^l, zeta^(l-1)
             for (int e = 0; e < l; ++e) {
                 qr = pr;
-                qi = pi;
-                const double t = pr * zr - pi * zi;
-                pi = pr * zi + pi * zr;
+                qi = pi_;
+                const double t = pr * zr - pi_ * zi;
+                pi_ = pr * zi + pi_ * zr;
                 pr = t;
             }
             const double br = L[2 * l], bi = L[2 * l + 1];
-            phr += br * pr - bi * pi;
+            phr += br * pr - bi * pi_;
             dr += l * (br * qr - bi * qi) / h;  // Phi' = (1/h) sum_l l b~_l zeta^(l-1)
             di += l * (br * qi + bi * qr) / h;
         }
         // W list: box c of width h/2 at offset (dx, dy) (units of h/4 in the pattern): zeta_w = 2 (zeta - D)
-        for (int e = a.wptr[b] + tid; e < a.wptr[b + 1]; e += 32) {
+        for (int e = a.wptr[b] + lane; e < a.wptr[b + 1]; e += 32) {
             const int c = a.widx[e];
             const int cfg = a.wcfg[e];
             int qx, qy;
@@ -164,84 +550,63 @@ __global__ void __launch_bounds__(kOffThreads) offnode_kernel(OffArgs a) {
             dr += __shfl_xor_sync(0xffffffffu, dr, o);
             di += __shfl_xor_sync(0xffffffffu, di, o);
         }
-        if (tid == 0) {
+        if (lane == 0) {
             s_far[0] = -inv2pi * phr;
             s_far[1] = -inv2pi * dr;
             s_far[2] = inv2pi * di;
         }
-    }
-    // near part, one neighbour leaf after another
-    double n0 = 0.0, n1 = 0.0, n2 = 0.0;
-    for (int e = a.uptr[b]; e < a.uptr[b + 1]; ++e) {
-        const int s = a.uidx[e];
-        const int ls = a.leaf_of_box[s];
-        const double hs = ldexp(a.width, -a.level[s]);
-        const double cxs = a.lox + ((double)a.ix[s] + 0.5) * hs, cys = a.loy + ((double)a.iy[s] + 0.5) * hs;
-        __syncthreads();  // sC, pcs free
-        // Chebyshev coefficients of f~_s: tmp[j][m] = sum_i A[m][i] V[j][i], C[n][m] = sum_j A[n][j] tmp[j][m]
-        const double* V = a.f + (size_t)ls * kk;
-        for (int q = tid; q < kk; q += blockDim.x) {
-            const int j = q / k, m = q - j * k;
-            double acc = 0.0;
-            for (int i = 0; i < k; ++i) acc += a.A[m * 16 + i] * V[j * k + i];
-            sTmp[q] = acc;
-        }
-        if (tid == 0) s_npc = make_pieces(px, py, cxs, cys, hs, pcs);
-        __syncthreads();
-        for (int q = tid; q < kk; q += blockDim.x) {
-            const int nn = q / k, m = q - nn * k;
-            double acc = 0.0;
-            for (int j = 0; j < k; ++j) acc += a.A[nn * 16 + j] * sTmp[j * k + m];
-            sC[q] = acc;
-        }
-        __syncthreads();
-        const int npc = s_npc;
-        // the rule: distance from the point to the boundary of the closed source box
-        const double lox = cxs - hs / 2, hix = cxs + hs / 2, loy = cys - hs / 2, hiy = cys + hs / 2;
-        const double ox = fmax(fmax(lox - px, px - hix), 0.0), oy = fmax(fmax(loy - py, py - hiy), 0.0);
-        const double din = fmin(fmin(px - lox, hix - px), fmin(py - loy, hiy - py));
-        const double d = (ox > 0.0 || oy > 0.0) ? sqrt(ox * ox + oy * oy) : din;  // 0 on the boundary
-        const int rule = (d <= 0.0 || d >= 0.25 * hs) ? 0 : (d >= 1e-3 * hs ? 1 : 2);
-        const int N = 2 * off_half(rule) + 1;
-        const int o0 = off_first(rule);
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-        const int total = npc * N * N;
-        for (int g = tid; g < total; g += blockDim.x) {
-            const int ip = g / (N * N), rem = g - ip * N * N;
-            const int js = o0 + rem / N, jt = o0 + rem % N;
-            const DENode ds{sDE[0][js], sDE[1][js], sDE[2][js]};
-            const DENode dt{sDE[0][jt], sDE[1][jt], sDE[2][jt]};
-            double w3[3], yx, yy;
-            node_weights(pcs[ip], px, py, ds, dt, w3, &yx, &yy);
-            // f~_s at y: sum_n T_n(y^) sum_m C[n][m] T_m(x^), x^, y^ in [-1, 1]
-            const double xh = 2.0 * (yx - cxs) / hs, yh = 2.0 * (yy - cys) / hs;
-            double tx[16];
-            tx[0] = 1.0;
-            if (k > 1) tx[1] = xh;
-            for (int m = 2; m < k; ++m) tx[m] = 2.0 * xh * tx[m - 1] - tx[m - 2];
-            double fv = 0.0, tm2 = 0.0, tm1 = 0.0;
-            for (int nn = 0; nn < k; ++nn) {
-                const double tn = nn == 0 ? 1.0 : (nn == 1 ? yh : 2.0 * yh * tm1 - tm2);
-                tm2 = tm1;
-                tm1 = tn;
-                double row = 0.0;
-                for (int m = 0; m < k; ++m) row += sC[nn * k + m] * tx[m];
-                fv += tn * row;
+    } else if (warp == 3) {
+        // 2 pi P and pi F in the leaves that hold the point (one, or those that share its edge or corner)
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int u = 0; u < nu; ++u) {
+            const OffLeaf L = lf[u];
+            if (!L.inside) continue;
+            __syncwarp();
+            if (lane < 2) {
+                const double x = L.d[2 * lane] - L.d[2 * lane + 1];  // 2 x in [-1, 1]
+                double p0 = 1.0, p1 = x, q0 = 0.0, q1 = 1.0;        // P_m, P_m' (p1, q1: m + 1)
+                for (int m = 0; m < N; ++m) {
+                    leg[2 * lane][m] = p0;
+                    leg[2 * lane + 1][m] = 2.0 * q0;
+                    const double4 c = a.t.C[m + 1];
+                    const double p2 = c.z * x * p1 - c.w * p0, q2 = fma((double)(2 * m + 3), p1, q0);
+                    p0 = p1;
+                    p1 = p2;
+                    q0 = q1;
+                    q1 = q2;
+                }
             }
-            a0 += w3[0] * fv;
-            a1 += w3[1] * fv;
-            a2 += w3[2] * fv;
+            __syncwarp();
+            double w[3] = {0.0, 0.0, 0.0};
+            for (int m = lane; m < N; m += 32)
+                for (int n = 0; m + n <= 2 * k; ++n) {
+                    const double cmn = cf[(off_row0(k, (m & 1) | ((n & 1) << 1), m >> 1) + (n >> 1)) * kOffMaxU + u];
+                    w[0] = fma(cmn, leg[0][m] * leg[2][n], w[0]);
+                    w[1] = fma(cmn, leg[1][m] * leg[2][n], w[1]);
+                    w[2] = fma(cmn, leg[0][m] * leg[3][n], w[2]);
+                }
+            v[0] = fma(L.h * L.h, w[0], v[0]);
+            v[1] = fma(L.h, w[1], v[1]);
+            v[2] = fma(L.h, w[2], v[2]);
         }
-        n0 += block_sum(a0, red);
-        n1 += block_sum(a1, red);
-        n2 += block_sum(a2, red);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+            if (lane == 0) s_in[i] = 2.0 * pi * v[i];
+        }
     }
     __syncthreads();
     if (tid == 0) {
-        a.u[p] = s_far[0] + n0;
-        a.ux[p] = s_far[1] + n1;
-        a.uy[p] = s_far[2] + n2;
+        // gradient: (u_x, u_y) = -(1/2pi) (Re Phi', -Im Phi')
+        a.u[pt] = s_far[0] - inv2pi * ((s_edge[0][0] + s_edge[1][0]) + s_in[0]);
+        a.ux[pt] = s_far[1] - inv2pi * ((s_edge[0][1] + s_edge[1][1]) + s_in[1]);
+        a.uy[pt] = s_far[2] - inv2pi * (s_in[2] - (s_edge[0][2] + s_edge[1][2]));
     }
+}
+
+static size_t off_smem(int k) {
+    const size_t rows = (size_t)off_first(k, 4) * kOffMaxU;
+    return (rows + std::max((size_t)k * k * kOffMaxU, (size_t)3 * (2 * k + 1) * kOffTasks)) * sizeof(double);
 }
 
 }  // namespace vfmm
@@ -291,18 +656,15 @@ extern "C" int vfmm_evaluate_points(const vfmm_tree* tree, const vfmm_ops* ops, 
     a.u = u_dev;
     a.ux = ux_dev;
     a.uy = uy_dev;
-    const int k = ops->k;
-    const double pi = 3.14159265358979323846;
-    for (int m = 0; m < 16; ++m)
-        for (int i = 0; i < 16; ++i) {
-            double v = 0.0;
-            if (m < k && i < k) {
-                const double th = pi * (2 * i + 1) / (2.0 * k);  // x_i = -cos(th), T_m(x_i) = cos(m (pi - th))
-                v = (m == 0 ? 1.0 : 2.0) / k * std::cos(m * (pi - th));
-            }
-            a.A[m * 16 + i] = v;
-        }
-    offnode_kernel<<<(unsigned)n_points, kOffThreads, 0, (cudaStream_t)stream>>>(a);
+    a.t = *(const OffTables*)ops->off;
+    static thread_local int attr_dev = -1;
+    int dev = 0;
+    VFMM_CUDA(cudaGetDevice(&dev));
+    if (attr_dev != dev) {
+        VFMM_CUDA(cudaFuncSetAttribute(offnode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)off_smem(16)));
+        attr_dev = dev;
+    }
+    offnode_kernel<<<(unsigned)n_points, kOffThreads, off_smem(ops->k), (cudaStream_t)stream>>>(a);
     VFMM_CUDA(cudaGetLastError());
     return VFMM_OK;
 }

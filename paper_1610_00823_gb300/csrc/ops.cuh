@@ -22,6 +22,8 @@ struct vfmm_ops {
     double* l2t = nullptr;    // [3kk][2(p+1)] real
     // FP64 form: every table product in the reflection classes of the square (SymTables, sym.cuh)
     void* sym = nullptr;
+    // leaf values -> inverse Laplacian, for the potential at arbitrary points (OffTables, offnode.cu)
+    void* off = nullptr;
     // split-precision near-field operands (VFMM_MIXED)
     void* mixed = nullptr;
     // plane-wave M2L (FP64 form, planewave.cu): rule length s, outgoing [p][s] lambda^(n-1)/(n-1)!,
@@ -42,6 +44,8 @@ void mixed_free(vfmm_ops* o);
 void free_ops(vfmm_ops* o);
 int planewave_prepare(vfmm_ops* o, cudaStream_t st);
 void planewave_free(vfmm_ops* o);
+int offnode_prepare(vfmm_ops* o, cudaStream_t st);
+void offnode_free(vfmm_ops* o);
 int pw_stride(int S);
 size_t planewave_work_doubles(int64_t n_boxes, const vfmm_ops& o);
 int planewave_m2l(const vfmm_ops& o, int begin, int n_boxes, const int32_t* vptr, const int32_t* vidx,

@@ -389,6 +389,7 @@ static int create(int k, int p, int precision, cudaStream_t st, vfmm_ops* o) {
     VFMM_CUDA(cudaMalloc(&o->near, (size_t)kNearCfg * 3 * kk * kk * sizeof(double)));
     near_table_kernel<<<dim3(kk, kNearCfg), 256, 0, st>>>(k, o->xhat, d_bw, o->near);
     VFMM_CUDA(cudaGetLastError());
+    VFMM_CHECK(offnode_prepare(o, st));  // its host work runs beside the tables' quadrature
     // S2M from 1-D moments
     std::vector<double> gx, gw;
     int ng = (k + p) / 2 + 4;
@@ -481,6 +482,7 @@ void free_ops(vfmm_ops* o) {
     mixed_free(o);
     planewave_free(o);
     sym_free(o);
+    offnode_free(o);
 }
 
 }  // namespace vfmm
