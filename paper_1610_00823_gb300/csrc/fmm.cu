@@ -1850,15 +1850,15 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
     struct Job {
         SplitPlan* P;
         const void* a;
-        const CUtensorMap* map;
+        const void* map;
         int Kp, Rp;
         float2* out;
         size_t rows;
         int slices;
-    } jobs[4] = {{&PS->near, w.mix.fsl, &mo->tm_near, mo->Kp, mo->Rp, w.mix.out, T.n_leaves * R, mo->slices[kCtrNear]},
-                 {&PS->m2l, w.mix.msl, &mo->tm_m2l, mo->Kx, mo->Rx, w.mix.m2l_out, T.n_boxes * R, mo->slices[kCtrM2L]},
-                 {&PS->s2l, w.mix.fsl, &mo->tm_s2l, mo->Kp, mo->Rx, w.mix.s2l_out, T.n_boxes * R, mo->slices[kCtrS2L]},
-                 {&PS->far, w.mix.aprep, &mo->tm_far, mo->Kx, mo->Rp, w.mix.far_out, T.n_leaves * R,
+    } jobs[4] = {{&PS->near, w.mix.fsl, mo->tsl, mo->Kp, mo->Rp, w.mix.out, T.n_leaves * R, mo->slices[kCtrNear]},
+                 {&PS->m2l, w.mix.msl, mo->m2l_sl, mo->Kx, mo->Rx, w.mix.m2l_out, T.n_boxes * R, mo->slices[kCtrM2L]},
+                 {&PS->s2l, w.mix.fsl, mo->s2l_sl, mo->Kp, mo->Rx, w.mix.s2l_out, T.n_boxes * R, mo->slices[kCtrS2L]},
+                 {&PS->far, w.mix.aprep, mo->far_sl, mo->Kx, mo->Rp, w.mix.far_out, T.n_leaves * R,
                   mo->slices[kCtrFar]}};
     cudaEvent_t e0, e1;
     VFMM_CUDA(cudaEventCreate(&e0));
@@ -1877,7 +1877,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
             float total = 0.0f;
             for (int rep = 0; rep < 4 && rc == VFMM_OK; ++rep) {
                 cudaEventRecord(e0, st);
-                rc = split_gemm(*P, jb.a, *jb.map, jb.Kp, jb.Rp, jb.out, w.mix.err, part, jb.rows, jb.slices, st);
+                rc = split_gemm(*P, jb.a, jb.map, jb.Kp, jb.Rp, jb.out, w.mix.err, part, jb.rows, jb.slices, st);
                 cudaEventRecord(e1, st);
                 if (rc != VFMM_OK) break;
                 cudaError_t e = cudaEventSynchronize(e1);
@@ -1908,7 +1908,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
             float total = 0.0f;
             for (int rep = 0; rep < 4 && rc == VFMM_OK; ++rep) {
                 cudaEventRecord(e0, st);
-                rc = split_gemm(*P, jb.a, *jb.map, jb.Kp, jb.Rp, jb.out, w.mix.err, part, jb.rows, jb.slices, st);
+                rc = split_gemm(*P, jb.a, jb.map, jb.Kp, jb.Rp, jb.out, w.mix.err, part, jb.rows, jb.slices, st);
                 cudaEventRecord(e1, st);
                 if (rc != VFMM_OK) break;
                 cudaError_t e = cudaEventSynchronize(e1);

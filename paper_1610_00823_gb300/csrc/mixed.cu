@@ -21,12 +21,15 @@
 //    2^(E_f + E_r) and by h^2 (potential) or h (gradient) in FP64.
 //
 // Tile: 128 rows on the M side (TMEM lanes) x 80 on the N side; which side holds the table rows
-// (by TMA) and which the gathered operand rows (by cp.async) depends on the contraction
+// (by bulk copies) and which the gathered operand rows (by cp.async) depends on the contraction
 // (near_transposed). For every table of a group and every K block of 32 values the S slices of
 // both go into a 64-byte-swizzled K-major stage (two stages); one thread issues the
 // S(S+1)/2 x 2 UMMAs (128 x N x 16) into the six TMEM accumulators; tcgen05.commit frees the
 // stage and, after the last K block of a drain group, hands the accumulators to the epilogue.
 // Every mbarrier wait is bounded and reports a timeout through an error word.
+// Table tiles lie in memory as the stage wants them (table_at), one bulk copy per stage; as 64-byte boxes
+// of a tensor map the same bytes took the longer part of a K block: near field 14.26 -> 13.27 ms on
+// 200,104 leaves, 184 -> 163 us on 1,378.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -76,13 +79,13 @@ __global__ void table_row_exp_kernel(const double* __restrict__ T, int R, int kk
     }
 }
 
-// tsl[cfg][r][i][k] (rows r >= R and columns k >= kk are zero)
-__global__ void table_slice_kernel(const double* __restrict__ T, int R, int kk, int Rp, int Kp,
+// slices of tables T[cfg][R][kk] in tiles (rows r >= R and columns k >= kk are zero)
+__global__ void table_slice_kernel(const double* __restrict__ T, int R, int kk, int Rp, int tile, int Kp,
                                    const int* __restrict__ Er, bf16* __restrict__ tsl) {
     const int cfg = blockIdx.y, r = blockIdx.x;
     for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
         double v = (r < R && k < kk) ? T[((size_t)cfg * R + r) * kk + k] : 0.0;
-        slice_fixed(v, r < R ? Er[r] : 0, tsl + slice_off((size_t)cfg * Rp + r, Kp, k), kKBlock);
+        slice_fixed(v, r < R ? Er[r] : 0, tsl + table_at(cfg, Rp, tile, Kp, r, k), tile * kKBlock);
     }
 }
 
@@ -134,7 +137,8 @@ __device__ __forceinline__ void named_bar_sync(int id, int count) {
 
 
 struct SplitArgs {
-    const bf16* asl;      // A rows [rows][Kp / 32][kSlices][32]; the tables come through the tensor map
+    const bf16* asl;      // A rows [rows][Kp / 32][kSlices][32]
+    const bf16* tab;      // tables (table_at)
     const int32_t* gptr;  // [n_groups + 1] into gcfg
     const int32_t* gcfg;  // table of each (group, table) entry
     const int32_t* gsrc;  // [entries][128] A row or -1
@@ -164,17 +168,22 @@ __device__ __forceinline__ void issue_unit(uint32_t tmem, uint64_t ad0, uint64_t
 #pragma unroll
     for (int i = 1; i <= S; ++i)
 #pragma unroll
-        for (int j = 1; j <= S; ++j) {
-            if (i + j > S + 1) continue;
-            const int acc = acc_of(i, j);
-            // first product of accumulator acc in (i, j) order: i == 1 for acc < kNumAcc - 1, else (1, kNumAcc)
-            const bool first_of_acc = (acc < kNumAcc - 1) ? (i == 1) : (i == 1 && j == kNumAcc);
+        for (int ks = 0; ks < kKBlock / 16; ++ks) {
+            // the S + 1 - i products of one A tile in a row: it is read from shared memory once
+            const uint64_t ad = ad0 + (((i - 1) * A_SLICE + ks * 32) >> 4);
+            const int n = S + 1 - i;
 #pragma unroll
-            for (int ks = 0; ks < kKBlock / 16; ++ks) {
-                const uint64_t ad = ad0 + (((i - 1) * A_SLICE + ks * 32) >> 4);
+            for (int j = 1; j <= n; ++j) {
+                const int acc = acc_of(i, j);
+                // first product of accumulator acc in (i, j) order: i == 1 for acc < kNumAcc - 1, else (1, kNumAcc)
+                const bool first_of_acc = (acc < kNumAcc - 1) ? (i == 1) : (i == 1 && j == kNumAcc);
                 const uint64_t bd = bd0 + (((j - 1) * B_SLICE + ks * 32) >> 4);
                 const uint32_t accum = (kFirst && first_of_acc && ks == 0) ? 0u : 1u;
-                tc::umma_bf16(tmem + acc * N, ad, bd, idesc, accum);
+                const uint32_t d = tmem + acc * N;
+                if (n == 1) tc::umma_bf16<tc::CollectA::kDiscard>(d, ad, bd, idesc, accum);
+                else if (j == 1) tc::umma_bf16<tc::CollectA::kFill>(d, ad, bd, idesc, accum);
+                else if (j < n) tc::umma_bf16<tc::CollectA::kUse>(d, ad, bd, idesc, accum);
+                else tc::umma_bf16<tc::CollectA::kLastUse>(d, ad, bd, idesc, accum);
             }
         }
 }
@@ -185,7 +194,7 @@ __device__ __forceinline__ void issue_unit(uint32_t tmem, uint64_t ad0, uint64_t
 // N: the MMA's N (TMEM columns per accumulator): 80, or 48 for the 48-row tables of small
 // expansions (targets on M only).
 template <int N>
-__global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, const __grid_constant__ CUtensorMap tmB) {
+__global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
     extern __shared__ unsigned char dsm[];
     __shared__ __align__(8) uint64_t bars[2 * kStages + 3];
     __shared__ uint32_t tmem_holder;
@@ -197,7 +206,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
     constexpr uint32_t B_SLICE = N * 64;
     constexpr uint32_t STAGE = kSlices * (A_SLICE + B_SLICE);
     constexpr int HALF = N / 2;  // columns per epilogue warp
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool tr = a.transposed != 0;     // table rows on M (TMA into the A region), targets on N
     const int G = tr ? kTileN : kTileM;    // gathered rows (targets) per group
     const uint32_t base = tc::smem_u32(dsm);
@@ -209,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
     const uint32_t mma_done = tc::smem_u32(&bars[2 * kStages + 2]);  // used only after an abort
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
-            tc::mbar_init(full0 + 8 * s, kProducerThreads + 1);  // cp.async producers + the TMA issuer
+            tc::mbar_init(full0 + 8 * s, kProducerThreads + 1);  // cp.async producers + the bulk copy's issuer
             tc::mbar_init(empty0 + 8 * s, 1);
         }
         tc::mbar_init(acc_full, 1);
@@ -226,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
-    const uint32_t tmem = tmem_holder;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_holder, 0);
     // Work items (group g, split share sp, row chunk rc), item = (g * split + sp) * nchunks + rc; this
     // CTA takes items blockIdx.x, blockIdx.x + gridDim.x, ... (one item per CTA unless the launch
     // caps the grid). Within an item, units = (table, K block) pairs of the group in table order;
@@ -255,14 +264,12 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
     int issued = 0;  // producers: units (CTA-wide count) whose copies were started
 
     if (warp >= kEpilogueWarps && warp < kMmaWarp) {
-        // ------------------------------------------------ producers: table tile by TMA (one thread),
+        // ------------------------------------------------ producers: table tile by a bulk copy (one thread),
         // gathered source rows by cp.async (all producer threads)
         const int ptid = tid - kEpilogueThreads;
-        if (ptid == 0) tc::tma_prefetch_desc(&tmB);
         int gu = 0;
         for (int it = blockIdx.x; it < n_items && !p_abort; it += gridDim.x) {
             const Item x = item(it);
-            const int r0 = x.rc * (tr ? kTileM : N);  // first table row of this item's tile
             for (int u = 0; u < x.U; ++u, ++gu) {
                 const int s = gu & 1;
                 if (gu >= 2 && !tc::mbar_wait(empty0 + 8 * s, ((gu >> 1) - 1) & 1, &abort_flag)) p_abort = 1;
@@ -282,15 +289,15 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
                     named_bar_sync(1, kProducerThreads);
                 }
                 const uint32_t sA = sbase + s * STAGE, sB = sA + kSlices * A_SLICE;
-                // table tile by TMA into the region of its side, gathered rows into the other
+                // table tile into the region of its side, gathered rows into the other
                 const uint32_t sT = tr ? sA : sB, sG = tr ? sB : sA;
                 const uint32_t T_SLICE = tr ? A_SLICE : B_SLICE, G_SLICE = tr ? B_SLICE : A_SLICE;
                 if (ptid == 0) {
-                    // boxes of (128 or 80) table rows x 64 bytes (one per slice), SW64-swizzled by TMA
+                    // the slices of one K block of the tile: one contiguous, already swizzled piece
                     tc::mbar_arrive_expect_tx(full0 + 8 * s, a.slices * T_SLICE);
-                    for (int sl_i = 0; sl_i < a.slices; ++sl_i)
-                        tc::tma_load_3d(sT + sl_i * T_SLICE, &tmB, 0, kb * kSlices + sl_i, cfg * a.Rp + r0,
-                                        full0 + 8 * s);
+                    const size_t tile = ((size_t)cfg * a.nchunks + x.rc) * nkb + kb;
+                    tc::bulk_copy_g2s(sT, reinterpret_cast<const char*>(a.tab) + tile * (kSlices * T_SLICE),
+                                      a.slices * T_SLICE, full0 + 8 * s);
                 }
                 // a warp instruction covers 8 rows x 64 bytes of one slice: 512 contiguous bytes of
                 // shared memory (no bank conflicts) from eight 64-byte pieces of global memory
@@ -311,26 +318,29 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
         }
         tc::cp_async_wait_all();
     } else if (warp == kMmaWarp) {
-        // ------------------------------------------------ MMA issuer: one unit at a time
-        if (lane == 0) {
+        // ------------------------------------------------ MMA issuer: one unit at a time, the whole
+        // warp in step (umma_bf16 and umma_commit elect the lane that issues)
+        {
             const uint64_t adesc_base = tc::smem_desc(sbase, 16, 512, tc::kLayoutSwizzle64B);
             int gu = 0, dg = 0;  // units and drain groups of this CTA so far
             bool stop = false;
+            auto wait = [&](uint32_t bar, uint32_t parity, int code) {
+                if (__all_sync(0xffffffffu, tc::mbar_wait(bar, parity, &abort_flag))) return true;
+                abort_flag = 1;
+                if (lane == 0) atomicExch(a.err, code);
+                return false;
+            };
             for (int it = blockIdx.x; it < n_items && !stop; it += gridDim.x) {
                 const Item x = item(it);
                 for (int u = 0; u < x.U; ++u, ++gu) {
                     // a drain group = DU consecutive units of an item summed in the same accumulators;
                     // before one starts, the epilogue must have drained the previous one
-                    if (u % DU == 0 && dg > 0 && !tc::mbar_wait(acc_empty, (dg - 1) & 1, &abort_flag)) {
-                        abort_flag = 1;
-                        atomicExch(a.err, 4);
+                    if (u % DU == 0 && dg > 0 && !wait(acc_empty, (dg - 1) & 1, 4)) {
                         stop = true;
                         break;
                     }
                     const int s = gu & 1;
-                    if (!tc::mbar_wait(full0 + 8 * s, (gu >> 1) & 1, &abort_flag)) {
-                        abort_flag = 1;
-                        atomicExch(a.err, 2);
+                    if (!wait(full0 + 8 * s, (gu >> 1) & 1, 2)) {
                         stop = true;
                         break;
                     }
@@ -443,9 +453,10 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
         if (tid == kEpilogueThreads)
             for (int u = issued - 2; u < issued; ++u)
                 if (u >= 0) tc::mbar_wait(full0 + 8 * (u & 1), (u >> 1) & 1, &never, 1ll << 27);
-        if (warp == kMmaWarp && lane == 0) {
+        if (warp == kMmaWarp) {
             tc::umma_commit(mma_done);
             tc::mbar_wait(mma_done, 0, &never, 1ll << 27);
+            __syncwarp();
         }
         __syncthreads();
     }
@@ -456,39 +467,6 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a, co
 }
 
 // ---------------------------------------------------------------- host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-int make_table_map(const void* base, int64_t rows, int Kp, int box_rows, CUtensorMap* out) {
-    static EncodeTiledFn encode = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            encode = (EncodeTiledFn)fn;
-    });
-    if (!encode) return fail(VFMM_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
-    if (Kp % kKBlock || rows < box_rows || rows > (int64_t)INT32_MAX || ((uintptr_t)base & 15) || box_rows < 1 ||
-        box_rows > 256)
-        return fail(VFMM_ERR_INTERNAL, "table shape not suitable for a tensor map");
-    // [rows][Kp / 32 K blocks][8 slices][32 values]: dim 0 = 32 values (64 bytes, one swizzle row),
-    // dim 1 = (K block, slice) segments, dim 2 = rows
-    const cuuint64_t nseg = (cuuint64_t)(Kp / kKBlock) * kSlices;
-    const cuuint64_t dims[3] = {(cuuint64_t)kKBlock, nseg, (cuuint64_t)rows};
-    const cuuint64_t strides[2] = {(cuuint64_t)kKBlock * 2, nseg * kKBlock * 2};
-    const cuuint32_t box[3] = {(cuuint32_t)kKBlock, 1, (cuuint32_t)box_rows};
-    const cuuint32_t es[3] = {1, 1, 1};
-    CUresult r = encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(VFMM_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
-    return VFMM_OK;
-}
-
 int mixed_prepare(vfmm_ops* o, cudaStream_t st) {
     if (o->k * o->k * 3 > 4096) return fail(VFMM_ERR_INVALID_ARG, "mixed precision supports k <= 16");
     MixedOps* mo = new MixedOps();
@@ -503,10 +481,10 @@ int mixed_prepare(vfmm_ops* o, cudaStream_t st) {
     VFMM_CUDA(cudaMemsetAsync(mo->Er, 0, mo->Rp * sizeof(int), st));
     VFMM_CUDA(cudaMalloc(&mo->tsl, (size_t)kNearCfg * mo->Rp * kSlices * mo->Kp * sizeof(bf16)));
     table_row_exp_kernel<<<R, 256, 0, st>>>(o->near, R, kk, mo->Er);
-    table_slice_kernel<<<dim3(mo->Rp, kNearCfg), 128, 0, st>>>(o->near, R, kk, mo->Rp, mo->Kp, mo->Er, (bf16*)mo->tsl);
+    table_slice_kernel<<<dim3(mo->Rp, kNearCfg), 128, 0, st>>>(o->near, R, kk, mo->Rp, tile_rows, mo->Kp, mo->Er,
+                                                               (bf16*)mo->tsl);
     VFMM_CUDA(cudaGetLastError());
     VFMM_CUDA(cudaStreamSynchronize(st));
-    VFMM_CHECK(make_table_map(mo->tsl, (int64_t)kNearCfg * mo->Rp, mo->Kp, tile_rows, &mo->tm_near));
     return far_prepare(o, st);
 }
 
@@ -705,7 +683,7 @@ void free_plan_set(PlanSet* ps) {
 static size_t smem_bytes(int N) { return (size_t)kStages * kSlices * (kTileM * 64 + N * 64) + 1024; }
 
 template <int N>
-static int launch_split(const SplitArgs& a, const CUtensorMap& bmap, int grid, cudaStream_t st) {
+static int launch_split(const SplitArgs& a, int grid, cudaStream_t st) {
     static thread_local int attr_dev = -1;  // the attribute is per device
     int dev = 0;
     VFMM_CUDA(cudaGetDevice(&dev));
@@ -714,13 +692,13 @@ static int launch_split(const SplitArgs& a, const CUtensorMap& bmap, int grid, c
                                        (int)smem_bytes(N)));
         attr_dev = dev;
     }
-    split_gemm_kernel<N><<<(unsigned)grid, kThreads, smem_bytes(N), st>>>(a, bmap);
+    split_gemm_kernel<N><<<(unsigned)grid, kThreads, smem_bytes(N), st>>>(a);
     VFMM_CUDA(cudaGetLastError());
     return VFMM_OK;
 }
 
-static int launch_split_n(int n, const SplitArgs& a, const CUtensorMap& bmap, int grid, cudaStream_t st) {
-    return n == kTileNSmall ? launch_split<kTileNSmall>(a, bmap, grid, st) : launch_split<kTileN>(a, bmap, grid, st);
+static int launch_split_n(int n, const SplitArgs& a, int grid, cudaStream_t st) {
+    return n == kTileNSmall ? launch_split<kTileNSmall>(a, grid, st) : launch_split<kTileN>(a, grid, st);
 }
 
 
@@ -752,7 +730,7 @@ __global__ void split_reduce_kernel(const float2* __restrict__ part, size_t stri
     out[o] = df_final(hi, lo);
 }
 
-int split_gemm(const SplitPlan& P, const void* asl, const CUtensorMap& bmap, int Kp, int Rp, float2* out, int* err,
+int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, int Rp, float2* out, int* err,
                float2* part, size_t n_out_rows, int slices, cudaStream_t st, cudaEvent_t* ev, int defer) {
     if (slices < kMinSlices || slices > kSlices) return fail(VFMM_ERR_INTERNAL, "slice count out of range");
     if (ev) VFMM_CUDA(cudaEventRecord(ev[0], st));
@@ -765,6 +743,7 @@ int split_gemm(const SplitPlan& P, const void* asl, const CUtensorMap& bmap, int
     const int n_mma = mma_n(P.transposed, Rp);
     SplitArgs a;
     a.asl = (const bf16*)asl;
+    a.tab = (const bf16*)tables;
     a.gptr = P.ptr;
     a.gcfg = P.cfg;
     a.gsrc = P.src;
@@ -787,7 +766,7 @@ int split_gemm(const SplitPlan& P, const void* asl, const CUtensorMap& bmap, int
         a.part_stride = 0;
         a.out = part;
         a.n_items = P.n_groups * a.nchunks;
-        VFMM_CHECK(launch_split_n(n_mma, a, bmap, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
+        VFMM_CHECK(launch_split_n(n_mma, a, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
         // deferred: the consumer sums each target's slab rows itself (same order)
         const int64_t n = (defer & kDeferSegments) ? 0 : (int64_t)P.n_seg * P.R * Rp;
         if (n > 0)
@@ -801,7 +780,7 @@ int split_gemm(const SplitPlan& P, const void* asl, const CUtensorMap& bmap, int
     a.part_stride = n_out_rows * (size_t)Rp;
     a.out = a.split > 1 ? part : out;
     a.n_items = P.n_groups * a.split * a.nchunks;
-    VFMM_CHECK(launch_split_n(n_mma, a, bmap, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
+    VFMM_CHECK(launch_split_n(n_mma, a, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
     if (a.split > 1 && !(defer & kDeferSplits)) {
         const int64_t n = (int64_t)P.n_groups * P.group * Rp;
         split_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part, a.part_stride, a.split, P.tgt,
@@ -945,7 +924,7 @@ int near_slices(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const
 
 int near_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const MixedWork& w, cudaStream_t st) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
-    return split_gemm(PS.near, w.fsl, mo->tm_near, mo->Kp, mo->Rp, w.out, w.err, w.part_side,
+    return split_gemm(PS.near, w.fsl, mo->tsl, mo->Kp, mo->Rp, w.out, w.err, w.part_side,
                       (size_t)T.n_leaves * PS.R, mo->slices[kCtrNear], st, w.cev ? w.cev + 0 : nullptr);
 }
 

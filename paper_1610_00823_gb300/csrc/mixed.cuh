@@ -1,7 +1,6 @@
 // Split-BF16 near field: constants and device buffers.
 #pragma once
 
-#include <cuda.h>  // CUtensorMap (the encoder is fetched through the runtime's driver entry point)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -160,26 +159,35 @@ __device__ __forceinline__ void slice8_fixed(const double* v, int E, __nv_bfloat
     for (int i = 0; i < kSlices; ++i) *reinterpret_cast<uint4*>(out + (size_t)i * stride) = *reinterpret_cast<uint4*>(tmp[i]);
 }
 
+// Sliced tables are stored tile by tile in the shared-memory image of a stage: [table][row tile][K block]
+// [slice][tile row][64 bytes], each 64-byte row (32 values) in the 64-byte swizzle of the MMA operand
+// (16-byte chunk c of row m at c ^ (m / 2 mod 4)). The slices that a contraction takes of one K block are
+// one contiguous piece, fetched by one bulk copy. Offset (elements) of (table, slice 0, row, k) for
+// tables of Rp rows in tiles of `tile` rows and Kp columns; slice i lies i * tile * kKBlock further on.
+__host__ __device__ inline size_t table_at(size_t table, int Rp, int tile, int Kp, int row, int k) {
+    const int rt = row / tile, m = row - rt * tile, kb = k / kKBlock, kk = k - kb * kKBlock;
+    return ((((table * (Rp / tile) + rt) * (Kp / kKBlock) + kb) * kSlices * tile) + m) * kKBlock +
+           ((((kk >> 3) ^ (m >> 1)) & 3) << 3) + (kk & 7);
+}
+
 struct MixedOps {
     int N = kTileN; // table rows per tile
     int Rp = 0;     // 3k^2 rounded up to N
     int Kp = 0;     // k^2 rounded up to kKBlock
-    void* tsl = nullptr;  // bf16 [33][Rp][kSlices][Kp]
+    void* tsl = nullptr;  // bf16 tables (table_at): near field, 33
     int* Er = nullptr;    // [Rp] row exponents
-    // TMA descriptors of the sliced tables (box = 80 rows x 64 bytes of one slice and K block)
-    CUtensorMap tm_near, tm_s2m, tm_m2l, tm_far, tm_s2l;
     // far field: expansion coefficients as reals (Re, Im of 0..p), Kx = 2(p+1) padded
     int Kx = 0;           // 2(p+1) rounded up to kKBlock
     int Rx = 0;           // 2p rounded up to 48 (2p <= 48) or to kTileN (rows of S2M and M2L without coefficient 0)
-    void* s2m_sl = nullptr;   // bf16 [1][Rx][kSlices][Kp]: S2M rows 2..2p+1
+    void* s2m_sl = nullptr;   // bf16 table: S2M rows 2..2p+1
     int* s2m_E = nullptr;     // [Rx]
     // M2L rows 2..2p+1 over input columns 0..2p+1, column k scaled by 2^-floor(k/4) (the decay
     // bound of multipole coefficient k/2), then per row by 2^-m2l_E[r]
-    void* m2l_sl = nullptr;   // bf16 [40][Rx][kSlices][Kx]
+    void* m2l_sl = nullptr;   // bf16 tables, 40
     int* m2l_E = nullptr;     // [Rx]
-    void* far_sl = nullptr;   // bf16 [21][Rp][kSlices][Kx]: L2T (0) and M2T per W configuration
+    void* far_sl = nullptr;   // bf16 tables, 21: L2T (0) and M2T per W configuration
     int* far_E = nullptr;     // [Rp]
-    void* s2l_sl = nullptr;   // bf16 [20][Rx][kSlices][Kp]: S2L rows of coefficients 1..p
+    void* s2l_sl = nullptr;   // bf16 tables, 20: S2L rows of coefficients 1..p
     int* s2l_E = nullptr;     // [Rx]
     double* s2l_r0 = nullptr; // [20][kk] FP64: Re of S2L row 0
     double* m2l_r0 = nullptr; // [40][p+1] complex FP64: M2L row 0 (output coefficient 0) per offset
@@ -276,11 +284,8 @@ int build_split_plan(const PlanItems& I, const std::vector<int32_t>& order, int 
 // whose slab fits keeps the form not chosen in P->alt.
 int build_contraction_plan(const PlanItems& I, int n_tables, int n_chunks, int R, bool transposed, int nkb,
                            double slab_overhead, size_t slab_row_bytes, PlanArena& A, SplitPlan* P);
-// Tensor map of a sliced table [rows][Kp / 32][kSlices][32] BF16 for the table operand of split_gemm
-// (box = box_rows rows x 64 bytes of one slice and K block).
-int make_table_map(const void* base, int64_t rows, int Kp, int box_rows, CUtensorMap* out);
 // ev (optional): a (start, stop) event pair recorded around the contraction and its reduction.
-int split_gemm(const SplitPlan& P, const void* asl, const CUtensorMap& bmap, int Kp, int Rp, float2* out, int* err,
+int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, int Rp, float2* out, int* err,
                float2* part, size_t n_out_rows, int slices, cudaStream_t st, cudaEvent_t* ev = nullptr,
                int defer = 0);
 // split_gemm's `defer` bits: the consumer of the output sums the entry-major slab rows of each

@@ -57,17 +57,17 @@ __global__ void rows_exp_kernel(const double* __restrict__ M, int nc, int R, int
     if (threadIdx.x == 0) E[r] = exp_of(red[0]);
 }
 
-// out[c][r][i][k] = slice i of M[c][r][k] / 2^E[r]; rows >= R and columns >= K are zero.
-__global__ void rows_slice_kernel(const double* __restrict__ M, int R, int K, int Rp, int Kp,
+// slices of M[c][r][k] / 2^E[r] in tiles; rows >= R and columns >= K are zero.
+__global__ void rows_slice_kernel(const double* __restrict__ M, int R, int K, int Rp, int tile, int Kp,
                                   const int* __restrict__ E, bf16* __restrict__ out) {
     const int r = blockIdx.x, c = blockIdx.y;
     for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
         double v = (r < R && k < K) ? M[((size_t)c * R + r) * K + k] : 0.0;
-        slice_fixed(v, r < R ? E[r] : 0, out + slice_at((size_t)c * Rp + r, Kp, k), kKBlock);
+        slice_fixed(v, r < R ? E[r] : 0, out + table_at(c, Rp, tile, Kp, r, k), tile * kKBlock);
     }
 }
 
-static int slice_table(const std::vector<double>& M, int nc, int R, int K, int Rp, int Kp, void** out, int** E,
+static int slice_table(const std::vector<double>& M, int nc, int R, int K, int Rp, int tile, int Kp, void** out, int** E,
                        cudaStream_t st) {
     double* dM = nullptr;
     VFMM_CUDA(cudaMalloc(&dM, M.size() * sizeof(double)));
@@ -76,7 +76,7 @@ static int slice_table(const std::vector<double>& M, int nc, int R, int K, int R
     VFMM_CUDA(cudaMemsetAsync(*E, 0, Rp * sizeof(int), st));
     VFMM_CUDA(cudaMalloc(out, (size_t)nc * Rp * kSlices * Kp * sizeof(bf16)));
     rows_exp_kernel<<<R, 256, 0, st>>>(dM, nc, R, K, *E);
-    rows_slice_kernel<<<dim3(Rp, nc), 128, 0, st>>>(dM, R, K, Rp, Kp, *E, (bf16*)*out);
+    rows_slice_kernel<<<dim3(Rp, nc), 128, 0, st>>>(dM, R, K, Rp, tile, Kp, *E, (bf16*)*out);
     VFMM_CUDA(cudaGetLastError());
     VFMM_CUDA(cudaStreamSynchronize(st));
     cudaFree(dM);
@@ -96,8 +96,7 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
     VFMM_CUDA(cudaMemcpy(s2m.data(), o->s2m, s2m.size() * sizeof(double), cudaMemcpyDeviceToHost));
     std::vector<double> S((size_t)2 * p * kk);
     std::copy(s2m.begin() + 2 * kk, s2m.end(), S.begin());
-    VFMM_CHECK(slice_table(S, 1, 2 * p, kk, mo->Rx, mo->Kp, &mo->s2m_sl, &mo->s2m_E, st));
-    VFMM_CHECK(make_table_map(mo->s2m_sl, mo->Rx, mo->Kp, rx_tile, &mo->tm_s2m));
+    VFMM_CHECK(slice_table(S, 1, 2 * p, kk, mo->Rx, rx_tile, mo->Kp, &mo->s2m_sl, &mo->s2m_E, st));
     // M2L as real matrices: rows 2..2p+1, columns 0..2p+1
     std::vector<double> mt((size_t)kVCfg * P * P * 2);
     VFMM_CUDA(cudaMemcpy(mt.data(), o->m2l_t, mt.size() * sizeof(double), cudaMemcpyDeviceToHost));
@@ -116,7 +115,7 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
     // n = k / 2) carries the bound 2^-floor(n/2); the operand is divided by it and the table times it
     for (size_t r = 0; r < (size_t)kVCfg * mo->Rx; ++r)
         for (int q = 0; q < mo->Kx; ++q) MR[r * mo->Kx + q] = std::ldexp(MR[r * mo->Kx + q], -(q >> 2));
-    VFMM_CHECK(slice_table(MR, kVCfg, mo->Rx, mo->Kx, mo->Rx, mo->Kx, &mo->m2l_sl, &mo->m2l_E, st));
+    VFMM_CHECK(slice_table(MR, kVCfg, mo->Rx, mo->Kx, mo->Rx, rx_tile, mo->Kx, &mo->m2l_sl, &mo->m2l_E, st));
     {
         // output coefficient 0 stays FP64: its row of every M2L matrix, [offset][n] complex
         std::vector<double> r0((size_t)kVCfg * P * 2);
@@ -128,7 +127,6 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
         VFMM_CUDA(cudaMalloc(&mo->m2l_r0, r0.size() * sizeof(double)));
         VFMM_CUDA(cudaMemcpy(mo->m2l_r0, r0.data(), r0.size() * sizeof(double), cudaMemcpyHostToDevice));
     }
-    VFMM_CHECK(make_table_map(mo->m2l_sl, (int64_t)kVCfg * mo->Rx, mo->Kx, rx_tile, &mo->tm_m2l));
     // leaf tables: 0 = L2T without coefficient 0, 1 + c = M2T of W configuration c
     std::vector<double> l2t((size_t)R * 2 * P), xh(k);
     VFMM_CUDA(cudaMemcpy(l2t.data(), o->l2t, l2t.size() * sizeof(double), cudaMemcpyDeviceToHost));
@@ -166,9 +164,7 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
             }
         }
     }
-    VFMM_CHECK(slice_table(F, 1 + kFarCfg, R, KX, mo->Rp, mo->Kx, &mo->far_sl, &mo->far_E, st));
-    VFMM_CHECK(make_table_map(mo->far_sl, (int64_t)(1 + kFarCfg) * mo->Rp, mo->Kx,
-                              table_rows_per_tile(near_transposed(o->k)), &mo->tm_far));
+    VFMM_CHECK(slice_table(F, 1 + kFarCfg, R, KX, mo->Rp, table_rows_per_tile(near_transposed(o->k)), mo->Kx, &mo->far_sl, &mo->far_E, st));
     // S2L: rows 2..2p+1 (Re, Im of coefficients 1..p) over the k*k source values; row 0 kept in FP64
     std::vector<double> st_((size_t)kFarCfg * kk * P * 2);
     VFMM_CUDA(cudaMemcpy(st_.data(), o->s2l_t, st_.size() * sizeof(double), cudaMemcpyDeviceToHost));
@@ -181,8 +177,7 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
                 XL[((size_t)c * 2 * p + 2 * (l - 1) + 1) * kk + s] = st_[(((size_t)c * kk + s) * P + l) * 2 + 1];
             }
         }
-    VFMM_CHECK(slice_table(XL, kFarCfg, 2 * p, kk, mo->Rx, mo->Kp, &mo->s2l_sl, &mo->s2l_E, st));
-    VFMM_CHECK(make_table_map(mo->s2l_sl, (int64_t)kFarCfg * mo->Rx, mo->Kp, rx_tile, &mo->tm_s2l));
+    VFMM_CHECK(slice_table(XL, kFarCfg, 2 * p, kk, mo->Rx, rx_tile, mo->Kp, &mo->s2l_sl, &mo->s2l_E, st));
     VFMM_CUDA(cudaMalloc(&mo->s2l_r0, X0.size() * sizeof(double)));
     VFMM_CUDA(cudaMemcpy(mo->s2l_r0, X0.data(), X0.size() * sizeof(double), cudaMemcpyHostToDevice));
     return VFMM_OK;
@@ -415,7 +410,7 @@ __global__ void s2m_finish_kernel(int nleaf, int R, int kk, int p, int Rx, const
 int s2m_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, double* Mexp,
               const MixedWork& w, cudaStream_t st) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
-    VFMM_CHECK(split_gemm(PS.s2m, w.fsl, mo->tm_s2m, mo->Kp, mo->Rx, w.s2m_out, w.err, w.part,
+    VFMM_CHECK(split_gemm(PS.s2m, w.fsl, mo->s2m_sl, mo->Kp, mo->Rx, w.s2m_out, w.err, w.part,
                           (size_t)T.n_leaves * PS.R, mo->slices[kCtrS2M], st, w.cev ? w.cev + 2 : nullptr,
                           kDeferSplits));
     // the split-K partials (when the plan splits) are summed by the finishing kernel
@@ -487,14 +482,14 @@ int m2l_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const d
                                                                           w.glev, (bf16*)w.msl);
     VFMM_CUDA(cudaGetLastError());
     // split-K partials (grouped form) are summed by the downward kernels that read the locals
-    return split_gemm(PS.m2l, w.msl, mo->tm_m2l, mo->Kx, mo->Rx, w.m2l_out, w.err, w.part, (size_t)T.n_boxes * R,
+    return split_gemm(PS.m2l, w.msl, mo->m2l_sl, mo->Kx, mo->Rx, w.m2l_out, w.err, w.part, (size_t)T.n_boxes * R,
                       mo->slices[kCtrM2L], st, w.cev ? w.cev + 4 : nullptr, kDeferSplits);
 }
 
 // ---------------------------------------------------------------- S2L
 int s2l_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const MixedWork& w, cudaStream_t st) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
-    return split_gemm(PS.s2l, w.fsl, mo->tm_s2l, mo->Kp, mo->Rx, w.s2l_out, w.err, w.part_s2l,
+    return split_gemm(PS.s2l, w.fsl, mo->s2l_sl, mo->Kp, mo->Rx, w.s2l_out, w.err, w.part_s2l,
                       (size_t)T.n_boxes * PS.R, mo->slices[kCtrS2L], st, w.cev ? w.cev + 6 : nullptr);
 }
 
@@ -557,7 +552,7 @@ int far_leaf_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, co
                                                           T.far_slot, T.lptr[VFMM_LIST_W], T.lidx[VFMM_LIST_W], Mexp,
                                                           Lexp, w.Et, (bf16*)w.aprep);
     VFMM_CUDA(cudaGetLastError());
-    return split_gemm(PS.far, w.aprep, mo->tm_far, mo->Kx, mo->Rp, w.far_out, w.err, w.part,
+    return split_gemm(PS.far, w.aprep, mo->far_sl, mo->Kx, mo->Rp, w.far_out, w.err, w.part,
                       (size_t)T.n_leaves * PS.R, mo->slices[kCtrFar], st, w.cev ? w.cev + 8 : nullptr,
                       kDeferSegments);
 }

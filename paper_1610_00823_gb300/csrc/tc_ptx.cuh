@@ -47,26 +47,13 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// ---------------------------------------------------------------- TMA (cp.async.bulk.tensor)
-// Tiled 3-D load of one box into shared memory (layout and swizzle from the tensor map); the
-// bytes count against the transaction count of `bar`. c0 (innermost) must be a multiple of
-// 16 bytes' worth of elements.
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int c0, int c1, int c2, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(dst),
-        "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-        : "memory");
-}
+// ---------------------------------------------------------------- bulk copies
 // Plain bulk copy global -> shared of `bytes` (both addresses 16-byte aligned, bytes a multiple
 // of 16), counted against the transaction count of `bar`.
 __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
 }
 
 // ---------------------------------------------------------------- cp.async (16 B, L2 only)
@@ -122,19 +109,41 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// MMAs and commits are issued by one elected lane of a warp whose lanes all run the issuing code with the
+// same operands (elect.sync picks the same lane each time): the operands then stay in uniform registers.
+// From one divergent lane an MMA takes 44.6 cycles to issue, which is more than N <= 80 needs.
+//
+// The A collector buffer holds the A operand of an MMA for those that follow with the same descriptor:
+// the first of a run fills it, the others use it, the last one releases it, and each B operand then costs
+// its own shared-memory read only. Measured per M128 x Nn x K16 MMA in the slice-product order, cycles,
+// one lane without / elected lane with the collector: N = 80 52.0 / 41.6, N = 64 48.1 / 35.6,
+// N = 48 44.6 / 29.5 (N / 2 at the tensor pipe's rate).
+enum class CollectA { kDiscard, kFill, kUse, kLastUse };
+
+template <CollectA kOp>
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+#define VFMM_UMMA(collect)                                                                      \
+    asm volatile(                                                                               \
+        "{\n\t.reg .pred p, q;\n\t"                                                            \
+        "elect.sync _|q, 0xffffffff;\n\t"                                                       \
+        "setp.ne.b32 p, %4, 0;\n\t"                                                             \
+        "@q tcgen05.mma.cta_group::1.kind::f16" collect " [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem), \
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                                     \
+        : "memory")
+    if constexpr (kOp == CollectA::kFill) VFMM_UMMA(".collector::a::fill");
+    else if constexpr (kOp == CollectA::kUse) VFMM_UMMA(".collector::a::use");
+    else if constexpr (kOp == CollectA::kLastUse) VFMM_UMMA(".collector::a::lastuse");
+    else VFMM_UMMA("");
+#undef VFMM_UMMA
 }
-// Arrives on the mbarrier once every tcgen05 operation issued so far by this thread completed.
+// Arrives on the mbarrier once every tcgen05 operation issued so far by the elected lane completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
 }
 
 // 32 lanes x 32 consecutive 32-bit columns (one register per column per lane).
