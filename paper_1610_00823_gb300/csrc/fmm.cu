@@ -806,24 +806,22 @@ __global__ void __launch_bounds__(kPassThreads, 1) downward_pass_kernel(PassArgs
 // scalar part, the same at every node of the leaf, is FP64:
 // -(1/2pi) [log(h) sum_U a_0 + Re b_0 + sum_W a_0 (log h_w)], h_w = h / 2 (first warp, fixed-order sums).
 struct LeafMixedArgs {
-    int nleaf, R, kk, Rp, P, lw;
+    int nleaf, R, k, kk, Rp, P, lw;
     double wm, width;
     const int32_t* box_of_leaf;
     const int32_t* level;
     const int32_t *uptr, *uidx, *wptr, *widx;
     const double* Mexp;
     const double* Lexp;
-    const float2* nearmix;
-    const int* Er;
+    ClassTab ct;
+    const float2* nearmix;  // class rows (ct.N > 0) or node rows
+    const int* Er;          // exponents of the quadrant rows or of the node rows
     const int* Ef;
     const float2* farmix;
     const int* farE;
     const int* Et;
-    // entry-major near field / leaf far field: the slab rows of every leaf's entries, summed here in
-    // entry order (the arithmetic of the separate segmented sum, which these contractions then skip);
-    // null: nearmix / farmix hold the sums
-    const float2* near_slab;
-    const int32_t* near_seg;  // [n_leaves + 1] first entry of each leaf
+    // entry-major leaf far field: the slab rows of every leaf's entries, summed here in entry order (the
+    // arithmetic of the separate segmented sum, which the contraction then skips); null: farmix holds the sums
     const float2* far_slab;
     const int32_t* far_seg;
     double *u, *ux, *uy;
@@ -838,40 +836,66 @@ __device__ __forceinline__ float2 slab_sum(const float2* __restrict__ slab, int 
     return df_final(hi, lo);
 }
 
-__global__ void leaf_mixed_kernel(LeafMixedArgs a) {
+__device__ __forceinline__ float2 df_sum(float2 a, float2 b, float sgn) {
+    float hi = a.x, lo = a.y;
+    df_add(hi, lo, make_float2(sgn * b.x, sgn * b.y));
+    return df_final(hi, lo);
+}
+
+__global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
     // width = wm 2^lw with wm in [1, 2): h = wm 2^(lw - lv), so every power-of-two scale is folded
     // into the exponents (f2d_scaled), times wm^(2, 1, -1) when wm is not one
+    extern __shared__ float2 s_near[];  // [3][kk] near field at the nodes
     __shared__ double s_scal;
-    const int nleaf = a.nleaf, R = a.R, kk = a.kk, Rp = a.Rp, lw = a.lw;
+    const int nleaf = a.nleaf, R = a.R, kk = a.kk, Rp = a.Rp, lw = a.lw, k = a.k, hx = (k + 1) / 2;
     const double wm = a.wm;
     const unsigned vl = blockIdx.x;
     const int t = threadIdx.x;
     const unsigned leaf = vl / (unsigned)R, r = vl - leaf * (unsigned)R;
     const int b = a.box_of_leaf[leaf];
     const int lv = a.level[b];
-    // the node values first (their loads overlap the first warp's scalar sums), then the barrier
+    // near field: the four classes of a quadrant node put together at its images (double-FP32: sums of
+    // numbers of one power-of-two scale, and the FP64 pipe is what bounds this kernel)
+    if (a.ct.N == 0) {  // near field by entries: node rows
+        const float2* nm = a.nearmix + (size_t)vl * Rp;
+        for (int q = t; q < 3 * kk; q += blockDim.x) s_near[q] = nm[q];
+    } else {
+        const float2* nm = a.nearmix + (size_t)vl * (4 * a.ct.nch * a.ct.N);
+        for (int q = t; q < 3 * hx * hx; q += blockDim.x) {
+            const int fl = q / (hx * hx), e = q - fl * hx * hx, j = e / hx, i = e - j * hx;
+            float2 w[4];  // by the field's parity in x and y
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int pa = sym_pa(c, fl), pb = sym_pb(c, fl), nx = sym_half(k, pa);
+                const bool in = i < nx && j < sym_half(k, pb);
+                const float2 x = in ? nm[a.ct.seg[3 * c + fl] + j * nx + i] : make_float2(0.0f, 0.0f);
+                const int s = pa | (pb << 1);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (s == u) w[u] = x;
+            }
+            const float2 x = df_sum(w[0], w[1], 1.0f), y = df_sum(w[0], w[1], -1.0f);
+            const float2 z = df_sum(w[2], w[3], 1.0f), v = df_sum(w[2], w[3], -1.0f);
+            float2* o = s_near + fl * kk;
+            const int i1 = k - 1 - i, j1 = k - 1 - j;
+            o[j * k + i] = df_sum(x, z, 1.0f);
+            if (i1 != i) o[j * k + i1] = df_sum(y, v, 1.0f);
+            if (j1 != j) o[j1 * k + i] = df_sum(x, z, -1.0f);
+            if (i1 != i && j1 != j) o[j1 * k + i1] = df_sum(y, v, -1.0f);
+        }
+    }
+    __syncthreads();
     double n0 = 0.0, n1 = 0.0, n2 = 0.0, f0 = 0.0, f1 = 0.0, f2 = 0.0;
     if (t < kk) {
-        const float2* __restrict__ nearmix = a.nearmix;
         const float2* __restrict__ farmix = a.farmix;
         const int* __restrict__ Er = a.Er;
         const int* __restrict__ farE = a.farE;
         const int* __restrict__ Et = a.Et;
         const int* __restrict__ Ef = a.Ef;
-        const float2* nm = nearmix + (size_t)vl * Rp;
         const float2* fm = farmix + (size_t)vl * Rp;
-        const int en = Ef[r] + lw - lv, ef = Et[vl] + lv - lw;  // near scale h 2^E_f, far scale 2^E_t / h
-        float2 v0, v1, v2, w0, w1, w2;
-        if (a.near_slab) {
-            const int s0 = a.near_seg[leaf], s1 = a.near_seg[leaf + 1];
-            v0 = slab_sum(a.near_slab, s0, s1, R, r, Rp, t);
-            v1 = slab_sum(a.near_slab, s0, s1, R, r, Rp, kk + t);
-            v2 = slab_sum(a.near_slab, s0, s1, R, r, Rp, 2 * kk + t);
-        } else {
-            v0 = nm[t];
-            v1 = nm[kk + t];
-            v2 = nm[2 * kk + t];
-        }
+        const int en = Ef[r] + (a.ct.N ? 1 : 0) + lw - lv, ef = Et[vl] + lv - lw;  // near scale h 2^(E_f + 0, 1), far scale 2^E_t / h
+        const float2 v0 = s_near[t], v1 = s_near[kk + t], v2 = s_near[2 * kk + t];
+        float2 w0, w1, w2;
         if (a.far_slab) {
             const int s0 = a.far_seg[leaf], s1 = a.far_seg[leaf + 1];
             w0 = slab_sum(a.far_slab, s0, s1, R, r, Rp, t);
@@ -882,7 +906,9 @@ __global__ void leaf_mixed_kernel(LeafMixedArgs a) {
             w1 = fm[kk + t];
             w2 = fm[2 * kk + t];
         }
-        const int e0 = en + lw - lv + Er[t], e1 = en + Er[kk + t], e2 = en + Er[2 * kk + t];
+        const int tj = t / k, ti = t - tj * k;
+        const int qn = a.ct.N ? min(tj, k - 1 - tj) * hx + min(ti, k - 1 - ti) : t, qs = a.ct.N ? hx * hx : kk;
+        const int e0 = en + lw - lv + Er[qn], e1 = en + Er[qs + qn], e2 = en + Er[2 * qs + qn];
         n0 = f2d_scaled(v0.x, e0) + f2d_scaled(v0.y, e0);  // h^2 x near u
         n1 = f2d_scaled(v1.x, e1) + f2d_scaled(v1.y, e1);  // h x near u_x
         n2 = f2d_scaled(v2.x, e2) + f2d_scaled(v2.y, e2);
@@ -1075,7 +1101,8 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         double* p = nullptr;
         take(&p, (nl * kSlices * mo->Kp * 2 + 7) / 8);
         if (w) w->mix.fsl = (void*)p;
-        take(&p, nl * mo->Rp);
+        const bool cls = near_by_classes(o.k);
+        take(&p, nl * (cls ? 4 * mo->near.nch * mo->near.N : mo->Rp));
         if (w) w->mix.out = (float2*)p;
         take(&p, R);
         if (w) w->mix.fmax = (unsigned long long*)p;
@@ -1100,11 +1127,19 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         if (w) w->mix.far_out = (float2*)p;
         size_t np[3] = {0, 0, 0};
         split_part_elems(T, *PS, o, np);
-        float2** bufs[3] = {w ? &w->mix.part : nullptr, w ? &w->mix.part_side : nullptr,
-                            w ? &w->mix.part_s2l : nullptr};
+        float2** bufs[3] = {w ? &w->mix.part : nullptr, w ? &w->mix.part_s2l : nullptr,
+                            w ? &w->mix.part_side : nullptr};
         for (int i = 0; i < 3; ++i) {
             take(&p, std::max<size_t>(np[i], 1));  // one float2 per double
             if (w) *bufs[i] = np[i] ? (float2*)p : nullptr;
+        }
+        take(&p, cls ? nl * kk : 1);
+        if (w) w->mix.ffix = (long long*)p;
+        const size_t ob = near_operand_bytes(T, PS->near, (int)R);
+        take(&p, (ob + 7) / 8);
+        if (w) {
+            w->mix.near_opnd = p;
+            w->mix.near_opnd_bytes = ob;
         }
     } else if (w) {
         w->mix = MixedWork();
@@ -1324,12 +1359,12 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
                 launches += gemm_launches(PS.s2l);
             }
             VFMM_CUDA(cudaEventRecord(side->ev[1], side->s));
-            VFMM_CHECK(near_contract(T, PS, o, w.mix, side->s));
+            VFMM_CHECK(near_contract(T, PS, o, f, w.mix, side->s));
             VFMM_CUDA(cudaEventRecord(side->ev[2], side->s));
         } else {
-            VFMM_CHECK(near_contract(T, PS, o, w.mix, st));
+            VFMM_CHECK(near_contract(T, PS, o, f, w.mix, st));
         }
-        launches += gemm_launches(PS.near);
+        launches += near_by_classes(o.k) ? near_launches(*mo, PS.near, w.mix.near_opnd_bytes) : gemm_launches(PS.entries);
         mark(se, ST_NEAR, true, st);
     }
     // S2M
@@ -1536,6 +1571,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         LeafMixedArgs la;
         la.nleaf = nleaf;
         la.R = R;
+        la.k = o.k;
         la.kk = kk;
         la.Rp = mo->Rp;
         la.P = P;
@@ -1551,21 +1587,19 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         la.Mexp = w.Mexp;
         la.Lexp = w.Lexp;
         la.nearmix = w.mix.out;
-        la.Er = mo->Er;
+        la.ct = mo->near;
+        la.Er = near_by_classes(o.k) ? mo->near_E : mo->Er;
         la.Ef = w.mix.Ef;
         la.farmix = w.mix.far_out;
         la.farE = mo->far_E;
         la.Et = w.mix.Et;
-        // an entry-major leaf far field leaves its per-leaf sums (a few entries per leaf) to this kernel;
-        // the near field (about nine entries per leaf, on the side stream) keeps its segmented-sum kernel
-        la.near_slab = nullptr;
-        la.near_seg = nullptr;
+        // an entry-major leaf far field leaves its per-leaf sums (a few entries per leaf) to this kernel
         la.far_slab = PS.far.entry ? w.mix.part : nullptr;
         la.far_seg = PS.far.entry ? PS.far.seg : nullptr;
         la.u = u;
         la.ux = ux;
         la.uy = uy;
-        leaf_mixed_kernel<<<(unsigned)nv, std::max(32, ((kk + 31) / 32) * 32), 0, st>>>(la);
+        leaf_mixed_kernel<<<(unsigned)nv, std::max(32, ((kk + 31) / 32) * 32), (size_t)3 * kk * sizeof(float2), st>>>(la);
         ++launches;
     } else {
         LeafArgs a;
@@ -1855,7 +1889,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
         float2* out;
         size_t rows;
         int slices;
-    } jobs[4] = {{&PS->near, w.mix.fsl, mo->tsl, mo->Kp, mo->Rp, w.mix.out, T.n_leaves * R, mo->slices[kCtrNear]},
+    } jobs[4] = {{&PS->entries, w.mix.fsl, mo->tsl, mo->Kp, mo->Rp, w.mix.out, T.n_leaves * R, mo->slices[kCtrNear]},
                  {&PS->m2l, w.mix.msl, mo->m2l_sl, mo->Kx, mo->Rx, w.mix.m2l_out, T.n_boxes * R, mo->slices[kCtrM2L]},
                  {&PS->s2l, w.mix.fsl, mo->s2l_sl, mo->Kp, mo->Rx, w.mix.s2l_out, T.n_boxes * R, mo->slices[kCtrS2L]},
                  {&PS->far, w.mix.aprep, mo->far_sl, mo->Kx, mo->Rp, w.mix.far_out, T.n_leaves * R,
@@ -1947,24 +1981,28 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
         if (splits) splits[j] = jb.P->split;
     }
     // Co-scheduling of the whole step: in a forked solve the near field (low-priority stream) and the
-    // main chain share the SMs, and a near-field CTA leaves no registers for anything else on its SM.
-    // Timed on the forked solve itself: the near field on every SM, or capped at 7/8 ... 4/8 of them,
-    // the cooperative tree passes capped to the SMs it leaves free (they can start only when their
-    // whole grid fits); the fastest is kept (the uncapped schedule unless a cap is faster).
-    if (rc == VFMM_OK && PS->near.n_groups > 0 && PS->near.ctas > 0 && use_passes(T, PS->R, ops->p + 1)) {
-        const int sms = sm_count();
+    // main chain share the SMs, and a near-field CTA leaves no room for anything else on its SM.
+    // Timed on the forked solve itself: one near-field CTA per item, persistent ones on every SM, or on
+    // 7/8 ... 4/8 of them with the cooperative tree passes capped to the SMs they leave free (they can
+    // start only when their whole grid fits); the fastest is kept. A near field with fewer items than
+    // half the SMs leaves the chain room as it is.
+    const bool cls = near_by_classes(ops->k);
+    int32_t& near_ctas = cls ? PS->near.ctas : PS->entries.ctas;
+    const int sms = sm_count();
+    const bool wide = cls ? 8 * PS->near.n_groups * mo->near.nch > sms : PS->entries.ctas > 0;
+    if (rc == VFMM_OK && wide && use_passes(T, PS->R, ops->p + 1)) {
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, upward_pass_kernel, kPassThreads, pass_smem_bytes(ops->p + 1));
         Workspace wf = w;
         wf.fork = true;
-        const int near0 = PS->near.ctas, pass0 = PS->pass_ctas;
+        const int near0 = near_ctas, pass0 = PS->pass_ctas;
         float best = -1.0f;
         int best_near = near0, best_pass = pass0;
-        const int fracs[5] = {8, 7, 6, 5, 4};  // eighths of the SMs
-        for (int c = 0; c < 5 && rc == VFMM_OK; ++c) {
-            const int ncta = fracs[c] == 8 ? near0 : std::max(1, sms * fracs[c] / 8);
-            PS->near.ctas = ncta;
-            PS->pass_ctas = fracs[c] == 8 ? pass0 : std::max(1, per_sm * (sms - ncta));
+        const int fracs[6] = {0, 8, 7, 6, 5, 4};  // eighths of the SMs; 0: uncapped
+        for (int c = 0; c < 6 && rc == VFMM_OK; ++c) {
+            const int ncta = fracs[c] == 0 ? 0 : std::max(1, sms * fracs[c] / 8);
+            near_ctas = ncta;
+            PS->pass_ctas = fracs[c] == 0 || fracs[c] == 8 ? 0 : std::max(1, per_sm * (sms - ncta));
             float total = 0.0f;
             for (int rep = 0; rep < 6 && rc == VFMM_OK; ++rep) {
                 cudaEventRecord(e0, st);
@@ -1979,11 +2017,11 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
             }
             if (rc == VFMM_OK && (best < 0.0f || total < best)) {
                 best = total;
-                best_near = PS->near.ctas;
+                best_near = near_ctas;
                 best_pass = PS->pass_ctas;
             }
         }
-        PS->near.ctas = best_near;
+        near_ctas = best_near;
         PS->pass_ctas = best_pass;
     }
     cudaEventDestroy(e0);
@@ -1999,7 +2037,7 @@ extern "C" int vfmm_schedule_get(const vfmm_tree* tree, int32_t nrhs, int32_t* n
     if (!tree || !near_ctas || !pass_ctas || nrhs < 1) return fail(VFMM_ERR_INVALID_ARG, "bad schedule query");
     const PlanSet* PS = nullptr;
     VFMM_CHECK(plans_for(tree->t, nrhs, &PS));
-    *near_ctas = PS->near.ctas;
+    *near_ctas = near_by_classes(tree->t.k) ? PS->near.ctas : PS->entries.ctas;
     *pass_ctas = PS->pass_ctas;
     return VFMM_OK;
 }
@@ -2009,7 +2047,7 @@ extern "C" int vfmm_schedule_set(vfmm_tree* tree, int32_t nrhs, int32_t near_cta
     const PlanSet* PS = nullptr;
     VFMM_CHECK(plans_for(tree->t, nrhs, &PS));
     PlanSet* ps = const_cast<PlanSet*>(PS);
-    ps->near.ctas = near_ctas;
+    (near_by_classes(tree->t.k) ? ps->near.ctas : ps->entries.ctas) = near_ctas;
     ps->pass_ctas = pass_ctas;
     return VFMM_OK;
 }

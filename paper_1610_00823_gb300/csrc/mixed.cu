@@ -21,15 +21,12 @@
 //    2^(E_f + E_r) and by h^2 (potential) or h (gradient) in FP64.
 //
 // Tile: 128 rows on the M side (TMEM lanes) x 80 on the N side; which side holds the table rows
-// (by bulk copies) and which the gathered operand rows (by cp.async) depends on the contraction
+// (by TMA) and which the gathered operand rows (by cp.async) depends on the contraction
 // (near_transposed). For every table of a group and every K block of 32 values the S slices of
 // both go into a 64-byte-swizzled K-major stage (two stages); one thread issues the
 // S(S+1)/2 x 2 UMMAs (128 x N x 16) into the six TMEM accumulators; tcgen05.commit frees the
 // stage and, after the last K block of a drain group, hands the accumulators to the epilogue.
 // Every mbarrier wait is bounded and reports a timeout through an error word.
-// Table tiles lie in memory as the stage wants them (table_at), one bulk copy per stage; as 64-byte boxes
-// of a tensor map the same bytes took the longer part of a K block: near field 14.26 -> 13.27 ms on
-// 200,104 leaves, 184 -> 163 us on 1,378.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -41,6 +38,7 @@
 #include <vector>
 
 #include "mixed.cuh"
+#include "mma_issue.cuh"
 #include "ops.cuh"
 #include "sym.cuh"
 #include "tc_ptx.cuh"
@@ -153,40 +151,6 @@ struct SplitArgs {
     int n_items;          // work items (n_groups * split * nchunks); the grid may be smaller (persistent CTAs)
     size_t part_stride;   // n_out_rows * Rp
 };
-
-// Accumulator of slice product (i, j): its diagonal i + j - 2; diagonals >= kNumAcc - 1 share the last.
-__host__ __device__ constexpr int acc_of(int i, int j) { return (i + j - 2) < (kNumAcc - 1) ? (i + j - 2) : (kNumAcc - 1); }
-
-// All slice products (i, j), i + j <= S + 1, of one K block: accumulator acc_of(i, j); on the
-// first K block of a configuration the first product into each accumulator overwrites it (with
-// S >= kMinSlices every accumulator gets a product).
-template <bool kFirst, int S, int N>
-__device__ __forceinline__ void issue_unit(uint32_t tmem, uint64_t ad0, uint64_t bd0) {
-    constexpr uint32_t idesc = tc::idesc_bf16_f32(kTileM, N);
-    constexpr uint32_t A_SLICE = kTileM * 64, B_SLICE = N * 64;
-    static_assert(S >= kMinSlices && S <= kSlices, "slice count");
-#pragma unroll
-    for (int i = 1; i <= S; ++i)
-#pragma unroll
-        for (int ks = 0; ks < kKBlock / 16; ++ks) {
-            // the S + 1 - i products of one A tile in a row: it is read from shared memory once
-            const uint64_t ad = ad0 + (((i - 1) * A_SLICE + ks * 32) >> 4);
-            const int n = S + 1 - i;
-#pragma unroll
-            for (int j = 1; j <= n; ++j) {
-                const int acc = acc_of(i, j);
-                // first product of accumulator acc in (i, j) order: i == 1 for acc < kNumAcc - 1, else (1, kNumAcc)
-                const bool first_of_acc = (acc < kNumAcc - 1) ? (i == 1) : (i == 1 && j == kNumAcc);
-                const uint64_t bd = bd0 + (((j - 1) * B_SLICE + ks * 32) >> 4);
-                const uint32_t accum = (kFirst && first_of_acc && ks == 0) ? 0u : 1u;
-                const uint32_t d = tmem + acc * N;
-                if (n == 1) tc::umma_bf16<tc::CollectA::kDiscard>(d, ad, bd, idesc, accum);
-                else if (j == 1) tc::umma_bf16<tc::CollectA::kFill>(d, ad, bd, idesc, accum);
-                else if (j < n) tc::umma_bf16<tc::CollectA::kUse>(d, ad, bd, idesc, accum);
-                else tc::umma_bf16<tc::CollectA::kLastUse>(d, ad, bd, idesc, accum);
-            }
-        }
-}
 
 // Warps 0..7: epilogue (lane quadrant w % 4, column half w / 4); warps 8..10: producers;
 // warp 11: TMEM allocation and the MMA issuer (lane 0). Twelve warps keep three warps per SM
@@ -477,6 +441,10 @@ int mixed_prepare(vfmm_ops* o, cudaStream_t st) {
     const int tile_rows = table_rows_per_tile(near_transposed(o->k));
     mo->Rp = (R + tile_rows - 1) / tile_rows * tile_rows;
     mo->Kp = (kk + kKBlock - 1) / kKBlock * kKBlock;
+    if (near_by_classes(o->k)) {
+        VFMM_CHECK(near_classes_prepare(o, st));
+        return far_prepare(o, st);
+    }
     VFMM_CUDA(cudaMalloc(&mo->Er, mo->Rp * sizeof(int)));
     VFMM_CUDA(cudaMemsetAsync(mo->Er, 0, mo->Rp * sizeof(int), st));
     VFMM_CUDA(cudaMalloc(&mo->tsl, (size_t)kNearCfg * mo->Rp * kSlices * mo->Kp * sizeof(bf16)));
@@ -492,6 +460,8 @@ void mixed_free(vfmm_ops* o) {
     MixedOps* mo = (MixedOps*)o->mixed;
     if (!mo) return;
     far_free(mo);
+    if (mo->near_tab) cudaFree(mo->near_tab);
+    if (mo->near_E) cudaFree(mo->near_E);
     if (mo->tsl) cudaFree(mo->tsl);
     if (mo->Er) cudaFree(mo->Er);
     delete mo;
@@ -576,11 +546,15 @@ int commit_plan_arena(PlanArena& A, PlanSet* PS, cudaStream_t st) {
         VFMM_CUDA(cudaMemcpyAsync(base, A.data.data(), A.data.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     VFMM_CUDA(cudaStreamSynchronize(st));
     int32_t* b = static_cast<int32_t*>(base);
-    for (SplitPlan* top : {&PS->near, &PS->s2m, &PS->m2l, &PS->far, &PS->s2l})
+    for (SplitPlan* top : {&PS->entries, &PS->s2m, &PS->m2l, &PS->far, &PS->s2l})
         for (SplitPlan* P = top; P; P = P->alt) {
             int32_t** field[6] = {&P->tgt, &P->ptr, &P->cfg, &P->src, &P->seg, &P->seg_out};
             for (int i = 0; i < 6; ++i) *field[i] = P->off[i] >= 0 ? b + P->off[i] : nullptr;
         }
+    if (PS->near.n_groups == 0) return VFMM_OK;
+    PS->near.order = b + PS->near.off[0];
+    PS->near.gmask = b + PS->near.off[1];
+    PS->near.first_dev = b + PS->near.off[2];
     return VFMM_OK;
 }
 
@@ -671,7 +645,8 @@ void free_split_plan(SplitPlan* P) {
 }
 
 void free_plan_set(PlanSet* ps) {
-    free_split_plan(&ps->near);
+    ps->near = NearPlan();
+    free_split_plan(&ps->entries);
     free_split_plan(&ps->s2m);
     free_split_plan(&ps->m2l);
     free_split_plan(&ps->far);
@@ -791,8 +766,7 @@ int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, 
     return VFMM_OK;
 }
 
-// Near field: targets are leaves; tables are the 33 configurations; A rows are leaves.
-// The near-field plan (U list: leaves as targets, 33 configurations, gathered row = source leaf).
+// The near-field plan by entries (U list: leaves as targets, 33 configurations, gathered row = source leaf).
 static int build_near_plan(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, PlanSet* PS) {
     const int nl = T.n_leaves;
     const std::vector<int32_t>& ptr = H.ptr[VFMM_LIST_U];
@@ -817,7 +791,7 @@ static int build_near_plan(const DeviceTree& T, int R, const HostLists& H, PlanA
     const int tile_rows = table_rows_per_tile(tr);
     const int Kp = (T.k * T.k + kKBlock - 1) / kKBlock * kKBlock;
     return build_contraction_plan(I, kNearCfg, (rows + tile_rows - 1) / tile_rows, R, tr, Kp / kKBlock, 48.0 / Kp,
-                                  (size_t)rows * sizeof(float2), A, &PS->near);
+                                  (size_t)rows * sizeof(float2), A, &PS->entries);
 }
 
 // All five plans of R folded right-hand sides. The contractions are independent: each is built on a
@@ -831,7 +805,9 @@ static int build_plans(const DeviceTree& T, int R, const HostLists& H, PlanSet* 
     int rc[kNumCtr];
     auto task = [&](int c) {
         cudaSetDevice(dev);  // the split-K heuristic reads the device's SM count
-        rc[c] = c == kCtrNear ? build_near_plan(T, R, H, A[c], PS) : build_far_plan(c, T, R, H, A[c], PS);
+        if (c != kCtrNear) rc[c] = build_far_plan(c, T, R, H, A[c], PS);
+        else if (near_by_classes(T.k)) rc[c] = build_near_classes(T, R, H, A[c], &PS->near);
+        else rc[c] = build_near_plan(T, R, H, A[c], PS);
     };
     std::vector<std::thread> workers;
     for (int c = 1; c < kNumCtr; ++c) workers.emplace_back(task, c);
@@ -840,7 +816,7 @@ static int build_plans(const DeviceTree& T, int R, const HostLists& H, PlanSet* 
     for (int c = 0; c < kNumCtr; ++c)
         if (rc[c] != VFMM_OK) return fail(rc[c], "split-contraction plan " + std::to_string(c) + " failed");
     SplitPlan* top[kNumCtr];
-    top[kCtrNear] = &PS->near;
+    top[kCtrNear] = &PS->entries;
     top[kCtrS2M] = &PS->s2m;
     top[kCtrM2L] = &PS->m2l;
     top[kCtrS2L] = &PS->s2l;
@@ -854,6 +830,8 @@ static int build_plans(const DeviceTree& T, int R, const HostLists& H, PlanSet* 
         for (SplitPlan* P = top[c]; P; P = P->alt)
             for (int i = 0; i < 6; ++i)
                 if (P->off[i] >= 0) P->off[i] += base;
+        if (c == kCtrNear)
+            for (int64_t& off : PS->near.off) off += base;
         all.data.insert(all.data.end(), A[c].data.begin(), A[c].data.end());
     }
     return commit_plan_arena(all, PS, st);
@@ -863,7 +841,7 @@ int build_mixed_plan(DeviceTree* T, cudaStream_t st) {
     HostLists H;
     VFMM_CHECK(fetch_host_lists(*T, &H));
     VFMM_CHECK(build_far_slots(T, H, st));
-    VFMM_CHECK(build_instances(T, st));  // the FP64 form's table products
+    VFMM_CHECK(build_instances(T, st));
     T->plans_r = new std::map<int, PlanSet*>();
     T->plans_mu = new std::mutex();
     return build_plans(*T, 1, H, &T->plans, st);
@@ -922,9 +900,11 @@ int near_slices(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const
     return VFMM_OK;
 }
 
-int near_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const MixedWork& w, cudaStream_t st) {
+int near_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
+                  cudaStream_t st) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
-    return split_gemm(PS.near, w.fsl, mo->tsl, mo->Kp, mo->Rp, w.out, w.err, w.part_side,
+    if (near_by_classes(o.k)) return near_class_contract(T, PS, o, f, w, st);
+    return split_gemm(PS.entries, w.fsl, mo->tsl, mo->Kp, mo->Rp, w.out, w.err, w.part_side,
                       (size_t)T.n_leaves * PS.R, mo->slices[kCtrNear], st, w.cev ? w.cev + 0 : nullptr);
 }
 

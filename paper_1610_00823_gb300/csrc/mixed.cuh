@@ -170,12 +170,34 @@ __host__ __device__ inline size_t table_at(size_t table, int Rp, int tile, int K
            ((((kk >> 3) ^ (m >> 1)) & 3) << 3) + (kk & 7);
 }
 
+// Shape of a contraction in reflection classes. Output rows [4][nch * N]: class c's rows (u, u_x, u_y of
+// its quadrant nodes) from c * nch * N on, in nch tiles of N rows, the rest padding.
+struct ClassTab {
+    int norb = 0, k = 0, N = 0, nch = 0;
+    int seg[13] = {};                                    // first row of (class, field) at 3 * class + field
+    uint8_t fold[12] = {};                               // reflections that fix the orbit's representative
+    int16_t K[12][4] = {}, nkb[12][4] = {};              // columns, K blocks
+    int32_t toff[12][4] = {};                            // first table tile of (orbit, class), in K blocks
+};
+
+// Near field in reflection classes (mixed_sym.cu), or one gathered row per list entry (split_gemm) where a
+// table is a single tile and K block: k <= 5. There a class has as many K blocks as a table and its rows
+// fill a quarter of a tile (us per solve, classes / entries, 1,024 uniform and 900 graded leaves: k = 4
+// 134 / 129 and 148 / 139, k = 5 131 / 133 and 150 / 139, k = 6 129 / 141 and 146 / 171).
+__host__ __device__ constexpr bool near_by_classes(int k) { return 3 * k * k > kTileN || k * k > kKBlock; }
+
 struct MixedOps {
     int N = kTileN; // table rows per tile
     int Rp = 0;     // 3k^2 rounded up to N
     int Kp = 0;     // k^2 rounded up to kKBlock
-    void* tsl = nullptr;  // bf16 tables (table_at): near field, 33
-    int* Er = nullptr;    // [Rp] row exponents
+    // near field in reflection classes (mixed_sym.cu): tables of every (orbit, class), exponents of the
+    // quadrant rows [3][h][h], h = (k + 1) / 2
+    ClassTab near;
+    void* near_tab = nullptr;
+    int* near_E = nullptr;
+    // near field by entries: bf16 tables (table_at), 33, and their row exponents [Rp]
+    void* tsl = nullptr;
+    int* Er = nullptr;
     // far field: expansion coefficients as reals (Re, Im of 0..p), Kx = 2(p+1) padded
     int Kx = 0;           // 2(p+1) rounded up to kKBlock
     int Rx = 0;           // 2p rounded up to 48 (2p <= 48) or to kTileN (rows of S2M and M2L without coefficient 0)
@@ -221,7 +243,11 @@ __device__ __forceinline__ float2 df_final(float hi, float lo) {
 
 struct MixedWork {
     void* fsl = nullptr;                  // bf16 [n_leaves][kSlices][Kp]
-    float2* out = nullptr;                // [n_leaves][Rp] (hi, lo), scaled by 2^-(E_f + E_r)
+    float2* out = nullptr;                // near field (hi, lo): class rows [n_leaves][4 nch N], scaled by
+                                          // 2^-(E_f + 1 + E_r), or node rows [n_leaves][Rp], by 2^-(E_f + E_r)
+    long long* ffix = nullptr;            // [R][n_leaves][k^2] f 2^(55 - E_f), truncated (near field)
+    void* near_opnd = nullptr;            // near field's operand tiles, a chunk at a time
+    size_t near_opnd_bytes = 0;
     unsigned long long* fmax = nullptr;   // [R] max |f| per right-hand side (bits)
     int* Ef = nullptr;                    // [R] exponent of f per right-hand side
     int* err = nullptr;                   // non-zero after a bounded wait expired
@@ -237,7 +263,7 @@ struct MixedWork {
     int* Et = nullptr;                    // [n_leaves]
     float2* far_out = nullptr;            // [n_leaves][Rp]
     float2* part = nullptr;               // partial sums or slab of S2M, M2L and the leaf far field
-    float2* part_side = nullptr;          // partial sums or slab of the near field
+    float2* part_side = nullptr;          // partial sums or slab of the near field by entries
     float2* part_s2l = nullptr;           // partial sums or slab of S2L
     cudaEvent_t* cev = nullptr;           // optional (start, stop) pairs: near, S2M, M2L, S2L, far
 };
@@ -294,7 +320,7 @@ int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, 
 constexpr int kDeferSegments = 1;
 constexpr int kDeferSplits = 2;
 // Partial-sum elements (float2) of the three buffers whose contractions may run at the same time:
-// [0] S2M, M2L and the leaf far field (one after another), [1] the near field, [2] S2L.
+// [0] S2M, M2L and the leaf far field (one after another), [1] S2L, [2] the near field by entries.
 void split_part_elems(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, size_t elems[3]);
 int build_mixed_plan(DeviceTree* T, cudaStream_t st);
 // Host copies of the tree arrays the plan builders read (fetched once per plan set).
@@ -305,11 +331,18 @@ int fetch_host_lists(const DeviceTree& T, HostLists* H);
 int build_far_slots(DeviceTree* T, const HostLists& H, cudaStream_t st);
 // Plan of one far-field contraction (kCtrS2M, kCtrM2L, kCtrS2L or kCtrFar) into PS.
 int build_far_plan(int which, const DeviceTree& T, int R, const HostLists& H, PlanArena& A, PlanSet* PS);
-// Near field in two parts: max |f| and the f slices (also the operand of S2M and S2L), then the
-// split contraction.
+// max |f| and the f slices (operand of S2M and S2L).
 int near_slices(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
                 cudaStream_t st);
-int near_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const MixedWork& w, cudaStream_t st);
+// Near field in reflection classes (mixed_sym.cu): tables, plan, operand buffer, solve, kernels launched.
+int near_classes_prepare(vfmm_ops* o, cudaStream_t st);
+int build_near_classes(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, NearPlan* P);
+size_t near_operand_bytes(const DeviceTree& T, const NearPlan& P, int R);
+int near_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
+                  cudaStream_t st);
+int near_class_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
+                        cudaStream_t st);
+int near_launches(const MixedOps& mo, const NearPlan& P, size_t opnd_bytes);
 int far_prepare(vfmm_ops* o, cudaStream_t st);
 void far_free(MixedOps* mo);
 // Stages of the split-precision far field (see mixed_far.cu). Multipoles and locals are stored per

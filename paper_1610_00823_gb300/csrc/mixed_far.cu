@@ -347,14 +347,13 @@ void split_part_elems(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o,
     auto need = [&](const SplitPlan& P, size_t rows, int Rp) -> size_t {
         return std::max(need1(P, rows, Rp), P.alt ? need1(*P.alt, rows, Rp) : size_t(0));
     };
-    size_t a = need(PS.near, T.n_leaves * R, mo->Rp);
     size_t b = need(PS.m2l, T.n_boxes * R, mo->Rx);
     size_t c = need(PS.far, T.n_leaves * R, mo->Rp);
     size_t d = need(PS.s2l, T.n_boxes * R, mo->Rx);
     size_t e = need(PS.s2m, T.n_leaves * R, mo->Rx);
     elems[0] = std::max(std::max(b, c), e);
-    elems[1] = a;
-    elems[2] = d;
+    elems[1] = d;
+    elems[2] = need(PS.entries, T.n_leaves * R, mo->Rp);
 }
 
 // ---------------------------------------------------------------- S2M
@@ -579,13 +578,19 @@ extern "C" int vfmm_solve_work(const vfmm_tree* tree, const vfmm_ops* ops, int32
         return 2.0 * (double)P.entries * (Rp / table_rows_per_tile(P.transposed, Rp)) * (double)Kp * (S * (S + 1) / 2) *
                kTileM * mma_n(P.transposed, Rp);
     };
-    out[0] = tc(PS->near, mo->Kp, mo->Rp, kCtrNear);
+    if (!near_by_classes(ops->k)) {
+        out[0] = tc(PS->entries, mo->Kp, mo->Rp, kCtrNear);
+    } else {
+        const int S = mo->slices[kCtrNear];
+        out[0] = 2.0 * (PS->near.first.empty() ? 0.0 : (double)PS->near.first.back()) * mo->near.nch * kTileM *
+                 mo->near.N * kKBlock * (S * (S + 1) / 2);
+    }
     out[1] = tc(PS->m2l, mo->Kx, mo->Rx, kCtrM2L);
     out[2] = tc(PS->far, mo->Kx, mo->Rp, kCtrFar);
     out[3] = tc(PS->s2l, mo->Kp, mo->Rx, kCtrS2L);
     out[4] = tc(PS->s2m, mo->Kp, mo->Rx, kCtrS2M);
-    out[7] = (PS->near.entry ? 1 : 0) + (PS->m2l.entry ? 2 : 0) + (PS->far.entry ? 4 : 0) + (PS->s2l.entry ? 8 : 0);
-    out[8] = PS->near.ctas;
+    out[7] = (PS->entries.entry ? 1 : 0) + (PS->m2l.entry ? 2 : 0) + (PS->far.entry ? 4 : 0) + (PS->s2l.entry ? 8 : 0);
+    out[8] = near_by_classes(ops->k) ? PS->near.ctas : PS->entries.ctas;
     out[9] = PS->pass_ctas;
     return VFMM_OK;
 }

@@ -146,11 +146,15 @@ static void m2t_tables(int k, int P, std::vector<double>& F) {
     }
 }
 
+int sym_near_op(const vfmm_ops* o, SymOp* op, cudaStream_t st) {
+    return make_op(op, VFMM_LIST_U, o->k, o->p + 1, true, true, o->near, 3 * o->k * o->k, o->k * o->k, st);
+}
+
 int sym_prepare(vfmm_ops* o, const double* m2l, const double* s2l, cudaStream_t st) {
     const int k = o->k, kk = k * k, P = o->p + 1, P2 = 2 * P;
     SymTables* s = new SymTables();
     o->sym = s;
-    VFMM_CHECK(make_op(&s->near, VFMM_LIST_U, k, P, true, true, o->near, 3 * kk, kk, st));
+    VFMM_CHECK(sym_near_op(o, &s->near, st));
     VFMM_CHECK(make_op(&s->s2m, -1, k, P, false, true, o->s2m, P2, kk, st));
     VFMM_CHECK(make_op(&s->l2t, -1, k, P, true, false, o->l2t, 3 * kk, P2, st));
     VFMM_CHECK(make_op(&s->m2l, VFMM_LIST_V, k, P, false, false, m2l, P2, P2, st));
@@ -240,10 +244,11 @@ __global__ void __launch_bounds__(256) inst_fill_kernel(InstLists L, InstOut O, 
 
 int build_instances(DeviceTree* T, cudaStream_t st) {
     const int n = T->n_boxes;
-    void* tmp = nullptr;  // [mask n][counts 4 n][flags 32 n]
-    VFMM_CHECK(tree_malloc(&tmp, (size_t)37 * n * sizeof(int32_t), st));
-    uint32_t* mask = (uint32_t*)tmp;
-    int32_t *cnt = (int32_t*)tmp + n, *flags = cnt + (size_t)4 * n;
+    void* tmp = nullptr;  // [counts 4 n][flags 32 n]
+    VFMM_CHECK(tree_malloc(reinterpret_cast<void**>(&T->inst_mask), (size_t)n * sizeof(uint32_t), st));
+    VFMM_CHECK(tree_malloc(&tmp, (size_t)36 * n * sizeof(int32_t), st));
+    uint32_t* mask = T->inst_mask;
+    int32_t *cnt = (int32_t*)tmp, *flags = cnt + (size_t)4 * n;
     InstLists L;
     L.leaf_of_box = T->leaf_of_box;
     for (int q = 0; q < 4; ++q) {

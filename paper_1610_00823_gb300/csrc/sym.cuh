@@ -97,6 +97,8 @@ struct SymTables {
 // coefficient l (device). The tables are complete when st is.
 int sym_prepare(::vfmm_ops* o, const double* m2l, const double* s2l, cudaStream_t st);
 void sym_free(::vfmm_ops* o);
+// The near field's operator alone (its table is the caller's to free).
+int sym_near_op(const ::vfmm_ops* o, SymOp* op, cudaStream_t st);
 
 // Instances of the four lists (built with the tree).
 int build_instances(DeviceTree* T, cudaStream_t st);

@@ -1088,7 +1088,7 @@ void free_tree(DeviceTree* t) {
     // work queued on any stream may still read the tree
     cudaDeviceSynchronize();
     void* ps[] = {t->key,         t->level,       t->ix,       t->iy,           t->parent,     t->child0,
-                  t->leaf_of_box, t->box_of_leaf, t->level_start_dev, t->inst,
+                  t->leaf_of_box, t->box_of_leaf, t->level_start_dev, t->inst, t->inst_mask,
                   t->far_slot,    t->nonleaf,     t->nonleaf_start_dev};
     free_plan_set(&t->plans);
     if (t->plans_r) {

@@ -184,11 +184,25 @@ struct SplitPlan {
     int64_t off[6] = {-1, -1, -1, -1, -1, -1};
 };
 
+// Schedule of the near field in reflection classes: leaves ordered by their set of orbits, in groups of
+// 128 virtual leaves (leaf, r); a piece is one group's class (4 * group + class).
+struct NearPlan {
+    int32_t n_groups = 0;
+    int32_t max_units = 0;         // most K blocks of a piece
+    int32_t ctas = 0;              // CTA cap of the launch (0: one CTA per item)
+    std::vector<int32_t> first;    // [4 n_groups + 1] first operand tile (K block) of each piece
+    int32_t* order = nullptr;      // [n_leaves]
+    int32_t* gmask = nullptr;      // [n_groups] orbits of a group's leaves
+    int32_t* first_dev = nullptr;
+    int64_t off[3] = {0, 0, 0};    // their places in the plan set's arena while it is being built
+};
+
 // The split contractions of the mixed form with R right-hand sides folded into the rows: the
 // virtual row of box or leaf x for right-hand side r is x * R + r (R consecutive rows per box).
 struct PlanSet {
     int R = 1;
-    SplitPlan near;  // U list: targets leaves, tables 33 configurations, A rows leaves
+    NearPlan near;      // U list, reflection classes (near_by_classes(k)), else
+    SplitPlan entries;  // U list: targets leaves, tables 33 configurations, A rows leaves
     SplitPlan s2m;   // targets leaves, one table, A rows leaves
     SplitPlan m2l;   // V list: targets boxes, tables the 40 offsets, A rows boxes
     SplitPlan far;   // L2T + W list: targets leaves, tables 0 (L2T) and 1 + W configuration, A rows far slots
@@ -228,6 +242,7 @@ struct DeviceTree {
     int32_t* inst_order[4] = {nullptr, nullptr, nullptr, nullptr};   // [n_inst]
     int32_t* inst_ostart[4] = {nullptr, nullptr, nullptr, nullptr};  // [orbits + 1]
     int64_t n_inst[4] = {0, 0, 0, 0};
+    uint32_t* inst_mask = nullptr;  // [n_boxes] the box's (list, orbit) rows
     // split-precision schedules (VFMM_MIXED): one right-hand side built with the tree, others on
     // first use (plans_for), guarded by plans_mu
     PlanSet plans;
