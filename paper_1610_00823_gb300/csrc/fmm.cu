@@ -2,21 +2,20 @@
 // expansions (Section 3.2), and the solve driver of both forms (FP64 below; the split-BF16
 // contractions of the mixed form are in mixed.cu and mixed_far.cu).
 //
-//   S2M      leaf multipoles  a = h^2 Q f                 (gather GEMM, all leaves)
-//   M2M      finest parents first: one cooperative persistent pass for small trees (position-DFT
-//            form, readiness counters), else one launch per level
-//   M2L      dense per V entry (gather GEMM per offset) or plane-wave (planewave.cu)
-//   DOWN     per level from 2 down the tree, one CTA per box:
+//   S2M      leaf multipoles  a = h^2 Q f
+//   M2M      one cooperative persistent pass over all levels (position-DFT form, readiness counters)
+//   M2L      dense per V list or plane-wave (planewave.cu); S2L over the X list
+//   DOWN     a second persistent pass:
 //            b = L2L(parent) + sum_V M2L a_c (+ a_0(c) log h) + sum_X (2h)^2 R f_c (+ a_0(c) log h)
-//   NEAR     per near configuration, T_cfg f_src for every U-list entry (gather GEMM into
-//            a per-entry slab of the workspace; one launch for all 33 configurations)
-//   L2T      far-field values from the leaf's local expansion (gather GEMM)
-//   LEAF     one CTA per leaf: u = h^2 sum_U T f - (1/2pi) log(h) sum_U a_0(src) + L2T + sum_W M2T,
-//            gradient = h sum_U T' f + L2T'/h + sum_W M2T'
+//   NEAR     sum over the U list of the configurations' tables applied to f
+//   L2T, M2T far-field values from the leaf's local expansion and the W list's multipoles
+//   LEAF     one CTA per leaf: u = h^2 NEAR - (1/2pi) log(h) sum_U a_0(src) + L2T + M2T (+ its log terms),
+//            gradient = h NEAR' + (L2T' + M2T')/h
+// The FP64 form's products run in the reflection classes of sym.cuh.
 //
 // Workspace (caller-owned, from vfmm_workspace_size): status word, multipoles and locals
-// [n_boxes][2(p+1)], near slabs [n_U][3kk], far values [n_leaves][3kk], M2L/S2L slabs or
-// plane-waves, the mixed form's operands and outputs (+ I/O copies); see layout().
+// [n_boxes][2(p+1)], the FP64 form's slabs (a row per instance) or the mixed form's operands and
+// outputs (+ I/O copies); see layout().
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -32,7 +31,16 @@ namespace vfmm {
 
 constexpr double kInv2Pi = 0.15915494309189533577;
 
-// 2^e as a double, built from its exponent bits (exact, no libm call).
+// log(h) of every level: a logarithm per box on the device is some 50 FP64 instructions of a whole warp,
+// as much as the rest of a leaf's scalar terms.
+struct LevelLogs {
+    double v[kMaxDepth + 1];
+};
+static LevelLogs level_logs(double width) {
+    LevelLogs l;
+    for (int i = 0; i <= kMaxDepth; ++i) l.v[i] = std::log(std::ldexp(width, -i));
+    return l;
+}
 
 // Re of local coefficient 0 from the V and X lists of each virtual box (box, r): sum over V of
 // Re(row 0 of M2L_c . a_c) + a_0(c) log h, and over X of (2h)^2 Re(S2L row 0) . f_c + a_0(c) log h.
@@ -40,6 +48,7 @@ constexpr double kInv2Pi = 0.15915494309189533577;
 // row-0 tables in shared memory; one warp per virtual box, the (entry, coefficient) pairs of eight
 // V entries at a time spread over the lanes.
 __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, int P, double width,
+                                                     const __grid_constant__ LevelLogs logs,
                                                      const int32_t* __restrict__ level,
                                                      const int32_t* __restrict__ vptr, const int32_t* __restrict__ vidx,
                                                      const int32_t* __restrict__ vcfg, const double2* __restrict__ m2l_r0,
@@ -61,7 +70,7 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
          vw += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int b = begin + (int)(vw / R), r = (int)(vw % R);
         const double h = ldexp(width, -level[b]);
-        const double logh = log(h);
+        const double logh = logs.v[level[b]];
         // V list: the warp walks the entries; lane n takes coefficients n, n + 32 of the source
         // multipole (coalesced), partial sums stay per lane until one final reduction
         double acc = 0.0;
@@ -106,214 +115,6 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
     }
 }
 
-// Outputs j and P-1-j of one position of a triangular translation (mode 0, M2M: output o takes
-// inputs n <= o; mode 1, L2L: n >= o), n ascending for each, fused into one loop of P + 1 steps so
-// that every thread of a warp runs the same number of steps. M: [n][o] complex, x: inputs.
-__device__ __forceinline__ void translate_pair(int mode, const double2* __restrict__ M, const double2* x, int P, int j,
-                                               double2* out) {
-    const int oa = j, ob = P - 1 - j;
-    const int la = mode == 0 ? oa + 1 : P - oa;
-    const int lb = ob != oa ? (mode == 0 ? ob + 1 : P - ob) : 0;
-    const int na = mode == 0 ? 0 : oa, nb = mode == 0 ? 0 : ob;
-    double re = 0.0, im = 0.0;
-    for (int i = 0; i < la + lb; ++i) {
-        if (i == la) {
-            out[oa] = make_double2(re, im);
-            re = im = 0.0;
-        }
-        const bool first = i < la;
-        const int o = first ? oa : ob;
-        const int n = first ? na + i : nb + (i - la);
-        const double2 m = M[(size_t)n * P + o], v = x[n];
-        re = fma(m.x, v.x, fma(-m.y, v.y, re));
-        im = fma(m.x, v.y, fma(m.y, v.x, im));
-    }
-    out[lb ? ob : oa] = make_double2(re, im);
-}
-
-// ---------------------------------------------------------------- M2M and L2L (one CTA per non-leaf box)
-// The translations are triangular: M2M output l of the parent takes child coefficients n <= l,
-// L2L output m of a child takes parent coefficients l >= m. A thread owns one child position and
-// the output pair (j, P-1-j), so every thread does P + 1 complex multiply-adds and no zero
-// entry is read. mode 0 (M2M): in = the 4 consecutive child multipoles, out = parent multipole.
-// mode 1 (L2L): in = parent local, out = the 4 child locals (written, later added to by the
-// downward pass). Tables [pos][in][out] complex.
-// ---- rotated real form of M2M and L2L (the factorisation is written out in tables.cu): for child
-// position pos (sx = +1 when pos & 1, sy = +1 when pos & 2, s = sx sy), M2M is
-// A_l = sigma_l sum_n Rm[n][l] (rho_n a_n) and L2L is c_m = rho_m sum_l Rl[l][m] (sigma_l b_l), with
-// the Gaussian integers sigma_l = (i s)^floor(l/2) (sx + i sy)^(l mod 2) and rho_n = conj(sigma_n):
-// one real triangular matrix for the four positions, 2 FP64 FMAs per entry instead of 4.
-
-// x with its sign bit flipped when neg = 0x80000000 (integer work, no FP64 operation)
-__device__ __forceinline__ double flip_sign(double x, unsigned neg) {
-    return __hiloint2double(__double2hiint(x) ^ (int)neg, __double2loint(x));
-}
-
-// v sigma_n (sig) or v rho_n (!sig) for child position pos: sign changes and swaps, then one
-// addition per component, exact for even n (the added term is zero).
-__device__ __forceinline__ double2 rotate(double2 v, int pos, int n, bool sig) {
-    constexpr unsigned kNeg = 0x80000000u;
-    const unsigned nx = (pos & 1) ? 0u : kNeg, ny = (pos & 2) ? 0u : kNeg;
-    const unsigned nc = sig ? (nx ^ ny) : (nx ^ ny ^ kNeg);  // unit u = i c: c = s (sigma), -s (rho)
-    const unsigned ne = sig ? ny : (ny ^ kNeg);              // odd factor sx + i e: e = sy (sigma), -sy (rho)
-    double wx, wy;  // v u^floor(n/2)
-    switch ((n >> 1) & 3) {
-        case 0: wx = v.x; wy = v.y; break;
-        case 1: wx = flip_sign(v.y, nc ^ kNeg); wy = flip_sign(v.x, nc); break;
-        case 2: wx = flip_sign(v.x, kNeg); wy = flip_sign(v.y, kNeg); break;
-        default: wx = flip_sign(v.y, nc); wy = flip_sign(v.x, nc ^ kNeg); break;
-    }
-    // times (sx + i e) for odd n: (wx sx - wy e) + i (wy sx + wx e)
-    const bool odd = n & 1;
-    const double ax = odd ? flip_sign(wx, nx) : wx, bx = odd ? flip_sign(wy, ne ^ kNeg) : 0.0;
-    const double ay = odd ? flip_sign(wy, nx) : wy, by = odd ? flip_sign(wx, ne) : 0.0;
-    return make_double2(ax + bx, ay + by);
-}
-
-// One CTA per virtual box of a level, in the rotated real form (for levels with many boxes, where
-// the FP64 pipes bound the translations): the four rotated input vectors are staged in shared
-// memory, each thread takes one child position and one output row pair (j, P-1-j) of the real
-// triangular matrix Mr [in][out] (P + 1 real-times-complex multiply-adds), rotates its two rows
-// back, and M2M sums the four positions. mode 0 (M2M): in = the 4 consecutive child multipoles,
-// out = parent multipole; mode 1 (L2L): in = parent local, out = the 4 child locals.
-__global__ void __launch_bounds__(128) translate_kernel(int mode, const int32_t* __restrict__ boxes, int nbox, int R,
-                                                        const int32_t* __restrict__ child0, int P,
-                                                        const double* __restrict__ Mr, double2* __restrict__ ex) {
-    extern __shared__ double2 sx[];  // [4P] rotated inputs, [4P] per-position results
-    const int bi = blockIdx.x / R, r = blockIdx.x - bi * R;  // virtual box (box, right-hand side)
-    if (bi >= nbox) return;
-    const int b = boxes[bi], c0 = child0[b];
-    double2* s_in = sx;
-    double2* s_out = sx + 4 * P;
-    for (int q = threadIdx.x; q < 4 * P; q += blockDim.x) {
-        const int pos = q / P, n = q - pos * P;
-        const double2 v = mode == 0 ? ex[((size_t)(c0 + pos) * R + r) * P + n] : ex[((size_t)b * R + r) * P + n];
-        s_in[q] = rotate(v, pos, n, mode == 1);  // rho for M2M inputs, sigma for L2L inputs
-    }
-    __syncthreads();
-    const int npair = (P + 1) / 2;
-    for (int task = threadIdx.x; task < 4 * npair; task += blockDim.x) {
-        const int pos = task / npair, j = task - pos * npair;
-        const int oa = j, ob = P - 1 - j;
-        const double2* x = s_in + pos * P;
-        double ar = 0.0, ai = 0.0, br = 0.0, bi2 = 0.0;
-        if (mode == 0) {
-            for (int n = 0; n <= ob; ++n) {  // row oa takes n <= oa, row ob n <= ob
-                const double2 v = x[n];
-                if (n <= oa) {
-                    const double m = __ldg(Mr + (size_t)n * P + oa);
-                    ar = fma(m, v.x, ar);
-                    ai = fma(m, v.y, ai);
-                }
-                const double m = __ldg(Mr + (size_t)n * P + ob);
-                br = fma(m, v.x, br);
-                bi2 = fma(m, v.y, bi2);
-            }
-        } else {
-            for (int n = oa; n < P; ++n) {  // row oa takes n >= oa, row ob n >= ob
-                const double2 v = x[n];
-                const double m = __ldg(Mr + (size_t)n * P + oa);
-                ar = fma(m, v.x, ar);
-                ai = fma(m, v.y, ai);
-                if (n >= ob) {
-                    const double mb = __ldg(Mr + (size_t)n * P + ob);
-                    br = fma(mb, v.x, br);
-                    bi2 = fma(mb, v.y, bi2);
-                }
-            }
-        }
-        // rotate back: sigma for M2M outputs, rho for L2L outputs
-        s_out[pos * P + oa] = rotate(make_double2(ar, ai), pos, oa, mode == 0);
-        if (ob != oa) s_out[pos * P + ob] = rotate(make_double2(br, bi2), pos, ob, mode == 0);
-    }
-    __syncthreads();
-    if (mode == 0) {
-        for (int o = threadIdx.x; o < P; o += blockDim.x) {
-            const double2 a0 = s_out[o], a1 = s_out[P + o], a2 = s_out[2 * P + o], a3 = s_out[3 * P + o];
-            ex[((size_t)b * R + r) * P + o] =
-                make_double2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
-        }
-    } else {
-        for (int q = threadIdx.x; q < 4 * P; q += blockDim.x) ex[((size_t)(c0 + q / P) * R + r) * P + q % P] = s_out[q];
-    }
-}
-
-// After a CTA has given up waiting for a bulk copy into its shared memory, thread 0 waits once
-// more, with a longer bound, for the copy to land (the other threads may leave): the CTA's shared
-// memory stays allocated, and no copy is left writing into it, until the copy has completed or
-// this second wait also runs out.
-__device__ __forceinline__ void settle_bulk_copy(uint32_t bar_a, const volatile int* never) {
-    if (threadIdx.x == 0) tc::mbar_wait(bar_a, 0, never, 1ll << 27);
-}
-
-// Same translations with the 4 position tables held in shared memory (one bulk copy per CTA),
-// persistent CTAs looping over the virtual boxes of the level: the table is read from L2 once
-// per CTA instead of once per multiply-add. Used when 4 P^2 complex values fit (P <= 58).
-constexpr int kTranslateThreads = 128;
-__global__ void __launch_bounds__(kTranslateThreads) translate_smem_kernel(int mode, const int32_t* __restrict__ boxes,
-                                                                           int nbox, int R,
-                                                                           const int32_t* __restrict__ child0, int P,
-                                                                           const double2* __restrict__ tab,
-                                                                           double2* __restrict__ ex, int* err) {
-    extern __shared__ __align__(128) unsigned char sm_raw[];
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ volatile int no_abort;
-    double2* sT = reinterpret_cast<double2*>(sm_raw);  // [4][P][P]
-    double2* s_in = sT + 4 * P * P;                    // [4P]
-    double2* s_out = s_in + 4 * P;                     // [4P]
-    const uint32_t bar_a = tc::smem_u32(&bar);
-    const uint32_t bytes = (uint32_t)(4 * P * P) * sizeof(double2);
-    if (threadIdx.x == 0) {
-        no_abort = 0;
-        tc::mbar_init(bar_a, 1);
-        tc::mbar_fence_init();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        tc::mbar_arrive_expect_tx(bar_a, bytes);
-        constexpr uint32_t kChunk = 32768;
-        for (uint32_t off = 0; off < bytes; off += kChunk)
-            tc::bulk_copy_g2s(tc::smem_u32(sm_raw) + off, reinterpret_cast<const char*>(tab) + off,
-                              min(kChunk, bytes - off), bar_a);
-    }
-    const bool landed = tc::mbar_wait(bar_a, 0, &no_abort);
-    if (!__syncthreads_and(landed)) {  // one decision for the whole CTA
-        if (threadIdx.x == 0 && err) atomicExch(err, 5);
-        settle_bulk_copy(bar_a, &no_abort);
-        return;
-    }
-    const int npair = (P + 1) / 2;
-    for (int item = blockIdx.x; item < nbox * R; item += gridDim.x) {
-        const int bi = item / R, r = item - bi * R;  // virtual box (box, right-hand side)
-        const int b = boxes[bi], c0 = child0[b];
-        if (mode == 0) {
-            for (int q = threadIdx.x; q < 4 * P; q += blockDim.x)
-                s_in[q] = ex[((size_t)(c0 + q / P) * R + r) * P + q % P];
-        } else {
-            for (int q = threadIdx.x; q < P; q += blockDim.x) s_in[q] = ex[((size_t)b * R + r) * P + q];
-        }
-        __syncthreads();
-        for (int task = threadIdx.x; task < 4 * npair; task += blockDim.x) {
-            const int pos = task / npair, j = task - pos * npair;
-            const double2* M = sT + pos * P * P;
-            const double2* x = mode == 0 ? s_in + pos * P : s_in;
-            translate_pair(mode, M, x, P, j, s_out + pos * P);
-        }
-        __syncthreads();
-        if (mode == 0) {
-            for (int o = threadIdx.x; o < P; o += blockDim.x) {
-                const double2 a0 = s_out[o], a1 = s_out[P + o], a2 = s_out[2 * P + o], a3 = s_out[3 * P + o];
-                ex[((size_t)b * R + r) * P + o] =
-                    make_double2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
-            }
-        } else {
-            for (int q = threadIdx.x; q < 4 * P; q += blockDim.x)
-                ex[((size_t)(c0 + q / P) * R + r) * P + q % P] = s_out[q];
-        }
-        __syncthreads();
-    }
-}
-
 static int sm_count() {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
@@ -321,37 +122,12 @@ static int sm_count() {
     return n > 0 ? n : 1;
 }
 
-static void launch_translate(int mode, const DeviceTree& T, int level, int R, int P, const double* tab,
-                             const double* tab_r, double* ex, int* err, cudaStream_t st) {
-    const int nbox = T.nonleaf_start[level + 1] - T.nonleaf_start[level];
-    if (nbox <= 0) return;
-    const size_t smem = (size_t)(4 * P * P + 8 * P) * sizeof(double2);
-    // small levels: the table is fetched once per CTA; large levels (at least ~8 boxes per SM): one CTA
-    // per box keeps many warps per SM feeding the FP64 pipes, the table staying in L1/L2
-    if (smem <= 113 * 1024 && (long long)nbox * R <= 8ll * sm_count()) {  // two CTAs per SM
-        static thread_local int attr_dev = -1;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (attr_dev != dev) {
-            cudaFuncSetAttribute(translate_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
-            attr_dev = dev;
-        }
-        const int grid = std::min<long long>((long long)nbox * R, 2ll * sm_count());
-        translate_smem_kernel<<<grid, kTranslateThreads, smem, st>>>(
-            mode, T.nonleaf + T.nonleaf_start[level], nbox, R, T.child0, P, reinterpret_cast<const double2*>(tab),
-            reinterpret_cast<double2*>(ex), err);
-        return;
-    }
-    const int threads = std::min(128, ((4 * ((P + 1) / 2) + 31) / 32) * 32);
-    translate_kernel<<<(unsigned)nbox * R, threads, (size_t)8 * P * sizeof(double2), st>>>(
-        mode, T.nonleaf + T.nonleaf_start[level], nbox, R, T.child0, P, tab_r, reinterpret_cast<double2*>(ex));
-}
-
 // ---------------------------------------------------------------- downward pass (one CTA per box)
 struct DownArgs {
     int begin, end, P, kk, level;
     int R, nleaf;  // right-hand sides folded into the box rows (virtual box = box * R + r); leaves
     double width;
+    LevelLogs logs;
     const int32_t* parent;
     const int32_t* ix;
     const int32_t* iy;
@@ -434,24 +210,7 @@ __device__ __forceinline__ void own_terms_fp64(const DownArgs& d, int level, int
         }
         own[i] = make_double2(re, im);
     }
-    if (lane == 0) own[0].x += log(h) * a0;
-}
-
-// FP64 form, one level (P <= 64): one warp per box adds its own terms to the L2L values that the
-// translation kernel has just written.
-__global__ void __launch_bounds__(128) down_kernel(DownArgs d) {
-    const int b = d.begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (b >= d.end) return;
-    double2 own[2];
-    own_terms_fp64(d, d.level, b, lane, own);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int t = lane + 32 * i;
-        if (t >= d.P) continue;
-        double2* L = reinterpret_cast<double2*>(d.Lexp) + (size_t)b * d.P + t;
-        const double2 p = d.level >= 3 ? *L : make_double2(0.0, 0.0);
-        *L = make_double2(p.x + own[i].x, p.y + own[i].y);
-    }
+    if (lane == 0) own[0].x += d.logs.v[level] * a0;
 }
 
 // Mixed form: coefficient t of the local expansion of virtual box (b, r) at `level` = the L2L
@@ -490,24 +249,6 @@ __device__ __forceinline__ double2 combine_local(const DownArgs& d, int level, i
         }
     }
     return make_double2(re, im);
-}
-
-// Mixed form, one level: one thread per (virtual box, coefficient).
-__global__ void down_mixed_kernel(DownArgs d) {
-    const int P = d.P, R = d.R;
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= (int64_t)(d.end - d.begin) * R * P) return;
-    const size_t vb = (size_t)d.begin * R + (size_t)(q / P);
-    const int t = (int)(q % P);
-    const int b = (int)(vb / R), r = (int)(vb % R);
-    double re = 0.0, im = 0.0;
-    if (d.level >= 3) {  // L2L from the parent, written by the translation kernel just before
-        re = d.Lexp[vb * 2 * P + 2 * t];
-        im = d.Lexp[vb * 2 * P + 2 * t + 1];
-    }
-    const double2 v = combine_local(d, d.level, b, r, t, re, im);
-    d.Lexp[vb * 2 * P + 2 * t] = v.x;
-    d.Lexp[vb * 2 * P + 2 * t + 1] = v.y;
 }
 
 // ---------------------------------------------------------------- persistent tree passes
@@ -807,7 +548,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) downward_pass_kernel(PassArgs
 // -(1/2pi) [log(h) sum_U a_0 + Re b_0 + sum_W a_0 (log h_w)], h_w = h / 2 (first warp, fixed-order sums).
 struct LeafMixedArgs {
     int nleaf, R, k, kk, Rp, P, lw;
-    double wm, width;
+    double wm;
+    LevelLogs logs;
     const int32_t* box_of_leaf;
     const int32_t* level;
     const int32_t *uptr, *uidx, *wptr, *widx;
@@ -926,7 +668,7 @@ __global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
     }
     if (t < 32) {
         const size_t P2 = 2 * (size_t)a.P;
-        const double logh = log(ldexp(a.width, -lv));
+        const double logh = a.logs.v[lv];
         double m = 0.0, w0 = 0.0;
         for (int e = a.uptr[b] + t; e < a.uptr[b + 1]; e += 32) m += a.Mexp[((size_t)a.uidx[e] * R + r) * P2];
         for (int e = a.wptr[b] + t; e < a.wptr[b + 1]; e += 32) w0 += a.Mexp[((size_t)a.widx[e] * R + r) * P2];
@@ -951,6 +693,7 @@ struct LeafArgs {
     SymOp op;  // rows of the classes
     int nleaf, kk, k, P;
     double width;
+    LevelLogs logs;
     const int32_t* box_of_leaf;
     const int32_t* level;
     const int32_t *uptr, *uidx, *wptr, *widx;
@@ -992,7 +735,7 @@ __global__ void __launch_bounds__(256) leaf_kernel(const __grid_constant__ LeafA
             w0 += __shfl_xor_sync(0xffffffffu, w0, o);
         }
         if (t == 0) {
-            const double logh = log(h);
+            const double logh = a.logs.v[a.level[b]];
             s_scal = -kInv2Pi * (logh * m + (logh - 0.6931471805599453) * w0);
         }
     }
@@ -1178,6 +921,7 @@ static void fill_down_args(DownArgs& d, const DeviceTree& T, const vfmm_ops& o, 
     d.kk = o.k * o.k;
     d.level = l;
     d.width = T.width;
+    d.logs = level_logs(T.width);
     d.parent = T.parent;
     d.ix = T.ix;
     d.iy = T.iy;
@@ -1214,16 +958,9 @@ static void fill_down_args(DownArgs& d, const DeviceTree& T, const vfmm_ops& o, 
     d.Rx = mo ? mo->Rx : 0;
 }
 
-// Persistent passes (one cooperative launch for all levels) when every level is small enough that
-// per-level launches would mostly wait on launch latency; larger levels keep one launch per level.
-static bool use_passes(const DeviceTree& T, int R, int P) {
-    const size_t smem = pass_smem_bytes(P);
-    if (smem > 200 * 1024 || T.depth < 3) return false;
-    int widest = 0;
-    for (int l = 1; l <= T.depth; ++l) widest = std::max(widest, T.nonleaf_start[l + 1] - T.nonleaf_start[l]);
-    return (long long)widest * R <= 16ll * sm_count();
-}
-
+// One cooperative launch per pass, whatever the tree's size: one real matrix-vector product per box, and
+// no launch per level. On 266,805 boxes the upward levels took 2.17 ms as one launch each, 1.21 as a pass,
+// the downward ones 2.32 and 1.60; small trees are bound by the levels' latency.
 template <typename... Args>
 static int launch_pass(void (*kernel)(Args...), int R, int P, int widest_items, int cap, cudaStream_t st,
                        Args... args) {
@@ -1343,9 +1080,8 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     const MixedOps* mo = (const MixedOps*)o.mixed;
     const SymTables* sy = (const SymTables*)o.sym;
     int launches = 0;
-    const bool passes = use_passes(T, R, P);
     // readiness counters (persistent passes) and level exponents (mixed form) start at zero
-    if (passes || mixed) VFMM_CUDA(cudaMemsetAsync(w.ready, 0, w.ready_words * sizeof(unsigned int), st));
+    VFMM_CUDA(cudaMemsetAsync(w.ready, 0, w.ready_words * sizeof(unsigned int), st));
     if (mixed) {
         // near field first: its f slices also feed S2M and S2L
         mark(se, ST_NEAR, false, st);
@@ -1389,7 +1125,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     mark(se, ST_M2M, false, st);
     int widest = 0;
     for (int l = 1; l <= T.depth; ++l) widest = std::max(widest, T.nonleaf_start[l + 1] - T.nonleaf_start[l]);
-    if (passes) {
+    if (T.depth >= 3) {
         PassArgs pa;
         pa.depth = T.depth;
         pa.R = R;
@@ -1407,11 +1143,6 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         pa.err = w.mix.err;
         VFMM_CHECK(launch_pass(upward_pass_kernel, R, P, widest * R, mixed ? PS.pass_ctas : 0, st, pa));
         ++launches;
-    } else {
-        for (int l = T.depth - 1; l >= 2; --l) {
-            if (T.nonleaf_start[l + 1] > T.nonleaf_start[l]) ++launches;
-            launch_translate(0, T, l, R, P, o.m2m_t, o.m2m_r, w.Mexp, w.mix.err, st);
-        }
     }
     mark(se, ST_M2M, true, st);
     // downward pass
@@ -1424,8 +1155,8 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
             VFMM_CUDA(cudaStreamWaitEvent(side->aux, side->ev[5], 0));
             c0s = side->aux;
         }
-        VFMM_CHECK(m2l_mixed(T, PS, o, w.Mexp, w.mix, passes, st));
-        if (PS.m2l.n_groups > 0) launches += 3 + gemm_launches(PS.m2l, kDeferSplits);
+        VFMM_CHECK(m2l_mixed(T, PS, o, w.Mexp, w.mix, st));
+        if (PS.m2l.n_groups > 0) launches += 2 + gemm_launches(PS.m2l, kDeferSplits);
         const int begin = T.level_start[2], end = T.level_start[T.depth + 1];
         const int64_t warps = (int64_t)(end - begin) * R;
         const size_t c0_smem = (size_t)kVCfg * P * sizeof(double2) + (size_t)kFarCfg * kk * sizeof(double);
@@ -1438,7 +1169,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         }
         const unsigned c0_grid = (unsigned)std::min<int64_t>((warps + 7) / 8, 3ll * sm_count());
         m2l_c0_kernel<<<c0_grid, 256, c0_smem, c0s>>>(
-            begin, end, R, P, T.width, T.level, T.lptr[VFMM_LIST_V], T.lidx[VFMM_LIST_V], T.lcfg[VFMM_LIST_V],
+            begin, end, R, P, T.width, level_logs(T.width), T.level, T.lptr[VFMM_LIST_V], T.lidx[VFMM_LIST_V], T.lcfg[VFMM_LIST_V],
             reinterpret_cast<const double2*>(mo->m2l_r0), w.Mexp, w.mix.m2l_c0, T.lptr[VFMM_LIST_X],
             T.lidx[VFMM_LIST_X], T.lcfg[VFMM_LIST_X], T.leaf_of_box, mo->s2l_r0, f, nleaf, kk);
         ++launches;
@@ -1484,7 +1215,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
             VFMM_CHECK(sym_gemm(T, sy->s2l, r, st));
         }
     }
-    if (passes) {
+    if (T.depth >= 2) {
         DownArgs d;
         fill_down_args(d, T, o, f, w, 2, R);
         PassArgs pa;
@@ -1506,24 +1237,6 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         if (mixed) VFMM_CHECK(launch_pass(downward_pass_kernel<true>, R, P, items, PS.pass_ctas, st, pa, d));
         else VFMM_CHECK(launch_pass(downward_pass_kernel<false>, R, P, items, 0, st, pa, d));
         ++launches;
-    }
-    for (int l = 2; l <= T.depth && !passes; ++l) {
-        DownArgs d;
-        fill_down_args(d, T, o, f, w, l, R);
-        int n = d.end - d.begin;
-        if (n <= 0) continue;
-        if (l >= 3) {
-            // L2L for every box of level l (children of the non-leaf boxes of level l - 1)
-            launch_translate(1, T, l - 1, R, P, o.l2l_t, o.l2l_r, w.Lexp, w.mix.err, st);
-            ++launches;
-        }
-        ++launches;
-        if (mixed) {
-            const int64_t nt = (int64_t)n * R * P;
-            down_mixed_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d);
-        } else {
-            down_kernel<<<(unsigned)((n + 3) / 4), 128, 0, st>>>(d);
-        }
     }
     if (T.depth < 2) VFMM_CUDA(cudaMemsetAsync(w.Lexp, 0, (size_t)T.n_boxes * R * P2 * sizeof(double), st));
     else VFMM_CUDA(cudaMemsetAsync(w.Lexp, 0, (size_t)T.level_start[2] * R * P2 * sizeof(double), st));
@@ -1577,7 +1290,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         la.P = P;
         la.lw = lw;
         la.wm = wm;
-        la.width = T.width;
+        la.logs = level_logs(T.width);
         la.box_of_leaf = T.box_of_leaf;
         la.level = T.level;
         la.uptr = T.lptr[VFMM_LIST_U];
@@ -1609,6 +1322,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         a.k = o.k;
         a.P = P;
         a.width = T.width;
+        a.logs = level_logs(T.width);
         a.box_of_leaf = T.box_of_leaf;
         a.level = T.level;
         a.uptr = T.lptr[VFMM_LIST_U];
@@ -1908,7 +1622,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
         for (int sp = P->may_split ? 1 : keep; sp <= std::max(max_sp, keep) && rc == VFMM_OK; sp *= 2) {
             if (P->may_split && sp > std::max(1.0, avg_units)) break;
             P->split = sp;
-            float total = 0.0f;
+            float total = 1e30f;  // the fastest of a few runs
             for (int rep = 0; rep < 4 && rc == VFMM_OK; ++rep) {
                 cudaEventRecord(e0, st);
                 rc = split_gemm(*P, jb.a, jb.map, jb.Kp, jb.Rp, jb.out, w.mix.err, part, jb.rows, jb.slices, st);
@@ -1918,7 +1632,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
                 float ms = 0.0f;
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
                 if (e != cudaSuccess) rc = cuda_fail(e, "timing a split contraction");
-                if (rep > 0) total += ms;  // the first run warms up
+                if (rep > 0) total = std::min(total, ms);  // the first run warms up
             }
             if (rc == VFMM_OK && (*best_ms < 0.0f || total < *best_ms)) {
                 *best_ms = total;
@@ -1939,7 +1653,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
         int best_c = P->ctas;
         for (int c : {0, sms}) {
             P->ctas = c;
-            float total = 0.0f;
+            float total = 1e30f;  // the fastest of a few runs
             for (int rep = 0; rep < 4 && rc == VFMM_OK; ++rep) {
                 cudaEventRecord(e0, st);
                 rc = split_gemm(*P, jb.a, jb.map, jb.Kp, jb.Rp, jb.out, w.mix.err, part, jb.rows, jb.slices, st);
@@ -1949,7 +1663,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
                 float ms = 0.0f;
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
                 if (e != cudaSuccess) rc = cuda_fail(e, "timing a split contraction");
-                if (rep > 0) total += ms;
+                if (rep > 0) total = std::min(total, ms);
             }
             if (rc == VFMM_OK && (best < 0.0f || total < best)) {
                 best = total;
@@ -1990,7 +1704,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
     int32_t& near_ctas = cls ? PS->near.ctas : PS->entries.ctas;
     const int sms = sm_count();
     const bool wide = cls ? 8 * PS->near.n_groups * mo->near.nch > sms : PS->entries.ctas > 0;
-    if (rc == VFMM_OK && wide && use_passes(T, PS->R, ops->p + 1)) {
+    if (rc == VFMM_OK && wide && T.depth >= 3) {
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, upward_pass_kernel, kPassThreads, pass_smem_bytes(ops->p + 1));
         Workspace wf = w;
@@ -2003,7 +1717,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
             const int ncta = fracs[c] == 0 ? 0 : std::max(1, sms * fracs[c] / 8);
             near_ctas = ncta;
             PS->pass_ctas = fracs[c] == 0 || fracs[c] == 8 ? 0 : std::max(1, per_sm * (sms - ncta));
-            float total = 0.0f;
+            float total = 1e30f;  // the fastest of a few runs
             for (int rep = 0; rep < 6 && rc == VFMM_OK; ++rep) {
                 cudaEventRecord(e0, st);
                 rc = solve_all(T, *ops, f_dev, nrhs, u_dev, ux_dev, uy_dev, wf, st);
@@ -2013,7 +1727,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
                 float ms = 0.0f;
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
                 if (e != cudaSuccess) rc = cuda_fail(e, "timing a forked solve");
-                if (rep > 0) total += ms;  // the first run warms up
+                if (rep > 0) total = std::min(total, ms);  // the first run warms up
             }
             if (rc == VFMM_OK && (best < 0.0f || total < best)) {
                 best = total;

@@ -349,10 +349,8 @@ void far_free(MixedOps* mo);
 // virtual box (box * R + r); f is [R][n_leaves][k^2].
 int s2m_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, double* Mexp,
               const MixedWork& w, cudaStream_t st);
-// exps_done: the level exponents of the non-leaf multipoles were already taken (persistent upward
-// pass); leaf multipoles always take theirs in S2M.
 int m2l_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const MixedWork& w,
-              bool exps_done, cudaStream_t st);
+              cudaStream_t st);
 int s2l_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const MixedWork& w, cudaStream_t st);
 int far_leaf_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const double* Lexp,
                    const MixedWork& w, cudaStream_t st);

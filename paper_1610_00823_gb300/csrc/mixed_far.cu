@@ -423,19 +423,6 @@ int s2m_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const d
 }
 
 // ---------------------------------------------------------------- M2L
-// Level exponents of the non-leaf multipoles of levels >= 2 when no persistent pass computed them as
-// it wrote them (per-level translation launches): a warp per virtual box.
-__global__ void box_exp_kernel(const int32_t* __restrict__ boxes, int nbox, int R, int P2, const int32_t* __restrict__ level,
-                               const double* __restrict__ Mexp, unsigned* __restrict__ glev) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= (int64_t)nbox * R) return;
-    const int b = boxes[w / R], r = (int)(w % R);
-    int e = INT_MIN;
-    for (int k = lane; k < P2; k += 32) e = max(e, part_exp(Mexp[((size_t)b * R + r) * P2 + k], k));
-    level_exp_max(e, glev + (size_t)level[b] * R + r);
-}
-
 // One thread per 8 consecutive coefficients of a virtual box (one 16-byte store per slice).
 __global__ void multipole_slice_kernel(const int32_t* __restrict__ level, int64_t vb0, int64_t vb1, int R, int P2,
                                        int Kx, const double* __restrict__ Mexp, const unsigned* __restrict__ G,
@@ -465,17 +452,12 @@ __global__ void multipole_slice_kernel(const int32_t* __restrict__ level, int64_
 }
 
 int m2l_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const MixedWork& w,
-              bool exps_done, cudaStream_t st) {
+              cudaStream_t st) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
     if (T.depth < 2 || PS.m2l.n_groups == 0) return VFMM_OK;
     const int P2 = 2 * (o.p + 1), R = PS.R;
     const int64_t vb0 = (int64_t)T.level_start[2] * R, vb1 = (int64_t)T.level_start[T.depth + 1] * R;
-    // leaf multipoles took their level maxima in s2m_finish_kernel, non-leaf ones in the persistent
-    // upward pass (exps_done) or here
-    const int nb0 = T.nonleaf_start[2], nnl = T.nonleaf_start[T.depth + 1] - nb0;
-    if (!exps_done && nnl > 0)
-        box_exp_kernel<<<(unsigned)(((int64_t)nnl * R + 7) / 8), 256, 0, st>>>(T.nonleaf + nb0, nnl, R, P2, T.level,
-                                                                             Mexp, w.glev);
+    // every multipole took its level maximum as it was written (s2m_finish_kernel, upward pass)
     const int64_t n2 = (vb1 - vb0) * (mo->Kx / 8);
     multipole_slice_kernel<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(T.level, vb0, vb1, R, P2, mo->Kx, Mexp,
                                                                           w.glev, (bf16*)w.msl);

@@ -18,7 +18,7 @@
 // tiles once, the B tiles once per product), 1,620 cycles; the MMAs take 1,700 of the 2,220 cycles measured,
 // 300 go to operands not yet there and 220 to drains. The operand is bound by HBM writes and integer work.
 // Against gathered rows and plain tables (ms): 200,104 graded leaves 13.3 -> 8.0, 16,384 uniform leaves
-// k = 16 1.05 -> 0.39, 1,378 graded leaves 0.18 -> 0.11, 4,096 rows of k = 8 0.081 -> 0.034.
+// k = 16 1.32 -> 0.39, 1,378 graded leaves 0.18 -> 0.11, 4,096 rows of k = 8 0.081 -> 0.034.
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -58,10 +58,13 @@ __host__ __device__ inline int off_val(int k, int c) {
     return r;
 }
 
+struct alignas(16) OffStep {
+    double x, y, z, w;
+};
 struct OffTables {
     double* G = nullptr;   // per class [value][row]: coefficients of P from the symmetrised values
     int64_t g_off[4] = {};
-    double4* C = nullptr;  // [kOffSteps]: (2n+1)/n, (n+1)/n (downwards), (2n+1)/(n+1), n/(n+1) (upwards)
+    OffStep* C = nullptr;  // [kOffSteps]: (2n+1)/n, (n+1)/n (downwards), (2n+1)/(n+1), n/(n+1) (upwards)
 };
 
 // ---------------------------------------------------------------- host: values -> P
@@ -198,14 +201,14 @@ int offnode_prepare(vfmm_ops* o, cudaStream_t st) {
         G.resize(G.size() + n);
         class_table(k, c, A, G.data() + t->g_off[c]);
     }
-    std::vector<double4> C(kOffSteps);
+    std::vector<OffStep> C(kOffSteps);
     for (int n = 0; n < kOffSteps; ++n)
-        C[n] = make_double4(n ? (2.0 * n + 1.0) / n : 0.0, n ? (n + 1.0) / n : 0.0, (2.0 * n + 1.0) / (n + 1.0),
-                            n / (n + 1.0));
+        C[n] = OffStep{n ? (2.0 * n + 1.0) / n : 0.0, n ? (n + 1.0) / n : 0.0, (2.0 * n + 1.0) / (n + 1.0),
+                            n / (n + 1.0)};
     VFMM_CUDA(cudaMalloc(&t->G, G.size() * sizeof(double)));
-    VFMM_CUDA(cudaMalloc(&t->C, C.size() * sizeof(double4)));
+    VFMM_CUDA(cudaMalloc(&t->C, C.size() * sizeof(OffStep)));
     VFMM_CUDA(cudaMemcpyAsync(t->G, G.data(), G.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    VFMM_CUDA(cudaMemcpyAsync(t->C, C.data(), C.size() * sizeof(double4), cudaMemcpyHostToDevice, st));
+    VFMM_CUDA(cudaMemcpyAsync(t->C, C.data(), C.size() * sizeof(OffStep), cudaMemcpyHostToDevice, st));
     VFMM_CUDA(cudaStreamSynchronize(st));
     return VFMM_OK;
 }
@@ -269,7 +272,7 @@ __device__ __forceinline__ void off_coeffs_n(int nu, const double* G, int K, int
 // p, g, T: Legendre coefficients of P, its outward and its tangential derivative, stride kOffTasks; logs is
 // log(h / 2); (tr, ti) the conjugate of the edge's direction.
 __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, const double* p, const double* g,
-                                           const double* T, int N, const double4* __restrict__ C, double logs,
+                                           const double* T, int N, const OffStep* __restrict__ C, double logs,
                                            double tr, double ti, double* out) {
     const double zr = 0.5 * (w2 - w1), n1 = w1 * w1 + zi * zi, n2 = w2 * w2 + zi * zi;
     const double l1 = 0.5 * log(n1);
@@ -303,7 +306,7 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
             add(n, qr, qi, gm, gn, gp);
             gm = gn;
             gn = gp;
-            const double4 c = C[n + 1];
+            const OffStep c = C[n + 1];
             const double xr = c.z * (zr * rr - zi * ri) - c.w * qr, xi = c.z * (zr * ri + zi * rr) - c.w * qi;
             qr = rr;
             qi = ri;
@@ -314,7 +317,7 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
         int n = N + 1 + (int)(18.5f / logf(rho));
         double qr = 1e-100, qi = 0.0, rr = 0.0, ri = 0.0;  // q_n, q_(n+1)
         for (; n > N; --n) {
-            const double4 c = C[n];
+            const OffStep c = C[n];
             const double xr = c.x * (zr * qr - zi * qi) - c.y * rr, xi = c.x * (zr * qi + zi * qr) - c.y * ri;
             rr = qr;
             ri = qi;
@@ -328,7 +331,7 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
             if (n == 0) break;
             gp = gn;
             gn = gm;
-            const double4 c = C[n];
+            const OffStep c = C[n];
             const double xr = c.x * (zr * qr - zi * qi) - c.y * rr, xi = c.x * (zr * qi + zi * qr) - c.y * ri;
             rr = qr;
             ri = qi;
@@ -568,7 +571,7 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
                 for (int m = 0; m < N; ++m) {
                     leg[2 * lane][m] = p0;
                     leg[2 * lane + 1][m] = 2.0 * q0;
-                    const double4 c = a.t.C[m + 1];
+                    const OffStep c = a.t.C[m + 1];
                     const double p2 = c.z * x * p1 - c.w * p0, q2 = fma((double)(2 * m + 3), p1, q0);
                     p0 = p1;
                     p1 = p2;
