@@ -236,7 +236,8 @@ int vfmm_ops_destroy(vfmm_ops* ops);
  * base-128 digits (56 bits below its power-of-two scale); a contraction that takes S of them
  * (6 <= S <= 8) issues the S (S + 1) / 2 slice products i + j <= S + 1 and rounds each operand at
  * 2^(-7 S - 1) of its scale: fewer tensor-core products and fewer gathered bytes, less accuracy.
- * slices[5] = near field, S2M, M2L, S2L, leaf far field (L2T + M2T); a new operator set takes 6
+ * slices[5] = near field, S2M, M2L, S2L, leaf far field (L2T + M2T; one more is taken for k >= 6, where it
+ * runs in the reflection classes of the square); a new operator set takes 6
  * for all, the fewest allowed: the error against the FP64 form stays at or below 6e-12 on the
  * adaptive 20-Gaussian (k = 16, p = 40), kinked and uniform depth-7 (k = 16) workloads.
  * Host-only; applies to later calls and graph captures (a graph keeps the counts it captured); not
@@ -355,8 +356,8 @@ int vfmm_evaluate_points(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
  * cudaMalloc is available to this library). It runs vfmm_volume_potential with its
  * workspace in a fixed 32 MiB static device array that every GPU loading the library
  * holds until the process exits, and never calls cudaMalloc or cudaFree.
- *  - Size limit: trees whose vfmm_workspace_size (nrhs = 1, with_io = 0) exceeds 32 MiB
- *    are rejected with VFMM_ERR_WORKSPACE (roughly a few hundred leaves at k = 8).
+ *  - Size limit: trees whose workspace for one right-hand side exceeds 32 MiB (the mixed form's
+ *    operand buffers at their smallest, so at most vfmm_workspace_size) are rejected with VFMM_ERR_WORKSPACE (roughly a few hundred leaves at k = 8).
  *  - Right-hand sides are solved one after another in the same scratch (the mixed form
  *    does not fold them here, since that would build new schedules in device memory),
  *    every launch on `stream` (no second stream is created).

@@ -546,6 +546,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) downward_pass_kernel(PassArgs
 // scalar, the split contraction outputs (hi, lo) scaled back by their power-of-two exponents. The
 // scalar part, the same at every node of the leaf, is FP64:
 // -(1/2pi) [log(h) sum_U a_0 + Re b_0 + sum_W a_0 (log h_w)], h_w = h / 2 (first warp, fixed-order sums).
+// q / d for q below 1024 and d up to 64: (q m) >> 16, m = floor(65535 / d) + 1.
+struct SmallDiv {
+    unsigned m;
+    __device__ __forceinline__ int operator()(int q) const { return (int)(((unsigned)q * m) >> 16); }
+};
+static SmallDiv small_div(int d) { return SmallDiv{65535u / (unsigned)d + 1u}; }
+
 struct LeafMixedArgs {
     int nleaf, R, k, kk, Rp, P, lw;
     double wm;
@@ -555,9 +562,11 @@ struct LeafMixedArgs {
     const int32_t *uptr, *uidx, *wptr, *widx;
     const double* Mexp;
     const double* Lexp;
-    ClassTab ct;
+    SmallDiv by_hh, by_h, by_k;
+    int near_split, far_split;  // partial sums by classes
+    ClassTab ct, ft;        // near field, far field (N = 0: by entries)
     const float2* nearmix;  // class rows (ct.N > 0) or node rows
-    const int* Er;          // exponents of the quadrant rows or of the node rows
+    const int* Er;          // exponents of these rows
     const int* Ef;
     const float2* farmix;
     const int* farE;
@@ -584,10 +593,51 @@ __device__ __forceinline__ float2 df_sum(float2 a, float2 b, float sgn) {
     return df_final(hi, lo);
 }
 
+// Node values s [3][kk] from class rows: the four classes of a quadrant node, brought to the largest of their
+// exponents, put together at its images (double-FP32: the FP64 pipe is what bounds the kernel), and
+// that exponent, se [3][quadrant nodes].
+__device__ __forceinline__ void class_nodes(const ClassTab& ct, const float2* __restrict__ rows,
+                                            int split, size_t stride, const int* __restrict__ E, int k, SmallDiv by_hh,
+                                            SmallDiv by_h, float2* s, int* se) {
+    const int hx = (k + 1) / 2, kk = k * k;
+    for (int q = threadIdx.x; q < 3 * hx * hx; q += blockDim.x) {
+        const int fl = by_hh(q), e = q - fl * hx * hx, j = by_h(e), i = e - j * hx;
+        float2 w[4];  // by the field's parity in x and y
+        int ew[4], emax = -1000;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int pa = u & 1, pb = u >> 1, c = (pa ^ (fl == 1)) | ((pb ^ (fl == 2)) << 1), nx = sym_half(k, pa);
+            const bool in = i < nx && j < sym_half(k, pb);
+            const int row = ct.seg[3 * c + fl] + j * nx + i;
+            w[u] = in ? rows[row] : make_float2(0.0f, 0.0f);
+            for (int sp = 1; in && sp < split; ++sp) w[u] = df_sum(w[u], rows[sp * stride + row], 1.0f);
+            ew[u] = in ? E[row] : -1000;
+            emax = max(emax, ew[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            // 2^(ew - emax); an exponent 100 below the largest is far beneath its last bit
+            const float sc = ew[u] > emax - 100 ? __int_as_float((127 + ew[u] - emax) << 23) : 0.0f;
+            w[u] = make_float2(w[u].x * sc, w[u].y * sc);
+        }
+        se[q] = emax;
+        const float2 x = df_sum(w[0], w[1], 1.0f), y = df_sum(w[0], w[1], -1.0f);
+        const float2 z = df_sum(w[2], w[3], 1.0f), v = df_sum(w[2], w[3], -1.0f);
+        float2* o = s + fl * kk;
+        const int i1 = k - 1 - i, j1 = k - 1 - j;
+        o[j * k + i] = df_sum(x, z, 1.0f);
+        if (i1 != i) o[j * k + i1] = df_sum(y, v, 1.0f);
+        if (j1 != j) o[j1 * k + i] = df_sum(x, z, -1.0f);
+        if (i1 != i && j1 != j) o[j1 * k + i1] = df_sum(y, v, -1.0f);
+    }
+}
+
 __global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
     // width = wm 2^lw with wm in [1, 2): h = wm 2^(lw - lv), so every power-of-two scale is folded
     // into the exponents (f2d_scaled), times wm^(2, 1, -1) when wm is not one
-    extern __shared__ float2 s_near[];  // [3][kk] near field at the nodes
+    // near field and far field at the nodes, [3][kk] each; by classes, their exponents [3][h][h]
+    extern __shared__ float2 s_near[];
+    __shared__ int s_ne[3 * 64], s_fe[3 * 64];
     __shared__ double s_scal;
     const int nleaf = a.nleaf, R = a.R, kk = a.kk, Rp = a.Rp, lw = a.lw, k = a.k, hx = (k + 1) / 2;
     const double wm = a.wm;
@@ -596,49 +646,32 @@ __global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
     const unsigned leaf = vl / (unsigned)R, r = vl - leaf * (unsigned)R;
     const int b = a.box_of_leaf[leaf];
     const int lv = a.level[b];
-    // near field: the four classes of a quadrant node put together at its images (double-FP32: sums of
-    // numbers of one power-of-two scale, and the FP64 pipe is what bounds this kernel)
-    if (a.ct.N == 0) {  // near field by entries: node rows
+    float2* s_far = s_near + 3 * kk;
+    if (a.ct.N == 0) {  // by entries: node rows
         const float2* nm = a.nearmix + (size_t)vl * Rp;
         for (int q = t; q < 3 * kk; q += blockDim.x) s_near[q] = nm[q];
     } else {
-        const float2* nm = a.nearmix + (size_t)vl * (4 * a.ct.nch * a.ct.N);
-        for (int q = t; q < 3 * hx * hx; q += blockDim.x) {
-            const int fl = q / (hx * hx), e = q - fl * hx * hx, j = e / hx, i = e - j * hx;
-            float2 w[4];  // by the field's parity in x and y
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int pa = sym_pa(c, fl), pb = sym_pb(c, fl), nx = sym_half(k, pa);
-                const bool in = i < nx && j < sym_half(k, pb);
-                const float2 x = in ? nm[a.ct.seg[3 * c + fl] + j * nx + i] : make_float2(0.0f, 0.0f);
-                const int s = pa | (pb << 1);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (s == u) w[u] = x;
-            }
-            const float2 x = df_sum(w[0], w[1], 1.0f), y = df_sum(w[0], w[1], -1.0f);
-            const float2 z = df_sum(w[2], w[3], 1.0f), v = df_sum(w[2], w[3], -1.0f);
-            float2* o = s_near + fl * kk;
-            const int i1 = k - 1 - i, j1 = k - 1 - j;
-            o[j * k + i] = df_sum(x, z, 1.0f);
-            if (i1 != i) o[j * k + i1] = df_sum(y, v, 1.0f);
-            if (j1 != j) o[j1 * k + i] = df_sum(x, z, -1.0f);
-            if (i1 != i && j1 != j) o[j1 * k + i1] = df_sum(y, v, -1.0f);
-        }
+        const size_t nrow = 4 * a.ct.nch * a.ct.N, frow = 4 * a.ft.nch * a.ft.N, nv = (size_t)nleaf * R;
+        class_nodes(a.ct, a.nearmix + vl * nrow, a.near_split, nv * nrow, a.Er, k, a.by_hh, a.by_h, s_near, s_ne);
+        class_nodes(a.ft, a.farmix + vl * frow, a.far_split, nv * frow, a.farE, k, a.by_hh, a.by_h, s_far, s_fe);
     }
     __syncthreads();
     double n0 = 0.0, n1 = 0.0, n2 = 0.0, f0 = 0.0, f1 = 0.0, f2 = 0.0;
     if (t < kk) {
         const float2* __restrict__ farmix = a.farmix;
-        const int* __restrict__ Er = a.Er;
-        const int* __restrict__ farE = a.farE;
+        const int* Er = a.ct.N ? s_ne : a.Er;
+        const int* farE = a.ct.N ? s_fe : a.farE;
         const int* __restrict__ Et = a.Et;
         const int* __restrict__ Ef = a.Ef;
         const float2* fm = farmix + (size_t)vl * Rp;
-        const int en = Ef[r] + (a.ct.N ? 1 : 0) + lw - lv, ef = Et[vl] + lv - lw;  // near scale h 2^(E_f + 0, 1), far scale 2^E_t / h
+        const int en = Ef[r] + (a.ct.N ? 1 : 0) + lw - lv, et = Et[vl], ef = et + lv - lw;  // near scale h 2^(E_f + 0, 1), far scale 2^E_t / h
         const float2 v0 = s_near[t], v1 = s_near[kk + t], v2 = s_near[2 * kk + t];
         float2 w0, w1, w2;
-        if (a.far_slab) {
+        if (a.ft.N) {
+            w0 = s_far[t];
+            w1 = s_far[kk + t];
+            w2 = s_far[2 * kk + t];
+        } else if (a.far_slab) {
             const int s0 = a.far_seg[leaf], s1 = a.far_seg[leaf + 1];
             w0 = slab_sum(a.far_slab, s0, s1, R, r, Rp, t);
             w1 = slab_sum(a.far_slab, s0, s1, R, r, Rp, kk + t);
@@ -648,13 +681,13 @@ __global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
             w1 = fm[kk + t];
             w2 = fm[2 * kk + t];
         }
-        const int tj = t / k, ti = t - tj * k;
+        const int tj = a.by_k(t), ti = t - tj * k;
         const int qn = a.ct.N ? min(tj, k - 1 - tj) * hx + min(ti, k - 1 - ti) : t, qs = a.ct.N ? hx * hx : kk;
         const int e0 = en + lw - lv + Er[qn], e1 = en + Er[qs + qn], e2 = en + Er[2 * qs + qn];
         n0 = f2d_scaled(v0.x, e0) + f2d_scaled(v0.y, e0);  // h^2 x near u
         n1 = f2d_scaled(v1.x, e1) + f2d_scaled(v1.y, e1);  // h x near u_x
         n2 = f2d_scaled(v2.x, e2) + f2d_scaled(v2.y, e2);
-        const int g0 = Et[vl] + farE[t], g1 = ef + farE[kk + t], g2 = ef + farE[2 * kk + t];
+        const int g0 = et + farE[qn], g1 = ef + farE[qs + qn], g2 = ef + farE[2 * qs + qn];
         f0 = f2d_scaled(w0.x, g0) + f2d_scaled(w0.y, g0);
         f1 = f2d_scaled(w1.x, g1) + f2d_scaled(w1.y, g1);  // far u_x / h
         f2 = f2d_scaled(w2.x, g2) + f2d_scaled(w2.y, g2);
@@ -782,10 +815,11 @@ struct Workspace {
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Workspace carving. The mixed form folds all nrhs right-hand sides into one solve (every
+// Workspace carving (tight: the mixed form's operand buffers at their smallest, for the fixed scratch). The mixed form folds all nrhs right-hand sides into one solve (every
 // per-box and per-leaf buffer has nrhs rows per box); the FP64 form solves them one at a time.
 static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Workspace* w, char* base,
-                  size_t* bytes) {
+                  size_t* bytes,
+                  bool tight = false) {
     const size_t P2 = 2 * (size_t)(o.p + 1), kk = (size_t)o.k * o.k;
     size_t off = 0;
     auto take = [&](double** p, size_t n) {
@@ -845,7 +879,13 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         take(&p, (nl * kSlices * mo->Kp * 2 + 7) / 8);
         if (w) w->mix.fsl = (void*)p;
         const bool cls = near_by_classes(o.k);
-        take(&p, nl * (cls ? 4 * mo->near.nch * mo->near.N : mo->Rp));
+        // partial sums of small trees' class contractions, in the scratch of fixed size none
+        const int ns = cls && !tight ? PS->near.split : 1, fs = cls && !tight ? PS->leaf.split : 1;
+        if (w) {
+            w->mix.near_split = ns;
+            w->mix.leaf_split = fs;
+        }
+        take(&p, nl * ns * (cls ? 4 * mo->near.nch * mo->near.N : mo->Rp));
         if (w) w->mix.out = (float2*)p;
         take(&p, R);
         if (w) w->mix.fmax = (unsigned long long*)p;
@@ -862,11 +902,18 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         if (w) w->mix.m2l_c0 = p;
         take(&p, nb * mo->Rx);
         if (w) w->mix.s2l_out = (float2*)p;
-        take(&p, ((size_t)T.n_far_slots * R * kSlices * mo->Kx * 2 + 7) / 8);
-        if (w) w->mix.aprep = (void*)p;
+        const size_t ab = cls ? class_operand_bytes(T, mo->leaf, PS->leaf, (int)R, 14, tight)
+                              : (size_t)T.n_far_slots * R * kSlices * mo->Kx * 2;
+        take(&p, (ab + 7) / 8);
+        if (w) {
+            w->mix.aprep = (void*)p;
+            w->mix.aprep_bytes = ab;
+        }
+        take(&p, cls ? (nb + 1) / 2 : 1);
+        if (w) w->mix.bexp = (int*)p;
         take(&p, (nl + 1) / 2);
         if (w) w->mix.Et = (int*)p;
-        take(&p, nl * mo->Rp);
+        take(&p, nl * fs * (cls ? 4 * mo->leaf.nch * mo->leaf.N : mo->Rp));
         if (w) w->mix.far_out = (float2*)p;
         size_t np[3] = {0, 0, 0};
         split_part_elems(T, *PS, o, np);
@@ -878,7 +925,7 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         }
         take(&p, cls ? nl * kk : 1);
         if (w) w->mix.ffix = (long long*)p;
-        const size_t ob = near_operand_bytes(T, PS->near, (int)R);
+        const size_t ob = class_operand_bytes(T, mo->near, PS->near, (int)R, 16, tight);
         take(&p, (ob + 7) / 8);
         if (w) {
             w->mix.near_opnd = p;
@@ -1100,7 +1147,9 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         } else {
             VFMM_CHECK(near_contract(T, PS, o, f, w.mix, st));
         }
-        launches += near_by_classes(o.k) ? near_launches(*mo, PS.near, w.mix.near_opnd_bytes) : gemm_launches(PS.entries);
+        launches += near_by_classes(o.k)
+                        ? 1 + class_launches(mo->near, PS.near, mo->slices[kCtrNear], w.mix.near_opnd_bytes)
+                        : gemm_launches(PS.entries);
         mark(se, ST_NEAR, true, st);
     }
     // S2M
@@ -1157,6 +1206,10 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         }
         VFMM_CHECK(m2l_mixed(T, PS, o, w.Mexp, w.mix, st));
         if (PS.m2l.n_groups > 0) launches += 2 + gemm_launches(PS.m2l, kDeferSplits);
+        if (near_by_classes(o.k)) {
+            VFMM_CHECK(leaf_class_bounds(T, PS, o, w.Mexp, w.mix, c0s));
+            ++launches;
+        }
         const int begin = T.level_start[2], end = T.level_start[T.depth + 1];
         const int64_t warps = (int64_t)(end - begin) * R;
         const size_t c0_smem = (size_t)kVCfg * P * sizeof(double2) + (size_t)kFarCfg * kk * sizeof(double);
@@ -1257,7 +1310,8 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     mark(se, ST_L2T, false, st);
     if (mixed) {
         VFMM_CHECK(far_leaf_mixed(T, PS, o, w.Mexp, w.Lexp, w.mix, st));
-        launches += 1 + gemm_launches(PS.far, kDeferSegments);
+        launches += near_by_classes(o.k) ? class_launches(mo->leaf, PS.leaf, leaf_class_slices(*mo), w.mix.aprep_bytes)
+                                         : 1 + gemm_launches(PS.far, kDeferSegments);
     } else {
         launches += T.n_inst[VFMM_LIST_W] > 0 ? 2 : 1;
         SymRun r;
@@ -1300,11 +1354,18 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         la.Mexp = w.Mexp;
         la.Lexp = w.Lexp;
         la.nearmix = w.mix.out;
+        const int hx = (o.k + 1) / 2;
+        la.by_hh = small_div(hx * hx);
+        la.by_h = small_div(hx);
+        la.by_k = small_div(o.k);
+        la.near_split = w.mix.near_split;
+        la.far_split = w.mix.leaf_split;
         la.ct = mo->near;
+        la.ft = mo->leaf;
         la.Er = near_by_classes(o.k) ? mo->near_E : mo->Er;
         la.Ef = w.mix.Ef;
         la.farmix = w.mix.far_out;
-        la.farE = mo->far_E;
+        la.farE = near_by_classes(o.k) ? mo->leaf_E : mo->far_E;
         la.Et = w.mix.Et;
         // an entry-major leaf far field leaves its per-leaf sums (a few entries per leaf) to this kernel
         la.far_slab = PS.far.entry ? w.mix.part : nullptr;
@@ -1312,7 +1373,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         la.u = u;
         la.ux = ux;
         la.uy = uy;
-        leaf_mixed_kernel<<<(unsigned)nv, std::max(32, ((kk + 31) / 32) * 32), (size_t)3 * kk * sizeof(float2), st>>>(la);
+        leaf_mixed_kernel<<<(unsigned)nv, std::max(32, ((kk + 31) / 32) * 32), (size_t)6 * kk * sizeof(float2), st>>>(la);
         ++launches;
     } else {
         LeafArgs a;
@@ -1358,6 +1419,11 @@ static int check_solve_args(const vfmm_tree* tree, const vfmm_ops* ops, int32_t 
     if (nrhs < 1) return fail(VFMM_ERR_INVALID_ARG, "nrhs must be >= 1");
     if (ops->p + 1 > 64) return fail(VFMM_ERR_INVALID_ARG, "p too large for the solve kernels");
     return VFMM_OK;
+}
+
+int vfmm::tight_workspace_bytes(const vfmm_tree* tree, const vfmm_ops* ops, size_t* bytes) {
+    VFMM_CHECK(check_solve_args(tree, ops, 1));
+    return layout(tree->t, *ops, 1, false, nullptr, nullptr, bytes, true);
 }
 
 extern "C" int vfmm_workspace_size(const vfmm_tree* tree, const vfmm_ops* ops, int32_t nrhs, int32_t with_io,
@@ -1410,12 +1476,12 @@ static int read_status(const Workspace& w) { return read_status_word(w.mix.err);
 
 int vfmm::volume_potential(const vfmm_tree* tree, const vfmm_ops* ops, const double* f_dev, int32_t nrhs,
                            double* u_dev, double* ux_dev, double* uy_dev, void* workspace_dev, size_t workspace_bytes,
-                           cudaStream_t st, bool fork, bool reset) {
+                           cudaStream_t st, bool fork, bool reset, bool tight) {
     VFMM_CHECK(check_solve_args(tree, ops, nrhs));
     if (!f_dev || !u_dev || !ux_dev || !uy_dev || !workspace_dev) return fail(VFMM_ERR_INVALID_ARG, "null buffer");
     Workspace w;
     size_t need = 0;
-    VFMM_CHECK(layout(tree->t, *ops, nrhs, false, &w, (char*)workspace_dev, &need));
+    VFMM_CHECK(layout(tree->t, *ops, nrhs, false, &w, (char*)workspace_dev, &need, tight));
     if (workspace_bytes < need) return fail(VFMM_ERR_WORKSPACE, "workspace too small");
     w.fork = fork;
     if (reset) VFMM_CHECK(reset_status(w, st));
@@ -1612,6 +1678,40 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
     VFMM_CUDA(cudaEventCreate(&e0));
     VFMM_CUDA(cudaEventCreate(&e1));
     int rc = VFMM_OK;
+    const bool cls = near_by_classes(ops->k);
+    int32_t& near_ctas = cls ? PS->near.ctas : PS->entries.ctas;
+    auto use_form = [](SplitPlan* P, bool entry) {
+        if (P->entry == entry || !P->alt) return;
+        SplitPlan* alt = P->alt;
+        P->alt = nullptr;
+        std::swap(*P, *alt);
+        P->alt = alt;
+    };
+    // the schedule as it stands, to go back to where its step is the faster one
+    struct Form {
+        bool entry;
+        int32_t split, ctas;
+    } forms0[4];
+    for (int j = 0; j < 4; ++j) forms0[j] = Form{jobs[j].P->entry, jobs[j].P->split, jobs[j].P->ctas};
+    const int near0 = near_ctas, pass0 = PS->pass_ctas;
+    // fastest of a few forked solves (the step as vfmm_volume_potential and its graphs run it)
+    auto time_step = [&]() -> float {
+        Workspace wf = w;
+        wf.fork = true;
+        float best = 1e30f;
+        for (int rep = 0; rep < 6 && rc == VFMM_OK; ++rep) {
+            cudaEventRecord(e0, st);
+            rc = solve_all(T, *ops, f_dev, nrhs, u_dev, ux_dev, uy_dev, wf, st);
+            cudaEventRecord(e1, st);
+            if (rc != VFMM_OK) break;
+            cudaError_t e = cudaEventSynchronize(e1);
+            float ms = 0.0f;
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+            if (e != cudaSuccess) rc = cuda_fail(e, "timing a forked solve");
+            if (rep > 0) best = std::min(best, ms);  // the first run warms up
+        }
+        return best;
+    };
     // fastest split-K factor of one form of a contraction (its current factor when it cannot split)
     auto time_form = [&](const Job& jb, SplitPlan* P, float2* part, int* best_sp, float* best_ms) {
         const double avg_units = (double)P->entries * (jb.Kp / kKBlock) / std::max(1, P->n_groups);
@@ -1684,15 +1784,9 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
             int sp_alt = 1;
             float ms_alt = -1.0f;
             time_form(jb, jb.P->alt, part, &sp_alt, &ms_alt);
-            if (rc == VFMM_OK && ms_alt >= 0.0f && ms_alt < ms) {
-                SplitPlan* alt = jb.P->alt;
-                jb.P->alt = nullptr;
-                std::swap(*jb.P, *alt);
-                jb.P->alt = alt;
-            }
+            if (rc == VFMM_OK && ms_alt >= 0.0f && ms_alt < ms) use_form(jb.P, !jb.P->entry);
         }
         if (rc == VFMM_OK) time_ctas(jb, jb.P, part);
-        if (splits) splits[j] = jb.P->split;
     }
     // Co-scheduling of the whole step: in a forked solve the near field (low-priority stream) and the
     // main chain share the SMs, and a near-field CTA leaves no room for anything else on its SM.
@@ -1700,44 +1794,51 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
     // 7/8 ... 4/8 of them with the cooperative tree passes capped to the SMs they leave free (they can
     // start only when their whole grid fits); the fastest is kept. A near field with fewer items than
     // half the SMs leaves the chain room as it is.
-    const bool cls = near_by_classes(ops->k);
-    int32_t& near_ctas = cls ? PS->near.ctas : PS->entries.ctas;
     const int sms = sm_count();
     const bool wide = cls ? 8 * PS->near.n_groups * mo->near.nch > sms : PS->entries.ctas > 0;
+    float best = 1e30f;
     if (rc == VFMM_OK && wide && T.depth >= 3) {
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, upward_pass_kernel, kPassThreads, pass_smem_bytes(ops->p + 1));
-        Workspace wf = w;
-        wf.fork = true;
-        const int near0 = near_ctas, pass0 = PS->pass_ctas;
-        float best = -1.0f;
         int best_near = near0, best_pass = pass0;
         const int fracs[6] = {0, 8, 7, 6, 5, 4};  // eighths of the SMs; 0: uncapped
         for (int c = 0; c < 6 && rc == VFMM_OK; ++c) {
             const int ncta = fracs[c] == 0 ? 0 : std::max(1, sms * fracs[c] / 8);
             near_ctas = ncta;
             PS->pass_ctas = fracs[c] == 0 || fracs[c] == 8 ? 0 : std::max(1, per_sm * (sms - ncta));
-            float total = 1e30f;  // the fastest of a few runs
-            for (int rep = 0; rep < 6 && rc == VFMM_OK; ++rep) {
-                cudaEventRecord(e0, st);
-                rc = solve_all(T, *ops, f_dev, nrhs, u_dev, ux_dev, uy_dev, wf, st);
-                cudaEventRecord(e1, st);
-                if (rc != VFMM_OK) break;
-                cudaError_t e = cudaEventSynchronize(e1);
-                float ms = 0.0f;
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                if (e != cudaSuccess) rc = cuda_fail(e, "timing a forked solve");
-                if (rep > 0) total = std::min(total, ms);  // the first run warms up
-            }
-            if (rc == VFMM_OK && (best < 0.0f || total < best)) {
-                best = total;
+            const float ms = time_step();
+            if (rc == VFMM_OK && ms < best) {
+                best = ms;
                 best_near = near_ctas;
                 best_pass = PS->pass_ctas;
             }
         }
         near_ctas = best_near;
         PS->pass_ctas = best_pass;
+    } else if (rc == VFMM_OK) {
+        best = time_step();
     }
+    // The contractions were timed alone; beside each other their fastest forms need not make the fastest
+    // step (1,378 leaves: 353 us as planned, 365 with the forms picked alone)
+    if (rc == VFMM_OK) {
+        const int near1 = near_ctas, pass1 = PS->pass_ctas;
+        Form forms1[4];
+        for (int j = 0; j < 4; ++j) forms1[j] = Form{jobs[j].P->entry, jobs[j].P->split, jobs[j].P->ctas};
+        auto set = [&](const Form* f, int nc, int pc) {
+            for (int j = 0; j < 4; ++j) {
+                use_form(jobs[j].P, f[j].entry);
+                jobs[j].P->split = f[j].split;
+                jobs[j].P->ctas = f[j].ctas;
+            }
+            near_ctas = nc;
+            PS->pass_ctas = pc;
+        };
+        set(forms0, near0, pass0);
+        const float ms = time_step();
+        if (rc == VFMM_OK && ms > best) set(forms1, near1, pass1);
+    }
+    if (splits)
+        for (int j = 0; j < 4; ++j) splits[j] = jobs[j].P->split;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     VFMM_CHECK(rc);

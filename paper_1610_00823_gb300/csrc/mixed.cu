@@ -462,6 +462,8 @@ void mixed_free(vfmm_ops* o) {
     far_free(mo);
     if (mo->near_tab) cudaFree(mo->near_tab);
     if (mo->near_E) cudaFree(mo->near_E);
+    if (mo->leaf_tab) cudaFree(mo->leaf_tab);
+    if (mo->leaf_E) cudaFree(mo->leaf_E);
     if (mo->tsl) cudaFree(mo->tsl);
     if (mo->Er) cudaFree(mo->Er);
     delete mo;
@@ -551,10 +553,12 @@ int commit_plan_arena(PlanArena& A, PlanSet* PS, cudaStream_t st) {
             int32_t** field[6] = {&P->tgt, &P->ptr, &P->cfg, &P->src, &P->seg, &P->seg_out};
             for (int i = 0; i < 6; ++i) *field[i] = P->off[i] >= 0 ? b + P->off[i] : nullptr;
         }
-    if (PS->near.n_groups == 0) return VFMM_OK;
-    PS->near.order = b + PS->near.off[0];
-    PS->near.gmask = b + PS->near.off[1];
-    PS->near.first_dev = b + PS->near.off[2];
+    for (ClassPlan* P : {&PS->near, &PS->leaf}) {
+        if (P->n_groups == 0) continue;
+        P->order = b + P->off[0];
+        P->gmask = b + P->off[1];
+        P->first_dev = b + P->off[2];
+    }
     return VFMM_OK;
 }
 
@@ -645,7 +649,8 @@ void free_split_plan(SplitPlan* P) {
 }
 
 void free_plan_set(PlanSet* ps) {
-    ps->near = NearPlan();
+    ps->near = ClassPlan();
+    ps->leaf = ClassPlan();
     free_split_plan(&ps->entries);
     free_split_plan(&ps->s2m);
     free_split_plan(&ps->m2l);
@@ -805,8 +810,9 @@ static int build_plans(const DeviceTree& T, int R, const HostLists& H, PlanSet* 
     int rc[kNumCtr];
     auto task = [&](int c) {
         cudaSetDevice(dev);  // the split-K heuristic reads the device's SM count
-        if (c != kCtrNear) rc[c] = build_far_plan(c, T, R, H, A[c], PS);
-        else if (near_by_classes(T.k)) rc[c] = build_near_classes(T, R, H, A[c], &PS->near);
+        if (near_by_classes(T.k) && c == kCtrNear) rc[c] = build_near_classes(T, R, H, A[c], &PS->near);
+        else if (near_by_classes(T.k) && c == kCtrFar) rc[c] = build_leaf_classes(T, R, H, A[c], &PS->leaf);
+        else if (c != kCtrNear) rc[c] = build_far_plan(c, T, R, H, A[c], PS);
         else rc[c] = build_near_plan(T, R, H, A[c], PS);
     };
     std::vector<std::thread> workers;
@@ -830,8 +836,8 @@ static int build_plans(const DeviceTree& T, int R, const HostLists& H, PlanSet* 
         for (SplitPlan* P = top[c]; P; P = P->alt)
             for (int i = 0; i < 6; ++i)
                 if (P->off[i] >= 0) P->off[i] += base;
-        if (c == kCtrNear)
-            for (int64_t& off : PS->near.off) off += base;
+        if (c == kCtrNear || c == kCtrFar)
+            for (int64_t& off : (c == kCtrNear ? PS->near : PS->leaf).off) off += base;
         all.data.insert(all.data.end(), A[c].data.begin(), A[c].data.end());
     }
     return commit_plan_arena(all, PS, st);
@@ -840,7 +846,7 @@ static int build_plans(const DeviceTree& T, int R, const HostLists& H, PlanSet* 
 int build_mixed_plan(DeviceTree* T, cudaStream_t st) {
     HostLists H;
     VFMM_CHECK(fetch_host_lists(*T, &H));
-    VFMM_CHECK(build_far_slots(T, H, st));
+    if (!near_by_classes(T->k)) VFMM_CHECK(build_far_slots(T, H, st));
     VFMM_CHECK(build_instances(T, st));
     T->plans_r = new std::map<int, PlanSet*>();
     T->plans_mu = new std::mutex();

@@ -191,10 +191,14 @@ struct MixedOps {
     int Rp = 0;     // 3k^2 rounded up to N
     int Kp = 0;     // k^2 rounded up to kKBlock
     // near field in reflection classes (mixed_sym.cu): tables of every (orbit, class), exponents of the
-    // quadrant rows [3][h][h], h = (k + 1) / 2
+    // output rows
     ClassTab near;
     void* near_tab = nullptr;
     int* near_E = nullptr;
+    // leaf far field the same way: orbit 0 L2T, 1..5 M2T
+    ClassTab leaf;
+    void* leaf_tab = nullptr;
+    int* leaf_E = nullptr;
     // near field by entries: bf16 tables (table_at), 33, and their row exponents [Rp]
     void* tsl = nullptr;
     int* Er = nullptr;
@@ -248,6 +252,7 @@ struct MixedWork {
     long long* ffix = nullptr;            // [R][n_leaves][k^2] f 2^(55 - E_f), truncated (near field)
     void* near_opnd = nullptr;            // near field's operand tiles, a chunk at a time
     size_t near_opnd_bytes = 0;
+    int near_split = 1, leaf_split = 1;   // partial sums in out and far_out, one row set after another (by classes)
     unsigned long long* fmax = nullptr;   // [R] max |f| per right-hand side (bits)
     int* Ef = nullptr;                    // [R] exponent of f per right-hand side
     int* err = nullptr;                   // non-zero after a bounded wait expired
@@ -259,9 +264,11 @@ struct MixedWork {
     float2* m2l_out = nullptr;            // [n_boxes][Rx]
     double* m2l_c0 = nullptr;             // [n_boxes] Re local coefficient 0 from the V and X lists
     float2* s2l_out = nullptr;            // [n_boxes][Rx]
-    void* aprep = nullptr;                // bf16 [n_far_slots][kSlices][Kx]
+    void* aprep = nullptr;                // bf16 [n_far_slots][kSlices][Kx], or the classes' operand tiles, a chunk at a time
+    size_t aprep_bytes = 0;
+    int* bexp = nullptr;                  // [n_boxes] exponent bounds of the multipoles (far field by classes)
     int* Et = nullptr;                    // [n_leaves]
-    float2* far_out = nullptr;            // [n_leaves][Rp]
+    float2* far_out = nullptr;            // [n_leaves][Rp], or class rows [n_leaves][4 nch N]
     float2* part = nullptr;               // partial sums or slab of S2M, M2L and the leaf far field
     float2* part_side = nullptr;          // partial sums or slab of the near field by entries
     float2* part_s2l = nullptr;           // partial sums or slab of S2L
@@ -334,15 +341,28 @@ int build_far_plan(int which, const DeviceTree& T, int R, const HostLists& H, Pl
 // max |f| and the f slices (operand of S2M and S2L).
 int near_slices(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
                 cudaStream_t st);
-// Near field in reflection classes (mixed_sym.cu): tables, plan, operand buffer, solve, kernels launched.
-int near_classes_prepare(vfmm_ops* o, cudaStream_t st);
-int build_near_classes(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, NearPlan* P);
-size_t near_operand_bytes(const DeviceTree& T, const NearPlan& P, int R);
+// Near field (by classes or by entries).
 int near_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
                   cudaStream_t st);
+// Reflection classes (mixed_sym.cu): tables, plans, operand buffers, contractions and the kernels they launch.
+int near_classes_prepare(vfmm_ops* o, cudaStream_t st);
+int leaf_classes_prepare(vfmm_ops* o, const std::vector<double>& F, cudaStream_t st);
+int build_near_classes(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, ClassPlan* P);
+int build_leaf_classes(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, ClassPlan* P);
+size_t class_operand_bytes(const DeviceTree& T, const ClassTab& ct, const ClassPlan& P, int R, int rows, bool tight);
+double class_tiles(const ClassTab& ct, const ClassPlan& P);  // operand tiles of all pieces
 int near_class_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
                         cudaStream_t st);
-int near_launches(const MixedOps& mo, const NearPlan& P, size_t opnd_bytes);
+// exponent bounds of the multipoles, before leaf_class_contract (trees of depth 2 and more)
+int leaf_class_bounds(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const MixedWork& w,
+                      cudaStream_t st);
+int leaf_class_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const double* Lexp,
+                        const MixedWork& w, cudaStream_t st);
+// Slices that the leaf far field takes in reflection classes: one more than set. A node's images share the
+// rounding of the largest of them, which cost 1.7 times the error of the gathered form at the same count
+// (1,378 leaves, largest of u_x: 6.7e-12 against 3.0e-12); with one more it is 1.4e-12, for 3 % of a solve.
+inline int leaf_class_slices(const MixedOps& mo) { return mo.slices[kCtrFar] < kSlices ? mo.slices[kCtrFar] + 1 : kSlices; }
+int class_launches(const ClassTab& ct, const ClassPlan& P, int S, size_t opnd_bytes);
 int far_prepare(vfmm_ops* o, cudaStream_t st);
 void far_free(MixedOps* mo);
 // Stages of the split-precision far field (see mixed_far.cu). Multipoles and locals are stored per

@@ -164,7 +164,12 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
             }
         }
     }
-    VFMM_CHECK(slice_table(F, 1 + kFarCfg, R, KX, mo->Rp, table_rows_per_tile(near_transposed(o->k)), mo->Kx, &mo->far_sl, &mo->far_E, st));
+    if (near_by_classes(k)) {
+        VFMM_CHECK(leaf_classes_prepare(o, F, st));
+    } else {
+        VFMM_CHECK(slice_table(F, 1 + kFarCfg, R, KX, mo->Rp, table_rows_per_tile(near_transposed(o->k)), mo->Kx,
+                               &mo->far_sl, &mo->far_E, st));
+    }
     // S2L: rows 2..2p+1 (Re, Im of coefficients 1..p) over the k*k source values; row 0 kept in FP64
     std::vector<double> st_((size_t)kFarCfg * kk * P * 2);
     VFMM_CUDA(cudaMemcpy(st_.data(), o->s2l_t, st_.size() * sizeof(double), cudaMemcpyDeviceToHost));
@@ -529,6 +534,7 @@ __global__ void far_operand_kernel(int nleaf, int R, int P2, int Kx, const int32
 int far_leaf_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const double* Lexp,
                    const MixedWork& w, cudaStream_t st) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
+    if (near_by_classes(o.k)) return leaf_class_contract(T, PS, o, Mexp, Lexp, w, st);
     far_operand_kernel<<<T.n_leaves * PS.R, 128, 0, st>>>(T.n_leaves, PS.R, 2 * (o.p + 1), mo->Kx, T.box_of_leaf,
                                                           T.far_slot, T.lptr[VFMM_LIST_W], T.lidx[VFMM_LIST_W], Mexp,
                                                           Lexp, w.Et, (bf16*)w.aprep);
@@ -564,11 +570,15 @@ extern "C" int vfmm_solve_work(const vfmm_tree* tree, const vfmm_ops* ops, int32
         out[0] = tc(PS->entries, mo->Kp, mo->Rp, kCtrNear);
     } else {
         const int S = mo->slices[kCtrNear];
-        out[0] = 2.0 * (PS->near.first.empty() ? 0.0 : (double)PS->near.first.back()) * mo->near.nch * kTileM *
-                 mo->near.N * kKBlock * (S * (S + 1) / 2);
+        out[0] = 2.0 * class_tiles(mo->near, PS->near) * mo->near.nch * kTileM * mo->near.N * kKBlock * (S * (S + 1) / 2);
     }
     out[1] = tc(PS->m2l, mo->Kx, mo->Rx, kCtrM2L);
-    out[2] = tc(PS->far, mo->Kx, mo->Rp, kCtrFar);
+    if (near_by_classes(ops->k)) {
+        const int S = leaf_class_slices(*mo);
+        out[2] = 2.0 * class_tiles(mo->leaf, PS->leaf) * mo->leaf.nch * kTileM * mo->leaf.N * kKBlock * (S * (S + 1) / 2);
+    } else {
+        out[2] = tc(PS->far, mo->Kx, mo->Rp, kCtrFar);
+    }
     out[3] = tc(PS->s2l, mo->Kp, mo->Rx, kCtrS2L);
     out[4] = tc(PS->s2m, mo->Kp, mo->Rx, kCtrS2M);
     out[7] = (PS->entries.entry ? 1 : 0) + (PS->m2l.entry ? 2 : 0) + (PS->far.entry ? 4 : 0) + (PS->s2l.entry ? 8 : 0);

@@ -64,7 +64,7 @@ extern "C" int vfmm_volume_potential_noalloc(const vfmm_tree* tree, const vfmm_o
     // tree, whereas folding several into one solve (the mixed form's usual path) would build new
     // schedules in device memory on first use.
     size_t need = 0;
-    VFMM_CHECK(vfmm_workspace_size(tree, ops, 1, 0, &need));
+    VFMM_CHECK(tight_workspace_bytes(tree, ops, &need));
     if (need > kStaticScratchBytes)
         return fail(VFMM_ERR_WORKSPACE, "tree needs " + std::to_string(need) +
                                             " bytes of scratch; the static scratch holds " +
@@ -80,6 +80,6 @@ extern "C" int vfmm_volume_potential_noalloc(const vfmm_tree* tree, const vfmm_o
     const size_t n = (size_t)tree->t.n_leaves * ops->k * ops->k;
     for (int r = 0; r < nrhs; ++r)
         VFMM_CHECK(volume_potential(tree, ops, f_dev + r * n, 1, u_dev + r * n, ux_dev + r * n, uy_dev + r * n,
-                                    scratch, kStaticScratchBytes, (cudaStream_t)stream, false, false));
+                                    scratch, kStaticScratchBytes, (cudaStream_t)stream, false, false, true));
     return VFMM_OK;
 }

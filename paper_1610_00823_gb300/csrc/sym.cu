@@ -60,10 +60,12 @@ __global__ void sym_table_kernel(SymOp op, RepCfg rep, const double* __restrict_
     }
 }
 
-// Shape of an operator over list q's orbits (q < 0: the leaf itself) and its table.
+// Shape of an operator over list q's orbits (q < 0: the leaf itself; kLeafFar: the leaf itself, then the W
+// list's) and its table.
+constexpr int kLeafFar = 4;
 static int make_op(SymOp* op, int q, int k, int P, bool node_rows, bool node_cols, const double* T, int trows, int tcols,
                    cudaStream_t st) {
-    op->norb = q < 0 ? 1 : sym_orbits(q);
+    op->norb = q < 0 ? 1 : (q == kLeafFar ? 1 + kFarOrb : sym_orbits(q));
     op->k = k;
     op->P = P;
     op->node_rows = node_rows;
@@ -71,6 +73,13 @@ static int make_op(SymOp* op, int q, int k, int P, bool node_rows, bool node_col
     RepCfg rep = {};
     if (q < 0) {
         op->fx[0] = op->fy[0] = 1;
+    } else if (q == kLeafFar) {
+        op->fx[0] = op->fy[0] = 1;
+        for (int cfg = 0; cfg < kFarCfg; ++cfg) {
+            int slots;
+            const int o = sym_orbit(VFMM_LIST_W, cfg, &slots);
+            if (slots & 1) rep.cfg[1 + o] = 1 + cfg;
+        }
     } else {
         const int ncfg = q == VFMM_LIST_U ? kNearCfg : (q == VFMM_LIST_V ? kVCfg : kFarCfg);
         for (int cfg = 0; cfg < ncfg; ++cfg) {
@@ -148,6 +157,10 @@ static void m2t_tables(int k, int P, std::vector<double>& F) {
 
 int sym_near_op(const vfmm_ops* o, SymOp* op, cudaStream_t st) {
     return make_op(op, VFMM_LIST_U, o->k, o->p + 1, true, true, o->near, 3 * o->k * o->k, o->k * o->k, st);
+}
+
+int sym_far_op(const vfmm_ops* o, const double* F, SymOp* op, cudaStream_t st) {
+    return make_op(op, kLeafFar, o->k, o->p + 1, true, false, F, 3 * o->k * o->k, 2 * (o->p + 1), st);
 }
 
 int sym_prepare(vfmm_ops* o, const double* m2l, const double* s2l, cudaStream_t st) {
@@ -260,8 +273,8 @@ int build_instances(DeviceTree* T, cudaStream_t st) {
     auto work = [&]() -> int {
         inst_count_kernel<<<grid, 256, 0, st>>>(L, n, mask, cnt, flags);
         VFMM_CUDA(cudaGetLastError());
-        int64_t total = 0, same = 0;
-        VFMM_CHECK(exclusive_scan(flags, flags, (int64_t)kSymRows * n, &same, st));
+        int64_t total = 0;
+        VFMM_CHECK(exclusive_scan(flags, flags, (int64_t)kSymRows * n, nullptr, st));
         int32_t start[5] = {};
         VFMM_CHECK(exclusive_scan(cnt, cnt, (int64_t)4 * n, &total, st));
         for (int q = 1; q < 4; ++q)

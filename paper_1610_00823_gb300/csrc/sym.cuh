@@ -97,7 +97,9 @@ struct SymTables {
 // coefficient l (device). The tables are complete when st is.
 int sym_prepare(::vfmm_ops* o, const double* m2l, const double* s2l, cudaStream_t st);
 void sym_free(::vfmm_ops* o);
-// The near field's operator alone (its table is the caller's to free).
+// Operator alone, its table the caller's to free: the near field; L2T (orbit 0, the leaf itself) and the five
+// orbits of M2T from the plain tables F [21][3 k^2][2(p+1)] (L2T, then every W configuration; device).
+int sym_far_op(const ::vfmm_ops* o, const double* F, SymOp* op, cudaStream_t st);
 int sym_near_op(const ::vfmm_ops* o, SymOp* op, cudaStream_t st);
 
 // Instances of the four lists (built with the tree).

@@ -191,7 +191,7 @@ __global__ void scan_add_kernel(int32_t* __restrict__ out, const int32_t* __rest
 
 int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, cudaStream_t st) {
     if (n <= 0) {
-        *total = 0;
+        if (total) *total = 0;
         return VFMM_OK;
     }
     int64_t nb = (n + kScanItems - 1) / kScanItems;
@@ -200,6 +200,7 @@ int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, c
     scan_blocks_kernel<<<(unsigned)nb, 256, 0, st>>>(in, out, sums.p, n);
     VFMM_CUDA(cudaGetLastError());
     if (nb == 1) {
+        if (!total) return VFMM_OK;
         int32_t h = 0;
         VFMM_CUDA(cudaMemcpyAsync(&h, sums.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         VFMM_CUDA(cudaStreamSynchronize(st));

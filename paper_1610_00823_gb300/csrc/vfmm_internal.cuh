@@ -184,16 +184,20 @@ struct SplitPlan {
     int64_t off[6] = {-1, -1, -1, -1, -1, -1};
 };
 
-// Schedule of the near field in reflection classes: leaves ordered by their set of orbits, in groups of
-// 128 virtual leaves (leaf, r); a piece is one group's class (4 * group + class).
-struct NearPlan {
+// Schedule of a contraction in reflection classes: leaves ordered by their set of orbits, in groups of
+// 128 virtual leaves (leaf, r); a piece is one group's class (4 * group + class). The operand tiles (K
+// blocks) before a piece: a table (near field), or from the number of orbits beside the first one in the
+// groups before (leaf far field, whose K blocks per orbit depend on the expansion order).
+struct ClassPlan {
     int32_t n_groups = 0;
-    int32_t max_units = 0;         // most K blocks of a piece
-    int32_t ctas = 0;              // CTA cap of the launch (0: one CTA per item)
-    std::vector<int32_t> first;    // [4 n_groups + 1] first operand tile (K block) of each piece
+    int32_t max_units = 0;         // most K blocks of a piece (near field), most such orbits (far field)
+    int32_t ctas = 0;              // CTA cap of the launch (0: one per SM)
+    int32_t split = 1;             // CTAs that share the K blocks of a piece and row tile
+    std::vector<int32_t> first;    // near field: [4 n_groups + 1] first tile of each piece
+    std::vector<int32_t> orbits;   // far field: [n_groups + 1] orbits before each group
     int32_t* order = nullptr;      // [n_leaves]
     int32_t* gmask = nullptr;      // [n_groups] orbits of a group's leaves
-    int32_t* first_dev = nullptr;
+    int32_t* first_dev = nullptr;  // `first` or `orbits`
     int64_t off[3] = {0, 0, 0};    // their places in the plan set's arena while it is being built
 };
 
@@ -201,10 +205,11 @@ struct NearPlan {
 // virtual row of box or leaf x for right-hand side r is x * R + r (R consecutive rows per box).
 struct PlanSet {
     int R = 1;
-    NearPlan near;      // U list, reflection classes (near_by_classes(k)), else
+    ClassPlan near;     // U list, reflection classes (near_by_classes(k)), else
     SplitPlan entries;  // U list: targets leaves, tables 33 configurations, A rows leaves
     SplitPlan s2m;   // targets leaves, one table, A rows leaves
     SplitPlan m2l;   // V list: targets boxes, tables the 40 offsets, A rows boxes
+    ClassPlan leaf;  // L2T + W list, reflection classes (near_by_classes(k)), else
     SplitPlan far;   // L2T + W list: targets leaves, tables 0 (L2T) and 1 + W configuration, A rows far slots
     SplitPlan s2l;   // X list: targets boxes, tables 20 configurations, A rows leaves
     // grid cap of the persistent tree passes (0: one CTA per box of the widest level, at most one per
@@ -266,14 +271,17 @@ int plans_for(const DeviceTree& T, int R, const PlanSet** out);
 // and is called once the device has finished with it (free_tree synchronises the device first).
 int tree_malloc(void** p, size_t bytes, cudaStream_t st);
 void tree_free(void* p);
-// out[i] = sum_{j < i} in[j]; *total = sum of all (host; synchronises st). `in` and `out` may alias.
+// out[i] = sum_{j < i} in[j]; *total = sum of all (host; synchronises st unless null). `in` and `out` may alias.
 int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, cudaStream_t st);
 // vfmm_volume_potential with flags: fork = false keeps every launch on `st` (no second stream);
 // reset = false leaves the workspace's status word as it is (a caller solving several right-hand
-// sides one after another clears it once, so that a timeout in an early one is not lost).
+// sides one after another clears it once, so that a timeout in an early one is not lost); tight = true
+// takes the smallest operand buffers and no split sums (the allocation-free scratch).
 int volume_potential(const vfmm_tree* tree, const vfmm_ops* ops, const double* f_dev, int32_t nrhs, double* u_dev,
                      double* ux_dev, double* uy_dev, void* workspace_dev, size_t workspace_bytes, cudaStream_t st,
-                     bool fork, bool reset = true);
+                     bool fork, bool reset = true, bool tight = false);
+// Workspace bytes of a one-right-hand-side solve with tight = true.
+int tight_workspace_bytes(const vfmm_tree* tree, const vfmm_ops* ops, size_t* bytes);
 // Reads a status word (device address) after the solve that wrote it has finished: VFMM_OK, or
 // VFMM_ERR_TIMEOUT naming the bounded wait that ran out.
 int read_status_word(const int* word);
