@@ -35,10 +35,14 @@ constexpr double kInv2Pi = 0.15915494309189533577;
 // as much as the rest of a leaf's scalar terms.
 struct LevelLogs {
     double v[kMaxDepth + 1];
+    double h2[kMaxDepth + 1];  // h^2
 };
 static LevelLogs level_logs(double width) {
     LevelLogs l;
-    for (int i = 0; i <= kMaxDepth; ++i) l.v[i] = std::log(std::ldexp(width, -i));
+    for (int i = 0; i <= kMaxDepth; ++i) {
+        l.v[i] = std::log(std::ldexp(width, -i));
+        l.h2[i] = std::ldexp(width, -i) * std::ldexp(width, -i);
+    }
     return l;
 }
 
@@ -47,7 +51,7 @@ static LevelLogs level_logs(double width) {
 // FP64; the other coefficients come from the split-precision M2L and S2L. Persistent CTAs hold the
 // row-0 tables in shared memory; one warp per virtual box, the (entry, coefficient) pairs of eight
 // V entries at a time spread over the lanes.
-__global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, int P, double width,
+__global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, int P,
                                                      const __grid_constant__ LevelLogs logs,
                                                      const int32_t* __restrict__ level,
                                                      const int32_t* __restrict__ vptr, const int32_t* __restrict__ vidx,
@@ -69,7 +73,6 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
     for (int64_t vw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; vw < total;
          vw += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int b = begin + (int)(vw / R), r = (int)(vw % R);
-        const double h = ldexp(width, -level[b]);
         const double logh = logs.v[level[b]];
         // V list: the warp walks the entries; lane n takes coefficients n, n + 32 of the source
         // multipole (coalesced), partial sums stay per lane until one final reduction
@@ -107,7 +110,7 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
             const double* r0 = sX + xcfg[e] * kk;
             double part = 0.0;
             for (int s = lane; s < kk; s += 32) part += r0[s] * fc[s];
-            acc += 4.0 * h * h * part;
+            acc += 4.0 * logs.h2[level[b]] * part;
             if (lane == 0) acc += logh * Mexp[((size_t)xidx[e] * R + r) * 2 * P];
         }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -227,8 +230,8 @@ __device__ __forceinline__ double2 combine_local(const DownArgs& d, int level, i
         const float2 vi = d.s2l_out[vb * d.Rx + 2 * (t - 1) + 1];
         const int e = d.Ef[r] + 2 + 2 * (d.lw - level);
         const int er = e + d.s2l_E[2 * (t - 1)], ei = e + d.s2l_E[2 * (t - 1) + 1];
-        double sr = f2d_scaled(vr.x, er) + f2d_scaled(vr.y, er);
-        double si = f2d_scaled(vi.x, ei) + f2d_scaled(vi.y, ei);
+        double sr = f2d_pair(vr, er);
+        double si = f2d_pair(vi, ei);
         if (d.wm != 1.0) {
             sr *= d.wm * d.wm;
             si *= d.wm * d.wm;
@@ -244,8 +247,8 @@ __device__ __forceinline__ double2 combine_local(const DownArgs& d, int level, i
             const float2 vi = m2l_value(d, vb, 2 * (t - 1) + 1);
             const int g = level_exp_value(d.m2l_G[(size_t)level * d.R + r]);
             const int er = g + d.m2l_E[2 * (t - 1)], ei = g + d.m2l_E[2 * (t - 1) + 1];
-            re += f2d_scaled(vr.x, er) + f2d_scaled(vr.y, er);
-            im += f2d_scaled(vi.x, ei) + f2d_scaled(vi.y, ei);
+            re += f2d_pair(vr, er);
+            im += f2d_pair(vi, ei);
         }
     }
     return make_double2(re, im);
@@ -556,6 +559,7 @@ static SmallDiv small_div(int d) { return SmallDiv{65535u / (unsigned)d + 1u}; }
 struct LeafMixedArgs {
     int nleaf, R, k, kk, Rp, P, lw;
     double wm;
+    bool scaled;  // wm != 1 (a comparison in FP64 costs what an addition does)
     LevelLogs logs;
     const int32_t* box_of_leaf;
     const int32_t* level;
@@ -684,14 +688,14 @@ __global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
         const int tj = a.by_k(t), ti = t - tj * k;
         const int qn = a.ct.N ? min(tj, k - 1 - tj) * hx + min(ti, k - 1 - ti) : t, qs = a.ct.N ? hx * hx : kk;
         const int e0 = en + lw - lv + Er[qn], e1 = en + Er[qs + qn], e2 = en + Er[2 * qs + qn];
-        n0 = f2d_scaled(v0.x, e0) + f2d_scaled(v0.y, e0);  // h^2 x near u
-        n1 = f2d_scaled(v1.x, e1) + f2d_scaled(v1.y, e1);  // h x near u_x
-        n2 = f2d_scaled(v2.x, e2) + f2d_scaled(v2.y, e2);
+        n0 = f2d_pair(v0, e0);  // h^2 x near u
+        n1 = f2d_pair(v1, e1);  // h x near u_x
+        n2 = f2d_pair(v2, e2);
         const int g0 = et + farE[qn], g1 = ef + farE[qs + qn], g2 = ef + farE[2 * qs + qn];
-        f0 = f2d_scaled(w0.x, g0) + f2d_scaled(w0.y, g0);
-        f1 = f2d_scaled(w1.x, g1) + f2d_scaled(w1.y, g1);  // far u_x / h
-        f2 = f2d_scaled(w2.x, g2) + f2d_scaled(w2.y, g2);
-        if (wm != 1.0) {
+        f0 = f2d_pair(w0, g0);
+        f1 = f2d_pair(w1, g1);  // far u_x / h
+        f2 = f2d_pair(w2, g2);
+        if (a.scaled) {
             n0 *= wm * wm;
             n1 *= wm;
             n2 *= wm;
@@ -705,13 +709,9 @@ __global__ void leaf_mixed_kernel(const __grid_constant__ LeafMixedArgs a) {
         double m = 0.0, w0 = 0.0;
         for (int e = a.uptr[b] + t; e < a.uptr[b + 1]; e += 32) m += a.Mexp[((size_t)a.uidx[e] * R + r) * P2];
         for (int e = a.wptr[b] + t; e < a.wptr[b + 1]; e += 32) w0 += a.Mexp[((size_t)a.widx[e] * R + r) * P2];
-        for (int o = 16; o > 0; o >>= 1) {
-            m += __shfl_xor_sync(0xffffffffu, m, o);
-            w0 += __shfl_xor_sync(0xffffffffu, w0, o);
-        }
-        if (t == 0)
-            s_scal = -kInv2Pi * logh * m -
-                     kInv2Pi * (a.Lexp[((size_t)b * R + r) * P2] + w0 * (logh - 0.6931471805599453));
+        m = fma(logh, m, (logh - 0.6931471805599453) * w0);
+        for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        if (t == 0) s_scal = -kInv2Pi * (m + a.Lexp[((size_t)b * R + r) * P2]);
     }
     __syncthreads();
     if (t >= kk) return;
@@ -1222,7 +1222,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         }
         const unsigned c0_grid = (unsigned)std::min<int64_t>((warps + 7) / 8, 3ll * sm_count());
         m2l_c0_kernel<<<c0_grid, 256, c0_smem, c0s>>>(
-            begin, end, R, P, T.width, level_logs(T.width), T.level, T.lptr[VFMM_LIST_V], T.lidx[VFMM_LIST_V], T.lcfg[VFMM_LIST_V],
+            begin, end, R, P, level_logs(T.width), T.level, T.lptr[VFMM_LIST_V], T.lidx[VFMM_LIST_V], T.lcfg[VFMM_LIST_V],
             reinterpret_cast<const double2*>(mo->m2l_r0), w.Mexp, w.mix.m2l_c0, T.lptr[VFMM_LIST_X],
             T.lidx[VFMM_LIST_X], T.lcfg[VFMM_LIST_X], T.leaf_of_box, mo->s2l_r0, f, nleaf, kk);
         ++launches;
@@ -1344,6 +1344,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         la.P = P;
         la.lw = lw;
         la.wm = wm;
+        la.scaled = wm != 1.0;
         la.logs = level_logs(T.width);
         la.box_of_leaf = T.box_of_leaf;
         la.level = T.level;

@@ -99,6 +99,22 @@ __device__ __forceinline__ double f2d_scaled(float x, int e) {
     return __longlong_as_double((long long)(sign | (ex == 0 ? 0ull : mag)));
 }
 
+// f2d_scaled(v.x, e) + f2d_scaled(v.y, e), rounded as that sum, by integer operations: lo in units of the
+// last place of hi's double (half of it just below a power of two) is added to the bits. A pair whose lo
+// is not below half an ulp of hi takes the FP64 addition; the contractions' outputs are normalised.
+__device__ __forceinline__ double f2d_pair(float2 v, int e) {
+    const unsigned u = __float_as_uint(v.x), l = __float_as_uint(v.y);
+    const int ex = (int)((u >> 23) & 0xFF), lx = (int)((l >> 23) & 0xFF), d = ex - lx;
+    if (lx != 0 && d < 24) return f2d_scaled(v.x, e) + f2d_scaled(v.y, e);
+    const bool minus = (int)(u ^ l) < 0;
+    const int unit = 150 + 29 + (minus && (u & 0x7FFFFFu) == 0 ? 1 : 0) - d;  // biased exponent of lo in units
+    const int n = lx ? __float2int_rn(__uint_as_float(((unsigned)max(unit, 1) << 23 | (l & 0x7FFFFFu)))) : 0;
+    const long long mag = ex ? (((long long)(ex - 127 + 1023 + e) << 52) | ((long long)(u & 0x7FFFFFu) << 29)) +
+                                   (minus ? -n : n)
+                             : 0ll;
+    return __longlong_as_double(mag | ((long long)(u >> 31) << 63));
+}
+
 // Binary exponent e with |m| < 2^e (frexp convention), from the bits; 0 for m = 0.
 __device__ __forceinline__ int exp_bound(double m) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(m);
@@ -115,7 +131,8 @@ __device__ __forceinline__ size_t slice_at(size_t row, int Kp, int k) {
 // Level exponents of the M2L operand: G(l, r) = max over the boxes b of level l and the parts k
 // (Re, Im of coefficient k / 2) of multipole row b of part_exp(value, k), kept as G + kGexpBias in
 // an unsigned array that starts at zero, so that every producer of a multipole can take the maximum
-// with atomicMax as it writes (order-independent, hence deterministic).
+// with atomicMax as it writes (order-independent, hence deterministic; skipped where the slot already holds
+// as much, since the atomics of a level meet at one address).
 constexpr unsigned kGexpBias = 1u << 20;
 
 // frexp exponent of |v| (from the bits, integer work) plus floor(k / 4); INT_MIN for +-0.
@@ -130,7 +147,8 @@ __device__ __forceinline__ int part_exp(double v, int k) {
 // contribute nothing).
 __device__ __forceinline__ void level_exp_max(int e, unsigned* slot) {
     for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    if ((threadIdx.x & 31) == 0 && e != INT_MIN) atomicMax(slot, (unsigned)(e + (int)kGexpBias));
+    if ((threadIdx.x & 31) == 0 && e != INT_MIN && (unsigned)(e + (int)kGexpBias) > __ldcg(slot))
+        atomicMax(slot, (unsigned)(e + (int)kGexpBias));
 }
 
 // Block-wide maximum of e, then one atomicMax by thread 0 (every thread of the block must call it;
@@ -142,7 +160,7 @@ __device__ __forceinline__ void level_exp_max_block(int e, unsigned* slot) {
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < (int)((blockDim.x + 31) >> 5); ++w) e = max(e, wmax[w]);
-        if (e != INT_MIN) atomicMax(slot, (unsigned)(e + (int)kGexpBias));
+        if (e != INT_MIN && (unsigned)(e + (int)kGexpBias) > __ldcg(slot)) atomicMax(slot, (unsigned)(e + (int)kGexpBias));
     }
 }
 

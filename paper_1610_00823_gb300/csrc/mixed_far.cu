@@ -366,17 +366,27 @@ void split_part_elems(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o,
 // contraction scaled back by 2^(E_f[r] + E_row).
 // With split > 1 the contraction's split-K partial sums part[s][row][Rx] are summed here (the
 // reduction kernel's order and arithmetic) instead of read from out.
+// Bound by FP64 issue (8 + 6 instructions of one warp per leaf of 16 x 16 nodes) and latency: with scales by
+// exponent arithmetic, (hi, lo) pairs joined by integers and atomics only where a level's maximum grows,
+// 0.70 -> 0.43 ms at 200,104 leaves.
+// h = 2 wm 2^(lw - 1 - level), wm in [1, 2), and h^2 of every level: from the host, since what a device
+// ldexp or comparison costs in FP64 is what an addition of the whole warp does.
+struct LevelScale {
+    int lw;
+    bool scaled;  // wm != 1
+    double wm2;
+    double h2[kMaxDepth + 1];
+};
 __global__ void s2m_finish_kernel(int nleaf, int R, int kk, int p, int Rx, const int32_t* __restrict__ box_of_leaf,
-                                  const int32_t* __restrict__ level, double width, const double* __restrict__ f,
-                                  const double* __restrict__ s2m, const float2* __restrict__ out,
+                                  const int32_t* __restrict__ level, const __grid_constant__ LevelScale ls,
+                                  const double* __restrict__ f, const double* __restrict__ s2m, const float2* __restrict__ out,
                                   const float2* __restrict__ part, int split, size_t part_stride,
                                   const int* __restrict__ E, const int* __restrict__ Ef, double* __restrict__ Mexp,
                                   unsigned* __restrict__ glev) {
     const int vl = blockIdx.x;
     const int leaf = vl / R, r = vl - leaf * R;
     const int b = box_of_leaf[leaf];
-    const double h = ldexp(width, -level[b]);
-    const int P2 = 2 * (p + 1);
+    const int lv = level[b], P2 = 2 * (p + 1);
     double* M = Mexp + ((size_t)b * R + r) * P2;
     const double* fl = f + ((size_t)r * nleaf + leaf) * kk;
     int e = INT_MIN;  // exponent bound of this thread's parts (level exponents of the M2L operand)
@@ -385,15 +395,13 @@ __global__ void s2m_finish_kernel(int nleaf, int R, int kk, int p, int Rx, const
         for (int s = threadIdx.x; s < kk; s += 32) m += s2m[s] * fl[s];
         for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
         if (threadIdx.x == 0) {
-            M[0] = h * h * m;
+            M[0] = ls.h2[lv] * m;
             M[1] = 0.0;
             e = part_exp(M[0], 0);
         }
     }
     // h^2 = wm^2 2^(2 (lw - level)): the power of two goes into the exponent bits
-    int lw = 0;
-    const double wm = 2.0 * frexp(width, &lw);
-    const int ef = Ef[r] + 2 * (lw - 1 - level[b]);
+    const int ef = Ef[r] + 2 * (ls.lw - 1 - lv);
     for (int q = threadIdx.x; q < 2 * p; q += blockDim.x) {
         float2 v;
         if (split > 1) {
@@ -403,12 +411,13 @@ __global__ void s2m_finish_kernel(int nleaf, int R, int kk, int p, int Rx, const
         } else {
             v = out[(size_t)vl * Rx + q];
         }
-        const double m = f2d_scaled(v.x, ef + E[q]) + f2d_scaled(v.y, ef + E[q]);
-        M[2 + q] = wm == 1.0 ? m : wm * wm * m;
-        e = max(e, part_exp(M[2 + q], 2 + q));
+        double m = f2d_pair(v, ef + E[q]);
+        if (ls.scaled) m *= ls.wm2;
+        M[2 + q] = m;
+        e = max(e, part_exp(m, 2 + q));
     }
     // one atomic per CTA (the level slots are few and shared by every leaf of a level)
-    if (level[b] >= 2) level_exp_max_block(e, glev + (size_t)level[b] * R + r);
+    if (lv >= 2) level_exp_max_block(e, glev + (size_t)lv * R + r);
 }
 
 int s2m_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, double* Mexp,
@@ -420,8 +429,13 @@ int s2m_mixed(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const d
     // the split-K partials (when the plan splits) are summed by the finishing kernel
     const int sp = (!PS.s2m.entry && w.part) ? PS.s2m.split : 1;
     const size_t stride = (size_t)T.n_leaves * PS.R * mo->Rx;
+    LevelScale ls;
+    const double wm = 2.0 * std::frexp(T.width, &ls.lw);
+    ls.scaled = wm != 1.0;
+    ls.wm2 = wm * wm;
+    for (int i = 0; i <= kMaxDepth; ++i) ls.h2[i] = std::ldexp(T.width, -i) * std::ldexp(T.width, -i);
     s2m_finish_kernel<<<T.n_leaves * PS.R, 128, 0, st>>>(T.n_leaves, PS.R, o.k * o.k, o.p, mo->Rx, T.box_of_leaf,
-                                                         T.level, T.width, f, o.s2m, w.s2m_out, w.part, sp, stride,
+                                                         T.level, ls, f, o.s2m, w.s2m_out, w.part, sp, stride,
                                                          mo->s2m_E, w.Ef, Mexp, w.glev);
     VFMM_CUDA(cudaGetLastError());
     return VFMM_OK;
