@@ -1,6 +1,6 @@
 // The FMM passes of the box code (Section 3.1), with the gradient from differentiated tables and
 // expansions (Section 3.2), and the solve driver of both forms (FP64 below; the split-BF16
-// contractions of the mixed form are in mixed.cu and mixed_far.cu).
+// contractions of the mixed form are in mixed.cu, mixed_far.cu and mixed_sym.cu).
 //
 //   S2M      leaf multipoles  a = h^2 Q f
 //   M2M      one cooperative persistent pass over all levels (position-DFT form, readiness counters)
@@ -48,7 +48,8 @@ static LevelLogs level_logs(double width) {
 
 // Re of local coefficient 0 from the V and X lists of each virtual box (box, r): sum over V of
 // Re(row 0 of M2L_c . a_c) + a_0(c) log h, and over X of (2h)^2 Re(S2L row 0) . f_c + a_0(c) log h.
-// FP64; the other coefficients come from the split-precision M2L and S2L. Persistent CTAs hold the
+// FP64, which bounds it (two FMAs per term; as product, FMA and addition 1.54 ms, now 1.14, at 266,805
+// boxes); the other coefficients come from the split-precision M2L and S2L. Persistent CTAs hold the
 // row-0 tables in shared memory; one warp per virtual box, the (entry, coefficient) pairs of eight
 // V entries at a time spread over the lanes.
 __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, int P,
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
         const double logh = logs.v[level[b]];
         // V list: the warp walks the entries; lane n takes coefficients n, n + 32 of the source
         // multipole (coalesced), partial sums stay per lane until one final reduction
-        double acc = 0.0;
+        double acc = 0.0, acc2 = 0.0;  // two FMAs per term, in chains of their own
         const int e_end = vptr[b + 1];
         // V list in batches of 8 entries: the batch's (entry, coefficient) pairs spread over the lanes,
         // so all 32 lanes work whatever p is (coalesced within an entry's multipole)
@@ -92,7 +93,8 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
                 const int e = e0 + j;
                 const double2 x = reinterpret_cast<const double2*>(Mexp + ((size_t)vidx[e] * R + r) * 2 * P)[n];
                 const double2 m = sM[vcfg[e] * P + n];
-                acc += m.x * x.x - m.y * x.y;
+                acc = fma(m.x, x.x, acc);
+                acc2 = fma(-m.y, x.y, acc2);
                 n += 32;
                 while (n >= P) {
                     n -= P;
@@ -103,7 +105,8 @@ __global__ void __launch_bounds__(256) m2l_c0_kernel(int begin, int end, int R, 
         // log(h) a_0(c) of every V entry: one lane per entry
         double a0 = 0.0;
         for (int e = vptr[b] + lane; e < e_end; e += 32) a0 += Mexp[((size_t)vidx[e] * R + r) * 2 * P];
-        acc += a0 * logh;
+        acc += acc2;
+        acc = fma(a0, logh, acc);
         // X list: (2h)^2 [Re(S2L row 0) . f_c + log(h) W . f_c], with W . f_c = a_0(c) / (2h)^2
         for (int e = xptr[b]; e < xptr[b + 1]; ++e) {
             const double* fc = f + ((size_t)r * nleaf + leaf_of_box[xidx[e]]) * kk;
@@ -310,14 +313,14 @@ __device__ __forceinline__ void group_sync(int grp) {
     asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kGroupThreads) : "memory");
 }
 
+// v, or -v where `on` (bit 0): on the bits, since a negation kept in a register costs an FP64 instruction.
+__device__ __forceinline__ double flip(double v, int on) {
+    return __hiloint2double(__double2hiint(v) ^ (on << 31), __double2loint(v));
+}
 // v i^m (sign changes and swaps; exact).
 __device__ __forceinline__ double2 mul_ipow(double2 v, int m) {
-    switch (m & 3) {
-        case 0: return v;
-        case 1: return make_double2(-v.y, v.x);
-        case 2: return make_double2(-v.x, -v.y);
-        default: return make_double2(v.y, -v.x);
-    }
+    const double x = m & 1 ? v.y : v.x, y = m & 1 ? v.x : v.y;
+    return make_double2(flip(x, (m ^ (m >> 1)) & 1), flip(y, (m >> 1) & 1));
 }
 // v sigma0_l = v i^floor(l/2) (1 + i)^(l mod 2): one addition per component for odd l.
 __device__ __forceinline__ double2 mul_sigma0(double2 v, int l) {
@@ -331,9 +334,9 @@ __device__ __forceinline__ double2 mul_rho0(double2 v, int n) {
 }
 // sum_e i^(e k) x_e (one output of a 4-point DFT): (x0 +- x2) + i^k (x1 +- x3).
 __device__ __forceinline__ double2 dft4(double2 x0, double2 x1, double2 x2, double2 x3, int k) {
-    const bool odd = k & 1;
-    const double2 u = odd ? make_double2(x0.x - x2.x, x0.y - x2.y) : make_double2(x0.x + x2.x, x0.y + x2.y);
-    const double2 w = mul_ipow(odd ? make_double2(x1.x - x3.x, x1.y - x3.y) : make_double2(x1.x + x3.x, x1.y + x3.y), k);
+    const int o = k & 1;  // one addition per component whichever k, not one for each parity in a mixed warp
+    const double2 u = make_double2(x0.x + flip(x2.x, o), x0.y + flip(x2.y, o));
+    const double2 w = mul_ipow(make_double2(x1.x + flip(x3.x, o), x1.y + flip(x3.y, o)), k);
     return make_double2(u.x + w.x, u.y + w.y);
 }
 // Child slot of DFT index e (g_pos = i^e (1 + i)).
@@ -413,19 +416,19 @@ __global__ void __launch_bounds__(kPassThreads, 1) upward_pass_kernel(PassArgs a
             const double2* ea = sE + (oa & 3) * P;
             const double2* eb = sE + (ob & 3) * P;
             double ar = 0.0, ai = 0.0, br = 0.0, bi2 = 0.0;
-            for (int i = s; i < la + lb; i += ns) {
-                if (i < la) {
-                    const double m = sR[i * P + oa];
-                    const double2 e = ea[i];
-                    ar = fma(m, e.x, ar);
-                    ai = fma(m, e.y, ai);
-                } else {
-                    const int n = i - la;
-                    const double m = sR[n * P + ob];
-                    const double2 e = eb[n];
-                    br = fma(m, e.x, br);
-                    bi2 = fma(m, e.y, bi2);
-                }
+            // one loop per row: in a common loop a warp whose lanes are in different rows issues both bodies
+            int i = s;
+            for (; i < la; i += ns) {
+                const double m = sR[i * P + oa];
+                const double2 e = ea[i];
+                ar = fma(m, e.x, ar);
+                ai = fma(m, e.y, ai);
+            }
+            for (i -= la; i < lb; i += ns) {
+                const double m = sR[i * P + ob];
+                const double2 e = eb[i];
+                br = fma(m, e.x, br);
+                bi2 = fma(m, e.y, bi2);
             }
             sPart[2 * g] = make_double2(ar, ai);
             sPart[2 * g + 1] = make_double2(br, bi2);
@@ -1007,7 +1010,9 @@ static void fill_down_args(DownArgs& d, const DeviceTree& T, const vfmm_ops& o, 
 
 // One cooperative launch per pass, whatever the tree's size: one real matrix-vector product per box, and
 // no launch per level. On 266,805 boxes the upward levels took 2.17 ms as one launch each, 1.21 as a pass,
-// the downward ones 2.32 and 1.60; small trees are bound by the levels' latency.
+// the downward ones 2.32 and 1.60; with one FP64 addition per term of the DFTs whatever the lane's index and
+// one loop per row 0.89 and 1.43. Bound by FP64 (2 FMA a clock and SM) and its latency at one CTA per SM;
+// small trees by the levels' latency.
 template <typename... Args>
 static int launch_pass(void (*kernel)(Args...), int R, int P, int widest_items, int cap, cudaStream_t st,
                        Args... args) {
