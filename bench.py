@@ -39,6 +39,8 @@ import workloads as W  # noqa: E402
 
 METRIC = "volume-FMM target pts/s at 1e-10 rel err: mixed/batched vs plain FP64, 1 GB300"
 UNIT = "target points/s"
+NEAR_FLOPS = ("issued: S(S+1)/2 slice products (S = the contraction's slices) of every tile of the reflection-class "
+              "form, which needs about a quarter of the products of one table per list entry; padded rows included")
 FP64_OVER_BF16 = 1.25 / 2250.0  # nominal dense FP64 / BF16 tensor ratio of GB300
 
 
@@ -312,7 +314,7 @@ def run_batch(args):
         from paper_1610_00823_gb300 import build as b
         b.build()
     import paper_1610_00823_gb300 as v
-    from paper_1610_00823_gb300.api import Batch, tune, volume_potential_profiled, workspace
+    from paper_1610_00823_gb300.api import Batch, solve_work, tune, volume_potential_profiled, workspace
     stream = torch.cuda.Stream()
     torch.cuda.set_stream(stream)
     t0 = time.perf_counter()
@@ -374,16 +376,13 @@ def run_batch(args):
     tc, near_ms, launches = 0.0, 0.0, 0
     for tree, ops, f, out, ws in items_mx:
         stages, nl = volume_potential_profiled(tree, ops, f, out, ws, stream=stream)
-        kk_m = tree.k * tree.k
-        sn = ops.slices["near"]
-        tc += sn * (sn + 1) / 2 * 2.0 * 3 * kk_m * kk_m * tree.list_len[0]  # algorithmic slice-product flops
+        tc += solve_work(tree, ops)["near_tc_flops"]  # slice products of the class tables
         near_ms += stages.get("near_tc") or stages["near"]
         launches += nl
     peaks, peak_kind = measured_peaks()
     achieved = tc / (near_ms / 1e3) / 1e12
-    roof = {"kernel": "split_gemm_kernel (near field, split-BF16 tcgen05), summed over members",
-            "flops": "algorithmic: S(S+1)/2 slice products (S = the near field's slices) x 2 x 3k^2 x k^2 "
-                     "per U-list entry",
+    roof = {"kernel": "class_gemm_kernel and its operands (near field, split-BF16 tcgen05), summed over members",
+            "flops": NEAR_FLOPS,
             "bound": "tensor", "achieved": achieved, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
             "frac": achieved / peaks["bf16_tflops"], "traffic": None, "peak_source": "%s bf16 burst" % peak_kind,
             "flops_per_launch": tc / n_members, "ms_per_launch": near_ms / n_members,
@@ -699,7 +698,7 @@ def main():
                                 "frac": iach / ipeak, "flops": "3 fields x 2 k^2 per point",
                                 "peak_source": "%s bf16 x nominal FP64/BF16 ratio (1.25/2250)" % peak_kind}}
         # V f~ itself at arbitrary points from the solve's stored expansions (vfmm_evaluate_points):
-        # the first 1024 of the same points; far part O(p), near part by on-the-fly quadrature (FP64)
+        # the first 1024 of the same points; far part O(p), near part in closed form on the leaves' edges (FP64)
         n_ev = 1024
         ex, ey = px[:n_ev].contiguous(), py[:n_ev].contiguous()
         v.evaluate_points(tree, ops, f, ws, ex, ey, stream=stream)
@@ -719,19 +718,23 @@ def main():
                                         "sample": "the first 1024 of the points above"}
     co_schedule = None
     if args.precision == "fp64":
-        flops = 2.0 * 3 * kk * kk * tree.list_len[0] * nrhs  # near-field table applies per step
+        # near-field table applies per step, one table per list entry; the reflection classes need about a quarter
+        flops = 2.0 * 3 * kk * kk * tree.list_len[0] * nrhs
         achieved = flops / (stage_ms["near"] / 1e3) / 1e12
         peak = peaks["bf16_tflops"] * FP64_OVER_BF16
-        roof = {"kernel": "near_gemm_kernel", "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        roof = {"kernel": "sym_gemm_kernel (near field)", "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": None,
                 "peak_source": "%s bf16 x nominal FP64/BF16 ratio (1.25/2250)" % peak_kind,
+                "flops": "2 x 3k^2 x k^2 per U-list entry; the reflection classes do about a quarter of these, so the "
+                         "fraction can pass one",
                 "flops_per_launch": flops, "ms_per_launch": stage_ms["near"]}
     else:
         work = solve_work(tree, ops, nrhs)
         # the tuner's co-schedule of the forked step (near-field CTA cap, tree-pass grid cap; 0 = none)
         co_schedule = {"near_field_ctas": int(work["near_ctas"]), "tree_pass_ctas": int(work["pass_ctas"])}
         peak = peaks["bf16_tflops"]
-        # algorithmic work of each split contraction: the S(S+1)/2 BF16 slice products (S = its slices) of every real
+        # near and leaf far field by reflection classes (k >= 6): the slice products issued, tile by tile.
+        # Other contractions, algorithmic work: the S(S+1)/2 BF16 slice products (S = its slices) of every real
         # multiply-add the method needs (list entries x rows x K, no zero rows, no padding); the
         # kernels also execute zero rows of targets lacking a table in their group and padded tiles
         # ("executed")
@@ -746,16 +749,18 @@ def main():
             ms_c = stage_ms.get(name + "_tc", 0.0)
             ex = work[name + "_tc_flops"]
             S = ops.slices[name]
-            alg = S * (S + 1) / 2 * alg_fp64eq[name] * nrhs
+            by_classes = name in ("near", "far") and wl.k >= 6
+            alg = ex if by_classes else S * (S + 1) / 2 * alg_fp64eq[name] * nrhs
             if ms_c > 0 and ex > 0:
                 contractions[name] = {"tflop_algorithmic": alg / 1e12, "tflop_executed": ex / 1e12, "ms": ms_c,
                                       "tflops": alg / (ms_c / 1e3) / 1e12,
                                       "frac_of_bf16_peak": alg / (ms_c / 1e3) / 1e12 / peak,
-                                      "executed_tflops": ex / (ms_c / 1e3) / 1e12, "useful_fraction": alg / ex,
-                                      "form": "entry-major" if int(work["entry_major_mask"]) & ENTRY_BIT.get(name, 0)
+                                      "executed_tflops": ex / (ms_c / 1e3) / 1e12,
+                                      "useful_fraction": None if by_classes else alg / ex,
+                                      "form": "reflection classes" if by_classes else "entry-major" if int(work["entry_major_mask"]) & ENTRY_BIT.get(name, 0)
                                       else "grouped"}
         sn = ops.slices["near"]
-        alg_near = sn * (sn + 1) / 2 * alg_fp64eq["near"] * nrhs
+        alg_near = work["near_tc_flops"] if wl.k >= 6 else sn * (sn + 1) / 2 * alg_fp64eq["near"] * nrhs
         near_ms = stage_ms.get("near_tc") or stage_ms["near"]
         # When the tuner caps the near field's CTAs so that it runs beside the main chain, the kernel's own
         # roofline is taken with the cap lifted to one persistent CTA per SM (one-stream profiled solves);
@@ -776,18 +781,10 @@ def main():
                        "note": "the capped launch of the timed step, alone on one stream"}
             near_ms = statistics.mean(full)
         achieved = alg_near / (near_ms / 1e3) / 1e12
-        # DRAM bytes read + written by this launch (tuned schedule, entry-major near field, 6 slices) in
-        # one ncu capture (--set full, the NVTX range stage_profile) of this command on this workload;
-        # null elsewhere and for other slice counts
-        traffic = None
-        if (wl.name == "adaptive_gauss20_k16_p40" and args.refine == "tail" and nrhs == 1 and not args.no_tune
-                and int(work["entry_major_mask"]) & 1 and ops.slices["near"] == 6):
-            traffic = 83487744 + 39357696
-        roof = {"kernel": "split_gemm_kernel (near field, split-BF16 tcgen05)", "bound": "tensor",
-                "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
+        roof = {"kernel": "class_gemm_kernel and its operands (near field, split-BF16 tcgen05)", "bound": "tensor",
+                "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                 "peak_source": "%s bf16 burst" % peak_kind, "flops_per_launch": alg_near, "ms_per_launch": near_ms,
-                "flops": "algorithmic: S(S+1)/2 slice products (S = the near field's slices) x 2 x 3k^2 x k^2 "
-                         "per U-list entry", "slices": ops.slices,
+                "flops": NEAR_FLOPS, "slices": ops.slices,
                 "executed_tflops": work["near_tc_flops"] / (near_ms / 1e3) / 1e12,
                 "in_step": in_step,
                 "fp64_equivalent_tflops": work["near_fp64eq_flops"] / (near_ms / 1e3) / 1e12,

@@ -439,16 +439,17 @@ int vfmm_batch_streams(const vfmm_batch* batch, int32_t* active);
 int vfmm_selftest_wait_timeout(int64_t polls, void* stream);
 
 /* Schedule autotuner (no counterpart in the paper): for the VFMM_MIXED form, times each small
- * split contraction of this tree and nrhs (near field, M2L, S2L, leaf far field: those with fewer
- * CTAs than two per SM) with split-K factors 1, 2, 4, 8, 16 on the caller's data, and where the
- * schedule holds both forms of a contraction (targets grouped, or one column per list entry with
- * a per-target sum) times both; keeps the fastest in the tree's schedule (used by every later
- * call with this nrhs) and returns the split-K factors in splits[4] (near, M2L, S2L, far; may be
- * NULL; 1 for the entry-major form, see vfmm_solve_work out[7]). Where the near field runs as one
- * persistent CTA per SM and the tree passes are persistent, it then times the whole forked solve
- * (near field beside the main chain, as vfmm_volume_potential and its graphs run it) with the near
- * field capped at 8/8, 7/8, 6/8, 5/8 and 4/8 of the SMs and the tree passes' grids capped to the SMs left
- * free, and keeps the fastest (out[8], out[9] of vfmm_solve_work). Runs two ordinary solves around the timing, so
+ * gathered split contraction of this tree and nrhs (M2L, S2L, and for k <= 5 the near field and the
+ * leaf far field: those with fewer CTAs than two per SM) with split-K factors 1, 2, 4, 8, 16 on the
+ * caller's data, and where the schedule holds both forms of a contraction (targets grouped, or one
+ * column per list entry with a per-target sum) times both. Where the tree passes are persistent it
+ * then times the whole forked solve (near field beside the main chain, as vfmm_volume_potential and
+ * its graphs run it) with the near field capped at 8/8 to 4/8 of the SMs and the tree passes' grids
+ * capped to the SMs left free (out[8], out[9] of vfmm_solve_work), and keeps the fastest step, the
+ * schedule from before the call included. It is used by every later call with this nrhs. splits[4]
+ * (near, M2L, S2L, far; may be NULL) returns the split-K factors; 1 for the entry-major form, see
+ * vfmm_solve_work out[7], and for the near and leaf far field by reflection classes (k >= 6), whose
+ * K blocks are shared by a rule on sizes. Runs two ordinary solves around the timing, so
  * u, u_x, u_y hold the solution afterwards; synchronises `stream`. Must not overlap other calls
  * on the same tree; graphs captured earlier keep the schedule they captured. No-op (splits = 1)
  * for VFMM_FP64. Errors as vfmm_volume_potential. */
@@ -456,23 +457,25 @@ int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const double* f_dev, i
               double* ux_dev, double* uy_dev, void* workspace_dev, size_t workspace_bytes, void* stream,
               int32_t* splits);
 
-/* Work accounting for roofline reports, for a call with nrhs right-hand sides: out[VFMM_N_WORK] =
+/* Work accounting for roofline reports, for a call with nrhs right-hand sides (the near and
+ * leaf far field run in the reflection classes of the square for k >= 6): out[VFMM_N_WORK] =
  * [0] BF16 tensor-core FLOPs the near-field contraction issues per call (VFMM_MIXED: every
  *     slice product of every tile at the operator set's slice counts, zero-padded rows included;
  *     0 for VFMM_FP64),
  * [1] the same for M2L, [2] for the leaf far field (L2T + M2T), [3] for S2L, [4] for S2M,
  * [5] FP64-equivalent FLOPs of the near field, 2 * 3k^2 * k^2 per U-list entry and right-hand side,
  * [6] number of U-list entries, [7] which contractions run in the entry-major form (one column
- *     per list entry, summed per target afterwards): bit 0 near field, 1 M2L, 2 leaf far field,
- *     3 S2L, [8] the near-field contraction's CTA cap (0: one CTA per work item), [9] the grid cap of
+ *     per list entry, summed per target afterwards): bit 0 near field (k <= 5), 1 M2L,
+ *     2 leaf far field (k <= 5), 3 S2L, [8] the near-field contraction's CTA cap (0: one CTA per work
+ *     item for k <= 5, at most one per SM above), [9] the grid cap of
  *     the persistent tree passes (0: one CTA per box of the widest level, at most one per SM).
  *     Host-only; no device work. */
 #define VFMM_N_WORK 10
 int vfmm_solve_work(const vfmm_tree* tree, const vfmm_ops* ops, int32_t nrhs, double* out);
 
 /* Co-schedule of a VFMM_MIXED solve with nrhs right-hand sides on this tree (no counterpart in the
- * paper): near_ctas caps the near-field contraction's grid (0: one CTA per work item; a positive
- * cap makes its CTAs persistent, each walking several work items), pass_ctas caps the grid of the
+ * paper): near_ctas caps the near-field contraction's grid (0: one CTA per work item for k <= 5, at most
+ * one per SM above; a positive cap makes its CTAs persistent, each walking several work items), pass_ctas caps the grid of the
  * persistent tree passes (0: one CTA per box of the widest level, at most one per SM). vfmm_tune
  * picks both by timing the forked solve; these calls read or override its choice (results do not
  * depend on either: every work item is computed the same way whichever CTA takes it). The set call

@@ -1,4 +1,5 @@
-// Split-BF16 tensor-core near field (VFMM_MIXED), tcgen05 on sm_103a.
+// Split-BF16 tensor-core contractions (VFMM_MIXED), tcgen05 on sm_103a: the arithmetic, the gathered engine of
+// S2M, M2L and S2L (and of near and leaf far field for k <= 5; mixed_sym.cu has these for larger k).
 //
 // The near-field sum of Section 3.1, out[t][r] = sum_{(cfg, s) in U(t)} sum_k T_cfg[r][k] f_s[k],
 // is an exact-enough FP64 contraction computed from BF16 tensor-core products:

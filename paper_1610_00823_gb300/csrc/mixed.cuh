@@ -1,4 +1,4 @@
-// Split-BF16 near field: constants and device buffers.
+// Split-BF16 contractions: constants and device buffers.
 #pragma once
 
 #include <cuda_bf16.h>
