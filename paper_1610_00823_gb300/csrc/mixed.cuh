@@ -10,13 +10,12 @@
 #include <utility>
 #include <vector>
 
+#include "mma_schedule.h"
 #include "ops.cuh"
 #include "vfmm_internal.cuh"
 
 namespace vfmm {
 
-constexpr int kSlices = 8;   // BF16 slice slots per operand (balanced base-128 digits, 56 bits)
-constexpr int kMinSlices = 6;  // fewest slices a contraction may take (every accumulator gets a product)
 // contractions of the mixed form, in the order of vfmm_ops_set_slices
 enum { kCtrNear = 0, kCtrS2M = 1, kCtrM2L = 2, kCtrS2L = 3, kCtrFar = 4, kNumCtr = 5 };
 constexpr int kTileM = 128;  // target leaves per tile (TMEM lanes)
@@ -24,7 +23,6 @@ constexpr int kKBlock = 32;  // K values per pipeline stage (64-byte rows)
 constexpr int kStages = 2;   // shared-memory stages
 constexpr int kTileN = 80;   // table rows per tile
 constexpr int kTileNSmall = 48;  // table rows per tile when 2p <= 48 (S2M, M2L, S2L at p <= 24)
-constexpr int kNumAcc = 6;   // TMEM accumulators (diagonals 0..4 exact, 5+ shared)
 constexpr int kTmemCols = 512;                  // allocation (power of two >= kNumAcc * kTileN)
 constexpr int kEpilogueWarps = 8;
 constexpr int kEpilogueThreads = 32 * kEpilogueWarps;
