@@ -239,7 +239,9 @@ struct OffArgs {
 
 // A U leaf as seen from the point, unit-box coordinates: distances to its sides (left, right, bottom,
 // top), positive inwards. On a side (all >= 0, some 0) the point counts as inside, by an amount that the
-// arithmetic of the edges cannot see.
+// arithmetic of the edges cannot see. Distances below 1e-150 of the width count as 0 (kOffOnEdge): of a point
+// that near to a corner from outside, the sum of the squares would underflow and its logarithm be infinite.
+constexpr double kOffOnEdge = 1e-150;
 struct OffLeaf {
     double d[4];
     double h;
@@ -267,6 +269,20 @@ __device__ __forceinline__ void off_coeffs_n(int nu, const double* G, int K, int
     else if constexpr (NU > 1) off_coeffs_n<NU - 1>(nu, G, K, ld, fs, out);
 }
 
+// Q_0 = log((z + 1)/(z - 1))/2 of an edge, z the point (w1, w2, zi as in edge_terms); l1 = log|z - 1|, dl and ang
+// twice its parts.
+struct EdgeLog {
+    double l1, dl, ang;
+};
+__device__ __forceinline__ EdgeLog edge_log(double w1, double w2, double zi) {
+    const double zr = 0.5 * (w2 - w1), n1 = w1 * w1 + zi * zi, n2 = w2 * w2 + zi * zi;
+    EdgeLog r;
+    r.l1 = 0.5 * log(n1);
+    r.dl = zr >= 0.0 ? 0.5 * log1p(4.0 * zr / n1) : -0.5 * log1p(-4.0 * zr / n2);  // log|z+1| - log|z-1|
+    r.ang = atan2(-2.0 * zi, zi * zi - w1 * w2);                                   // arg(z+1) - arg(z-1)
+    return r;
+}
+
 // (V, Re Phi', Im Phi') of one edge of a unit box at the point: w1, w2 the distances along the edge from
 // the point to its end and from its start (edge coordinate, length 2), zi the one across (positive inside);
 // p, g, T: Legendre coefficients of P, its outward and its tangential derivative, stride kOffTasks; logs is
@@ -275,9 +291,8 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
                                            const double* T, int N, const OffStep* __restrict__ C, double logs,
                                            double tr, double ti, double* out) {
     const double zr = 0.5 * (w2 - w1), n1 = w1 * w1 + zi * zi, n2 = w2 * w2 + zi * zi;
-    const double l1 = 0.5 * log(n1);
-    const double dl = zr >= 0.0 ? 0.5 * log1p(4.0 * zr / n1) : -0.5 * log1p(-4.0 * zr / n2);  // log|z+1| - log|z-1|
-    const double ang = atan2(-2.0 * zi, zi * zi - w1 * w2);                                   // arg(z+1) - arg(z-1)
+    const EdgeLog lg = edge_log(w1, w2, zi);
+    const double l1 = lg.l1, dl = lg.dl, ang = lg.ang;
     const double q0r = 0.5 * dl, q0i = 0.5 * ang;
     // rho = |z + sqrt(z^2 - 1)|, the growth of the recurrence
     const float s = 0.5f * (sqrtf((float)n1) + sqrtf((float)n2));
@@ -356,6 +371,37 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
     out[2] = -2.0 * cr;
 }
 
+// Next to a corner Q_n grows like -log(r)/2 on both its edges. The parts cancel, since the two series have one
+// value there, but only to a rounding of each times the logarithm (u_x of one leaf, k = 16, width 1/4, random
+// values of size 1, against extended precision: 1e-13 at r = 1e-10, 3e-13 at 1e-100; now 8e-15 at any r). So the conjugate gradient at the corner, C, is taken off all four edges, and its own
+// integral around the leaf, -2 pi C inside and 0 outside, is put back.
+// An edge with the corner at its end sg = 1 or start sg = -1: sum over n of (T_n + i g_n)(Q_n - sg^n Q_0). With
+// S_n = sg^n Q_n - Q_0, D_n = S_(n+1) - S_n and delta = 1 - sg z the three-term recurrence reads
+//   D_n = (n D_(n-1) - (2n + 1) delta (S_n + Q_0)) / (n + 1),   D_0 = -sg - delta Q_0,
+// in which z, whose last bit the derivative of P_n blows up by n^2, stands no more.
+__device__ __noinline__ double2 edge_corner(double w1, double w2, double zi, double sg, const double* g, const double* T,
+                                            int N, const OffStep* __restrict__ C) {
+    const EdgeLog lg = edge_log(w1, w2, zi);
+    const double qr = 0.5 * lg.dl, qi = 0.5 * lg.ang;
+    const double ar = sg > 0.0 ? w1 : w2, ai = -sg * zi;  // delta
+    double sr = 0.0, si = 0.0, dr = -sg - (ar * qr - ai * qi), di = -(ar * qi + ai * qr);  // S_n, D_n
+    double Br = 0.0, Bi = 0.0, sn = 1.0;                                                  // sg^n
+    for (int n = 0; n < N; ++n) {
+        const double tn = sn * T[n * kOffTasks], gn = sn * g[n * kOffTasks];
+        Br = fma(tn, sr, fma(-gn, si, Br));
+        Bi = fma(tn, si, fma(gn, sr, Bi));
+        sn *= sg;
+        sr += dr;
+        si += di;
+        const OffStep c = C[n + 1];
+        const double xr = sr + qr, xi = si + qi;
+        dr = c.w * dr - c.z * (ar * xr - ai * xi);
+        di = c.w * di - c.z * (ar * xi + ai * xr);
+    }
+    return make_double2(Br, Bi);
+}
+constexpr double kOffCorner = 1e-3;  // of the leaf's width; both edges' recurrences then run upwards
+
 __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_constant__ OffArgs a) {
     extern __shared__ double off_sm[];
     __shared__ OffLeaf lf[kOffMaxU];
@@ -406,6 +452,8 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
         L.d[1] = (x0 + h - px) / h;
         L.d[2] = (py - y0) / h;
         L.d[3] = (y0 + h - py) / h;
+        for (int i = 0; i < 4; ++i)
+            if (fabs(L.d[i]) < kOffOnEdge) L.d[i] = 0.0;
         L.inside = L.d[0] >= 0.0 && L.d[1] >= 0.0 && L.d[2] >= 0.0 && L.d[3] >= 0.0;
         if (L.inside)
             for (int i = 0; i < 4; ++i) L.d[i] = fmax(L.d[i], 1e-30);
@@ -475,20 +523,61 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
     if (warp < 2) {
         // one edge per lane
         const int e = tid;
-        double v[3] = {0.0, 0.0, 0.0};
+        double v[3] = {0.0, 0.0, 0.0}, w1 = 0.0, w2 = 0.0, zi = 0.0, hl = 0.0, tr = 0.0, ti = 0.0;
+        int corner = -1;  // c where edge c starts, if the point is next to it
+        const int s = e & 3;
+        bool inside = false;
         if (e < 4 * nu) {
             const OffLeaf L = lf[e >> 2];
-            const int s = e & 3;
             // (end - point, point - start) along the edge, distance inwards
-            const double w1 = 2.0 * (s == 0 ? L.d[1] : (s == 1 ? L.d[3] : (s == 2 ? L.d[0] : L.d[2])));
-            const double w2 = 2.0 * (s == 0 ? L.d[0] : (s == 1 ? L.d[2] : (s == 2 ? L.d[1] : L.d[3])));
-            const double zi = 2.0 * (s == 0 ? L.d[2] : (s == 1 ? L.d[1] : (s == 2 ? L.d[3] : L.d[0])));
-            edge_terms(w1, w2, zi, tp + e, tg + e, tt + e, N, a.t.C, log(0.5 * L.h),
-                       s == 0 ? 1.0 : (s == 2 ? -1.0 : 0.0), s == 1 ? -1.0 : (s == 3 ? 1.0 : 0.0), v);
-            v[0] *= L.h * L.h;
-            v[1] *= L.h;
-            v[2] *= L.h;
+            w1 = 2.0 * (s == 0 ? L.d[1] : (s == 1 ? L.d[3] : (s == 2 ? L.d[0] : L.d[2])));
+            w2 = 2.0 * (s == 0 ? L.d[0] : (s == 1 ? L.d[2] : (s == 2 ? L.d[1] : L.d[3])));
+            zi = 2.0 * (s == 0 ? L.d[2] : (s == 1 ? L.d[1] : (s == 2 ? L.d[3] : L.d[0])));
+            hl = L.h;
+            tr = s == 0 ? 1.0 : (s == 2 ? -1.0 : 0.0);
+            ti = s == 1 ? -1.0 : (s == 3 ? 1.0 : 0.0);
+            edge_terms(w1, w2, zi, tp + e, tg + e, tt + e, N, a.t.C, log(0.5 * hl), tr, ti, v);
+            const double cx = fmin(fabs(L.d[0]), fabs(L.d[1])), cy = fmin(fabs(L.d[2]), fabs(L.d[3]));
+            if (cx < kOffCorner && cy < kOffCorner) {
+                const bool left = fabs(L.d[0]) < fabs(L.d[1]);
+                corner = fabs(L.d[2]) < fabs(L.d[3]) ? (left ? 0 : 1) : (left ? 3 : 2);
+                inside = L.inside;
+            }
         }
+        if (__any_sync(0xffffffffu, corner >= 0)) {
+            double cr = 0.0, ci = 0.0;  // C, from the edge that starts there
+            if (s == corner) {
+                double fr = 0.0, fi = 0.0;
+                for (int n = N - 1; n >= 0; --n) {  // T + i g at the start, P_n = (-1)^n there
+                    fr = tt[n * kOffTasks + e] - fr;
+                    fi = tg[n * kOffTasks + e] - fi;
+                }
+                cr = tr * fr - ti * fi;
+                ci = tr * fi + ti * fr;
+            }
+            const int from = (lane & ~3) | max(corner, 0);
+            cr = __shfl_sync(0xffffffffu, cr, from);
+            ci = __shfl_sync(0xffffffffu, ci, from);
+            if (corner >= 0) {
+                const bool start = s == corner, end = s == ((corner + 3) & 3);
+                if (start || end) {
+                    const double2 B = edge_corner(w1, w2, zi, end ? 1.0 : -1.0, tg + e, tt + e, N, a.t.C);
+                    v[1] = 2.0 * (tr * B.y + ti * B.x);
+                    v[2] = -2.0 * (tr * B.x - ti * B.y);
+                } else {  // -2 i (sum - C Q_0)
+                    const EdgeLog q = edge_log(w1, w2, zi);
+                    v[1] -= cr * q.ang + ci * q.dl;
+                    v[2] += cr * q.dl - ci * q.ang;
+                }
+                if (start && inside) {
+                    v[1] -= 2.0 * pi * cr;
+                    v[2] -= 2.0 * pi * ci;
+                }
+            }
+        }
+        v[0] *= hl * hl;
+        v[1] *= hl;
+        v[2] *= hl;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
@@ -566,15 +655,18 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
             if (!L.inside) continue;
             __syncwarp();
             if (lane < 2) {
-                const double x = L.d[2 * lane] - L.d[2 * lane + 1];  // 2 x in [-1, 1]
-                double p0 = 1.0, p1 = x, q0 = 0.0, q1 = 1.0;        // P_m, P_m' (p1, q1: m + 1)
+                // 2 x = sg (1 - delta) in [-1, 1]; P_m by its differences, as in edge_corner
+                const double dl = L.d[2 * lane], dr = L.d[2 * lane + 1], delta = 2.0 * fmin(dl, dr);
+                const double sg = dl < dr ? -1.0 : 1.0;
+                double p0 = 1.0, dp = -delta, q0 = 0.0, q1 = 1.0, sn = 1.0;  // sg^m P_m, difference, P_m', P_(m+1)', sg^m
                 for (int m = 0; m < N; ++m) {
-                    leg[2 * lane][m] = p0;
+                    leg[2 * lane][m] = sn * p0;
                     leg[2 * lane + 1][m] = 2.0 * q0;
                     const OffStep c = a.t.C[m + 1];
-                    const double p2 = c.z * x * p1 - c.w * p0, q2 = fma((double)(2 * m + 3), p1, q0);
-                    p0 = p1;
-                    p1 = p2;
+                    p0 += dp;
+                    sn *= sg;
+                    const double q2 = fma((double)(2 * m + 3), sn * p0, q0);
+                    dp = c.w * dp - c.z * (delta * p0);
                     q0 = q1;
                     q1 = q2;
                 }
