@@ -51,7 +51,8 @@ __host__ __device__ constexpr int mma_n(bool transposed, int Rp) {
 // Splits v / 2^E (|v| < 2^E) into kSlices balanced base-128 digits, out[(i - 1) * stride] =
 // d_i 2^(-7 i), with v / 2^E = sum_i d_i 2^(-7 i) + (|v| 2^(56 - E) - floor(|v| 2^(56 - E))) 2^-56:
 // q = floor(|v| 2^(56 - E)) is written in base 128 from its low end, a digit of 64 or more becoming
-// d - 128 with a carry into the next higher one, so d_2..d_8 lie in [-64, 63] and d_1 in [0, 128];
+// d - 128 with a carry into the next higher one, so d_2..d_8 lie in [-64, 63] and d_1 in [0, 128] (up to
+// 256 for the tables in reflection classes, whose scale may be half of that);
 // a negative v negates every digit. Each is an integer of at most 8 significant bits (exact in
 // BF16), the products of two are below 2^14, and the first S digits are v / 2^E rounded to the
 // nearest multiple of 2^(-7 S) (error at most 2^(-7 S - 1) of the scale 2^E). Integer work on the
@@ -62,14 +63,14 @@ __device__ __forceinline__ void slice_fixed(double v, int E, __nv_bfloat16* out,
     unsigned long long mant = bits & ((1ull << 52) - 1);
     if (ev) mant |= 1ull << 52;
     else ev = 1;
-    // |v| 2^(56 - E) = mant 2^(ev - 1075 + 56 - E): a right shift by 1019 - ev + E (>= -3 when |v| < 2^E)
+    // |v| 2^(56 - E) = mant 2^(ev - 1075 + 56 - E): a right shift by 1019 - ev + E (>= -4)
     const int shift = 1019 - ev + E;
     const unsigned long long q = shift >= 64 ? 0ull : (shift >= 0 ? mant >> shift : mant << (-shift));
     const bool neg = (bits >> 63) != 0;
     int carry = 0;
 #pragma unroll
     for (int i = kSlices; i >= 1; --i) {
-        int d = (int)((q >> (7 * (kSlices - i))) & 127ull) + carry;
+        int d = (int)((q >> (7 * (kSlices - i))) & (i > 1 ? 127ull : 511ull)) + carry;
         carry = (i > 1 && d >= 64) ? 1 : 0;
         d -= carry << 7;
         const float s = (float)(neg ? -d : d) * __int_as_float((127 - 7 * i) << 23);
@@ -265,7 +266,7 @@ struct MixedWork {
     void* fsl = nullptr;                  // bf16 [n_leaves][kSlices][Kp]
     float2* out = nullptr;                // near field (hi, lo): class rows [n_leaves][4 nch N], scaled by
                                           // 2^-(E_f + 1 + E_r), or node rows [n_leaves][Rp], by 2^-(E_f + E_r)
-    long long* ffix = nullptr;            // [R][n_leaves][k^2] f 2^(55 - E_f), truncated (near field)
+    long long* ffix = nullptr;            // [R][n_leaves][k^2] f 2^(59 - E_f), truncated (near field)
     void* near_opnd = nullptr;            // near field's operand tiles, a chunk at a time
     size_t near_opnd_bytes = 0;
     int near_split = 1, leaf_split = 1;   // partial sums in out and far_out, one row set after another (by classes)

@@ -9,8 +9,14 @@
 //    a tile in the order and swizzle in which the MMA reads it. A stage of the pipeline is then two bulk
 //    copies of contiguous memory by one thread.
 //  * |f| < 2^E makes |g| < 2^(E+2); E + 1 is the scale all the same: the top digit of a tile may be as
-//    large as 256, which BF16 holds, at the price of draining every 448 K values instead of 512
-//    (36,864 units per K value on diagonal 4, 448 of them below 2^24).
+//    large as 256, which BF16 holds. What this costs an orbit with a single member, its last slice makes up
+//    for: not a whole digit but all that is left, rounded to BF16 (at most 1/8 of the digit's unit).
+//  * a table row's scale is half its largest entry's power of two (top digits up to 256) wherever the entries of
+//    a K block are on average no larger than that scale (all but some 4 % of the rows): half the weight of
+//    the slice products left out. Per K value diagonals 0 to 4 then sum to at most 36,864 units, 448 of
+//    them below 2^24: diagonal 0 to 256 x 128 (the table's average), diagonal 4 to 256 x 64 + 3 x 64^2
+//    + 64 x 128. The sixth accumulator (diagonals from 5 on, 40,960 units at S = 6) may round by 2^-49 of
+//    the scales' product where its sum is past 2^24 units, 1/400 of what the products left out may weigh.
 //  * the outputs of a class are put together at the nodes by the leaf kernel (double-FP32).
 // The leaf far field does the same with the leaf's local (one K block per class) and its W orbits, scaled
 // per leaf: with E_t the exponent of its largest coefficient and m the most boxes in one of its orbits,
@@ -51,26 +57,42 @@ constexpr size_t kClsSmem = 224 * 1024;
 constexpr size_t kClsUnit = kTileM * 64;  // bytes of one slice of an operand tile
 
 // ---------------------------------------------------------------- tables
-// E[output row] = exponent of the largest entry of that row over the orbits (0: padding). A class has its own:
-// for the smooth potential tables the odd ones are far smaller than the even one.
-__global__ void class_row_exp_kernel(SymOp op, ClassTab ct, int* __restrict__ E) {
-    __shared__ double red[256];
+// E[output row] = scale of that row over the orbits (0: padding). A class has its own: for the smooth
+// potential tables the odd ones are far smaller than the even one. With e the exponent of the row's largest
+// entry it is e - 1 if no K block's entries sum to more than 31.8 2^(e - 1) (32 top digits then sum to at
+// most 31.8 x 128 and 32 carries, below 32 x 128), else e.
+__global__ void __launch_bounds__(256) class_row_exp_kernel(SymOp op, ClassTab ct, int* __restrict__ E) {
+    __shared__ double red[8], reds[8];
     const int c = blockIdx.x / (ct.nch * ct.N), r = blockIdx.x - c * (ct.nch * ct.N);
-    double m = 0.0;
+    double m = 0.0, ms = 0.0;
     if (r < op.M[c])
         for (int o = 0; o < op.norb; ++o) {
             const double* A = op.A + op.off[o][c] + r;
-            for (int col = threadIdx.x; col < op.K[o][c]; col += blockDim.x)
-                m = fmax(m, fabs(A[(size_t)col * op.M[c]]));
+            const int Kp = ct.nkb[o][c] * kKBlock;  // a warp takes whole K blocks
+            for (int col = threadIdx.x; col < Kp; col += blockDim.x) {
+                const double v = col < op.K[o][c] ? fabs(A[(size_t)col * op.M[c]]) : 0.0;
+                double s = v;
+                for (int x = 16; x > 0; x >>= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
+                m = fmax(m, v);
+                ms = fmax(ms, s);
+            }
         }
-    red[threadIdx.x] = m;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
-        __syncthreads();
+    for (int x = 16; x > 0; x >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, x));
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = m;
+        reds[threadIdx.x >> 5] = ms;
     }
-    if (threadIdx.x == 0) E[blockIdx.x] = red[0] > 0.0 ? exp_bound(red[0]) : 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            m = fmax(m, red[w]);
+            ms = fmax(ms, reds[w]);
+        }
+        const int e = m > 0.0 ? exp_bound(m) : 0;
+        E[blockIdx.x] = m > 0.0 && ms <= ldexp(31.8, e - 1) ? e - 1 : e;
+    }
 }
+static_assert(kKBlock == 32, "a K block per warp");
 
 // Digits of every table, tile by tile (table_at with one orbit's class as a table of nch * N rows).
 __global__ void class_table_kernel(SymOp op, ClassTab ct, const int* __restrict__ E, bf16* __restrict__ out) {
@@ -331,6 +353,7 @@ int class_launches(const ClassTab& ct, const ClassPlan& P, int S, size_t opnd_by
 struct ClassOperandArgs {
     ClassTab ct;
     int S, R, nleaf, nv;
+    long long bias;      // class_bias(S)
     int p0, p1;          // pieces (4 * group + class) of this chunk
     const int32_t* order;
     const int32_t* gmask;
@@ -348,51 +371,64 @@ struct ClassOperandArgs {
     unsigned char* out;  // chunk's tiles: K block u of piece p at (span(p) - span(p0) + u) * S * kClsUnit
 };
 
-// floor(|v| 2^(56 - E)) with v's sign (|v| < 2^E), integer work.
-__device__ __forceinline__ long long fixed56(double v, int E) {
+// floor(|v| 2^(60 - E)) with v's sign (|v| < 2^(E + 1)), integer work.
+__device__ __forceinline__ long long fixed60(double v, int E) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
     int ev = (int)((bits >> 52) & 0x7FF);
     unsigned long long mant = bits & ((1ull << 52) - 1);
     if (ev) mant |= 1ull << 52;
     else ev = 1;
-    const int shift = 1019 - ev + E;
+    const int shift = 1015 - ev + E;
     const long long q = (long long)(shift >= 64 ? 0ull : (shift >= 0 ? mant >> shift : mant << (-shift)));
     return (bits >> 63) ? -q : q;
 }
 
-// q[r][i] = f[r][i] 2^(55 - E_f[r]), truncated: the fixed-point values that the operand sums.
+// q[r][i] = f[r][i] 2^(59 - E_f[r]), truncated: the fixed-point values that the operand sums.
 __global__ void __launch_bounds__(256) class_fixed_kernel(const double* __restrict__ f, int64_t n,
                                                           const int* __restrict__ Ef, long long* __restrict__ q) {
     const int E = Ef[blockIdx.y] + 1;
     const size_t base = (size_t)blockIdx.y * n;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        q[base + i] = fixed56(f[base + i], E);
+        q[base + i] = fixed60(f[base + i], E);
 }
 
-// Balanced base-128 digits of 4 values q 2^-56 (|q| < 2^57): d_i = digit 8 - i of q + 64 (128^6 + ... + 1),
-// less 64, the top one the rest; S 8-byte stores, slice i at out + i * kClsUnit.
-__device__ __forceinline__ void class_digits4(const long long* q, int S, unsigned char* out) {
-    constexpr long long kBias = 64ll * (((1ll << 49) - 1) / 127);
+// S slices of 4 values q 2^-60 (|q| < 2^61): slices 1 .. S - 1 balanced base-128 digits, d_i = digit i of
+// q + bias less 64 (the top one as it is), bias = 64 of each later digit's unit; the last slice what is left,
+// less than 64 units of 2^(-7 S), rounded to BF16. 8-byte stores, slice i at out + i * kClsUnit.
+__device__ __forceinline__ void class_digits4(const long long* q, int S, long long bias, unsigned char* out) {
     constexpr float kMagic = 12582912.0f;  // 1.5 2^23: an integer below 2^22 added to its bits is added to it
     long long b[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) b[e] = q[e] + kBias;
+    for (int e = 0; e < 4; ++e) b[e] = q[e] + bias;
+    auto store = [&](int i, const float* v) {
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[0], v[1]), h1 = __floats2bfloat162_rn(v[2], v[3]);
+        *reinterpret_cast<uint2*>(out + (size_t)i * kClsUnit) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+    };
+    float v[4];
 #pragma unroll
-    for (int i = 0; i < kSlices; ++i) {
-        if (i >= S) break;
-        const int shift = 7 * (kSlices - 1 - i);
+    for (int i = 0; i < kSlices - 1; ++i) {
+        if (i >= S - 1) break;
+        const int shift = 53 - 7 * i;
         const float sc = __int_as_float((127 - 7 * (i + 1)) << 23);
         const float zero = (i == 0 ? kMagic : kMagic + 64.0f) * sc;
-        float v[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int d = (int)(b[e] >> shift);
             v[e] = fmaf(__int_as_float(0x4B400000 + (i == 0 ? d : d & 127)), sc, -zero);
         }
-        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[0], v[1]), h1 = __floats2bfloat162_rn(v[2], v[3]);
-        *reinterpret_cast<uint2*>(out + (size_t)i * kClsUnit) =
-            make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+        store(i, v);
     }
+    const int low = 67 - 7 * S;  // bits below digit S - 1 (25 at S = 6); exact in FP32
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        v[e] = (float)(((int)b[e] & ((1 << low) - 1)) - (1 << (low - 1))) * __int_as_float((127 - 60) << 23);
+    store(S - 1, v);
+}
+static long long class_bias(int S) {
+    long long b = 0;
+    for (int i = 1; i < S; ++i) b += 64ll << (53 - 7 * i);
+    return b;
 }
 
 // One CTA per (group, orbit) and share of its K blocks, thread = (target row, 4 columns of a 64-byte row), so that
@@ -466,10 +502,10 @@ __global__ void __launch_bounds__(1024) class_operand_kernel(const __grid_consta
                 s2[e] = x - z;
                 s3[e] = y - w;
             }
-            if (shared ? mine(0) : c0 == 0) class_digits4(s0, a.S, tile(0));
-            if (shared ? mine(1) : c0 == 1) class_digits4(s1, a.S, tile(1));
-            if (shared ? mine(2) : c0 == 2) class_digits4(s2, a.S, tile(2));
-            if (shared ? mine(3) : c0 == 3) class_digits4(s3, a.S, tile(3));
+            if (shared ? mine(0) : c0 == 0) class_digits4(s0, a.S, a.bias, tile(0));
+            if (shared ? mine(1) : c0 == 1) class_digits4(s1, a.S, a.bias, tile(1));
+            if (shared ? mine(2) : c0 == 2) class_digits4(s2, a.S, a.bias, tile(2));
+            if (shared ? mine(3) : c0 == 3) class_digits4(s3, a.S, a.bias, tile(3));
         }
     }
 }
@@ -552,9 +588,9 @@ __global__ void __launch_bounds__(1024) class_far_operand_kernel(const __grid_co
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int part = sym_part(c, c4 * 4 + e);
-                q[e] = src.x >= 0 && part >= 2 && part < P2 ? fixed56(L[part], E) : 0;
+                q[e] = src.x >= 0 && part >= 2 && part < P2 ? fixed60(L[part], E) : 0;
             }
-            class_digits4(q, a.S, tile(c, 0));
+            class_digits4(q, a.S, a.bias, tile(c, 0));
         }
         return;
     }
@@ -569,10 +605,10 @@ __global__ void __launch_bounds__(1024) class_far_operand_kernel(const __grid_co
         for (int e = 0; e < 4; ++e) {
             const int part = col0 + e;
             const bool in = part < P2;
-            long long s0 = in && src.x >= 0 ? fixed56(__ldg(M0 + part), E) : 0;
-            long long s1 = in && src.y >= 0 ? fixed56(__ldg(M1 + part), E) : 0;
-            long long s2 = in && src.z >= 0 ? fixed56(__ldg(M2 + part), E) : 0;
-            long long s3 = in && src.w >= 0 ? fixed56(__ldg(M3 + part), E) : 0;
+            long long s0 = in && src.x >= 0 ? fixed60(__ldg(M0 + part), E) : 0;
+            long long s1 = in && src.y >= 0 ? fixed60(__ldg(M1 + part), E) : 0;
+            long long s2 = in && src.z >= 0 ? fixed60(__ldg(M2 + part), E) : 0;
+            long long s3 = in && src.w >= 0 ? fixed60(__ldg(M3 + part), E) : 0;
             if (sym_part_sign(part, 1)) s1 = -s1;
             if (sym_part_sign(part, 2)) s2 = -s2;
             if (sym_part_sign(part, 3)) s3 = -s3;
@@ -582,10 +618,10 @@ __global__ void __launch_bounds__(1024) class_far_operand_kernel(const __grid_co
             q2[e] = x - z;
             q3[e] = y - w;
         }
-        if (mine(0)) class_digits4(q0, a.S, tile(0, kb));
-        if (mine(1)) class_digits4(q1, a.S, tile(1, kb));
-        if (mine(2)) class_digits4(q2, a.S, tile(2, kb));
-        if (mine(3)) class_digits4(q3, a.S, tile(3, kb));
+        if (mine(0)) class_digits4(q0, a.S, a.bias, tile(0, kb));
+        if (mine(1)) class_digits4(q1, a.S, a.bias, tile(1, kb));
+        if (mine(2)) class_digits4(q2, a.S, a.bias, tile(2, kb));
+        if (mine(3)) class_digits4(q3, a.S, a.bias, tile(3, kb));
     }
 }
 
@@ -872,6 +908,7 @@ static ClassOperandArgs operand_args(const DeviceTree& T, const ClassTab& ct, co
     ClassOperandArgs oa = {};
     oa.ct = ct;
     oa.S = S;
+    oa.bias = class_bias(S);
     oa.R = R;
     oa.nleaf = T.n_leaves;
     oa.nv = T.n_leaves * R;
