@@ -356,8 +356,9 @@ int vfmm_evaluate_points(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
  * cudaMalloc is available to this library). It runs vfmm_volume_potential with its
  * workspace in a fixed 32 MiB static device array that every GPU loading the library
  * holds until the process exits, and never calls cudaMalloc or cudaFree.
- *  - Size limit: trees whose workspace for one right-hand side exceeds 32 MiB (the mixed form's
- *    operand buffers at their smallest, so at most vfmm_workspace_size) are rejected with VFMM_ERR_WORKSPACE (roughly a few hundred leaves at k = 8).
+ *  - Size limit: trees that need more than 32 MiB for one right-hand side are rejected with
+ *    VFMM_ERR_WORKSPACE (roughly a few hundred leaves at k = 8). The mixed form's operand tiles
+ *    take turns in what the rest leaves, so it takes trees whose vfmm_workspace_size is larger.
  *  - Right-hand sides are solved one after another in the same scratch (the mixed form
  *    does not fold them here, since that would build new schedules in device memory),
  *    every launch on `stream` (no second stream is created).

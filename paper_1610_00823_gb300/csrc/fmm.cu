@@ -818,11 +818,12 @@ struct Workspace {
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Workspace carving (tight: the mixed form's operand buffers at their smallest, for the fixed scratch). The mixed form folds all nrhs right-hand sides into one solve (every
-// per-box and per-leaf buffer has nrhs rows per box); the FP64 form solves them one at a time.
+// Workspace carving. The mixed form folds all nrhs right-hand sides into one solve (every per-box and
+// per-leaf buffer has nrhs rows per box); the FP64 form solves them one at a time. room (not 0): bytes of a
+// scratch of fixed size, for a solve on one stream; its near field and leaf far field then take no split sums
+// and, one after the other, the same operand buffer, which gets what the rest leaves.
 static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Workspace* w, char* base,
-                  size_t* bytes,
-                  bool tight = false) {
+                  size_t* bytes, size_t room = 0) {
     const size_t P2 = 2 * (size_t)(o.p + 1), kk = (size_t)o.k * o.k;
     size_t off = 0;
     auto take = [&](double** p, size_t n) {
@@ -882,8 +883,7 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         take(&p, (nl * kSlices * mo->Kp * 2 + 7) / 8);
         if (w) w->mix.fsl = (void*)p;
         const bool cls = near_by_classes(o.k);
-        // partial sums of small trees' class contractions, in the scratch of fixed size none
-        const int ns = cls && !tight ? PS->near.split : 1, fs = cls && !tight ? PS->leaf.split : 1;
+        const int ns = cls && !room ? PS->near.split : 1, fs = cls && !room ? PS->leaf.split : 1;  // partial sums
         if (w) {
             w->mix.near_split = ns;
             w->mix.leaf_split = fs;
@@ -905,8 +905,8 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         if (w) w->mix.m2l_c0 = p;
         take(&p, nb * mo->Rx);
         if (w) w->mix.s2l_out = (float2*)p;
-        const size_t ab = cls ? class_operand_bytes(T, mo->leaf, PS->leaf, (int)R, 14, tight)
-                              : (size_t)T.n_far_slots * R * kSlices * mo->Kx * 2;
+        const size_t ab = !cls ? (size_t)T.n_far_slots * R * kSlices * mo->Kx * 2
+                               : (room ? 0 : class_operand_bytes(mo->leaf, PS->leaf, 0));
         take(&p, (ab + 7) / 8);
         if (w) {
             w->mix.aprep = (void*)p;
@@ -928,11 +928,17 @@ static int layout(const DeviceTree& T, const vfmm_ops& o, int nrhs, bool io, Wor
         }
         take(&p, cls ? nl * kk : 1);
         if (w) w->mix.ffix = (long long*)p;
-        const size_t ob = class_operand_bytes(T, mo->near, PS->near, (int)R, 16, tight);
+        const size_t left = room > off ? (room - off) & ~(size_t)255 : size_t(1);
+        size_t ob = class_operand_bytes(mo->near, PS->near, room ? left : 0);
+        if (room && cls) ob = std::max(ob, class_operand_bytes(mo->leaf, PS->leaf, left));
         take(&p, (ob + 7) / 8);
         if (w) {
             w->mix.near_opnd = p;
             w->mix.near_opnd_bytes = ob;
+            if (room && cls) {
+                w->mix.aprep = p;
+                w->mix.aprep_bytes = ob;
+            }
         }
     } else if (w) {
         w->mix = MixedWork();
@@ -1427,9 +1433,9 @@ static int check_solve_args(const vfmm_tree* tree, const vfmm_ops* ops, int32_t 
     return VFMM_OK;
 }
 
-int vfmm::tight_workspace_bytes(const vfmm_tree* tree, const vfmm_ops* ops, size_t* bytes) {
+int vfmm::scratch_bytes(const vfmm_tree* tree, const vfmm_ops* ops, size_t room, size_t* bytes) {
     VFMM_CHECK(check_solve_args(tree, ops, 1));
-    return layout(tree->t, *ops, 1, false, nullptr, nullptr, bytes, true);
+    return layout(tree->t, *ops, 1, false, nullptr, nullptr, bytes, room);
 }
 
 extern "C" int vfmm_workspace_size(const vfmm_tree* tree, const vfmm_ops* ops, int32_t nrhs, int32_t with_io,
@@ -1482,14 +1488,14 @@ static int read_status(const Workspace& w) { return read_status_word(w.mix.err);
 
 int vfmm::volume_potential(const vfmm_tree* tree, const vfmm_ops* ops, const double* f_dev, int32_t nrhs,
                            double* u_dev, double* ux_dev, double* uy_dev, void* workspace_dev, size_t workspace_bytes,
-                           cudaStream_t st, bool fork, bool reset, bool tight) {
+                           cudaStream_t st, bool fork, bool reset, bool fixed) {
     VFMM_CHECK(check_solve_args(tree, ops, nrhs));
     if (!f_dev || !u_dev || !ux_dev || !uy_dev || !workspace_dev) return fail(VFMM_ERR_INVALID_ARG, "null buffer");
     Workspace w;
     size_t need = 0;
-    VFMM_CHECK(layout(tree->t, *ops, nrhs, false, &w, (char*)workspace_dev, &need, tight));
+    VFMM_CHECK(layout(tree->t, *ops, nrhs, false, &w, (char*)workspace_dev, &need, fixed ? workspace_bytes : 0));
     if (workspace_bytes < need) return fail(VFMM_ERR_WORKSPACE, "workspace too small");
-    w.fork = fork;
+    w.fork = fork && !fixed;
     if (reset) VFMM_CHECK(reset_status(w, st));
     return solve_all(tree->t, *ops, f_dev, nrhs, u_dev, ux_dev, uy_dev, w, st);
 }

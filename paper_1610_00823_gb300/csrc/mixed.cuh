@@ -366,7 +366,7 @@ int near_classes_prepare(vfmm_ops* o, cudaStream_t st);
 int leaf_classes_prepare(vfmm_ops* o, const std::vector<double>& F, cudaStream_t st);
 int build_near_classes(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, ClassPlan* P);
 int build_leaf_classes(const DeviceTree& T, int R, const HostLists& H, PlanArena& A, ClassPlan* P);
-size_t class_operand_bytes(const DeviceTree& T, const ClassTab& ct, const ClassPlan& P, int R, int rows, bool tight);
+size_t class_operand_bytes(const ClassTab& ct, const ClassPlan& P, size_t room);
 double class_tiles(const ClassTab& ct, const ClassPlan& P);  // operand tiles of all pieces
 int near_class_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* f, const MixedWork& w,
                         cudaStream_t st);

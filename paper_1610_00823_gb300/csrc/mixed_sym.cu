@@ -313,15 +313,13 @@ double class_tiles(const ClassTab& ct, const ClassPlan& P) {
     return P.n_groups ? (double)class_span(host_spans(ct, P), 4 * P.n_groups, nullptr) : 0.0;
 }
 
-// Bytes of the operand buffer: all tiles at once, up to 768 MB; more take turns in it. tight: no more than
-// `rows` rows of outputs per leaf (what the gathered form keeps for its partial sums) or 8 MB.
-size_t class_operand_bytes(const DeviceTree& T, const ClassTab& ct, const ClassPlan& P, int R, int rows, bool tight) {
+// Bytes of the operand buffer: all tiles at once, up to 768 MB; more take turns in it. room (not 0): as many
+// as fit in it. At least the largest piece's.
+size_t class_operand_bytes(const ClassTab& ct, const ClassPlan& P, size_t room) {
     if (P.n_groups == 0) return 0;
     const size_t all = (size_t)class_tiles(ct, P) * kSlices * kClsUnit;
     const size_t most = P.first.empty() ? 1 + (size_t)P.max_units * ct.nkb[1][0] : (size_t)P.max_units;
-    const size_t share = std::max((size_t)T.n_leaves * R * rows * 3 * T.k * T.k * sizeof(float2), size_t(8) << 20);
-    const size_t cap = std::min(tight ? share : SIZE_MAX, size_t(768) << 20);
-    return std::max(std::min(all, cap), most * kSlices * kClsUnit);
+    return std::max(std::min(all, room ? room : size_t(768) << 20), most * kSlices * kClsUnit);
 }
 
 // Chunks of pieces [p0, p1) whose tiles fit the buffer.

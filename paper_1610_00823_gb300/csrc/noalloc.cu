@@ -64,7 +64,7 @@ extern "C" int vfmm_volume_potential_noalloc(const vfmm_tree* tree, const vfmm_o
     // tree, whereas folding several into one solve (the mixed form's usual path) would build new
     // schedules in device memory on first use.
     size_t need = 0;
-    VFMM_CHECK(tight_workspace_bytes(tree, ops, &need));
+    VFMM_CHECK(scratch_bytes(tree, ops, kStaticScratchBytes, &need));
     if (need > kStaticScratchBytes)
         return fail(VFMM_ERR_WORKSPACE, "tree needs " + std::to_string(need) +
                                             " bytes of scratch; the static scratch holds " +

@@ -275,13 +275,14 @@ void tree_free(void* p);
 int exclusive_scan(const int32_t* in, int32_t* out, int64_t n, int64_t* total, cudaStream_t st);
 // vfmm_volume_potential with flags: fork = false keeps every launch on `st` (no second stream);
 // reset = false leaves the workspace's status word as it is (a caller solving several right-hand
-// sides one after another clears it once, so that a timeout in an early one is not lost); tight = true
-// takes the smallest operand buffers and no split sums (the allocation-free scratch).
+// sides one after another clears it once, so that a timeout in an early one is not lost); fixed = true
+// carves a scratch of fixed size (the allocation-free one): one stream, operand buffers in what is left of it.
 int volume_potential(const vfmm_tree* tree, const vfmm_ops* ops, const double* f_dev, int32_t nrhs, double* u_dev,
                      double* ux_dev, double* uy_dev, void* workspace_dev, size_t workspace_bytes, cudaStream_t st,
-                     bool fork, bool reset = true, bool tight = false);
-// Workspace bytes of a one-right-hand-side solve with tight = true.
-int tight_workspace_bytes(const vfmm_tree* tree, const vfmm_ops* ops, size_t* bytes);
+                     bool fork, bool reset = true, bool fixed = false);
+// Bytes that a one-right-hand-side solve with fixed = true takes of a scratch of `room` bytes (more than room:
+// it does not fit).
+int scratch_bytes(const vfmm_tree* tree, const vfmm_ops* ops, size_t room, size_t* bytes);
 // Reads a status word (device address) after the solve that wrote it has finished: VFMM_OK, or
 // VFMM_ERR_TIMEOUT naming the bounded wait that ran out.
 int read_status_word(const int* word);
