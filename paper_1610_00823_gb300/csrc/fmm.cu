@@ -1757,7 +1757,7 @@ extern "C" int vfmm_tune(const vfmm_tree* tree, const vfmm_ops* ops, const doubl
     // persistent CTAs (one per SM, each walking several work items) against one CTA per item, for a
     // contraction with more items than SMs; the faster is kept
     auto time_ctas = [&](const Job& jb, SplitPlan* P, float2* part) {
-        const int nchunks = jb.Rp / table_rows_per_tile(P->transposed, jb.Rp);
+        const int nchunks = jb.Rp / table_rows_per_tile(jb.Rp);
         const long long items = (long long)P->n_groups * (P->entry ? 1 : P->split) * nchunks;
         const int sms = sm_count();
         if (items <= sms) return;

@@ -21,12 +21,12 @@
 //    registers; at the end of an item they store (hi, lo). The leaf pass scales by
 //    2^(E_f + E_r) and by h^2 (potential) or h (gradient) in FP64.
 //
-// Tile: 128 rows on the M side (TMEM lanes) x 80 on the N side; which side holds the table rows
-// (by TMA) and which the gathered operand rows (by cp.async) depends on the contraction
-// (near_transposed). For every table of a group and every K block of 32 values the S slices of
-// both go into a 64-byte-swizzled K-major stage (two stages); one thread issues the
-// S(S+1)/2 x 2 UMMAs (128 x N x 16) into the six TMEM accumulators; tcgen05.commit frees the
-// stage and, after the last K block of a drain group, hands the accumulators to the epilogue.
+// Tile: 128 targets on the M side (TMEM lanes), their operand rows gathered by cp.async, x 80 (or 48) table
+// rows on the N side, one bulk copy per K block. For every table of a group and every K block of 32
+// values the S slices of both go into a 64-byte-swizzled K-major stage (two stages); one elected lane
+// issues the MMAs of the S(S+1)/2 slice products (mma_issue.cuh) into the six TMEM accumulators;
+// tcgen05.commit frees the stage and, after the last K block of a drain group, hands the accumulators
+// to the epilogue.
 // Every mbarrier wait is bounded and reports a timeout through an error word.
 #include <cuda_bf16.h>
 
@@ -147,17 +147,15 @@ struct SplitArgs {
     int Kp, Rp, nchunks;
     int split;            // CTAs sharing one group's tables (split-K over tables)
     int drain_every;      // configurations accumulated in TMEM between two drains (exactness bound)
-    int transposed;       // table rows on the M side (see near_transposed)
     int slices;           // slices of each operand taken, kMinSlices .. kSlices (products i + j <= slices + 1)
     int n_items;          // work items (n_groups * split * nchunks); the grid may be smaller (persistent CTAs)
     size_t part_stride;   // n_out_rows * Rp
 };
 
 // Warps 0..7: epilogue (lane quadrant w % 4, column half w / 4); warps 8..10: producers;
-// warp 11: TMEM allocation and the MMA issuer (lane 0). Twelve warps keep three warps per SM
+// warp 11: TMEM allocation and the MMA issuer. Twelve warps keep three warps per SM
 // sub-partition, which leaves each thread up to 168 registers.
-// N: the MMA's N (TMEM columns per accumulator): 80, or 48 for the 48-row tables of small
-// expansions (targets on M only).
+// N: the MMA's N (TMEM columns per accumulator): 80, or 48 for the 48-row tables of small expansions.
 template <int N>
 __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
     extern __shared__ unsigned char dsm[];
@@ -172,8 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
     constexpr uint32_t STAGE = kSlices * (A_SLICE + B_SLICE);
     constexpr int HALF = N / 2;  // columns per epilogue warp
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const bool tr = a.transposed != 0;     // table rows on M (TMA into the A region), targets on N
-    const int G = tr ? kTileN : kTileM;    // gathered rows (targets) per group
+    constexpr int G = kTileM;  // gathered rows (targets) per group
     const uint32_t base = tc::smem_u32(dsm);
     const uint32_t sbase = (base + 1023u) & ~1023u;
     const uint32_t full0 = tc::smem_u32(&bars[0]);
@@ -254,15 +251,12 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
                     named_bar_sync(1, kProducerThreads);
                 }
                 const uint32_t sA = sbase + s * STAGE, sB = sA + kSlices * A_SLICE;
-                // table tile into the region of its side, gathered rows into the other
-                const uint32_t sT = tr ? sA : sB, sG = tr ? sB : sA;
-                const uint32_t T_SLICE = tr ? A_SLICE : B_SLICE, G_SLICE = tr ? B_SLICE : A_SLICE;
                 if (ptid == 0) {
                     // the slices of one K block of the tile: one contiguous, already swizzled piece
-                    tc::mbar_arrive_expect_tx(full0 + 8 * s, a.slices * T_SLICE);
+                    tc::mbar_arrive_expect_tx(full0 + 8 * s, a.slices * B_SLICE);
                     const size_t tile = ((size_t)cfg * a.nchunks + x.rc) * nkb + kb;
-                    tc::bulk_copy_g2s(sT, reinterpret_cast<const char*>(a.tab) + tile * (kSlices * T_SLICE),
-                                      a.slices * T_SLICE, full0 + 8 * s);
+                    tc::bulk_copy_g2s(sB, reinterpret_cast<const char*>(a.tab) + tile * (kSlices * B_SLICE),
+                                      a.slices * B_SLICE, full0 + 8 * s);
                 }
                 // a warp instruction covers 8 rows x 64 bytes of one slice: 512 contiguous bytes of
                 // shared memory (no bank conflicts) from eight 64-byte pieces of global memory
@@ -273,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
                     const int src = s_src[m];
                     const bf16* gp =
                         a.asl + (((size_t)(src < 0 ? 0 : src) * nkb + kb) * kSlices + sl_i) * kKBlock + ch * 8;
-                    const uint32_t dst = sG + sl_i * G_SLICE + m * 64 + ((ch ^ ((m >> 1) & 3)) << 4);
+                    const uint32_t dst = sA + sl_i * A_SLICE + m * 64 + ((ch ^ ((m >> 1) & 3)) << 4);
                     tc::cp_async16(dst, gp, src < 0 ? 0u : 16u);
                 }
                 // the stage's full barrier gets this thread's arrival when its copies have landed
@@ -377,31 +371,18 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
             if (!ok) break;
             float2* outp = a.split > 1 ? a.out + (size_t)x.sp * a.part_stride : a.out;
             const int m = quad * 32 + lane;  // TMEM lane
-            const int r0 = x.rc * (tr ? kTileM : N);
-            if (tr) {
-                // lane = table row r0 + m, columns = targets half * HALF + j of the group
-                const int row = r0 + m;
+            const int r0 = x.rc * N;
+            // lane = target m of the group, columns = table rows r0 + half * HALF + j
+            const int tgt = a.gtgt[(size_t)x.g * G + m];
+            if (tgt >= 0) {
+                float4* o = reinterpret_cast<float4*>(outp + (size_t)tgt * a.Rp + r0 + half * HALF);
 #pragma unroll
-                for (int j = 0; j < HALF; ++j) {
-                    const int tgt = a.gtgt[(size_t)x.g * G + half * HALF + j];
-                    if (tgt < 0) continue;
-                    const float h = __fadd_rn(hi[j], lo[j]);
-                    const float l = __fsub_rn(lo[j], __fsub_rn(h, hi[j]));
-                    outp[(size_t)tgt * a.Rp + row] = make_float2(h, l);
-                }
-            } else {
-                // lane = target m of the group, columns = table rows r0 + half * HALF + j
-                const int tgt = a.gtgt[(size_t)x.g * G + m];
-                if (tgt >= 0) {
-                    float4* o = reinterpret_cast<float4*>(outp + (size_t)tgt * a.Rp + r0 + half * HALF);
-#pragma unroll
-                    for (int j = 0; j < HALF / 2; ++j) {
-                        float h0 = __fadd_rn(hi[2 * j], lo[2 * j]);
-                        float l0 = __fsub_rn(lo[2 * j], __fsub_rn(h0, hi[2 * j]));
-                        float h1 = __fadd_rn(hi[2 * j + 1], lo[2 * j + 1]);
-                        float l1 = __fsub_rn(lo[2 * j + 1], __fsub_rn(h1, hi[2 * j + 1]));
-                        o[j] = make_float4(h0, l0, h1, l1);
-                    }
+                for (int j = 0; j < HALF / 2; ++j) {
+                    float h0 = __fadd_rn(hi[2 * j], lo[2 * j]);
+                    float l0 = __fsub_rn(lo[2 * j], __fsub_rn(h0, hi[2 * j]));
+                    float h1 = __fadd_rn(hi[2 * j + 1], lo[2 * j + 1]);
+                    float l1 = __fsub_rn(lo[2 * j + 1], __fsub_rn(h1, hi[2 * j + 1]));
+                    o[j] = make_float4(h0, l0, h1, l1);
                 }
             }
         }
@@ -412,7 +393,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_gemm_kernel(SplitArgs a) {
         // after an abort (a bounded wait ran out somewhere): wait, with a longer bound, for the work
         // still in flight, so that no copy writes this CTA's shared memory and no MMA its
         // accumulators once they are released. Units may have been started that no MMA consumed
-        // (their table tiles come by TMA; the cp.async rows are complete after cp.async.wait_all),
+        // (their table tiles come by bulk copies; the cp.async rows are complete after cp.async.wait_all),
         // and MMAs issued before the abort may still run.
         const volatile int never = 0;
         if (tid == kEpilogueThreads)
@@ -439,7 +420,7 @@ int mixed_prepare(vfmm_ops* o, cudaStream_t st) {
     const int kk = o->k * o->k;
     const int R = 3 * kk;
     mo->N = kTileN;
-    const int tile_rows = table_rows_per_tile(near_transposed(o->k));
+    const int tile_rows = kTileN;
     mo->Rp = (R + tile_rows - 1) / tile_rows * tile_rows;
     mo->Kp = (kk + kKBlock - 1) / kKBlock * kKBlock;
     if (near_by_classes(o->k)) {
@@ -472,8 +453,8 @@ void mixed_free(vfmm_ops* o) {
 }
 
 int build_split_plan(const PlanItems& I, const std::vector<int32_t>& order, int n_tables, int n_chunks, int R,
-                     bool transposed, int nkb, PlanArena& A, SplitPlan* P) {
-    const int G = transposed ? kTileN : kTileM;  // targets per group
+                     int nkb, PlanArena& A, SplitPlan* P) {
+    constexpr int G = kTileM;  // targets per group
     // target t stands for the R consecutive virtual targets t * R + r, whose gathered rows are
     // src * R + r: the right-hand sides of one target share its set of tables
     const int nt0 = (int)I.tgt.size();
@@ -507,8 +488,6 @@ int build_split_plan(const PlanItems& I, const std::vector<int32_t>& order, int 
     }
     P->n_groups = ng;
     P->entries = (int64_t)gcfg.size();
-    P->transposed = transposed;
-    P->group = G;
     {
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
@@ -571,12 +550,12 @@ static std::vector<int32_t> key_order(const PlanItems& I) {
     return order;
 }
 
-int build_contraction_plan(const PlanItems& I, int n_tables, int n_chunks, int R, bool transposed, int nkb,
+int build_contraction_plan(const PlanItems& I, int n_tables, int n_chunks, int R, int nkb,
                            double slab_overhead, size_t slab_row_bytes, PlanArena& A, SplitPlan* P) {
     constexpr size_t kMaxSlabBytes = size_t(256) << 20;
-    VFMM_CHECK(build_split_plan(I, key_order(I), n_tables, n_chunks, R, transposed, nkb, A, P));
+    VFMM_CHECK(build_split_plan(I, key_order(I), n_tables, n_chunks, R, nkb, A, P));
     const int nt = (int)I.tgt.size();
-    const int64_t G = P->group;
+    constexpr int64_t G = kTileM;
     const int64_t n_entries = (int64_t)I.tab.size();
     std::vector<int64_t> per_table(n_tables + 1, 0);
     for (int64_t e = 0; e < n_entries; ++e) ++per_table[I.tab[e] + 1];
@@ -609,7 +588,7 @@ int build_contraction_plan(const PlanItems& I, int n_tables, int n_chunks, int R
     }
     seg[nt] = (int32_t)n_entries;
     SplitPlan* E_plan = new SplitPlan();
-    int rc = build_split_plan(E, e_order, n_tables, n_chunks, R, transposed, nkb, A, E_plan);
+    int rc = build_split_plan(E, e_order, n_tables, n_chunks, R, nkb, A, E_plan);
     if (rc == VFMM_OK) {
         E_plan->entry = true;  // the slab occupies the partial-sum buffer: no split-K
         E_plan->may_split = false;
@@ -719,9 +698,8 @@ int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, 
         if (ev) VFMM_CUDA(cudaEventRecord(ev[1], st));
         return VFMM_OK;
     }
-    const int tile_rows = table_rows_per_tile(P.transposed, Rp);
+    const int tile_rows = table_rows_per_tile(Rp);
     if (Kp % kKBlock || Rp % tile_rows) return fail(VFMM_ERR_INTERNAL, "split GEMM shape not tiled");
-    const int n_mma = mma_n(P.transposed, Rp);
     SplitArgs a;
     a.asl = (const bf16*)asl;
     a.tab = (const bf16*)tables;
@@ -733,7 +711,6 @@ int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, 
     a.Kp = Kp;
     a.Rp = Rp;
     a.nchunks = Rp / tile_rows;
-    a.transposed = P.transposed ? 1 : 0;
     a.slices = slices;
     // Per K value the slice products of an exact diagonal (d <= 4) sum to at most
     // 2 * 128 * 64 + 3 * 64^2 = 28672 units (balanced digits), so those accumulators stay exact while
@@ -747,7 +724,7 @@ int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, 
         a.part_stride = 0;
         a.out = part;
         a.n_items = P.n_groups * a.nchunks;
-        VFMM_CHECK(launch_split_n(n_mma, a, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
+        VFMM_CHECK(launch_split_n(tile_rows, a, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
         // deferred: the consumer sums each target's slab rows itself (same order)
         const int64_t n = (defer & kDeferSegments) ? 0 : (int64_t)P.n_seg * P.R * Rp;
         if (n > 0)
@@ -761,11 +738,11 @@ int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, 
     a.part_stride = n_out_rows * (size_t)Rp;
     a.out = a.split > 1 ? part : out;
     a.n_items = P.n_groups * a.split * a.nchunks;
-    VFMM_CHECK(launch_split_n(n_mma, a, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
+    VFMM_CHECK(launch_split_n(tile_rows, a, P.ctas > 0 ? std::min(P.ctas, a.n_items) : a.n_items, st));
     if (a.split > 1 && !(defer & kDeferSplits)) {
-        const int64_t n = (int64_t)P.n_groups * P.group * Rp;
+        const int64_t n = (int64_t)P.n_groups * kTileM * Rp;
         split_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part, a.part_stride, a.split, P.tgt,
-                                                                          P.n_groups * P.group, Rp, out);
+                                                                          P.n_groups * kTileM, Rp, out);
         VFMM_CUDA(cudaGetLastError());
     }
     if (ev) VFMM_CUDA(cudaEventRecord(ev[1], st));
@@ -793,10 +770,8 @@ static int build_near_plan(const DeviceTree& T, int R, const HostLists& H, PlanA
         I.close(t, sig, (uint64_t)t);
     }
     const int rows = 3 * T.k * T.k;
-    const bool tr = near_transposed(T.k);
-    const int tile_rows = table_rows_per_tile(tr);
     const int Kp = (T.k * T.k + kKBlock - 1) / kKBlock * kKBlock;
-    return build_contraction_plan(I, kNearCfg, (rows + tile_rows - 1) / tile_rows, R, tr, Kp / kKBlock, 48.0 / Kp,
+    return build_contraction_plan(I, kNearCfg, (rows + kTileN - 1) / kTileN, R, Kp / kKBlock, 48.0 / Kp,
                                   (size_t)rows * sizeof(float2), A, &PS->entries);
 }
 

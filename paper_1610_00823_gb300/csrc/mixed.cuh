@@ -32,21 +32,9 @@ constexpr int kThreads = 32 * (kMmaWarp + 1);                     // 384: 3 warp
 constexpr int kMaxSplit = 16;  // largest split-K factor (partial sums held for small contractions only)
 static_assert(kNumAcc * kTileN <= kTmemCols, "TMEM budget");
 
-// Orientation of the near-field and leaf far-field contractions: with 3k^2 a multiple of 128
-// (k = 16) the table rows are the M side (128 per tile, TMA) and the targets the N side (80 per
-// group, gathered), which gathers 40 % fewer bytes; otherwise targets are the M side (128 per group)
-// and table rows the N side (80 per tile). M2L, S2L and S2M (2p rows) always use the latter.
-__host__ __device__ constexpr bool near_transposed(int k) { return (3 * k * k) % kTileM == 0; }
-// Table rows per tile of a contraction whose tables have Rp rows: 128 (transposed), else 80, or 48
-// for the 48-row tables of small expansions.
-__host__ __device__ constexpr int table_rows_per_tile(bool transposed, int Rp = kTileN) {
-    return transposed ? kTileM : (Rp % kTileN == 0 ? kTileN : kTileNSmall);
-}
-// N of the MMAs (TMEM columns per accumulator): the gathered targets (80) when transposed, else the
-// table rows per tile.
-__host__ __device__ constexpr int mma_n(bool transposed, int Rp) {
-    return transposed ? kTileN : table_rows_per_tile(false, Rp);
-}
+// Table rows per tile (the MMA's N, TMEM columns per accumulator) of a gathered contraction whose tables have
+// Rp rows: 80, or 48 for the 48-row tables of small expansions. The targets are its M side, 128 per group.
+__host__ __device__ constexpr int table_rows_per_tile(int Rp) { return Rp % kTileN == 0 ? kTileN : kTileNSmall; }
 
 // Splits v / 2^E (|v| < 2^E) into kSlices balanced base-128 digits, out[(i - 1) * stride] =
 // d_i 2^(-7 i), with v / 2^E = sum_i d_i 2^(-7 i) + (|v| 2^(56 - E) - floor(|v| 2^(56 - E))) 2^-56:
@@ -76,12 +64,6 @@ __device__ __forceinline__ void slice_fixed(double v, int E, __nv_bfloat16* out,
         const float s = (float)(neg ? -d : d) * __int_as_float((127 - 7 * i) << 23);
         out[(i - 1) * stride] = __float2bfloat16_rn(s);
     }
-}
-
-// 2^e as a double built from its exponent bits (e clamped to the normal range).
-__device__ __forceinline__ double pow2(int e) {
-    e = max(-1022, min(1023, e));
-    return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
 // (double)x * 2^e for a float x from the bits, with integer operations only (the FP64 units are
@@ -323,16 +305,16 @@ struct PlanItems {
         key.push_back({k0, k1});
     }
 };
-// Groups of 128 (80 when transposed) targets taken in the given order; per group the tables present
+// Groups of 128 targets taken in the given order; per group the tables present
 // and, per table, the gathered row of each target (-1 when the target has no entry for that table).
 int build_split_plan(const PlanItems& I, const std::vector<int32_t>& order, int n_tables, int n_chunks, int R,
-                     bool transposed, int nkb, PlanArena& A, SplitPlan* P);
+                     int nkb, PlanArena& A, SplitPlan* P);
 // build_split_plan, or its entry-major form when that executes enough fewer columns: chosen when
 // (entry-major columns) x (1 + slab_overhead) < 0.85 x (grouped columns, padding included) and the
 // slab (entries x R x slab_row_bytes) stays within 256 MB. slab_overhead = the slab's write and read
 // time per column relative to its tensor time. A small contraction (fewer CTAs than two per SM)
 // whose slab fits keeps the form not chosen in P->alt.
-int build_contraction_plan(const PlanItems& I, int n_tables, int n_chunks, int R, bool transposed, int nkb,
+int build_contraction_plan(const PlanItems& I, int n_tables, int n_chunks, int R, int nkb,
                            double slab_overhead, size_t slab_row_bytes, PlanArena& A, SplitPlan* P);
 // ev (optional): a (start, stop) event pair recorded around the contraction and its reduction.
 int split_gemm(const SplitPlan& P, const void* asl, const void* tables, int Kp, int Rp, float2* out, int* err,

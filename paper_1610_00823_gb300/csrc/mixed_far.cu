@@ -89,7 +89,7 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
     const int R = 3 * kk;
     mo->Kx = (2 * P + kKBlock - 1) / kKBlock * kKBlock;
     mo->Rx = 2 * p <= kTileNSmall ? kTileNSmall : (2 * p + kTileN - 1) / kTileN * kTileN;
-    const int rx_tile = table_rows_per_tile(false, mo->Rx);
+    const int rx_tile = table_rows_per_tile(mo->Rx);
     const double inv2pi = 1.0 / (2.0 * 3.14159265358979323846);
     // S2M rows 2..2p+1 (coefficients 1..p)
     std::vector<double> s2m((size_t)2 * P * kk);
@@ -167,7 +167,7 @@ int far_prepare(vfmm_ops* o, cudaStream_t st) {
     if (near_by_classes(k)) {
         VFMM_CHECK(leaf_classes_prepare(o, F, st));
     } else {
-        VFMM_CHECK(slice_table(F, 1 + kFarCfg, R, KX, mo->Rp, table_rows_per_tile(near_transposed(o->k)), mo->Kx,
+        VFMM_CHECK(slice_table(F, 1 + kFarCfg, R, KX, mo->Rp, kTileN, mo->Kx,
                                &mo->far_sl, &mo->far_E, st));
     }
     // S2L: rows 2..2p+1 (Re, Im of coefficients 1..p) over the k*k source values; row 0 kept in FP64
@@ -300,15 +300,15 @@ int build_far_plan(int which, const DeviceTree& T, int R, const HostLists& H, Pl
             }
             std::vector<int32_t> order(nl);
             for (int t = 0; t < nl; ++t) order[t] = t;
-            return build_split_plan(I, order, 1, 1, R, false, Kp / kKBlock, A, &PS->s2m);
+            return build_split_plan(I, order, 1, 1, R, Kp / kKBlock, A, &PS->s2m);
         }
         case kCtrM2L:  // boxes with a V list, tables = the 40 offsets, gathered row = source box
             list_items(VFMM_LIST_V, false, &I);
             // slab costs relative to the tensor work per column: K = 2(p+1) padded (about 96), rows <= 128
-            return build_contraction_plan(I, kVCfg, 1, R, false, kFarKb, 0.5, 128 * sizeof(float2), A, &PS->m2l);
+            return build_contraction_plan(I, kVCfg, 1, R, kFarKb, 0.5, 128 * sizeof(float2), A, &PS->m2l);
         case kCtrS2L:  // boxes with an X list, tables 20 configurations, gathered row = source leaf
             list_items(VFMM_LIST_X, true, &I);
-            return build_contraction_plan(I, kFarCfg, 1, R, false, Kp / kKBlock, 48.0 / Kp, 128 * sizeof(float2), A,
+            return build_contraction_plan(I, kFarCfg, 1, R, Kp / kKBlock, 48.0 / Kp, 128 * sizeof(float2), A,
                                           &PS->s2l);
         case kCtrFar: {  // leaf far field: slot 0 = own local (L2T), slot 1 + j = j-th W entry (table 1 + its configuration)
             const std::vector<int32_t>& ptr = H.ptr[VFMM_LIST_W];
@@ -326,9 +326,7 @@ int build_far_plan(int which, const DeviceTree& T, int R, const HostLists& H, Pl
                 I.close(t, sig, (uint64_t)t);
             }
             const int rows = 3 * T.k * T.k;
-            const bool tr = near_transposed(T.k);
-            const int tile_rows = table_rows_per_tile(tr);
-            return build_contraction_plan(I, 1 + kFarCfg, (rows + tile_rows - 1) / tile_rows, R, tr, kFarKb, 0.5,
+            return build_contraction_plan(I, 1 + kFarCfg, (rows + kTileN - 1) / kTileN, R, kFarKb, 0.5,
                                           (size_t)rows * sizeof(float2), A, &PS->far);
         }
         default:
@@ -574,11 +572,10 @@ extern "C" int vfmm_solve_work(const vfmm_tree* tree, const vfmm_ops* ops, int32
     if (ops->precision != VFMM_MIXED || !mo) return VFMM_OK;
     const PlanSet* PS = nullptr;
     VFMM_CHECK(plans_for(T, nrhs, &PS));
-    // per table of a tile and per K value: S (S + 1) / 2 products of 128 x 80 MACs
+    // per table of a tile and per K value: S (S + 1) / 2 products of 128 x (80 or 48) MACs
     auto tc = [&](const SplitPlan& P, int Kp, int Rp, int ctr) {
         const int S = mo->slices[ctr];
-        return 2.0 * (double)P.entries * (Rp / table_rows_per_tile(P.transposed, Rp)) * (double)Kp * (S * (S + 1) / 2) *
-               kTileM * mma_n(P.transposed, Rp);
+        return 2.0 * (double)P.entries * Rp * (double)Kp * (S * (S + 1) / 2) * kTileM;
     };
     if (!near_by_classes(ops->k)) {
         out[0] = tc(PS->entries, mo->Kp, mo->Rp, kCtrNear);

@@ -166,8 +166,6 @@ struct SplitPlan {
     int32_t split = 1;       // CTAs per group (each takes a share of the group's tables)
     int32_t ctas = 0;        // CTA cap of the launch (persistent CTAs walk several work items); 0: one CTA per item
     bool may_split = false;  // small contraction (fewer CTAs than two per SM): split-K allowed
-    bool transposed = false; // table rows on the M side (128 per tile), targets on the N side
-    int32_t group = 128;     // targets per group: 128, or 80 when transposed
     // Entry-major form: every (target, table) entry is a column of its own, grouped by table, so
     // no column is empty; the contraction writes one slab row per entry (in the partial-sum
     // buffer) and a segmented reduction sums each target's entries into its output row.
