@@ -128,24 +128,14 @@ static int sm_count() {
     return n > 0 ? n : 1;
 }
 
-// ---------------------------------------------------------------- downward pass (one CTA per box)
+// ---------------------------------------------------------------- a box's own terms of the downward pass
 struct DownArgs {
-    int begin, end, P, kk, level;
-    int R, nleaf;  // right-hand sides folded into the box rows (virtual box = box * R + r); leaves
+    int P, R;  // R right-hand sides folded into the box rows (virtual box = box * R + r)
     double width;
     LevelLogs logs;
-    const int32_t* parent;
-    const int32_t* ix;
-    const int32_t* iy;
-    const int32_t *vptr, *vidx, *vcfg;
-    const int32_t *xptr, *xidx, *xcfg;
-    const int32_t* leaf_of_box;
-    const double* l2l_t;
-    const double* m2l_t;
-    const double* s2l_t;
+    const int32_t *vptr, *vidx;
+    const int32_t *xptr, *xidx;
     const double* Mexp;
-    const double* f;
-    double* Lexp;
     // split-precision M2L rows 2..2p+1 (null in the FP64 form): (hi, lo) scaled by 2^-E[level][r]
     const float2* m2l_out;
     // split-K M2L: its partial sums [split][n_boxes * R][Rx], summed here when m2l_split > 1 (the
@@ -350,7 +340,6 @@ struct PassArgs {
     const int32_t* child0;
     const double* tab;     // the real triangular matrix of the rotated form, [in][out]
     double2* ex;           // Mexp (upward) or Lexp (downward), [n_boxes * R][P] complex
-    const int32_t* parent;
     unsigned int* ready;   // [n_boxes * R] readiness counters, zero at launch
     unsigned* glev;        // upward pass, mixed form: biased level exponents of the M2L operand (or null)
     const int32_t* level;
@@ -964,36 +953,19 @@ static inline void mark(StageEvents* se, int stage, bool stop, cudaStream_t st) 
     if (se) cudaEventRecord(se->ev[2 * stage + (stop ? 1 : 0)], st);
 }
 
-static void fill_down_args(DownArgs& d, const DeviceTree& T, const vfmm_ops& o, const double* f, const Workspace& w,
-                           int l, int R) {
+static void fill_down_args(DownArgs& d, const DeviceTree& T, const vfmm_ops& o, const Workspace& w, int R) {
     const MixedOps* mo = (const MixedOps*)o.mixed;
     d.R = R;
-    d.nleaf = T.n_leaves;
     d.wm = 2.0 * std::frexp(T.width, &d.lw);
     d.lw -= 1;
-    d.begin = T.level_start[l];
-    d.end = T.level_start[l + 1];
     d.P = o.p + 1;
-    d.kk = o.k * o.k;
-    d.level = l;
     d.width = T.width;
     d.logs = level_logs(T.width);
-    d.parent = T.parent;
-    d.ix = T.ix;
-    d.iy = T.iy;
     d.vptr = T.lptr[VFMM_LIST_V];
     d.vidx = T.lidx[VFMM_LIST_V];
-    d.vcfg = T.lcfg[VFMM_LIST_V];
     d.xptr = T.lptr[VFMM_LIST_X];
     d.xidx = T.lidx[VFMM_LIST_X];
-    d.xcfg = T.lcfg[VFMM_LIST_X];
-    d.leaf_of_box = T.leaf_of_box;
-    d.l2l_t = o.l2l_t;
-    d.m2l_t = o.m2l_t;
-    d.s2l_t = o.s2l_t;
     d.Mexp = w.Mexp;
-    d.f = f;
-    d.Lexp = w.Lexp;
     d.vslab = w.vslab;
     d.xslab = w.xslab;
     d.viptr = T.inst_ptr[VFMM_LIST_V];
@@ -1196,7 +1168,6 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         pa.child0 = T.child0;
         pa.tab = o.m2m_r;
         pa.ex = reinterpret_cast<double2*>(w.Mexp);
-        pa.parent = T.parent;
         pa.ready = w.ready;
         pa.glev = mixed ? w.mix.glev : nullptr;
         pa.level = T.level;
@@ -1281,7 +1252,7 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
     }
     if (T.depth >= 2) {
         DownArgs d;
-        fill_down_args(d, T, o, f, w, 2, R);
+        fill_down_args(d, T, o, w, R);
         PassArgs pa;
         pa.depth = T.depth;
         pa.R = R;
@@ -1292,7 +1263,6 @@ static int solve_steps(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o
         pa.child0 = T.child0;
         pa.tab = o.l2l_r;
         pa.ex = reinterpret_cast<double2*>(w.Lexp);
-        pa.parent = T.parent;
         pa.ready = w.ready + (size_t)T.n_boxes * R;
         pa.glev = nullptr;
         pa.level = T.level;
@@ -1466,7 +1436,6 @@ static const char* status_site(int code) {
         case 2: return "the tensor-core MMA issuer waiting for operands";
         case 3: return "a tensor-core epilogue waiting for its accumulators";
         case 4: return "the tensor-core MMA issuer waiting for drained accumulators";
-        case 5: return "a translation-table copy into shared memory";
         case 6: return "a persistent tree pass waiting for an expansion another unit writes";
         case 7: return "the failure-path self-test's wait on an mbarrier nothing arrives on (expected)";
         default: return "an unknown site";
