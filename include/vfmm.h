@@ -236,9 +236,11 @@ int vfmm_ops_destroy(vfmm_ops* ops);
  * base-128 digits (56 bits below its power-of-two scale); a contraction that takes S of them
  * (6 <= S <= 8) issues the S (S + 1) / 2 slice products i + j <= S + 1 and rounds each operand at
  * 2^(-7 S - 1) of its scale: fewer tensor-core products and fewer gathered bytes, less accuracy.
+ * (In the reflection classes of k >= 6 an operand is a sum of up to four values under twice their scale; its last
+ * slice holds what the digits before it leave, to 1/8 of that digit's unit, so a value is rounded no more coarsely.)
  * slices[5] = near field, S2M, M2L, S2L, leaf far field (L2T + M2T; one more is taken for k >= 6, where it
  * runs in the reflection classes of the square); a new operator set takes 6
- * for all, the fewest allowed: the error against the FP64 form stays at or below 6e-12 on the
+ * for all, the fewest allowed: the error against the FP64 form stays at or below 3e-12 on the
  * adaptive 20-Gaussian (k = 16, p = 40), kinked and uniform depth-7 (k = 16) workloads.
  * Host-only; applies to later calls and graph captures (a graph keeps the counts it captured); not
  * while a solve with these operators is being launched. Errors: INVALID_ARG (null pointer, not
@@ -271,6 +273,9 @@ int vfmm_ops_get_m2l(const vfmm_ops* ops, int32_t* form, int32_t* n_waves);
 /* Device workspace the solve needs for this tree, operator set and nrhs
  * (multipole and local expansions, near-field partial products). with_io != 0
  * adds room for the device copies vfmm_volume_potential_host stages through.
+ * VFMM_MIXED with k >= 6 also holds the operand tiles of the near field and of the leaf far field: all of them up
+ * to 768 MB each, beyond that they take turns (k = 16, p = 40: 8 MB for 64 uniform leaves, 0.35 GB for 4,096,
+ * 1.3 GB for 16,384, 2.8 GB for 50,000 graded ones).
  * VFMM_MIXED with nrhs > 1 builds (once per tree and nrhs, host-side, cached in the
  * tree under a lock) the contraction schedules with the right-hand sides folded in. */
 int vfmm_workspace_size(const vfmm_tree* tree, const vfmm_ops* ops, int32_t nrhs, int32_t with_io,

@@ -358,8 +358,8 @@ int leaf_class_bounds(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o,
 int leaf_class_contract(const DeviceTree& T, const PlanSet& PS, const vfmm_ops& o, const double* Mexp, const double* Lexp,
                         const MixedWork& w, cudaStream_t st);
 // Slices that the leaf far field takes in reflection classes: one more than set. A node's images share the
-// rounding of the largest of them, which cost 1.7 times the error of the gathered form at the same count
-// (1,378 leaves, largest of u_x: 6.7e-12 against 3.0e-12); with one more it is 1.4e-12, for 3 % of a solve.
+// rounding of the largest of them. On 1,219 leaves its error is 2.3e-12 of the largest u_x at 6 slices
+// (gathered form: 3.0e-12) and 2.4e-14 at 7, on 200,104 leaves 4.2e-12 (5.2e-12) and 4.1e-14, for 3 % of a solve.
 inline int leaf_class_slices(const MixedOps& mo) { return mo.slices[kCtrFar] < kSlices ? mo.slices[kCtrFar] + 1 : kSlices; }
 int class_launches(const ClassTab& ct, const ClassPlan& P, int S, size_t opnd_bytes);
 int far_prepare(vfmm_ops* o, cudaStream_t st);

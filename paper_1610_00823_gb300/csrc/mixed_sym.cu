@@ -12,8 +12,8 @@
 //    large as 256, which BF16 holds. What this costs an orbit with a single member, its last slice makes up
 //    for: not a whole digit but all that is left, rounded to BF16 (at most 1/8 of the digit's unit).
 //  * a table row's scale is half its largest entry's power of two (top digits up to 256) wherever the entries of
-//    a K block are on average no larger than that scale (all but some 4 % of the rows): half the weight of
-//    the slice products left out. Per K value diagonals 0 to 4 then sum to at most 36,864 units, 448 of
+//    a K block are on average no larger than that scale (755 of the near field's 768 rows at k = 16): half the
+//    weight of the slice products left out. Per K value diagonals 0 to 4 then sum to at most 36,864 units, 448 of
 //    them below 2^24: diagonal 0 to 256 x 128 (the table's average), diagonal 4 to 256 x 64 + 3 x 64^2
 //    + 64 x 128. The sixth accumulator (diagonals from 5 on, 40,960 units at S = 6) may round by 2^-49 of
 //    the scales' product where its sum is past 2^24 units, 1/400 of what the products left out may weigh.
@@ -27,9 +27,10 @@
 // What bounds it: a K block of 128 x 64 outputs moves 207 KB through shared memory (72 KB written, the A
 // tiles once, the B tiles once per product), 1,620 cycles; the MMAs take 1,700 of the 2,220 cycles measured,
 // 300 go to operands not yet there and 220 to drains. The operand is bound by HBM writes and integer work.
-// Against gathered rows and plain tables (ms): 200,104 graded leaves 13.3 -> 8.0, 16,384 uniform leaves
+// Against gathered rows and plain tables (ms): 200,104 graded leaves 13.3 -> 8.1, 16,384 uniform leaves
 // k = 16 1.32 -> 0.39, 1,378 graded leaves 0.18 -> 0.11, 4,096 rows of k = 8 0.081 -> 0.034; the far field of
-// the 200,104 leaves 4.1 -> 1.9 and its error at the nodes of 1,378 leaves 3.0e-12 -> 1.4e-12 of the largest u_x.
+// the 200,104 leaves 4.1 -> 1.9. Error against the FP64 form at 6 slices, largest of u_x: near field on 1,219
+// graded leaves 3.5e-12 -> 1.7e-12, far field (7 slices here) 3.0e-12 -> 2.4e-14.
 // k <= 5 keeps the gathered rows: its class rows fill half a tile of 48.
 #include <cuda_bf16.h>
 

@@ -372,9 +372,10 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
 }
 
 // Next to a corner Q_n grows like -log(r)/2 on both its edges. The parts cancel, since the two series have one
-// value there, but only to a rounding of each times the logarithm (u_x of one leaf, k = 16, width 1/4, random
-// values of size 1, against extended precision: 1e-13 at r = 1e-10, 3e-13 at 1e-100; now 8e-15 at any r). So the conjugate gradient at the corner, C, is taken off all four edges, and its own
-// integral around the leaf, -2 pi C inside and 0 outside, is put back.
+// value there, but only to a rounding of each times the logarithm. So the conjugate gradient at the corner, C,
+// is taken off all four edges, and its own integral around the leaf, -2 pi C inside and 0 outside, is put back
+// (u_x of one leaf, k = 16, width 1/4, random values of size 1, against extended precision: 1e-13 -> 8e-15 at
+// r = 1e-10, 3e-13 -> 8e-15 at 1e-100).
 // An edge with the corner at its end sg = 1 or start sg = -1: sum over n of (T_n + i g_n)(Q_n - sg^n Q_0). With
 // S_n = sg^n Q_n - Q_0, D_n = S_(n+1) - S_n and delta = 1 - sg z the three-term recurrence reads
 //   D_n = (n D_(n-1) - (2n + 1) delta (S_n + Q_0)) / (n + 1),   D_0 = -sg - delta Q_0,

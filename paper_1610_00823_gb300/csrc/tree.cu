@@ -1061,7 +1061,7 @@ static int finalize(std::vector<DBuf<uint32_t>>& keys, std::vector<int64_t>& cnt
     VFMM_CHECK(compute_lists(T, st));
     VFMM_CUDA(cudaStreamSynchronize(st));
     {
-        // non-leaf boxes per level (for the per-level M2M and L2L GEMMs)
+        // non-leaf boxes per level (units of the M2M and L2L passes)
         std::vector<int32_t> c0(n);
         VFMM_CUDA(cudaMemcpy(c0.data(), T->child0, n * sizeof(int32_t), cudaMemcpyDeviceToHost));
         std::vector<int32_t> nl;
