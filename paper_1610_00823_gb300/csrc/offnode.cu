@@ -239,13 +239,21 @@ struct OffArgs {
 
 // A U leaf as seen from the point, unit-box coordinates: distances to its sides (left, right, bottom,
 // top), positive inwards. On a side (all >= 0, some 0) the point counts as inside, by an amount that the
-// arithmetic of the edges cannot see. Distances below 1e-150 of the width count as 0 (kOffOnEdge): of a point
-// that near to a corner from outside, the sum of the squares would underflow and its logarithm be infinite.
-constexpr double kOffOnEdge = 1e-150;
+// arithmetic of the edges cannot see. Distances below 2^-498 (1.2e-150) of the width count as 0 (kOffOnEdge): of
+// a point that near to a corner from outside, the sum of the squares would underflow and its logarithm be
+// infinite. Both lines are drawn by exponents: a comparison in FP64 takes a warp as long as an addition.
+constexpr int kOffOnEdge = 1023 - 498;
+constexpr int kOffCorner = 1023 - 10;  // within 2^-10 of the leaf's width; both edges' recurrences then run upwards
+// -d where `on` (bit 0), on the bits.
+__device__ __forceinline__ double off_flip(double d, int on) {
+    return __hiloint2double(__double2hiint(d) ^ (on << 31), __double2loint(d));
+}
+__device__ __forceinline__ int off_exp(double d) { return (__double2hiint(d) >> 20) & 0x7FF; }
 struct OffLeaf {
     double d[4];
     double h;
     int leaf, inside;
+    int corner;  // c where edge c starts, if the point is next to it, or -1
 };
 
 // sum over this thread's values v of the table columns, for NU leaves: cf[row][u] = sum_v G[v][row] fs[v][u]
@@ -380,7 +388,7 @@ __device__ __forceinline__ void edge_terms(double w1, double w2, double zi, cons
 // S_n = sg^n Q_n - Q_0, D_n = S_(n+1) - S_n and delta = 1 - sg z the three-term recurrence reads
 //   D_n = (n D_(n-1) - (2n + 1) delta (S_n + Q_0)) / (n + 1),   D_0 = -sg - delta Q_0,
 // in which z, whose last bit the derivative of P_n blows up by n^2, stands no more.
-__device__ __noinline__ double2 edge_corner(double w1, double w2, double zi, double sg, const double* g, const double* T,
+__device__ __forceinline__ double2 edge_corner(double w1, double w2, double zi, double sg, const double* g, const double* T,
                                             int N, const OffStep* __restrict__ C) {
     const EdgeLog lg = edge_log(w1, w2, zi);
     const double qr = 0.5 * lg.dl, qi = 0.5 * lg.ang;
@@ -401,7 +409,42 @@ __device__ __noinline__ double2 edge_corner(double w1, double w2, double zi, dou
     }
     return make_double2(Br, Bi);
 }
-constexpr double kOffCorner = 1e-3;  // of the leaf's width; both edges' recurrences then run upwards
+
+// The warp's edges (lanes 4 u + s) with the corner taken off where their leaf has one next to the point (corner >= 0):
+// (Re Phi', Im Phi') of this lane's edge, `own` without. A call of its own: rare, and the kernel keeps its registers.
+__device__ __noinline__ double2 corner_edges(double w1, double w2, double zi, int s, int corner, bool inside, const double* g,
+                                             const double* T, int N, const OffStep* __restrict__ C, double2 own) {
+    const double tr = s == 0 ? 1.0 : (s == 2 ? -1.0 : 0.0), ti = s == 1 ? -1.0 : (s == 3 ? 1.0 : 0.0);
+    double cr = 0.0, ci = 0.0;  // C, from the edge that starts there
+    if (s == corner) {
+        double fr = 0.0, fi = 0.0;
+        for (int n = N - 1; n >= 0; --n) {  // T + i g at the start, P_n = (-1)^n there
+            fr = T[n * kOffTasks] - fr;
+            fi = g[n * kOffTasks] - fi;
+        }
+        cr = tr * fr - ti * fi;
+        ci = tr * fi + ti * fr;
+    }
+    const int from = ((threadIdx.x & 31) & ~3) | max(corner, 0);
+    cr = __shfl_sync(0xffffffffu, cr, from);
+    ci = __shfl_sync(0xffffffffu, ci, from);
+    if (corner < 0) return own;
+    const bool start = s == corner, end = s == ((corner + 3) & 3);
+    if (start || end) {
+        const double2 B = edge_corner(w1, w2, zi, end ? 1.0 : -1.0, g, T, N, C);
+        own = make_double2(2.0 * (tr * B.y + ti * B.x), -2.0 * (tr * B.x - ti * B.y));
+    } else {  // -2 i (sum - C Q_0)
+        const EdgeLog q = edge_log(w1, w2, zi);
+        own.x -= cr * q.ang + ci * q.dl;
+        own.y += cr * q.dl - ci * q.ang;
+    }
+    if (start && inside) {
+        const double two_pi = 6.28318530717958647693;
+        own.x -= two_pi * cr;
+        own.y -= two_pi * ci;
+    }
+    return own;
+}
 
 __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_constant__ OffArgs a) {
     extern __shared__ double off_sm[];
@@ -454,10 +497,13 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
         L.d[2] = (py - y0) / h;
         L.d[3] = (y0 + h - py) / h;
         for (int i = 0; i < 4; ++i)
-            if (fabs(L.d[i]) < kOffOnEdge) L.d[i] = 0.0;
+            if (off_exp(L.d[i]) < kOffOnEdge) L.d[i] = 0.0;
         L.inside = L.d[0] >= 0.0 && L.d[1] >= 0.0 && L.d[2] >= 0.0 && L.d[3] >= 0.0;
         if (L.inside)
             for (int i = 0; i < 4; ++i) L.d[i] = fmax(L.d[i], 1e-30);
+        const int dl = off_exp(L.d[0]), dr = off_exp(L.d[1]), db = off_exp(L.d[2]), dt = off_exp(L.d[3]);
+        L.corner = -1;
+        if (min(dl, dr) < kOffCorner && min(db, dt) < kOffCorner) L.corner = db < dt ? (dl < dr ? 0 : 1) : (dl < dr ? 3 : 2);
         lf[tid] = L;
     }
     __syncthreads();
@@ -525,9 +571,8 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
         // one edge per lane
         const int e = tid;
         double v[3] = {0.0, 0.0, 0.0}, w1 = 0.0, w2 = 0.0, zi = 0.0, hl = 0.0, tr = 0.0, ti = 0.0;
-        int corner = -1;  // c where edge c starts, if the point is next to it
+        int corner = -1;
         const int s = e & 3;
-        bool inside = false;
         if (e < 4 * nu) {
             const OffLeaf L = lf[e >> 2];
             // (end - point, point - start) along the edge, distance inwards
@@ -538,43 +583,13 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
             tr = s == 0 ? 1.0 : (s == 2 ? -1.0 : 0.0);
             ti = s == 1 ? -1.0 : (s == 3 ? 1.0 : 0.0);
             edge_terms(w1, w2, zi, tp + e, tg + e, tt + e, N, a.t.C, log(0.5 * hl), tr, ti, v);
-            const double cx = fmin(fabs(L.d[0]), fabs(L.d[1])), cy = fmin(fabs(L.d[2]), fabs(L.d[3]));
-            if (cx < kOffCorner && cy < kOffCorner) {
-                const bool left = fabs(L.d[0]) < fabs(L.d[1]);
-                corner = fabs(L.d[2]) < fabs(L.d[3]) ? (left ? 0 : 1) : (left ? 3 : 2);
-                inside = L.inside;
-            }
+            corner = L.corner;
         }
         if (__any_sync(0xffffffffu, corner >= 0)) {
-            double cr = 0.0, ci = 0.0;  // C, from the edge that starts there
-            if (s == corner) {
-                double fr = 0.0, fi = 0.0;
-                for (int n = N - 1; n >= 0; --n) {  // T + i g at the start, P_n = (-1)^n there
-                    fr = tt[n * kOffTasks + e] - fr;
-                    fi = tg[n * kOffTasks + e] - fi;
-                }
-                cr = tr * fr - ti * fi;
-                ci = tr * fi + ti * fr;
-            }
-            const int from = (lane & ~3) | max(corner, 0);
-            cr = __shfl_sync(0xffffffffu, cr, from);
-            ci = __shfl_sync(0xffffffffu, ci, from);
-            if (corner >= 0) {
-                const bool start = s == corner, end = s == ((corner + 3) & 3);
-                if (start || end) {
-                    const double2 B = edge_corner(w1, w2, zi, end ? 1.0 : -1.0, tg + e, tt + e, N, a.t.C);
-                    v[1] = 2.0 * (tr * B.y + ti * B.x);
-                    v[2] = -2.0 * (tr * B.x - ti * B.y);
-                } else {  // -2 i (sum - C Q_0)
-                    const EdgeLog q = edge_log(w1, w2, zi);
-                    v[1] -= cr * q.ang + ci * q.dl;
-                    v[2] += cr * q.dl - ci * q.ang;
-                }
-                if (start && inside) {
-                    v[1] -= 2.0 * pi * cr;
-                    v[2] -= 2.0 * pi * ci;
-                }
-            }
+            const double2 w = corner_edges(w1, w2, zi, s, corner, corner >= 0 && lf[e >> 2].inside, tg + e, tt + e, N,
+                                           a.t.C, make_double2(v[1], v[2]));
+            v[1] = w.x;
+            v[2] = w.y;
         }
         v[0] *= hl * hl;
         v[1] *= hl;
@@ -658,16 +673,15 @@ __global__ void __launch_bounds__(kOffThreads, 2) offnode_kernel(const __grid_co
             if (lane < 2) {
                 // 2 x = sg (1 - delta) in [-1, 1]; P_m by its differences, as in edge_corner
                 const double dl = L.d[2 * lane], dr = L.d[2 * lane + 1], delta = 2.0 * fmin(dl, dr);
-                const double sg = dl < dr ? -1.0 : 1.0;
-                double p0 = 1.0, dp = -delta, q0 = 0.0, q1 = 1.0, sn = 1.0;  // sg^m P_m, difference, P_m', P_(m+1)', sg^m
+                const int neg = dl < dr ? 1 : 0;
+                double p0 = 1.0, dp = -delta, q0 = 0.0, q1 = 2.0;  // sg^m P_m, its difference, 2 P_m', 2 P_(m+1)'
                 for (int m = 0; m < N; ++m) {
-                    leg[2 * lane][m] = sn * p0;
-                    leg[2 * lane + 1][m] = 2.0 * q0;
+                    leg[2 * lane][m] = off_flip(p0, m & neg);
+                    leg[2 * lane + 1][m] = q0;
                     const OffStep c = a.t.C[m + 1];
                     p0 += dp;
-                    sn *= sg;
-                    const double q2 = fma((double)(2 * m + 3), sn * p0, q0);
-                    dp = c.w * dp - c.z * (delta * p0);
+                    const double q2 = fma((double)(4 * m + 6), off_flip(p0, (m + 1) & neg), q0);
+                    dp = fma(-(c.z * delta), p0, c.w * dp);  // two operations in the chain
                     q0 = q1;
                     q1 = q2;
                 }
